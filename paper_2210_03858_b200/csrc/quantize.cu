@@ -1,11 +1,22 @@
 // BCQ post-training quantizer (greedy and alternating) and the dequantize helper.
 //
-// One "team" of threads owns one (row, group) problem and keeps the group's residual in
-// registers: thread `tid` of a team of NT threads holds elements e*NT + tid, e < EPT.  A team is
-// one warp for g <= 1024 and a whole CTA above that.  Sums are fp64 and are reduced in a fixed
-// tree order (shuffles inside a warp, then a sequential pass over the per-warp partials), so a
-// result never depends on scheduling.  Sign bits leave the team as __ballot words, which is
-// exactly the container format: 32 consecutive weights of one plane per 32-bit word.
+// One "team" of threads owns one (row, group) problem and keeps its weights in registers.
+//
+// team_quantize_kernel (greedy for every q, alternating for q <= 4): a thread holds up to 32 weights, so
+// a group of 128 is four lanes and a warp works on eight groups; a team is up to a warp for g <= 1024
+// and a whole CTA above that.  Four lanes share 128 consecutive weights, lane l taking the 16-byte
+// pieces l, l + 4, ...: full 32-byte sectors from memory, and the four lanes' sign bits make four
+// container words with one 4 x 4 byte transpose.  With a warp per group (four weights a lane), as
+// this kernel worked before, a plane of 128 weights cost five rounds of 64-bit shuffles and a
+// ballot per 32 weights; now two rounds, and per weight and plane two fp64 additions and one shift
+// that collects the sign.  Measured, before and after: greedy q = 4, g = 128, the four linears of a
+// layer of width 1600 (30.7 M weights) 162 -> 69 us (2.1 TB/s; the logic pipe is 55 % busy, the fp64
+// pipe 21 %); five alternating rounds, q = 3, g = 128, 5120 x 5120: 1119 -> 373 us (instruction fetch of
+// the unrolled rounds and fp64 latency at 2.6 warps per scheduler bound it).
+//
+// Sums are fp64 and are reduced in a fixed order, so a result never depends on scheduling.
+//
+// quantize_kernel (alternating, q > 4): one warp per group up to 1024 weights, a CTA above.
 //
 // Appendix "Details on BCQ Format": Eq. ap:1-ap:3 (greedy), Eq. ap:4 and the following
 // paragraph (alternating).
@@ -22,6 +33,10 @@ struct QuantParams {
     float* alpha;
     double* sq_err;
     long long items;  // d_out * G
+    int vec;          // rows and groups start on 16-byte boundaries
+    double inv_g;     // 1 / g where that is exact (a power of two), else 0
+    uint32_t g_magic; // where not 0: row of an item = hi32(item * g_magic) >> g_shift
+    uint32_t g_shift;
 };
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -139,17 +154,15 @@ __device__ __forceinline__ bool solve_ls_static(double m, double (&A)[Q][Q + 1],
     return true;
 }
 
-// QT > 0: the number of planes as a compile-time constant (alternating path for q = 2, 3, 4: the
-// scales and the normal equations then live in registers); QT = 0: p.q at run time.
-template <int EPT, int TW, bool ALT, int QT>
+// Alternating method for any number of planes.
+template <int EPT, int TW>
 __global__ void __launch_bounds__(TW == 1 ? 128 : TW * 32)
 quantize_kernel(const QuantParams p) {
-    constexpr int QN = QT > 0 ? QT : BCQ_MAX_Q;
-    const int q = QT > 0 ? QT : p.q;
+    const int q = p.q;
     constexpr int NT = TW * 32;
     constexpr int TEAMS = (TW == 1) ? 4 : 1;
     __shared__ double red_scratch[32];
-    __shared__ double level_smem[TEAMS][ALT ? (1 << BCQ_MAX_Q) : 1];
+    __shared__ double level_smem[TEAMS][1 << BCQ_MAX_Q];
 
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
@@ -171,22 +184,20 @@ quantize_kernel(const QuantParams p) {
         const double inv_m = 1.0 / md;
 
         double r[EPT];
-        float w[ALT ? EPT : 1];
-        uint32_t code[ALT ? EPT : 1];
+        float w[EPT];
+        uint32_t code[EPT];
         const float* wrow = p.W + (long long)j * p.ldw + k0;
 #pragma unroll
         for (int e = 0; e < EPT; ++e) {
             const int kl = e * NT + tid;
             const float v = (kl < m) ? __ldg(wrow + kl) : 0.0f;
             r[e] = (double)v;
-            if (ALT) {
-                w[e] = v;
-                code[e] = 0u;
-            }
+            w[e] = v;
+            code[e] = 0u;
         }
 
-        float a[QN];
-        // ---- greedy planes (q is a constant for QT > 0: the loops over planes unroll by themselves)
+        float a[BCQ_MAX_Q];
+        // ---- greedy planes
         for (int i = 0; i < q; ++i) {
             double local = 0.0;
 #pragma unroll
@@ -196,24 +207,19 @@ quantize_kernel(const QuantParams p) {
             // a power-of-two group size divides exactly by multiplying with its reciprocal
             a[i] = (float)(m_pow2 ? __dmul_rn(S, inv_m) : __ddiv_rn(S, md));
             const double ad = (double)a[i];
-            uint32_t* brow = p.bits + ((long long)i * p.d_out + j) * p.pitch + (k0 >> 5);
 #pragma unroll
             for (int e = 0; e < EPT; ++e) {
-                const int kl = e * NT + tid;
-                const bool valid = kl < m;
                 const bool pos = r[e] >= 0.0;
-                const uint32_t word = __ballot_sync(0xffffffffu, valid && pos);
-                if (!ALT && lane == 0 && (e * NT + twarp * 32) < m) brow[e * TW + twarp] = word;
-                if (valid) r[e] = pos ? r[e] - ad : r[e] + ad;
-                if (ALT && pos) code[e] |= (1u << i);
+                if (e * NT + tid < m) r[e] = pos ? r[e] - ad : r[e] + ad;
+                if (pos) code[e] |= (1u << i);
             }
         }
 
-        if (ALT) {
+        {
             const int ncodes = 1 << q;
             for (int it = 0; it <= p.alt_iters; ++it) {
                 // ---- least-squares alpha for the current signs
-                double A[QN][QN + 1];
+                double A[BCQ_MAX_Q][BCQ_MAX_Q + 1];
                 for (int i = 0; i < q; ++i) {
                     double local = 0.0;
 #pragma unroll
@@ -231,8 +237,7 @@ quantize_kernel(const QuantParams p) {
                         A[l][i] = A[i][l];
                     }
                 }
-                if constexpr (QT > 0) solve_ls_static<QT>(md, A, a);
-                else solve_ls(q, md, A, a);
+                solve_ls(q, md, A, a);
                 if (it == p.alt_iters) break;  // the last pass is the final refit only
                 // ---- every weight moves to the nearest level; largest code wins ties
                 team_sync<TW>();
@@ -271,13 +276,7 @@ quantize_kernel(const QuantParams p) {
         }
 
         // ---- scales, zero padding words of the row, optional squared error
-        if constexpr (QT > 0) {
-#pragma unroll
-            for (int i = 0; i < QT; ++i)
-                if (tid == i) p.alpha[((long long)i * p.d_out + j) * p.G + c] = a[i];
-        } else {
-            if (tid < q) p.alpha[((long long)tid * p.d_out + j) * p.G + c] = a[tid];
-        }
+        if (tid < q) p.alpha[((long long)tid * p.d_out + j) * p.G + c] = a[tid];
         if (c == p.G - 1) {
             const int first_pad = (p.d_in + 31) >> 5;
             const int npad = p.pitch - first_pad;  // 0..3
@@ -288,25 +287,492 @@ quantize_kernel(const QuantParams p) {
         }
         if (p.sq_err != nullptr) {
             double local = 0.0;
-            if (ALT) {
 #pragma unroll
-                for (int e = 0; e < EPT; ++e)
-                    if (e * NT + tid < m) {
-                        double wh = 0.0;
-                        for (int i = 0; i < q; ++i)
-                            wh = ((code[e] >> i) & 1u) ? wh + (double)a[i] : wh - (double)a[i];
-                        const double d = (double)w[e] - wh;
-                        local += d * d;
-                    }
-            } else {
-#pragma unroll
-                for (int e = 0; e < EPT; ++e)
-                    if (e * NT + tid < m) local += r[e] * r[e];
-            }
+            for (int e = 0; e < EPT; ++e)
+                if (e * NT + tid < m) {
+                    double wh = 0.0;
+                    for (int i = 0; i < q; ++i)
+                        wh = ((code[e] >> i) & 1u) ? wh + (double)a[i] : wh - (double)a[i];
+                    const double d = (double)w[e] - wh;
+                    local += d * d;
+                }
             const double E = team_sum<TW>(local, red_scratch);
             if (tid == 0) p.sq_err[(long long)j * p.G + c] = E;
         }
     }
+}
+
+// ------------------------------------------------------------------------------------------
+// the team kernel
+// ------------------------------------------------------------------------------------------
+
+// Sum over a team of L lanes (TW = 1) or TW warps.
+template <int L, int TW>
+__device__ __forceinline__ double lanes_sum(double v, double* scratch) {
+#pragma unroll
+    for (int o = L / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (TW == 1) return v;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double t = 0.0;
+#pragma unroll 1
+    for (int w = 0; w < TW; ++w) t += scratch[w];
+    return t;
+}
+
+// Four lanes hold the bits of 128 consecutive weights: bit 4 i + e of a lane's word is weight
+// 16 i + 4 l + e.  Returns container word l (weights 32 l .. 32 l + 31) to lane l.
+__device__ __forceinline__ uint32_t transpose_bits(uint32_t v) {
+    const uint32_t l = threadIdx.x & 3u;
+    uint32_t o = __shfl_xor_sync(0xffffffffu, v, 1);
+    v = (l & 1u) ? __byte_perm(v, o, 0x3715u) : __byte_perm(v, o, 0x6240u);
+    o = __shfl_xor_sync(0xffffffffu, v, 2);
+    v = (l & 2u) ? __byte_perm(v, o, 0x3276u) : __byte_perm(v, o, 0x5410u);
+    // byte l' = (low nibble: weights 4 l' .. + 3, high nibble: weights 16 + 4 l' .. + 3)
+    uint32_t lo = v & 0x0F0F0F0Fu, hi = (v >> 4) & 0x0F0F0F0Fu;
+    lo |= lo >> 4;
+    hi |= hi >> 4;
+    return __byte_perm(lo, hi, 0x6420u);
+}
+
+// (value, code) pairs into ascending order of the values.
+template <int N>
+__device__ __forceinline__ void sort_levels(double (&L)[N], uint32_t (&c)[N]) {
+    auto ce = [&](int x, int y) {
+        if (L[y] < L[x]) {
+            const double t = L[x]; L[x] = L[y]; L[y] = t;
+            const uint32_t u = c[x]; c[x] = c[y]; c[y] = u;
+        }
+    };
+    if constexpr (N == 2) ce(0, 1);
+    if constexpr (N == 4) { ce(0, 1); ce(2, 3); ce(0, 2); ce(1, 3); ce(1, 2); }
+    if constexpr (N == 8) {
+        ce(0, 1); ce(2, 3); ce(4, 5); ce(6, 7);
+        ce(0, 2); ce(1, 3); ce(4, 6); ce(5, 7);
+        ce(1, 2); ce(5, 6); ce(0, 4); ce(3, 7);
+        ce(1, 5); ce(2, 6);
+        ce(1, 4); ce(3, 6);
+        ce(2, 4); ce(3, 5);
+        ce(3, 4);
+    }
+}
+
+// Nearest of the 2^Q levels, the largest code among equidistant ones: the definition.
+template <int Q>
+__device__ __noinline__ uint32_t nearest_code(double w, const float (&a)[Q]) {
+    uint32_t best = 0u;
+    double dbest = 0.0;
+#pragma unroll 1
+    for (int s = (1 << Q) - 1; s >= 0; --s) {
+        double L = 0.0;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) L = ((s >> i) & 1) ? L + (double)a[i] : L - (double)a[i];
+        const double d = fabs(w - L);
+        if (s == (1 << Q) - 1 || d < dbest) {
+            dbest = d;
+            best = (uint32_t)s;
+        }
+    }
+    return best;
+}
+
+// What a round of the alternating method needs to know about the levels of a group.  They come in
+// pairs +-L, so only the positive ones are kept: sorted, as fp32 midpoints, with the code of each
+// (bit i set where plane i is -1) in a nibble of `codes`.  A magnitude finds its level in Q - 1
+// comparisons instead of 2^Q fp64 distances.
+template <int Q>
+struct LevelSearch {
+    static constexpr int N = 1 << (Q - 1);
+    float mid[N];     // mid[k], k >= 1: between level k - 1 and level k
+    uint32_t codes;
+    float delta;      // a weight closer than this to a midpoint (or to 0) is decided by nearest_code
+
+    // amax: at least the group's largest magnitude
+    __device__ __forceinline__ void build(const float (&a)[Q], float amax) {
+        double L[N];
+        uint32_t c[N];
+#pragma unroll
+        for (int s = 0; s < N; ++s) {
+            double v = 0.0;
+#pragma unroll
+            for (int i = 0; i < Q; ++i) v = (i == Q - 1 || ((s >> i) & 1)) ? v + (double)a[i] : v - (double)a[i];
+            const uint32_t neg = ~((uint32_t)s | (1u << (Q - 1))) & ((1u << Q) - 1u);
+            const bool flip = v < 0.0;
+            L[s] = flip ? -v : v;
+            c[s] = flip ? neg ^ ((1u << Q) - 1u) : neg;
+        }
+        sort_levels<N>(L, c);
+        codes = 0u;
+        double gap = 2.0 * L[0];
+        mid[0] = 0.f;
+#pragma unroll
+        for (int s = 0; s < N; ++s) {
+            codes |= c[s] << (4 * s);
+            if (s > 0) {
+                gap = fmin(gap, L[s] - L[s - 1]);
+                mid[s] = (float)(0.5 * (L[s] + L[s - 1]));
+            }
+        }
+        // fp32 decides exactly as the fp64 distances do when the weight is 2^-21 of the largest level
+        // away from every midpoint: the midpoint is rounded by 2^-24 of itself, the distances by
+        // 2^-53 of the weight.  Levels (almost) on top of each other, or far below the weights, are
+        // left to the definition: delta then covers everything.
+        const float top = (float)L[N - 1];
+        delta = (gap > 9.6e-7 * fmax((double)top, (double)amax * 2.5e-4)) ? top * 4.8e-7f : __int_as_float(0x7F800000);
+        if (!(top < 3.0e38f)) delta = __int_as_float(0x7F800000);
+    }
+    // the code (as in `codes`) of magnitude x in the low Q bits of the result; near = min(near, distances)
+    __device__ __forceinline__ uint32_t find(float x, float& near) const {
+        if constexpr (Q == 1) return codes;
+        float d = x - mid[N / 2];
+        near = fminf(near, fabsf(d));
+        bool p0 = d >= 0.f;
+        if constexpr (Q == 2) return p0 ? codes >> 4 : codes;
+        if constexpr (Q == 3) {
+            d = x - (p0 ? mid[3] : mid[1]);
+            near = fminf(near, fabsf(d));
+            const uint32_t h = p0 ? codes >> 8 : codes;
+            return d >= 0.f ? h >> 4 : h;
+        }
+        if constexpr (Q == 4) {
+            const float lo = p0 ? mid[5] : mid[1], hi = p0 ? mid[7] : mid[3];
+            d = x - (p0 ? mid[6] : mid[2]);
+            near = fminf(near, fabsf(d));
+            const bool p1 = d >= 0.f;
+            d = x - (p1 ? hi : lo);
+            near = fminf(near, fabsf(d));
+            uint32_t h = p0 ? codes >> 16 : codes;
+            h = p1 ? h >> 8 : h;
+            return d >= 0.f ? h >> 4 : h;
+        }
+    }
+};
+
+// Q = 0: greedy, p.q planes; Q > 0: alternating with Q planes.  A thread holds 4 NI weights, a team is L
+// lanes (TW = 1) or TW warps.
+template <int NI, int L, int TW, int Q>
+__global__ void __launch_bounds__(TW == 1 ? 128 : TW * 32, TW == 1 ? (Q == 0 ? 5 : 3) : TW <= 4 ? 12 / TW : 1)
+team_quantize_kernel(const QuantParams p) {
+    constexpr bool ALT = Q > 0;
+    constexpr int EPT = 4 * NI;
+    constexpr int NT = L * TW;                       // threads of a team
+    constexpr int TEAMS = TW == 1 ? 128 / L : 1;     // per CTA
+    __shared__ double scratch[TW == 1 ? 1 : 32];
+    const int tl = TW == 1 ? (int)(threadIdx.x & (L - 1)) : (int)threadIdx.x;
+    const long long item0 = (long long)blockIdx.x * TEAMS + (TW == 1 ? threadIdx.x / L : 0);
+    // teams past the last item repeat it (the shuffles need every lane) and store nothing
+    const bool live = item0 < p.items;
+    const long long item = live ? item0 : p.items - 1;
+    int j, c;
+    if (p.g_magic != 0u) {
+        j = (int)(__umulhi((uint32_t)item, p.g_magic) >> p.g_shift);
+        c = (int)((uint32_t)item - (uint32_t)j * (uint32_t)p.G);
+    } else {
+        j = (int)(item / p.G);
+        c = (int)(item - (long long)j * p.G);
+    }
+    const int k0 = c * p.g;
+    const int m = min(p.g, p.d_in - k0);
+    const double md = (double)m;
+    const int kt = (tl >> 2) * (16 * NI) + (tl & 3) * 4;  // first weight of the thread; piece i is 16 i further
+
+    // ---- load; bit t of `valid`: the thread's t-th weight exists
+    const float* src = p.W + (long long)j * p.ldw + k0 + kt;
+    float w[EPT];
+    constexpr uint32_t kAll = EPT == 32 ? 0xFFFFFFFFu : (1u << (EPT & 31)) - 1u;
+    uint32_t valid = kAll;
+    int pieces = NI;       // 16-byte pieces that hold weights
+    bool partial = false;  // the last of them is not full
+    double inv_m = p.inv_g;
+    if (m == EPT * NT && p.vec) {
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(src + 16 * i));
+            w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
+        }
+    } else {
+        valid = 0u;
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+            const int left = m - (kt + 16 * i);
+            if (p.vec && left >= 4) {
+                const float4 v = __ldg(reinterpret_cast<const float4*>(src + 16 * i));
+                w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) w[4 * i + e] = (e < left) ? __ldg(src + 16 * i + e) : 0.0f;
+            }
+            valid |= (left >= 4 ? 0xFu : left > 0 ? (1u << left) - 1u : 0u) << (4 * i);
+        }
+        pieces = min(NI, max(0, (m - kt + 15) >> 4));
+        partial = pieces > 0 && m - (kt + 16 * (pieces - 1)) < 4;
+        inv_m = (m & (m - 1)) == 0 ? 1.0 / md : 0.0;
+    }
+
+    // ---- greedy planes.  A residual is kept as a magnitude |t| and a sign bit in `negs`: taking a off in
+    // the direction of its sign leaves |t| - a with the sign kept, or a - |t| with the sign turned.
+    // t = a - |t| is one addition, and the collected sign bits of all t turn `negs` at once.
+    // Weights that do not exist are zeros throughout.  (-0.0 as an input counts as positive.)
+    double t[EPT];
+    uint32_t negs = 0u;
+#pragma unroll
+    for (int e = EPT - 1; e >= 0; --e) {
+        w[e] += 0.0f;
+        negs = __funnelshift_l(__float_as_uint(w[e]), negs, 1);
+        t[e] = (double)w[e];
+    }
+    const int q = ALT ? Q : p.q;
+    constexpr int QN = ALT ? Q : 1;
+    float a[QN];
+    uint32_t neg[QN];  // bit t: plane i of the thread's t-th weight is -1
+    const int wi = (tl >> 2) * (NI / 2) + (tl & 3);           // container word of the group this thread writes
+    const bool writes = live && (tl & 3) < NI / 2 && 32 * wi < m;
+    const uint32_t word_mask = m - 32 * wi >= 32 ? 0xFFFFFFFFu : (1u << ((m - 32 * wi) & 31)) - 1u;
+    uint32_t* dst = p.bits + (long long)j * p.pitch + (k0 >> 5) + wi;
+    const long long plane_words = (long long)p.d_out * p.pitch, plane_alpha = (long long)p.d_out * p.G;
+    float* adst = p.alpha + (long long)j * p.G + c;
+    // scale of the next plane; `negs` are its signs
+    auto scale_of = [&]() {
+        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+#pragma unroll
+        for (int e = 0; e < EPT; e += 4) {
+            s0 += fabs(t[e]);
+            s1 += fabs(t[e + 1]);
+            s2 += fabs(t[e + 2]);
+            s3 += fabs(t[e + 3]);
+        }
+        const double S = lanes_sum<L, TW>((s0 + s1) + (s2 + s3), scratch);
+        // a power-of-two group size divides exactly by multiplying with its reciprocal
+        return (float)(inv_m != 0.0 ? __dmul_rn(S, inv_m) : __ddiv_rn(S, md));
+    };
+    // the residual after a plane with scale ai
+    auto next_residual = [&](float ai) {
+        const double ad = (double)ai;
+        uint32_t kept = 0u, least = 0xFFFFFFFFu;
+        if (__all_sync(0xffffffffu, valid == kAll)) {
+#pragma unroll
+            for (int e = EPT - 1; e >= 0; --e) {
+                t[e] = ad - fabs(t[e]);
+                kept = __funnelshift_l((uint32_t)__double2hiint(t[e]), kept, 1);
+                least = min(least, (uint32_t)__double2hiint(t[e]));
+            }
+        } else {
+#pragma unroll
+            for (int i4 = NI - 1; i4 >= 0; --i4) {  // a piece without weights: -0.0 - 0.0 is -0.0
+                const double ap = i4 < pieces ? ad : -0.0;
+#pragma unroll
+                for (int e = 4 * i4 + 3; e >= 4 * i4; --e) {
+                    t[e] = ap - fabs(t[e]);
+                    kept = __funnelshift_l((uint32_t)__double2hiint(t[e]), kept, 1);
+                    least = min(least, (uint32_t)__double2hiint(t[e]));
+                }
+            }
+            if (partial) {
+#pragma unroll
+                for (int e = 0; e < EPT; ++e)
+                    if (!((valid >> e) & 1u)) t[e] = -0.0;
+            }
+        }
+        negs ^= ~kept;
+        if (least == 0u) {  // a residual of exactly zero counts as positive
+#pragma unroll
+            for (int e = 0; e < EPT; ++e)
+                if (t[e] == 0.0 && ((valid >> e) & 1u)) negs &= ~(1u << e);
+        }
+    };
+    if constexpr (!ALT) {
+        for (int i = 0; i < q; ++i) {
+            const float ai = scale_of();
+            const uint32_t word = transpose_bits(~negs);
+            if (writes) dst[i * plane_words] = word & word_mask;
+            if (live && tl == 0) adst[i * plane_alpha] = ai;
+            if (i + 1 < q || p.sq_err != nullptr) next_residual(ai);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            a[i] = scale_of();
+            neg[i] = negs;
+            if (i + 1 < Q) next_residual(a[i]);
+        }
+
+        // ---- alternating rounds.  From here on only magnitudes count: b_i w = (b_i sign(w)) |w|, so the
+        // sums run over |w| with the signs `neg` relative to sign(w), and so do the mismatch counts.
+        uint32_t sgn = 0u, zero = 0u;
+        float tiny = __int_as_float(0x7F800000), amax = 0.f;
+#pragma unroll
+        for (int e = EPT - 1; e >= 0; --e) {
+            sgn = __funnelshift_l(__float_as_uint(w[e]), sgn, 1);
+            w[e] = fabsf(w[e]);
+            zero = (zero << 1) | (w[e] == 0.f ? 1u : 0u);
+            if (w[e] != 0.f) tiny = fminf(tiny, w[e]);
+            amax = fmaxf(amax, w[e]);
+        }
+        zero &= valid;
+#pragma unroll
+        for (int o = L / 2; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+        if (TW > 1) amax = (float)lanes_sum<1, TW>((double)amax, scratch);  // a bound: the sum over the warps
+#pragma unroll
+        for (int i = 0; i < Q; ++i) neg[i] ^= sgn;
+
+        double S[Q];
+        auto sums_from_signs = [&]() {
+#pragma unroll
+            for (int i = 0; i < Q; ++i) S[i] = 0.0;
+#pragma unroll
+            for (int e = 0; e < EPT; ++e) {
+                const double x = (double)w[e];
+                const int hi = __double2hiint(x), lo = __double2loint(x);
+#pragma unroll
+                for (int i = 0; i < Q; ++i)
+                    S[i] += __hiloint2double(hi ^ (int)((neg[i] << (31 - e)) & 0x80000000u), lo);
+            }
+        };
+        sums_from_signs();
+        uint32_t flip0 = 0u;  // the code of an exact zero is the complement of the smallest level's
+        for (int it = 0;; ++it) {
+            // ---- least-squares alpha for the current signs
+            double A[Q][Q + 1];
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                A[i][Q] = lanes_sum<L, TW>(S[i], scratch);
+                A[i][i] = md;
+            }
+            // mismatch counts, two to a word (at most 1024 weights to a warp)
+            constexpr int PAIRS = Q * (Q - 1) / 2;
+            uint32_t cnt[PAIRS > 0 ? (PAIRS + 1) / 2 : 1] = {};
+            {
+                int n = 0;
+#pragma unroll
+                for (int i = 0; i < Q; ++i)
+#pragma unroll
+                    for (int l = i + 1; l < Q; ++l, ++n)
+                        cnt[n / 2] += (uint32_t)__popc((neg[i] ^ neg[l]) & valid) << (16 * (n & 1));
+            }
+            if (PAIRS > 0) {
+#pragma unroll
+                for (int v = 0; v < (PAIRS + 1) / 2; ++v) {
+#pragma unroll
+                    for (int o = L / 2; o > 0; o >>= 1) cnt[v] += __shfl_xor_sync(0xffffffffu, cnt[v], o);
+                }
+                int n = 0;
+#pragma unroll
+                for (int i = 0; i < Q; ++i)
+#pragma unroll
+                    for (int l = i + 1; l < Q; ++l, ++n) {
+                        double mism = (double)((cnt[n / 2] >> (16 * (n & 1))) & 0xFFFFu);
+                        if (TW > 1) mism = lanes_sum<1, TW>(mism, scratch);
+                        A[i][l] = md - 2.0 * mism;
+                        A[l][i] = A[i][l];
+                    }
+            }
+            solve_ls_static<Q>(md, A, a);
+            if (it == p.alt_iters) break;  // the last pass is the final refit only
+            // ---- every weight moves to the nearest level
+            // (opaque to the compiler, which would keep all fp64 copies across the rounds and spill)
+#pragma unroll
+            for (int e = 0; e < EPT; ++e) asm volatile("" : "+f"(w[e]));
+            LevelSearch<Q> ls;
+            ls.build(a, amax);
+            flip0 = (ls.codes >> (Q - 1)) & 1u;
+            float near = tiny;
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                S[i] = 0.0;
+                neg[i] = 0u;
+            }
+#pragma unroll
+            for (int e = EPT - 1; e >= 0; --e) {
+                const uint32_t y = ls.find(w[e], near);
+                const double x = (double)w[e];
+                const int hi = __double2hiint(x), lo = __double2loint(x);
+#pragma unroll
+                for (int i = 0; i < Q; ++i) {
+                    const uint32_t b = y << (31 - i);
+                    neg[i] = __funnelshift_l(b, neg[i], 1);
+                    S[i] += __hiloint2double(hi ^ (int)(b & 0x80000000u), lo);
+                }
+            }
+            if (!(near > ls.delta)) {
+                // some weight of this thread is too close to call in fp32
+                flip0 = 0u;
+#pragma unroll
+                for (int i = 0; i < Q; ++i) neg[i] = 0u;
+#pragma unroll
+                for (int e = EPT - 1; e >= 0; --e) {
+                    const uint32_t code = nearest_code<Q>(((sgn >> e) & 1u) ? -(double)w[e] : (double)w[e], a);
+#pragma unroll
+                    for (int i = 0; i < Q; ++i) neg[i] |= (~(code >> i) & 1u) << e;
+                }
+#pragma unroll
+                for (int i = 0; i < Q; ++i) neg[i] ^= sgn;
+                sums_from_signs();
+            }
+        }
+        // ---- write the planes
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            // flip0: a zero is equidistant from +L and -L, the larger code (plane Q - 1 at +1) wins
+            neg[i] ^= sgn ^ (flip0 ? zero : 0u);
+            const uint32_t word = transpose_bits(~neg[i]);
+            if (writes) dst[i * plane_words] = word & word_mask;
+            if (live && tl == 0) adst[i * plane_alpha] = a[i];
+        }
+        if (p.sq_err != nullptr) {
+#pragma unroll
+            for (int e = 0; e < EPT; ++e) {
+                double wh = 0.0;
+#pragma unroll
+                for (int i = 0; i < Q; ++i) wh = ((neg[i] >> e) & 1u) ? wh - (double)a[i] : wh + (double)a[i];
+                t[e] = ((valid >> e) & 1u) ? (((sgn >> e) & 1u) ? -(double)w[e] : (double)w[e]) - wh : 0.0;
+            }
+        }
+    }
+
+    // ---- zero padding words of the row, optional squared error
+    if (c == p.G - 1 && live) {
+        const int first_pad = (p.d_in + 31) >> 5;
+        const int npad = p.pitch - first_pad;  // 0..3
+        for (int e = tl; e < npad * q; e += NT) {
+            const int i = e / npad;
+            p.bits[i * plane_words + (long long)j * p.pitch + first_pad + (e - i * npad)] = 0u;
+        }
+    }
+    if (p.sq_err != nullptr) {
+        double local = 0.0;
+#pragma unroll
+        for (int e = 0; e < EPT; ++e) local += t[e] * t[e];
+        const double E = lanes_sum<L, TW>(local, scratch);
+        if (live && tl == 0) p.sq_err[(long long)j * p.G + c] = E;
+    }
+}
+
+template <int NI, int L, int TW, int Q>
+cudaError_t launch_team(const QuantParams& p, cudaStream_t stream) {
+    constexpr int TEAMS = TW == 1 ? 128 / L : 1;
+    const int threads = TW == 1 ? 128 : TW * 32;
+    const unsigned blocks = (unsigned)((p.items + TEAMS - 1) / TEAMS);
+    team_quantize_kernel<NI, L, TW, Q><<<blocks, threads, 0, stream>>>(p);
+    bcq::count_launch();
+    return cudaGetLastError();
+}
+
+// The smallest team that holds a group at 32 weights a thread (8 or 16 for groups of 32 or 64).
+template <int Q>
+cudaError_t launch_team_size(const QuantParams& p, cudaStream_t s) {
+    const int g = p.g;
+    if (g <= 32) return launch_team<2, 4, 1, Q>(p, s);
+    if (g <= 64) return launch_team<4, 4, 1, Q>(p, s);
+    if (g <= 128) return launch_team<8, 4, 1, Q>(p, s);
+    if (g <= 256) return launch_team<8, 8, 1, Q>(p, s);
+    if (g <= 512) return launch_team<8, 16, 1, Q>(p, s);
+    if (g <= 1024) return launch_team<8, 32, 1, Q>(p, s);
+    if (g <= 2048) return launch_team<8, 32, 2, Q>(p, s);
+    if (g <= 4096) return launch_team<8, 32, 4, Q>(p, s);
+    if (g <= 8192) return launch_team<8, 32, 8, Q>(p, s);
+    if (g <= 16384) return launch_team<8, 32, 16, Q>(p, s);
+    return launch_team<8, 32, 32, Q>(p, s);
 }
 
 template <int EPT, int TW>
@@ -316,14 +782,7 @@ cudaError_t launch_quantize(const QuantParams& p, cudaStream_t stream) {
     long long blocks = (p.items + TEAMS - 1) / TEAMS;
     const long long cap = (long long)bcq::sm_count() * 64;  // grid-stride beyond this
     if (blocks > cap) blocks = cap;
-    if (p.alt_iters > 0) {
-        if (p.q == 2) quantize_kernel<EPT, TW, true, 2><<<(unsigned)blocks, threads, 0, stream>>>(p);
-        else if (p.q == 3) quantize_kernel<EPT, TW, true, 3><<<(unsigned)blocks, threads, 0, stream>>>(p);
-        else if (p.q == 4) quantize_kernel<EPT, TW, true, 4><<<(unsigned)blocks, threads, 0, stream>>>(p);
-        else quantize_kernel<EPT, TW, true, 0><<<(unsigned)blocks, threads, 0, stream>>>(p);
-    } else {
-        quantize_kernel<EPT, TW, false, 0><<<(unsigned)blocks, threads, 0, stream>>>(p);
-    }
+    quantize_kernel<EPT, TW><<<(unsigned)blocks, threads, 0, stream>>>(p);
     bcq::count_launch();
     return cudaGetLastError();
 }
@@ -364,9 +823,24 @@ extern "C" bcq_status bcq_quantize(int d_out, int d_in, int q, int g, const floa
     p.pitch = (int)bcq_pitch_words(d_in);
     p.W = W; p.bits = bits; p.alpha = alpha; p.sq_err = sq_err;
     p.items = (long long)d_out * p.G;
+    p.vec = bcq::aligned16(W) && ldw % 4 == 0;
+    p.inv_g = (g & (g - 1)) == 0 ? 1.0 / g : 0.0;
+    p.g_magic = 0; p.g_shift = 0;
+    if (p.G > 1 && p.items < (1ll << 31)) {
+        // ceil(2^(32 + s) / G) with 2^s < G <= 2^(s+1): exact for every item below 2^31
+        int sh = 0;
+        while ((2ll << sh) < p.G) ++sh;
+        p.g_shift = (uint32_t)sh;
+        p.g_magic = (uint32_t)(((1ull << (32 + sh)) + p.G - 1) / p.G);
+    }
     cudaStream_t s = (cudaStream_t)stream;
     cudaError_t e;
-    if (g <= 128) e = launch_quantize<4, 1>(p, s);
+    if (alt_iters == 0) e = launch_team_size<0>(p, s);
+    else if (q == 1) e = launch_team_size<1>(p, s);
+    else if (q == 2) e = launch_team_size<2>(p, s);
+    else if (q == 3) e = launch_team_size<3>(p, s);
+    else if (q == 4) e = launch_team_size<4>(p, s);
+    else if (g <= 128) e = launch_quantize<4, 1>(p, s);
     else if (g <= 256) e = launch_quantize<8, 1>(p, s);
     else if (g <= 512) e = launch_quantize<16, 1>(p, s);
     else if (g <= 1024) e = launch_quantize<32, 1>(p, s);

@@ -111,6 +111,29 @@ def test_quantize_matches_oracle(d_out, d_in, q, g, alt, outl):
     np.testing.assert_allclose(sq_err[same], sq_ref[same], rtol=1e-6, atol=1e-18)
 
 
+@pytest.mark.parametrize("alt", [0, 3])
+@pytest.mark.parametrize("d_in,g", [(96, 32), (200, 64), (420, 96), (520, 160), (900, 256), (1100, 512), (1023, 1023),
+                                    (2050, 2050), (5000, 2528), (8192, 8192), (12001, 12001), (20000, 20000)])
+def test_quantize_team_sizes_with_exact_ties(d_in, g, alt):
+    # Multiples of 1/64 with many zeros (also -0.0) and repeated magnitudes: every sum the quantizer
+    # forms from them is exact in fp64 whatever its order (values below 2, at most 2^15 of them, 24
+    # bits each), so ties are ties on both sides and the bits have to be the oracle's, one for one.
+    rng = np.random.default_rng(d_in + alt)
+    for q in (1, 2, 3, 4) if d_in < 3000 else (3,):
+        W = (rng.integers(-6, 7, size=(5, d_in)) / 64.0).astype(np.float32)
+        W[0, ::3] = -0.0
+        W[1] = 0.0
+        W[2, : d_in // 2] = 0.25
+        Wd = torch.zeros((5, d_in + 1), dtype=torch.float32, device="cuda")[:, 1:]   # rows not 16-byte aligned
+        Wd.copy_(torch.from_numpy(W))
+        bits_ref, alpha_ref, sq_ref, _ = oracle.quantize(W, q, g, alt_iters=alt)
+        for src in (Wd, torch.from_numpy(W).cuda()):
+            bits, alpha, sq = bcq.quantize(src, q, g, alt, want_sq_err=True)
+            np.testing.assert_array_equal(host_bits(bits), bits_ref)
+            np.testing.assert_allclose(alpha.cpu().numpy(), alpha_ref, rtol=1e-6, atol=1e-9)
+            np.testing.assert_allclose(sq.cpu().numpy(), sq_ref, rtol=1e-6, atol=1e-12)
+
+
 def test_quantize_strided_input_and_determinism():
     W = synth.weights(48, 384, (101, 0, 0))
     Wp = np.zeros((48, 400), dtype=np.float32)
