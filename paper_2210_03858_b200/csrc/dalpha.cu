@@ -1,15 +1,21 @@
 // Scale gradient of the BCQ linear layer (Eq. 4):
 //     dalpha_i[j, c] = scale * sum_{k in group c} b_i[j,k] * (dY^T X)[j,k].
 //
-// D[j, k] = sum_t dY[t, j] X[t, k] is a 128 x TN x 64 UMMA tile product with both operands
-// MN-major (tokens are the K index; dY and X rows are contiguous in j and k), loaded by TMA in
-// 64 x 64 boxes.  The epilogue never writes D: thread = (row j, half of the tile's columns) reads
+// D[j, k] = sum_t dY[t, j] X[t, k] is a 256 x 256 x 64 UMMA tile product of a CTA pair with both
+// operands MN-major (tokens are the K index; dY and X rows are contiguous in j and k), loaded by TMA
+// in 64 x 64 boxes.  A pair, because operand traffic bounds this kernel: per 512 tensor-core cycles a
+// 128 x 256 tile of a CTA alone takes 48 KiB into shared memory and reads 48 KiB back, 192 bytes a
+// cycle against the 128 of shared memory; in a pair each CTA holds half of the columns, 128 bytes a
+// cycle.  Measured, CTA alone and pair: 1600 -> 6400 with 4096 tokens 75.5 and 68.5 us, 5120 -> 20480
+// with 2048 tokens 326 and 276 us (1558 TFLOP/s).  The epilogue never writes D: thread = (row j, half of the tile's columns) reads
 // its accumulator row from tensor memory 32 columns at a time, applies the signs of every
 // requested plane from one 32-bit word of the packed planes, and sums per group.  Partial sums
 // (one per split over tokens, column sub-tile and group piece) go to the workspace and a second
 // kernel adds them in a fixed order, so the result does not depend on scheduling.  When every
 // output has exactly one partial (no token split and a group per column sub-tile, e.g. g = 128)
 // the epilogue writes dalpha itself and the second kernel is not launched.
+#include <algorithm>
+
 #include "gemm_common.cuh"
 
 namespace {
@@ -24,7 +30,7 @@ struct DalphaParams {
     int kb_per_split;
     int splits;
     int m_tiles, n_tiles;
-    int n_subtiles;      // column sub-tiles of width TN/2 over d_in
+    int n_subtiles;      // column sub-tiles of width kHN over d_in
     int slots;           // partial slots per sub-tile
     uint32_t plane_mask;
     const uint32_t* bits;
@@ -41,61 +47,73 @@ struct DalphaParams {
 // dalpha: D[j, k] = sum_t dY[t, j] X[t, k], sign-weighted group sums in the epilogue
 // ------------------------------------------------------------------------------------------
 
-// Persistent: every CTA walks over (row tile, column tile, token split) tiles; two accumulators
-// in tensor memory, so the sign-and-sum epilogue of one tile runs under the main loop of the next.
-//   warp 0      TMA producer (dY and X boxes of every K block of 64 tokens)
-//   warp 1      UMMA issuer, owner of the tensor-memory allocation
-//   warps 2..9  epilogue: thread = (row j, half of the tile's columns)
-template <int TN, int STAGES>
+constexpr int kTN = 256;       // columns of a tile
+constexpr int kHN = kTN / 2;   // of an epilogue sub-tile, and of the half of B that one CTA holds
+constexpr int kTM = 2 * kBlockM;
+constexpr int kStages = 6;
+constexpr uint32_t kStageBytes = kABytes + kHN * kBlockK * 2;  // 32 KiB
+constexpr size_t kDalphaSmem = (size_t)kStages * kStageBytes + 1024 + 256;
+
+// Persistent: every pair of CTAs walks over (row tile, column tile, token split) tiles; two
+// accumulators in tensor memory, so the sign-and-sum epilogue of one tile runs under the main loop of
+// the next.  In each CTA:
+//   warp 0      TMA producer (its dY and X boxes of every K block of 64 tokens)
+//   warp 1      owner of the tensor-memory allocation; in the leader, UMMA issuer for both
+//   warps 2..9  epilogue: thread = (row j of this CTA's 128, half of the tile's columns)
+// `full` and `acc_empty` are the leader's barriers; `empty` and `accum` exist in both CTAs and are
+// signalled by one commit to both.
 __global__ void __launch_bounds__(kThreads, 1)
 dalpha_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ CUtensorMap tmap_x,
               const DalphaParams p) {
-    constexpr uint32_t kBBytes = TN * kBlockK * 2;
-    constexpr uint32_t kStageBytes = kABytes + kBBytes;
-    constexpr int HN = TN / 2;
+    constexpr int HN = kHN;
     constexpr int NCH = HN / 32;
-    constexpr uint32_t kAccCols = TmemCols<TN>::value;
+    constexpr uint32_t kAccCols = kTN;
     constexpr uint32_t kTmemCols = 2 * kAccCols;
 
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* smem_gen = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
-    const uint32_t ctl_base = smem_base + STAGES * kStageBytes;
-    uint8_t* ctl_gen = smem_gen + STAGES * kStageBytes;
+    const uint32_t ctl_base = smem_base + kStages * kStageBytes;
+    uint8_t* ctl_gen = smem_gen + kStages * kStageBytes;
 
     Ctl ctl;
     ctl.full = ctl_base;
     ctl.aready = 0;
-    ctl.empty = ctl_base + 8 * STAGES;
-    ctl.accum = ctl_base + 16 * STAGES;         // + 8c : accumulator c complete
-    const uint32_t acc_empty = ctl.accum + 16;  // + 8c : accumulator c drained
+    ctl.empty = ctl_base + 8 * kStages;
+    ctl.accum = ctl_base + 16 * kStages;        // + 8c : accumulator c complete
+    const uint32_t acc_empty = ctl.accum + 16;  // + 8c : accumulator c drained by both CTAs
     ctl.spare = ctl.accum + 32;
-    volatile uint32_t* tmem_holder = reinterpret_cast<volatile uint32_t*>(ctl_gen + 16 * STAGES + 40);
-    ctl.abort_flag = reinterpret_cast<volatile int*>(ctl_gen + 16 * STAGES + 44);
+    volatile uint32_t* tmem_holder = reinterpret_cast<volatile uint32_t*>(ctl_gen + 16 * kStages + 40);
+    ctl.abort_flag = reinterpret_cast<volatile int*>(ctl_gen + 16 * kStages + 44);
     ctl.device_flag = &g_timeout_flag;
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
+    const int rank = (int)ptx::cluster_rank();
     const int num_tiles = p.m_tiles * p.n_tiles * p.splits;
-    // row tile fastest: CTAs running together share the X boxes of a column tile in L2
+    const int pair0 = (int)blockIdx.x >> 1, num_pairs = (int)gridDim.x >> 1;
+    // row tile fastest: pairs running together share the X boxes of a column tile in L2
     auto tile_coords = [&](int tile, int& j0, int& k0, int& z, int& kb_begin, int& iters) {
         const int mt = tile % p.m_tiles;
         const int rest = tile / p.m_tiles;
-        j0 = mt * kBlockM;
-        k0 = (rest % p.n_tiles) * TN;
+        j0 = mt * kTM + rank * kBlockM;
+        k0 = (rest % p.n_tiles) * kTN;
         z = rest / p.n_tiles;
         kb_begin = z * p.kb_per_split;
         iters = min(p.num_kb, kb_begin + p.kb_per_split) - kb_begin;
     };
+    // a column tile that reaches past d_in multiplies only the 64-column blocks that hold columns of
+    // the matrix; half of them are in each CTA
+    auto tile_width = [&](int k0) { return min(kTN, (p.d_in - k0 + 63) / 64 * 64); };
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
+        for (int s = 0; s < kStages; ++s) {
             ptx::mbar_init(ctl.full + 8 * s, 1);
             ptx::mbar_init(ctl.empty + 8 * s, 1);
         }
         for (int c = 0; c < 2; ++c) {
             ptx::mbar_init(ctl.accum + 8 * c, 1);
-            ptx::mbar_init(acc_empty + 8 * c, kWorkerWarps);
+            ptx::mbar_init(acc_empty + 8 * c, 2 * kWorkerWarps);
         }
         ptx::mbar_init(ctl.spare, 1);
         *ctl.abort_flag = 0;
@@ -103,57 +121,53 @@ dalpha_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant
         ptx::prefetch_tmap(&tmap_dy);
         ptx::prefetch_tmap(&tmap_x);
     }
+    __syncwarp();
     if (warp == 1) {
-        ptx::tmem_alloc(ptx::smem_u32(const_cast<uint32_t*>(tmem_holder)), kTmemCols);
-        ptx::tmem_relinquish();
+        ptx::tmem_alloc_pair(ptx::smem_u32(const_cast<uint32_t*>(tmem_holder)), kTmemCols);
+        ptx::tmem_relinquish_pair();
     }
     ptx::tc_fence_before_sync();
     __syncthreads();
+    ptx::cluster_sync();  // the peer's barriers exist
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_holder;
 
     if (warp == 0) {
         if (lane == 0) {
             bool ok = true;
-            int s = 0, in_flight = 0;
+            int s = 0;
             uint32_t ph = 0;
-            for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+            for (int tile = pair0; tile < num_tiles && ok; tile += num_pairs) {
                 int j0, k0, z, kb_begin, iters;
                 tile_coords(tile, j0, k0, z, kb_begin, iters);
-                // a column tile that reaches past d_in brings (and multiplies) only the 64-column
-                // blocks that hold columns of the matrix
-                const int boxes = min(TN / 64, (p.d_in - k0 + 63) / 64);
+                const int half = tile_width(k0) / 2;  // columns this CTA brings
+                const int boxes = (half + 63) / 64;
+                const int kx = k0 + rank * half;
                 for (int it = 0; it < iters; ++it) {
                     ok = wait_bar(ctl.empty + 8 * s, ph ^ 1u, ctl, 11);
                     if (!ok) break;
                     const uint32_t sa = smem_base + s * kStageBytes;
+                    const uint32_t bar = ptx::leader_addr(ctl.full + 8 * s);
                     const int tok = (kb_begin + it) * kBlockK;
-                    ptx::mbar_arrive_expect_tx(ctl.full + 8 * s, kABytes + (uint32_t)boxes * 8192u);
-                    // A: two blocks of 64 rows j (inner) x 64 tokens; B: TN/64 blocks of 64 k x 64 tokens
-                    ptx::tma_load_2d(sa, &tmap_dy, j0, tok, ctl.full + 8 * s);
-                    ptx::tma_load_2d(sa + 8192, &tmap_dy, j0 + 64, tok, ctl.full + 8 * s);
-#pragma unroll
-                    for (int b = 0; b < TN / 64; ++b)
-                        if (b < boxes) ptx::tma_load_2d(sa + kABytes + b * 8192, &tmap_x, k0 + b * 64, tok, ctl.full + 8 * s);
-                    in_flight = min(in_flight + 1, STAGES);
-                    if (++s == STAGES) { s = 0; ph ^= 1u; }
+                    if (rank == 0) ptx::mbar_arrive_expect_tx(ctl.full + 8 * s, 2u * (kABytes + (uint32_t)boxes * 8192u));
+                    // A: two blocks of 64 rows j (inner) x 64 tokens; B: blocks of 64 k x 64 tokens
+                    ptx::tma_load_2d_pair(sa, &tmap_dy, j0, tok, bar);
+                    ptx::tma_load_2d_pair(sa + 8192, &tmap_dy, j0 + 64, tok, bar);
+                    ptx::tma_load_2d_pair(sa + kABytes, &tmap_x, kx, tok, bar);
+                    if (boxes > 1) ptx::tma_load_2d_pair(sa + kABytes + 8192, &tmap_x, kx + 64, tok, bar);
+                    if (++s == kStages) { s = 0; ph ^= 1u; }
                 }
             }
-            if (!ok) {
-                int bs = s;
-                uint32_t bph = ph;
-                for (int i = 0; i < in_flight; ++i) {
-                    if (bs == 0) { bs = STAGES; bph ^= 1u; }
-                    --bs;
-                    wait_bar(ctl.full + 8 * bs, bph, ctl, 12);
-                }
-            }
+            // giving up: the copies in flight are counted on the leader's barriers, which may never
+            // complete; they land within microseconds, so wait a thousand times as long
+            if (!ok) for (int i = 0; i < 1000; ++i) __nanosleep(2000);
         }
+        __syncwarp();
     } else if (warp == 1) {
         // One elected thread runs the whole loop: between two stages it has a barrier check, a
         // fence, four UMMAs and a commit to get through in less time than the tensor core needs
         // for a stage, so nothing warp-wide (election, reconvergence) is left inside the loop.
-        if (ptx::elect_one()) {
+        if (rank == 0 && ptx::elect_one()) {
             bool ok = true;
             int s = 0, lt = 0;
             uint32_t ph = 0;
@@ -161,7 +175,7 @@ dalpha_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant
             // rows, stride 1024 B between groups of eight token lines); a UMMA steps the start by 2048 B
             constexpr uint32_t kHi = (1024u >> 4) | (1u << 14) | (2u << 29);
             constexpr uint32_t kLoExtra = (8192u >> 4) << 16;
-            for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++lt) {
+            for (int tile = pair0; tile < num_tiles && ok; tile += num_pairs, ++lt) {
                 int j0, k0, z, kb_begin, iters;
                 tile_coords(tile, j0, k0, z, kb_begin, iters);
                 const int acc = lt & 1;
@@ -169,8 +183,7 @@ dalpha_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
                 const uint32_t d_tmem = tmem_base + (uint32_t)acc * kAccCols;
-                const int boxes = min(TN / 64, (p.d_in - k0 + 63) / 64);
-                const uint32_t idesc = ptx::make_idesc_bf16(kBlockM, boxes * 64, 1, 1);  // the UMMA is as wide as the tile's columns
+                const uint32_t idesc = ptx::make_idesc_bf16(kTM, tile_width(k0), 1, 1);
                 for (int it = 0; it < iters; ++it) {
                     ok = wait_bar(ctl.full + 8 * s, ph, ctl, 13, 32u);
                     if (!ok) break;
@@ -179,15 +192,15 @@ dalpha_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant
                     const uint32_t b_lo = a_lo + (kABytes >> 4);
 #pragma unroll
                     for (int kk = 0; kk < kBlockK / 16; ++kk)
-                        ptx::umma_f16_halves(d_tmem, a_lo + kk * (2048u >> 4), kHi, b_lo + kk * (2048u >> 4), kHi, idesc,
-                                             (it > 0 || kk > 0) ? 1u : 0u);
-                    ptx::umma_commit(ctl.empty + 8 * s);
-                    if (++s == STAGES) { s = 0; ph ^= 1u; }
+                        ptx::umma_f16_pair(d_tmem, a_lo + kk * (2048u >> 4), kHi, b_lo + kk * (2048u >> 4), kHi, idesc,
+                                           (it > 0 || kk > 0) ? 1u : 0u);
+                    ptx::umma_commit_pair(ctl.empty + 8 * s);
+                    if (++s == kStages) { s = 0; ph ^= 1u; }
                 }
-                if (ok) ptx::umma_commit(ctl.accum + 8 * acc);
+                if (ok) ptx::umma_commit_pair(ctl.accum + 8 * acc);
             }
             if (!ok) {
-                ptx::umma_commit(ctl.spare);
+                ptx::umma_commit_pair(ctl.spare);
                 wait_bar(ctl.spare, 0, ctl, 15);
             }
         }
@@ -199,14 +212,14 @@ dalpha_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant
         const long long plane_words = (long long)p.d_out * p.pitch;
         bool ok = true;
         int lt = 0;
-        for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++lt) {
+        for (int tile = pair0; tile < num_tiles && ok; tile += num_pairs, ++lt) {
             int j0, k0, z, kb_begin, iters;
             tile_coords(tile, j0, k0, z, kb_begin, iters);
             const int acc = lt & 1;
             const int j = j0 + quarter * 32 + lane;
             const bool j_ok = j < p.d_out;
             const int kbase = k0 + half * HN;
-            const int subtile = (k0 / TN) * 2 + half;
+            const int subtile = (k0 / kTN) * 2 + half;
 
             // the sign words do not depend on the accumulator: fetch them while the main loop runs
             uint32_t nw[NCH][BCQ_MAX_Q];
@@ -279,15 +292,16 @@ dalpha_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant
             // the accumulator may be overwritten by the tile after next
             ptx::tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(acc_empty + 8 * acc);
+            if (lane == 0) ptx::mbar_arrive_cluster(ptx::leader_addr(acc_empty + 8 * acc));
         }
     }
 
     ptx::tc_fence_before_sync();
     __syncthreads();
+    ptx::cluster_sync();  // neither CTA's memory goes away under the other
     if (warp == 1) {
         ptx::tc_fence_after_sync();
-        ptx::tmem_dealloc(tmem_base, kTmemCols);
+        ptx::tmem_dealloc_pair(tmem_base, kTmemCols);
     }
 }
 
@@ -331,26 +345,21 @@ dalpha_reduce_kernel(int d_out, int d_in, int q, int g, int G, int HN, int split
 }
 
 struct DalphaPlan {
-    int TN, HN, splits, kb_per_split, num_kb, m_tiles, n_tiles, n_subtiles, slots;
+    int splits, kb_per_split, num_kb, m_tiles, n_tiles, n_subtiles, slots;
 };
 
 DalphaPlan plan_dalpha(int d_out, int d_in, int g, int n) {
     DalphaPlan pl;
-    const int sms = sm_count();
-    pl.m_tiles = ceil_div(d_out, kBlockM);
+    const int pairs = std::max(1, sm_count() / 2);
+    pl.m_tiles = ceil_div(d_out, kTM);
     pl.num_kb = ceil_div(n, kBlockK);
-    // The UMMA-issuing thread needs about 0.3 us per 64-token stage whatever the tile width, more
-    // than a 128 x 128 x 64 UMMA group takes to execute, so wide tiles (and a token split when
-    // they do not fill the SMs) beat twice as many narrow ones.
-    pl.TN = (d_in <= 128) ? 128 : 256;
-    pl.HN = pl.TN / 2;
-    pl.n_tiles = ceil_div(d_in, pl.TN);
+    pl.n_tiles = ceil_div(d_in, kTN);
     pl.n_subtiles = pl.n_tiles * 2;
-    if (g % pl.HN == 0) pl.slots = 1;
-    else if (pl.HN % g == 0) pl.slots = pl.HN / g;
-    else pl.slots = pl.HN / g + 2;
+    if (g % kHN == 0) pl.slots = 1;
+    else if (kHN % g == 0) pl.slots = kHN / g;
+    else pl.slots = kHN / g + 2;
     const int tiles = pl.m_tiles * pl.n_tiles;
-    int splits = sms / tiles;
+    int splits = pairs / tiles;
     if (splits < 1) splits = 1;
     const int max_splits = (pl.num_kb + 3) / 4;
     if (splits > max_splits) splits = max_splits;
@@ -360,16 +369,6 @@ DalphaPlan plan_dalpha(int d_out, int d_in, int g, int n) {
     return pl;
 }
 
-
-template <int TN>
-constexpr int stages_for() {
-    return TN == 256 ? 4 : 6;
-}
-
-template <int TN>
-constexpr size_t smem_for() {
-    return (size_t)stages_for<TN>() * (kABytes + TN * kBlockK * 2) + 1024 + 256;
-}
 
 size_t dalpha_ws_bytes(const DalphaPlan& pl, int d_out, int q) {
     return (size_t)pl.splits * pl.n_subtiles * q * pl.slots * d_out * sizeof(float);
@@ -424,29 +423,33 @@ extern "C" bcq_status bcq_linear_bwd_alpha(int d_out, int d_in, int q, int g, in
     p.m_tiles = pl.m_tiles; p.n_tiles = pl.n_tiles;
     p.n_subtiles = pl.n_subtiles; p.slots = pl.slots; p.plane_mask = plane_mask;
     p.bits = bits; p.partial = reinterpret_cast<float*>(ws);
-    p.direct = (pl.splits == 1 && g == pl.HN) ? 1 : 0;
+    p.direct = (pl.splits == 1 && g == kHN) ? 1 : 0;
     p.accumulate = accumulate; p.scale = scale; p.dalpha = dalpha;
     cudaStream_t s = (cudaStream_t)stream;
-    // persistent, one CTA per SM; every CTA gets the same number of tiles (as many as the busiest
+    // persistent, one CTA per SM; every pair gets the same number of tiles (as many as the busiest
     // would get anyway), which leaves whole SMs to other kernels instead of a ragged last wave
     const int tiles = pl.m_tiles * pl.n_tiles * pl.splits;
-    const int per_cta = ceil_div(tiles, sm_count());
-    const unsigned grid = (unsigned)ceil_div(tiles, per_cta);
-    if (pl.TN == 256) {
-        auto kern = dalpha_kernel<256, stages_for<256>()>;
-        if ((st = ensure_dynamic_smem(kern, smem_for<256>())) != BCQ_OK) return st;
-        kern<<<grid, kThreads, smem_for<256>(), s>>>(tm_dy, tm_x, p);
-    } else {
-        auto kern = dalpha_kernel<128, stages_for<128>()>;
-        if ((st = ensure_dynamic_smem(kern, smem_for<128>())) != BCQ_OK) return st;
-        kern<<<grid, kThreads, smem_for<128>(), s>>>(tm_dy, tm_x, p);
-    }
+    const int per_pair = ceil_div(tiles, std::max(1, sm_count() / 2));
+    if ((st = ensure_dynamic_smem(dalpha_kernel, kDalphaSmem)) != BCQ_OK) return st;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2u * (unsigned)ceil_div(tiles, per_pair));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kDalphaSmem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    BCQ_CUDA_TRY(cudaLaunchKernelEx(&cfg, dalpha_kernel, tm_dy, tm_x, p));
     bcq::count_launch();
     BCQ_CUDA_TRY(cudaGetLastError());
     if (p.direct) return BCQ_OK;
     const long long rblocks = (long long)q * p.G * ((d_out + 31) / 32);
     dalpha_reduce_kernel<<<(unsigned)rblocks, 256, 0, s>>>(
-        d_out, d_in, q, g, p.G, pl.HN, pl.splits, pl.n_subtiles, pl.slots, plane_mask, scale, accumulate,
+        d_out, d_in, q, g, p.G, kHN, pl.splits, pl.n_subtiles, pl.slots, plane_mask, scale, accumulate,
         p.partial, dalpha);
     bcq::count_launch();
     BCQ_CUDA_TRY(cudaGetLastError());

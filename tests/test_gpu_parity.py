@@ -229,6 +229,17 @@ def test_bwd_alpha_matches_oracle(n, d_in, d_out, q, g):
     assert np.abs(o[0] - 3.0 - ref[0] / g).max() <= TOL * np.abs(ref[0] / g).max() + 1e-6
 
 
+@pytest.mark.parametrize("n,d_in,d_out,q,g", [(65, 40, 136, 2, 40), (64, 64, 256, 3, 32), (127, 136, 264, 1, 136),
+                                              (200, 320, 384, 4, 64), (640, 456, 104, 2, 128)])
+def test_bwd_alpha_partial_tiles_of_a_cta_pair(n, d_in, d_out, q, g):
+    # last column tiles of 64, 128 and 192 columns (32, 64 and 96 in each CTA of the pair), and row tiles
+    # that hold rows for one CTA of the pair only
+    _, X, dY, bits, alpha, _, _ = make_case(40 + n, n, d_in, d_out, q, g)
+    Xd, dYd, bd, _ = _upload(X, dY, bits, alpha)
+    ref = oracle.bwd_alpha(dY, X, bits, d_in, g)
+    assert rel_err(bcq.linear_bwd_alpha(dYd, Xd, bd, d_in, g).cpu().numpy(), ref) <= TOL
+
+
 @pytest.mark.parametrize("n", [1, 4, 16, 5])
 @pytest.mark.parametrize("d_in,d_out,q,g", [(4096, 1536, 3, 128), (1024, 520, 4, 128), (2048, 256, 3, 2048)])
 def test_decode_matches_oracle(n, d_in, d_out, q, g):
