@@ -27,6 +27,7 @@
 //     of every byte as 0,2,4,6,1,3,5,7, so that the expanded tile is in natural k order.  Decode
 //     has no pre-pass: there the tile keeps the PRMT order and the workers write the activations
 //     in the same order.
+#include <algorithm>
 #include <mutex>
 
 #include "gemm_common.cuh"
@@ -254,7 +255,7 @@ struct WsHeader {
 
 // Power of two for the weights: q * max|alpha| lands in [2^13, 2^14).  Called by whole warps.
 __device__ __forceinline__ int weight_shift(const WsHeader* hdr, int q) {
-    const int nb = (int)__ldg(&hdr->nblocks);
+    const int nb = (int)min(__ldg(&hdr->nblocks), (uint32_t)kMaxAlphaBlocks);  // never past the header
     uint32_t m = 0u;
     for (int b = threadIdx.x & 31; b < nb; b += 32) m = max(m, __ldg(&hdr->block_max[b]));
 #pragma unroll
@@ -541,12 +542,13 @@ struct ExpandParams {
     int num_kb;        // K blocks of 64 over d_in (fwd) or d_out (dX)
     int kb_per_split;
     int splits;
-    int m_tiles, n_tiles;
+    int m_tiles;           // row tiles of 128 of the regrouped planes
+    int m_pairs, n_tiles;  // output tiles: pairs of row tiles, token tiles
     int tn;                // token tile width
     uint32_t acc_cols;     // tensor-memory columns per accumulator
     // pipeline geometry (chosen on the host)
     int a_slots;           // ring of expanded weight tiles (16 KiB each), >= the number of worker groups
-    int b_slots;           // ring of activation tiles (TN x 128 B each), filled by TMA
+    int b_slots;           // ring of activation tiles (TN / 2 x 128 B each), filled by TMA
     int epi_bufs;          // staging buffers per epilogue warp: 1 or 2
     uint32_t chunk_words;  // words of one stage's chunk of the regrouped planes
     const uint32_t* bits_t;      // regrouped plane words (see PrepParams)
@@ -576,35 +578,46 @@ struct StageLayout {
     static constexpr uint32_t kStageBytes = kBitsOff + kBitsBytes;
 };
 
-// Prefill kernel.  Persistent: every CTA walks over output tiles (m-tile fastest, so that CTAs
-// running at the same time share activation tiles in L2).  32 warps:
-//   warps 0..11   workers in three groups of four; group g takes the pipeline stages whose running
-//                 index is g mod 3.  A thread expands 64 weights of one row per stage (one 128-byte
-//                 line of the operand tile), so a group rebuilds one 128 x 64 weight tile.  The
-//                 thread reads its selector codes (or plane words) and scales straight from the
-//                 regrouped arrays in global memory, one task ahead of the one it expands, so the
-//                 loads are hidden behind a whole turn of the group
-//   warp 12       UMMA issuer, owner of the tensor-memory allocation (two accumulators)
-//   warp 13       producer of the activation tiles (TMA)
+// Prefill kernel.  Persistent: every pair of CTAs walks over output tiles of 256 rows x TN tokens (rows
+// fastest, so that pairs running at the same time share activation tiles in L2).  A pair, because
+// shared memory bounds a CTA alone: per 64-wide stage of a 128 x 256 tile (512 tensor-core cycles) the
+// workers write 16 KiB, TMA writes 32 KiB and the tensor core reads 48 KiB, 768 cycles at 128 bytes a
+// cycle (measured: 755 - 820 cycles a stage).  In a pair each CTA expands its own 128 rows but holds
+// only half of the tokens: 512 cycles (measured: 600 - 700, now set by the workers).
+// Each CTA has 22 warps:
+//   warps 0..15   workers in four groups of four; group g takes the pipeline stages whose running
+//                 index is g mod 4 (the workers set the pace by latency, not by issue rate: 6400 -> 1600
+//                 with 4096 tokens takes 106 us with three groups, 97 with four, 100 with five).  A
+//                 thread expands 64 weights of one row per stage (one 128-byte line of the operand
+//                 tile), so a group rebuilds one 128 x 64 weight tile.  The thread reads its selector
+//                 codes (or plane words) and scales straight from the regrouped arrays in global
+//                 memory, one task ahead of the one it expands, so the loads are hidden behind a
+//                 whole turn of the group
 //   warps 16..19  epilogue: drain one accumulator while the main loop fills the other (warp w
 //                 reaches the tensor-memory lanes 32 * (w % 4) .. + 31)
-// Shared memory: a ring of weight tiles (16 KiB each; few, the workers refill one as soon as the
-// tensor core is done with it), a deeper ring of activation tiles (TN x 128 B each; a TMA load
-// takes about a microsecond to land), the epilogue's staging, barriers and output scales.
-constexpr int kPfGroups = 3;
+//   warp 20       owner of the tensor-memory allocation (two accumulators); in the leader of the
+//                 pair, UMMA issuer for both CTAs
+//   warp 21       producer of this CTA's half of the activation tiles (TMA)
+// Shared memory: a ring of weight tiles (16 KiB each; the workers refill one as soon as the tensor core
+// is done with it), a ring of activation tiles (TN / 2 x 128 B each; a TMA load takes about a
+// microsecond to land), the epilogue's staging, barriers and output scales.  The barriers "operand
+// in place" and "accumulator drained" are the leader's and count both CTAs; the others exist in both
+// CTAs and are signalled by one commit to both.
+constexpr int kPfGroups = 4;
 constexpr int kPfGroupWarps = 4;
-constexpr int kPfWorkerWarps = kPfGroups * kPfGroupWarps;  // 12
-constexpr int kPfMmaWarp = kPfWorkerWarps;                 // 12
-constexpr int kPfProdWarp = kPfMmaWarp + 1;                // 13
-constexpr int kPfEpiWarp0 = 16;
+constexpr int kPfWorkerWarps = kPfGroups * kPfGroupWarps;  // 16
+constexpr int kPfEpiWarp0 = kPfWorkerWarps;
 constexpr int kPfEpiWarps = 4;
-constexpr int kPfWarps = kPfEpiWarp0 + kPfEpiWarps;        // 20
-constexpr int kPfThreads = kPfWarps * 32;                  // 640
+constexpr int kPfMmaWarp = kPfEpiWarp0 + kPfEpiWarps;
+constexpr int kPfProdWarp = kPfMmaWarp + 1;
+constexpr int kPfThreads = (kPfProdWarp + 1) * 32;         // 704
 static_assert(kPfEpiWarp0 % 4 == 0, "epilogue warp e must sit on tensor-memory lane quarter e");
 __device__ __forceinline__ int pf_worker_index(int warp) { return warp < kPfWorkerWarps ? warp : -1; }
-__device__ __forceinline__ int pf_epilogue_index(int warp) { return warp >= kPfEpiWarp0 ? warp - kPfEpiWarp0 : -1; }
+__device__ __forceinline__ int pf_epilogue_index(int warp) {
+    return warp >= kPfEpiWarp0 && warp < kPfEpiWarp0 + kPfEpiWarps ? warp - kPfEpiWarp0 : -1;
+}
 constexpr int kPfMaxSlots = 8;                                // per ring
-constexpr uint32_t kPfGroupBar0 = 4;                           // named barriers 4, 5, 6: one per worker group
+constexpr uint32_t kPfGroupBar0 = 4;                           // named barriers 4..7: one per worker group
 constexpr uint32_t kPfCtlBytes = 384;                          // barriers, TMEM handle, abort flag
 constexpr uint32_t kPfScaleBytes = 256 * 4;                    // [TN] output scales of the tile being drained
 constexpr uint32_t kPfStagingBuf = kPfEpiWarps * 1024;         // per epilogue warp one 1 KiB buffer of 32 rows x 16 bf16 (8 fp32) tokens; one or two such sets
@@ -614,14 +627,14 @@ __global__ void __launch_bounds__(kPfThreads, 1)
 expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant__ CUtensorMap tmap_out,
                    const ExpandParams p) {
     const int TN = p.tn;                                   // token tile: a multiple of 16, <= 256
-    const uint32_t kBBytes = (uint32_t)TN * kBlockK * 2;
+    const uint32_t kBBytes = (uint32_t)(TN / 2) * kBlockK * 2;  // this CTA's half of the tokens
     const uint32_t kAccCols = p.acc_cols;                  // tensor-memory columns of one accumulator
     const uint32_t kTmemCols = 2 * kAccCols;               // a power of two >= 32
     constexpr int kRows = (MODE == MODE_FWD) ? 128 : 64;  // weight rows of one stage
     constexpr int kUnit = (MODE == MODE_FWD) ? 2 : 4;     // 32-weight blocks per row and stage
     constexpr int NW = NumWords<QM>::value;
     // fp16 x fp16 -> fp32; A is MN-major for dX
-    const uint32_t kIdesc = (ptx::make_idesc_bf16(kBlockM, TN, MODE == MODE_BWDX ? 1 : 0, 0)) &
+    const uint32_t kIdesc = (ptx::make_idesc_bf16(2 * kBlockM, TN, MODE == MODE_BWDX ? 1 : 0, 0)) &
                             ~((1u << 7) | (1u << 10));
 
     extern __shared__ uint8_t smem_raw[];
@@ -650,19 +663,21 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
+    const int rank = (int)ptx::cluster_rank();
+    const int pair0 = (int)blockIdx.x >> 1, num_pairs = (int)gridDim.x >> 1;
 
     if (warp == 0) {
         // the barriers are initialised by the lanes of one warp side by side (one after the other
         // they cost a few tenths of a microsecond before any copy can start)
         if (lane < NA) {
-            ptx::mbar_init(ctl.aready + 8 * lane, kPfGroupWarps);
+            ptx::mbar_init(ctl.aready + 8 * lane, 2 * kPfGroupWarps);
             ptx::mbar_init(ctl.empty + 8 * lane, 1);
         } else if (lane >= 8 && lane < 8 + NB) {
             ptx::mbar_init(ctl.full + 8 * (lane - 8), 1);
             ptx::mbar_init(b_empty + 8 * (lane - 8), 1);
         } else if (lane >= 16 && lane < 18) {
             ptx::mbar_init(ctl.accum + 8 * (lane - 16), 1);
-            ptx::mbar_init(acc_empty + 8 * (lane - 16), kPfEpiWarps);
+            ptx::mbar_init(acc_empty + 8 * (lane - 16), 2 * kPfEpiWarps);
         } else if (lane == 18) {
             ptx::mbar_init(ctl.spare, 1);
             *ctl.abort_flag = 0;
@@ -671,22 +686,24 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
             if (p.fast_epi) ptx::prefetch_tmap(&tmap_out);
         }
         ptx::fence_mbar_init();
+        __syncwarp();
     }
     if (warp == kPfMmaWarp) {
-        ptx::tmem_alloc(ptx::smem_u32(const_cast<uint32_t*>(tmem_holder)), kTmemCols);
-        ptx::tmem_relinquish();
+        ptx::tmem_alloc_pair(ptx::smem_u32(const_cast<uint32_t*>(tmem_holder)), kTmemCols);
+        ptx::tmem_relinquish_pair();
     }
     ptx::tc_fence_before_sync();
     __syncthreads();
+    ptx::cluster_sync();  // the peer's barriers exist
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_holder;
 
     // every role walks the same sequence of tiles and pipeline stages
-    const int num_tiles = p.m_tiles * p.n_tiles * p.splits;
+    const int num_tiles = p.m_pairs * p.n_tiles * p.splits;
     auto tile_coords = [&](int tile, int& m0, int& t0, int& z, int& kb_begin, int& iters) {
-        const int mt = tile % p.m_tiles;
-        const int rest = tile / p.m_tiles;
-        m0 = mt * kBlockM;
+        const int mt = tile % p.m_pairs;
+        const int rest = tile / p.m_pairs;
+        m0 = (2 * mt + rank) * kBlockM;
         t0 = (rest % p.n_tiles) * TN;
         z = rest / p.n_tiles;
         kb_begin = z * p.kb_per_split;
@@ -726,50 +743,42 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
         }
     };
     // On the last tile of a CTA the worker warps have nothing left to expand, so they share its
-    // epilogue: of the four warps on a tensor-memory lane quarter (one epilogue warp, three workers)
-    // warp h takes the boxes h, h + 4, ...
-    constexpr int kPfHelpers = 1 + kPfWorkerWarps / 4;  // 4
-    auto is_last_tile = [&](int tile) { return tile + (int)gridDim.x >= num_tiles; };
+    // epilogue: of the five warps on a tensor-memory lane quarter (one epilogue warp, four workers)
+    // warp h takes the boxes h, h + 5, ...
+    constexpr int kPfHelpers = 1 + kPfWorkerWarps / 4;  // 5
+    auto is_last_tile = [&](int tile) { return tile + num_pairs >= num_tiles; };
 
     if (warp == kPfProdWarp) {
         // ---------------- producer: the activation tile of every stage (TMA), into a ring of its
         // own that runs as far ahead of the tensor core as shared memory allows
         if (lane == 0) {
             bool ok = true;
-            int s = 0, in_flight = 0;
+            int s = 0;
             uint32_t ph = 0;
-            for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+            for (int tile = pair0; tile < num_tiles && ok; tile += num_pairs) {
                 int m0, t0, z, kb_begin, iters;
                 tile_coords(tile, m0, t0, z, kb_begin, iters);
                 for (int it = 0; it < iters; ++it) {
                     ok = wait_bar(b_empty + 8 * s, ph ^ 1u, ctl, 1, 256u);
                     if (!ok) break;
-                    const uint32_t bar = ctl.full + 8 * s;
-                    ptx::mbar_arrive_expect_tx(bar, kBBytes);
-                    ptx::tma_load_2d(b_base + s * kBBytes, &tmap_b, (kb_begin + it) * kBlockK, t0, bar);
-                    in_flight = min(in_flight + 1, NB);
+                    if (rank == 0) ptx::mbar_arrive_expect_tx(ctl.full + 8 * s, 2u * kBBytes);
+                    ptx::tma_load_2d_pair(b_base + s * kBBytes, &tmap_b, (kb_begin + it) * kBlockK, t0 + rank * (TN / 2),
+                                          ptx::leader_addr(ctl.full + 8 * s));
                     if (++s == NB) { s = 0; ph ^= 1u; }
                 }
             }
-            if (!ok) {
-                // giving up: let the copies already issued land before the CTA exits.  The last
-                // `in_flight` slots before (s, ph) were issued with the phase they had then.
-                int bs = s;
-                uint32_t bph = ph;
-                for (int i = 0; i < in_flight; ++i) {
-                    if (bs == 0) { bs = NB; bph ^= 1u; }
-                    --bs;
-                    wait_bar(ctl.full + 8 * bs, bph, ctl, 2);
-                }
-            }
+            // giving up: the copies in flight are counted on the leader's barriers, which may never
+            // complete; they land within microseconds, so wait a thousand times as long
+            if (!ok) for (int i = 0; i < 1000; ++i) __nanosleep(2000);
         }
+        __syncwarp();
     } else if (warp == kPfMmaWarp) {
         // ---------------- UMMA issuer.  One elected thread runs the whole loop: per stage it has
         // to get through two barrier checks, a fence, four UMMAs and two commits in less time
         // than the tensor core needs for the stage (512 cycles at the full width), so nothing
         // warp-wide (election, reconvergence) is left inside the loop and the two barrier checks
         // are issued together.
-        if (ptx::elect_one()) {
+        if (rank == 0 && ptx::elect_one()) {
             bool ok = true;
             int sa = 0, sb = 0, lt = 0;
             uint32_t pha = 0, phb = 0;
@@ -782,7 +791,7 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
             constexpr uint32_t kAStep = (MODE == MODE_FWD) ? (32u >> 4) : (2048u >> 4);
             const uint32_t a_lo0 = ((smem_base >> 4) & 0x3FFFu) | kALoExtra;
             const uint32_t b_lo0 = ((b_base >> 4) & 0x3FFFu) | kBLoExtra;
-            for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++lt) {
+            for (int tile = pair0; tile < num_tiles && ok; tile += num_pairs, ++lt) {
                 int m0, t0, z, kb_begin, iters;
                 tile_coords(tile, m0, t0, z, kb_begin, iters);
                 const int acc = lt & 1;
@@ -805,24 +814,24 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
                     const uint32_t b_lo = b_lo0 + (uint32_t)sb * (kBBytes >> 4);
 #pragma unroll
                     for (int kk = 0; kk < kBlockK / 16; ++kk)
-                        ptx::umma_f16_halves(d_tmem, a_lo + kk * kAStep, kAHi, b_lo + kk * 2, kBHi, kIdesc,
-                                             (it > 0 || kk > 0) ? 1u : 0u);
-                    ptx::umma_commit(ctl.empty + 8 * sa);
-                    ptx::umma_commit(b_empty + 8 * sb);
+                        ptx::umma_f16_pair(d_tmem, a_lo + kk * kAStep, kAHi, b_lo + kk * 2, kBHi, kIdesc,
+                                           (it > 0 || kk > 0) ? 1u : 0u);
+                    ptx::umma_commit_pair(ctl.empty + 8 * sa);
+                    ptx::umma_commit_pair(b_empty + 8 * sb);
                     if (++sa == NA) { sa = 0; pha ^= 1u; }
                     if (++sb == NB) { sb = 0; phb ^= 1u; }
                 }
-                if (ok) ptx::umma_commit(ctl.accum + 8 * acc);
+                if (ok) ptx::umma_commit_pair(ctl.accum + 8 * acc);
             }
             if (!ok) {
-                ptx::umma_commit(ctl.spare);
+                ptx::umma_commit_pair(ctl.spare);
                 wait_bar(ctl.spare, 0, ctl, 5);
             }
         }
         __syncwarp();
     } else if (pf_worker_index(warp) >= 0) {
         // ---------------- workers
-        const int wid = pf_worker_index(warp);  // 0..11
+        const int wid = pf_worker_index(warp);  // 0..15
         const int group = wid / kPfGroupWarps;  // takes the stages whose running index is `group` mod kPfGroups
         const int wl = wid % kPfGroupWarps;
         const float wscale = pow2f(weight_shift(p.hdr, p.q));
@@ -861,7 +870,7 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
         auto enter_tile = [&](Cur& x) {
             int m0, t0, z;
             tile_coords(x.tile, m0, t0, z, x.kb_begin, x.iters);
-            x.mt = m0 >> 7;
+            x.mt = min(m0 >> 7, p.m_tiles - 1);  // a pair whose second row tile does not exist expands the first again
         };
         const uint32_t code_step = kPfGroups * chunk_words;
         const uint32_t alpha_step = kPfGroups * (uint32_t)p.G * alpha_block;  // dX: the next task's rows
@@ -880,7 +889,7 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
             bool moved = false;
             while (x.it >= x.iters) {
                 x.it -= x.iters;
-                x.tile += gridDim.x;
+                x.tile += num_pairs;
                 if (x.tile >= num_tiles) { x.valid = false; return; }
                 enter_tile(x);
                 moved = true;
@@ -983,14 +992,14 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
             }
             ptx::fence_proxy_async_smem();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(ctl.aready + 8 * s);
+            if (lane == 0) ptx::mbar_arrive_cluster(ptx::leader_addr(ctl.aready + 8 * s));
             s += kPfGroups;
             if (s >= NA) { s -= NA; ph ^= 1u; }
             return true;
         };
 
         Cur cur;
-        cur.tile = (int)blockIdx.x;
+        cur.tile = pair0;
         cur.valid = cur.tile < num_tiles;
         cur.fresh = true;
         cur.split = false;
@@ -1001,7 +1010,7 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
             enter_tile(cur);
             while (cur.it >= cur.iters) {
                 cur.it -= cur.iters;
-                cur.tile += gridDim.x;
+                cur.tile += num_pairs;
                 if (cur.tile >= num_tiles) { cur.valid = false; break; }
                 enter_tile(cur);
             }
@@ -1033,18 +1042,18 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
                 cur = nxt;
             }
         }
-        if (p.helpers && ok && (int)blockIdx.x < num_tiles) {
+        if (p.helpers && ok && pair0 < num_tiles) {
             // share the epilogue of this CTA's last tile.  Its operand slots are free once the
             // accumulator is complete, so each warp stages its boxes in 1 KiB of the first slots.
-            const int lt = (num_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x;
-            const int tile = (int)blockIdx.x + lt * (int)gridDim.x;
+            const int lt = (num_tiles - 1 - pair0) / num_pairs;
+            const int tile = pair0 + lt * num_pairs;
             int m0, t0, z, kb_begin, iters;
             tile_coords(tile, m0, t0, z, kb_begin, iters);
             const int acc = lt & 1;
             ok = wait_bar(ctl.accum + 8 * acc, (uint32_t)(lt >> 1) & 1u, ctl, 10);
             if (ok) {
                 ptx::tc_fence_after_sync();
-                const int quarter = warp & 3, helper = 1 + (warp >> 2);  // 1..3
+                const int quarter = warp & 3, helper = 1 + (warp >> 2);  // 1..4
                 const int m0w = m0 + quarter * 32;
                 const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)acc * kAccCols;
                 const uint32_t buf = smem_base + (uint32_t)warp * 1024u;
@@ -1086,7 +1095,7 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
         bool ok = true;
         int lt = 0;
         uint32_t chunks = 0;  // output boxes stored so far (fast path): selects the staging buffer
-        for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++lt) {
+        for (int tile = pair0; tile < num_tiles && ok; tile += num_pairs, ++lt) {
             int m0, t0, z, kb_begin, iters;
             tile_coords(tile, m0, t0, z, kb_begin, iters);
             const int acc = lt & 1;
@@ -1193,16 +1202,17 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
             // the accumulator (and this tile's scale row) may be reused
             ptx::tc_fence_before_sync();
             asm volatile("bar.sync 2, %0;" ::"n"(kPfEpiWarps * 32) : "memory");
-            if (lane == 0) ptx::mbar_arrive(acc_empty + 8 * acc);
+            if (lane == 0) ptx::mbar_arrive_cluster(ptx::leader_addr(acc_empty + 8 * acc));
         }
         if (p.fast_epi && lane == 0) ptx::bulk_wait_group<0>();  // all output boxes written before the CTA ends
     }
 
     ptx::tc_fence_before_sync();
     __syncthreads();
+    ptx::cluster_sync();  // neither CTA's memory goes away under the other
     if (warp == kPfMmaWarp) {
         ptx::tc_fence_after_sync();
-        ptx::tmem_dealloc(tmem_base, kTmemCols);
+        ptx::tmem_dealloc_pair(tmem_base, kTmemCols);
     }
 }
 
@@ -1503,7 +1513,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tmap_bits, const DecodeParams 
 // ------------------------------------------------------------------------------------------
 
 struct ExpandPlan {
-    int TN, splits, kb_per_split, num_kb, m_tiles, n_tiles;
+    int TN, splits, kb_per_split, num_kb, m_tiles, m_pairs, n_tiles;
     int a_slots, b_slots, epi_bufs;
     uint32_t bits_bytes, alpha_bytes;                                    // one stage's chunk of the planes; the scales of one (row block, group)
     size_t planes_bytes;                                                 // the regrouped planes (codes for q <= 4)
@@ -1513,7 +1523,6 @@ struct ExpandPlan {
 };
 
 constexpr int kPfStageFixed = 224;                                     // fixed cost of a pipeline stage, in token-tile columns
-constexpr size_t kSmemLimit = 232448;                                   // 227 KiB per CTA
 constexpr size_t kPfFixedBytes = 1024 + kPfCtlBytes + kPfScaleBytes;   // alignment slack, barriers, output scales
 
 // Tile width over tokens, the K split and the pipeline geometry.  Wide token tiles amortise the
@@ -1521,11 +1530,12 @@ constexpr size_t kPfFixedBytes = 1024 + kPfCtlBytes + kPfScaleBytes;   // alignm
 // tiles.
 ExpandPlan plan_expand(int mode, int d_out, int d_in, int q, int g, int n) {
     ExpandPlan pl;
-    const int sms = sm_count();
+    const int pairs = std::max(1, sm_count() / 2);
     const int Mdim = (mode == MODE_FWD) ? d_out : d_in;
     const int Kdim = (mode == MODE_FWD) ? d_in : d_out;
     const int G = (int)bcq_num_groups(d_in, g);
     pl.m_tiles = ceil_div(Mdim, kBlockM);
+    pl.m_pairs = ceil_div(pl.m_tiles, 2);
     pl.num_kb = ceil_div(Kdim, kBlockK);
     int tn;
     if (n <= 32) tn = 32;
@@ -1542,8 +1552,8 @@ ExpandPlan plan_expand(int mode, int d_out, int d_in, int q, int g, int n) {
         long long best = -1;
         tn = 256;
         for (int c = 256; c >= 128; c -= 16) {
-            const long long tiles = (long long)pl.m_tiles * ceil_div(n, c);
-            const long long per_cta = (tiles + sms - 1) / sms;
+            const long long tiles = (long long)pl.m_pairs * ceil_div(n, c);
+            const long long per_cta = (tiles + pairs - 1) / pairs;
             const long long stage = c + kPfStageFixed;
             const long long cost = (per_cta * stage) * (tiles * stage);
             if (best < 0 || cost < best) { best = cost; tn = c; }
@@ -1551,10 +1561,10 @@ ExpandPlan plan_expand(int mode, int d_out, int d_in, int q, int g, int n) {
     }
     pl.TN = tn;
     pl.n_tiles = ceil_div(n, tn);
-    const int tiles = pl.m_tiles * pl.n_tiles;
+    const int tiles = pl.m_pairs * pl.n_tiles;
     // The K split goes through fp32 partials, a slower epilogue and a second kernel: only for
     // problems that would otherwise leave most of the SMs idle.
-    int splits = (4 * tiles <= sms) ? sms / tiles : 1;
+    int splits = (4 * tiles <= pairs) ? pairs / tiles : 1;
     if (splits < 1) splits = 1;
     const int max_splits = (pl.num_kb + 3) / 4;  // at least 4 K blocks per CTA
     if (splits > max_splits) splits = max_splits;
@@ -1565,24 +1575,14 @@ ExpandPlan plan_expand(int mode, int d_out, int d_in, int q, int g, int n) {
     const int rows = (mode == MODE_FWD) ? 128 : 64;
     pl.bits_bytes = (q <= 3 ? 3u : (uint32_t)q) * 1024u;  // q <= 4: selector codes (3 or 4 words per 32 weights)
     pl.alpha_bytes = (uint32_t)(q * rows * 4);
-    // Shared memory.  A worker group takes a few hundred nanoseconds from "the tensor core is done
-    // with my slot" to "the slot holds the next tile", and a TMA load about a microsecond to land;
-    // both rings must be deep enough to cover that at one stage per ~0.3 us.  First choice that fits:
-    const size_t b_bytes = (size_t)tn * kBlockK * 2;
-    auto smem_of = [&](int a_slots, int b_slots, int epi_bufs) {
-        return a_slots * (size_t)kABytes + b_slots * b_bytes + epi_bufs * (size_t)kPfStagingBuf + kPfFixedBytes;
-    };
-    const int rings[8][2] = {{6, 5}, {5, 5}, {6, 4}, {5, 4}, {4, 4}, {4, 3}, {3, 3}, {3, 2}};
+    // Shared memory.  A worker group takes about a microsecond from "the tensor core is done with my
+    // slot" to "the slot holds the next tile", and a TMA load as long to land; both rings must be deep
+    // enough to cover that at one stage per ~0.3 us.  These fit at every token-tile width.
     pl.epi_bufs = 2;
-    pl.a_slots = kPfGroups;
-    pl.b_slots = 2;
-    for (int r = 0; r < 8; ++r)
-        if (smem_of(rings[r][0], rings[r][1], pl.epi_bufs) <= kSmemLimit) {
-            pl.a_slots = rings[r][0];
-            pl.b_slots = rings[r][1];
-            break;
-        }
-    pl.smem = smem_of(pl.a_slots, pl.b_slots, pl.epi_bufs);
+    pl.a_slots = 6;
+    pl.b_slots = 6;
+    pl.smem = pl.a_slots * (size_t)kABytes + pl.b_slots * (size_t)(tn / 2) * kBlockK * 2 +
+              pl.epi_bufs * (size_t)kPfStagingBuf + kPfFixedBytes;
 
     const size_t chunks_bits = (size_t)pl.m_tiles * pl.num_kb;                       // [m_tile][kb] or [u][jb]
     const size_t blocks_alpha = (size_t)((mode == MODE_FWD) ? pl.m_tiles : pl.num_kb) * G;  // [m_tile][G] or [jb][G]
@@ -1631,13 +1631,24 @@ bcq_status launch_expand(const CUtensorMap& tm, const CUtensorMap& tmo, const Ex
     auto kern = expand_gemm_kernel<MODE, QM>;
     bcq_status st0 = ensure_dynamic_smem(kern, pl.smem);
     if (st0 != BCQ_OK) return st0;
-    const int tiles = pl.m_tiles * pl.n_tiles * pl.splits;
-    // persistent, at most one CTA per SM; with more tiles than SMs every CTA gets the same number of
+    const int tiles = pl.m_pairs * pl.n_tiles * pl.splits;
+    // persistent, at most one CTA per SM; with more tiles than pairs every pair gets the same number of
     // tiles (as many as the busiest would get anyway): fewer CTAs pay the prologue, more epilogues
     // overlap the next tile's main loop, and the SMs left over can run other kernels
-    const int per_cta = ceil_div(tiles, sm_count());
-    const int grid = ceil_div(tiles, per_cta);
-    kern<<<grid, kPfThreads, pl.smem, stream>>>(tm, tmo, p);
+    const int per_pair = ceil_div(tiles, std::max(1, sm_count() / 2));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2u * (unsigned)ceil_div(tiles, per_pair));
+    cfg.blockDim = dim3(kPfThreads);
+    cfg.dynamicSmemBytes = pl.smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    BCQ_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, tm, tmo, p));
     bcq::count_launch();
     BCQ_CUDA_TRY(cudaGetLastError());
     return BCQ_OK;
@@ -1692,7 +1703,7 @@ bcq_status run_expand(int d_out, int d_in, int q, int g, int n, const void* act,
     const int pitch = (int)bcq_pitch_words(d_in);
 
     CUtensorMap tm;
-    bcq_status st = make_tmap_16bit(&tm, act16, 1, pl.ld_act, n, (size_t)pl.ld_act, pl.TN);
+    bcq_status st = make_tmap_16bit(&tm, act16, 1, pl.ld_act, n, (size_t)pl.ld_act, pl.TN / 2);
     if (st != BCQ_OK) return st;
 
     // everything that can fail is done before the first launch: the output tensor map and the
@@ -1747,7 +1758,7 @@ bcq_status run_expand(int d_out, int d_in, int q, int g, int n, const void* act,
     p.G = (int)bcq_num_groups(d_in, g);
     p.pitch = pitch;
     p.n = n; p.Mdim = Mdim; p.num_kb = pl.num_kb; p.kb_per_split = pl.kb_per_split; p.splits = pl.splits;
-    p.m_tiles = pl.m_tiles; p.n_tiles = pl.n_tiles;
+    p.m_tiles = pl.m_tiles; p.m_pairs = pl.m_pairs; p.n_tiles = pl.n_tiles;
     p.tn = pl.TN;
     p.acc_cols = 32;
     while ((int)p.acc_cols < pl.TN) p.acc_cols *= 2;
