@@ -285,6 +285,8 @@ struct PrepParams {
     const uint32_t* bits;
     float* alpha_t;
     uint32_t* bits_t;
+    uint32_t* counters;  // zeroed for the GEMM kernel (arrivals at tiles that several pairs share)
+    int num_counters;
 };
 
 // One warp per token row; VPL = 16-byte vectors a lane keeps in registers between finding the
@@ -434,6 +436,8 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
     }
     if (bid >= p.act_blocks) {
         // ---- max |alpha| of this block's share of the scales
+        if (bid == p.act_blocks)
+            for (int i = threadIdx.x; i < p.num_counters; i += 256) p.counters[i] = 0u;
         const long long nb = p.amax_blocks;
         uint32_t m = 0u;
         for (long long o = ((long long)bid - p.act_blocks) * 256 + threadIdx.x; o < p.alpha_count;
@@ -540,8 +544,9 @@ struct ExpandParams {
     int d_out, d_in, q, g, G, pitch, n;
     int Mdim;          // d_out (fwd) or d_in (dX)
     int num_kb;        // K blocks of 64 over d_in (fwd) or d_out (dX)
-    int kb_per_split;
-    int splits;
+    // The first full_tiles output tiles go whole to the pairs in turn; the res_tiles tiles after them
+    // are cut into `pieces` pieces of piece_len stages, one for each of the first res_tiles * pieces pairs
+    int full_tiles, res_tiles, pieces, piece_len;
     int m_tiles;           // row tiles of 128 of the regrouped planes
     int m_pairs, n_tiles;  // output tiles: pairs of row tiles, token tiles
     int tn;                // token tile width
@@ -549,7 +554,6 @@ struct ExpandParams {
     // pipeline geometry (chosen on the host)
     int a_slots;           // ring of expanded weight tiles (16 KiB each), >= the number of worker groups
     int b_slots;           // ring of activation tiles (TN / 2 x 128 B each), filled by TMA
-    int epi_bufs;          // staging buffers per epilogue warp: 1 or 2
     uint32_t chunk_words;  // words of one stage's chunk of the regrouped planes
     const uint32_t* bits_t;      // regrouped plane words (see PrepParams)
     const float* alpha_t;        // regrouped scales
@@ -561,7 +565,8 @@ struct ExpandParams {
     int out_bf16;
     int fast_epi;                // bf16 output written by TMA stores (aligned base and pitch, no K split)
     int helpers;                 // the worker warps share the epilogue of a CTA's last tile (see run_expand)
-    float* partial;              // [splits][n][Mdim] when splits > 1
+    float* partial;              // [pair][rank][TN columns][128 rows]
+    uint32_t* counters;          // [shared tile][rank][quarter][box class]
 };
 
 // One pipeline stage in shared memory: | A tile 16 KiB | B tile TN x 128 B | plane words |.
@@ -603,6 +608,12 @@ struct StageLayout {
 // microsecond to land), the epilogue's staging, barriers and output scales.  The barriers "operand
 // in place" and "accumulator drained" are the leader's and count both CTAs; the others exist in both
 // CTAs and are signalled by one commit to both.
+//
+// Where a ragged last wave of tiles (or a problem with few tiles) would leave at least half of the pairs
+// idle, its tiles are cut along K into as many pieces as there are pairs for; a pair does its piece
+// first.  It writes its fp32 sums to the workspace, and for each box of the output the warp that arrives
+// last (a counter) adds the pieces in order and writes the result, so no warp waits for another and the
+// result does not depend on which one is last.
 constexpr int kPfGroups = 4;
 constexpr int kPfGroupWarps = 4;
 constexpr int kPfWorkerWarps = kPfGroups * kPfGroupWarps;  // 16
@@ -620,7 +631,7 @@ constexpr int kPfMaxSlots = 8;                                // per ring
 constexpr uint32_t kPfGroupBar0 = 4;                           // named barriers 4..7: one per worker group
 constexpr uint32_t kPfCtlBytes = 384;                          // barriers, TMEM handle, abort flag
 constexpr uint32_t kPfScaleBytes = 256 * 4;                    // [TN] output scales of the tile being drained
-constexpr uint32_t kPfStagingBuf = kPfEpiWarps * 1024;         // per epilogue warp one 1 KiB buffer of 32 rows x 16 bf16 (8 fp32) tokens; one or two such sets
+constexpr uint32_t kPfStagingBuf = kPfEpiWarps * 1024;         // per epilogue warp one 1 KiB buffer of 32 rows x 16 bf16 (8 fp32) tokens; two such sets
 
 template <int MODE, int QM>
 __global__ void __launch_bounds__(kPfThreads, 1)
@@ -643,7 +654,7 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
     uint8_t* smem_gen = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
     const uint32_t b_base = smem_base + NA * kABytes;
     const uint32_t staging_base = b_base + NB * kBBytes;  // 1 KiB aligned: the output boxes are swizzled
-    const uint32_t staging_bytes = (uint32_t)p.epi_bufs * kPfStagingBuf;
+    constexpr uint32_t staging_bytes = 2 * kPfStagingBuf;
     const uint32_t ctl_base = staging_base + staging_bytes;
     uint8_t* ctl_gen = smem_gen + NA * kABytes + NB * kBBytes + staging_bytes;
 
@@ -699,15 +710,26 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
     const uint32_t tmem_base = *tmem_holder;
 
     // every role walks the same sequence of tiles and pipeline stages
-    const int num_tiles = p.m_pairs * p.n_tiles * p.splits;
-    auto tile_coords = [&](int tile, int& m0, int& t0, int& z, int& kb_begin, int& iters) {
-        const int mt = tile % p.m_pairs;
-        const int rest = tile / p.m_pairs;
-        m0 = (2 * mt + rank) * kBlockM;
-        t0 = (rest % p.n_tiles) * TN;
-        z = rest / p.n_tiles;
-        kb_begin = z * p.kb_per_split;
-        iters = min(p.num_kb, kb_begin + p.kb_per_split) - kb_begin;
+    // every role walks the same sequence of segments (a tile, or this pair's part of one) and pipeline
+    // stages
+    const int nres = pair0 < p.res_tiles * p.pieces ? 1 : 0;
+    const int nseg = nres + (pair0 < p.full_tiles ? (p.full_tiles - 1 - pair0) / num_pairs + 1 : 0);
+    // res: index of the shared tile of which the segment is a part, or -1 for a whole tile
+    auto tile_coords = [&](int seg, int& m0, int& t0, int& res, int& kb_begin, int& iters) {
+        int tile;
+        res = -1;
+        if (seg < nres) {
+            res = pair0 / p.pieces;
+            kb_begin = (pair0 - res * p.pieces) * p.piece_len;
+            iters = min(p.piece_len, p.num_kb - kb_begin);
+            tile = p.full_tiles + res;
+        } else {
+            kb_begin = 0;
+            iters = p.num_kb;
+            tile = pair0 + (seg - nres) * num_pairs;
+        }
+        m0 = (2 * (tile % p.m_pairs) + rank) * kBlockM;
+        t0 = (tile / p.m_pairs) * TN;
     };
 
     // bf16 output through TMA stores, 16 tokens x 32 rows at a time: the accumulator is read as MMA
@@ -742,11 +764,125 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
             ptx::bulk_commit_group();
         }
     };
-    // On the last tile of a CTA the worker warps have nothing left to expand, so they share its
+    // Any other output, 16 tokens x 32 rows at a time: transposed through the staging buffer `stg`
+    // ([token][row]), then 16-byte pieces of one token's 32 rows as coalesced stores.  sc: the output
+    // scales of the 16 tokens.
+    auto store_box_any = [&](uint32_t t_row, int col, uint32_t stg, const float (&sc)[16], float bias, int m0w, int t0) {
+        const int esz = p.out_bf16 ? 2 : 4;
+        uint8_t* out_base = reinterpret_cast<uint8_t*>(p.out);
+        // 16-byte stores need an aligned base and pitch
+        const bool full_rows = ((reinterpret_cast<uintptr_t>(out_base) & 15u) == 0) && ((p.ldo * esz) % 16 == 0) &&
+                               (m0w + 32 <= p.Mdim);
+        const int pieces = 2 * esz;          // 16-byte vectors of one token's 32 rows
+        const int toks = 1024 / (32 * esz);  // tokens per staging round: 16 (bf16) or 8 (fp32)
+        uint32_t v[16];
+        ptx::tmem_ld_x16(t_row + (uint32_t)col, v);
+        ptx::tmem_ld_wait();
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            if (esz == 2) {
+                if (half == 1) break;
+#pragma unroll
+                for (int c = 0; c < 16; ++c) {
+                    const __nv_bfloat16 h = __float2bfloat16_rn(__uint_as_float(v[c]) * sc[c] + bias);
+                    asm volatile("st.shared.b16 [%0], %1;" ::"r"(stg + c * 64 + lane * 2),
+                                 "h"(*reinterpret_cast<const unsigned short*>(&h)) : "memory");
+                }
+            } else {
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const float f = __uint_as_float(v[8 * half + c]) * sc[8 * half + c] + bias;
+                    asm volatile("st.shared.b32 [%0], %1;" ::"r"(stg + c * 128 + lane * 4), "f"(f) : "memory");
+                }
+            }
+            __syncwarp();
+            const int tbase = t0 + col + ((esz == 4) ? 8 * half : 0);
+            for (int pc = lane; pc < toks * pieces; pc += 32) {
+                const int c = pc / pieces, piece = pc - c * pieces;
+                const int t = tbase + c;
+                if (t >= p.n) continue;
+                uint32_t x0, x1, x2, x3;
+                asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(x0), "=r"(x1), "=r"(x2), "=r"(x3)
+                             : "r"(stg + pc * 16) : "memory");
+                uint8_t* dst = out_base + ((long long)t * p.ldo + m0w) * esz + piece * 16;
+                if (full_rows) {
+                    *reinterpret_cast<uint4*>(dst) = make_uint4(x0, x1, x2, x3);
+                } else {
+                    const uint32_t rr[4] = {x0, x1, x2, x3};
+                    const int per = 16 / esz;  // elements in this piece
+#pragma unroll
+                    for (int e2 = 0; e2 < 8; ++e2) {
+                        if (e2 < per && m0w + piece * per + e2 < p.Mdim) {
+                            if (esz == 2)
+                                reinterpret_cast<unsigned short*>(dst)[e2] =
+                                    (unsigned short)(rr[e2 >> 1] >> ((e2 & 1) * 16));
+                            else
+                                reinterpret_cast<uint32_t*>(dst)[e2] = rr[e2 & 3];
+                        }
+                    }
+                }
+            }
+            __syncwarp();
+        }
+    };
+    // Output of a segment: emit(col) for the boxes first, first + step, ... of this warp's 32 rows.  For
+    // a part of a shared tile the sums go to the workspace, and emit() follows for those classes of
+    // boxes (box mod kPfHelpers) of which this warp's part is the last to arrive.
+    constexpr int kPfHelpers = 1 + kPfWorkerWarps / 4;  // 5
+    auto drain = [&](int res, int m0w, int t0, uint32_t t_row, int quarter, int first, int step, auto&& emit) {
+        if (m0w >= p.Mdim) return;
+        const int nbox = min(TN >> 4, (p.n - t0 + 15) >> 4);
+        if (res < 0) {
+#pragma unroll 1
+            for (int b = first; b < nbox; b += step) emit(16 * b);
+            return;
+        }
+        const size_t part = (size_t)TN * 256;  // floats of one contribution, both CTAs
+        const int e0 = rank * TN * 128 + quarter * 32 + lane;
+        float* mine = p.partial + (size_t)pair0 * part + e0;
+#pragma unroll 1
+        for (int b = first; b < nbox; b += step) {
+            uint32_t v[16];
+            ptx::tmem_ld_x16(t_row + 16u * b, v);
+            ptx::tmem_ld_wait();
+#pragma unroll
+            for (int c = 0; c < 16; ++c) __stcg(mine + (16 * b + c) * 128, __uint_as_float(v[c]));
+        }
+        __threadfence();
+        __syncwarp();
+        const int p_first = res * p.pieces, p_last = p_first + p.pieces - 1;
+        uint32_t* cnt = p.counters + ((res * 2 + rank) * 4 + quarter) * kPfHelpers;
+        const int cl_end = min(nbox, step == 1 ? kPfHelpers : first + 1);
+#pragma unroll 1
+        for (int cl = first; cl < cl_end; ++cl) {
+            uint32_t before = 0u;
+            if (lane == 0) before = atomicAdd(cnt + cl, 1u);
+            before = __shfl_sync(0xffffffffu, before, 0);
+            if (before != (uint32_t)(p_last - p_first)) continue;
+            __threadfence();
+#pragma unroll 1
+            for (int b = cl; b < nbox; b += kPfHelpers) {
+                float sum[16];
+#pragma unroll
+                for (int c = 0; c < 16; ++c) sum[c] = 0.0f;
+#pragma unroll 2
+                for (int q = p_first; q <= p_last; ++q) {
+                    const float* src = p.partial + (size_t)q * part + e0 + (size_t)(16 * b) * 128;
+                    float x[16];
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) x[c] = __ldcg(src + c * 128);
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) sum[c] += x[c];
+                }
+                ptx::tmem_st_x16(t_row + 16u * b, sum);
+                ptx::tmem_st_wait();
+                emit(16 * b);
+            }
+        }
+    };
+    // On the last segment of a CTA the worker warps have nothing left to expand, so they share its
     // epilogue: of the five warps on a tensor-memory lane quarter (one epilogue warp, four workers)
     // warp h takes the boxes h, h + 5, ...
-    constexpr int kPfHelpers = 1 + kPfWorkerWarps / 4;  // 5
-    auto is_last_tile = [&](int tile) { return tile + num_pairs >= num_tiles; };
 
     if (warp == kPfProdWarp) {
         // ---------------- producer: the activation tile of every stage (TMA), into a ring of its
@@ -755,9 +891,9 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
             bool ok = true;
             int s = 0;
             uint32_t ph = 0;
-            for (int tile = pair0; tile < num_tiles && ok; tile += num_pairs) {
-                int m0, t0, z, kb_begin, iters;
-                tile_coords(tile, m0, t0, z, kb_begin, iters);
+            for (int seg = 0; seg < nseg && ok; ++seg) {
+                int m0, t0, res, kb_begin, iters;
+                tile_coords(seg, m0, t0, res, kb_begin, iters);
                 for (int it = 0; it < iters; ++it) {
                     ok = wait_bar(b_empty + 8 * s, ph ^ 1u, ctl, 1, 256u);
                     if (!ok) break;
@@ -791,9 +927,9 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
             constexpr uint32_t kAStep = (MODE == MODE_FWD) ? (32u >> 4) : (2048u >> 4);
             const uint32_t a_lo0 = ((smem_base >> 4) & 0x3FFFu) | kALoExtra;
             const uint32_t b_lo0 = ((b_base >> 4) & 0x3FFFu) | kBLoExtra;
-            for (int tile = pair0; tile < num_tiles && ok; tile += num_pairs, ++lt) {
-                int m0, t0, z, kb_begin, iters;
-                tile_coords(tile, m0, t0, z, kb_begin, iters);
+            for (; lt < nseg && ok; ++lt) {
+                int m0, t0, res, kb_begin, iters;
+                tile_coords(lt, m0, t0, res, kb_begin, iters);
                 const int acc = lt & 1;
                 const uint32_t acc_ph = (lt >> 1) & 1;
                 ok = wait_bar(acc_empty + 8 * acc, acc_ph ^ 1u, ctl, 8);  // the epilogue has drained it
@@ -859,7 +995,7 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
         // The task stream of this thread: the stages whose running index over all tiles of the CTA
         // is `group` mod kPfGroups.  A cursor names one of them.
         struct Cur {
-            int tile, it, iters, kb_begin, mt;
+            int seg, it, iters, kb_begin, mt;
             int c, kpos, next_edge;  // group index of the task's first 32 k (forward: advances with the stage)
             uint32_t code_idx;       // this thread's first word of the task in the regrouped planes
             uint32_t alpha_idx;      // its first scale (plane 0, group c) in the regrouped scales
@@ -868,13 +1004,13 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
             bool valid;
         };
         auto enter_tile = [&](Cur& x) {
-            int m0, t0, z;
-            tile_coords(x.tile, m0, t0, z, x.kb_begin, x.iters);
+            int m0, t0, res;
+            tile_coords(x.seg, m0, t0, res, x.kb_begin, x.iters);
             x.mt = min(m0 >> 7, p.m_tiles - 1);  // a pair whose second row tile does not exist expands the first again
         };
         const uint32_t code_step = kPfGroups * chunk_words;
         const uint32_t alpha_step = kPfGroups * (uint32_t)p.G * alpha_block;  // dX: the next task's rows
-        auto locate = [&](Cur& x) {  // group index and array positions at (tile, it), from scratch
+        auto locate = [&](Cur& x) {  // group index and array positions at (seg, it), from scratch
             x.kpos = (MODE == MODE_FWD) ? (x.kb_begin + x.it) * kBlockK : x.mt * kBlockM + half * 64;
             x.c = min(x.kpos / p.g, p.G - 1);
             x.next_edge = (x.c + 1) * p.g;
@@ -889,8 +1025,7 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
             bool moved = false;
             while (x.it >= x.iters) {
                 x.it -= x.iters;
-                x.tile += num_pairs;
-                if (x.tile >= num_tiles) { x.valid = false; return; }
+                if (++x.seg >= nseg) { x.valid = false; return; }
                 enter_tile(x);
                 moved = true;
             }
@@ -999,8 +1134,8 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
         };
 
         Cur cur;
-        cur.tile = pair0;
-        cur.valid = cur.tile < num_tiles;
+        cur.seg = 0;
+        cur.valid = nseg > 0;
         cur.fresh = true;
         cur.split = false;
         cur.it = group;
@@ -1010,8 +1145,7 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
             enter_tile(cur);
             while (cur.it >= cur.iters) {
                 cur.it -= cur.iters;
-                cur.tile += num_pairs;
-                if (cur.tile >= num_tiles) { cur.valid = false; break; }
+                if (++cur.seg >= nseg) { cur.valid = false; break; }
                 enter_tile(cur);
             }
             if (cur.valid) locate(cur);
@@ -1042,15 +1176,15 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
                 cur = nxt;
             }
         }
-        if (p.helpers && ok && pair0 < num_tiles) {
-            // share the epilogue of this CTA's last tile.  Its operand slots are free once the
+        if (p.helpers && ok && nseg > 0) {
+            // share the output of this CTA's last segment.  Its operand slots are free once the
             // accumulator is complete, so each warp stages its boxes in 1 KiB of the first slots.
-            const int lt = (num_tiles - 1 - pair0) / num_pairs;
-            const int tile = pair0 + lt * num_pairs;
-            int m0, t0, z, kb_begin, iters;
-            tile_coords(tile, m0, t0, z, kb_begin, iters);
+            const int lt = nseg - 1;
+            int m0, t0, res, kb_begin, iters;
+            tile_coords(lt, m0, t0, res, kb_begin, iters);
             const int acc = lt & 1;
             ok = wait_bar(ctl.accum + 8 * acc, (uint32_t)(lt >> 1) & 1u, ctl, 10);
+            ok = __all_sync(0xffffffffu, ok);
             if (ok) {
                 ptx::tc_fence_after_sync();
                 const int quarter = warp & 3, helper = 1 + (warp >> 2);  // 1..4
@@ -1058,26 +1192,31 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
                 const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)acc * kAccCols;
                 const uint32_t buf = smem_base + (uint32_t)warp * 1024u;
                 const float winv = 1.0f / wscale;  // a power of two
-                const int g = lane >> 2, tq = lane & 3;
-                float b4[4];
+                auto scale_of = [&](int t) { return (t < p.n) ? winv * __ldg(p.tok_inv_scale + t) : 0.0f; };
+                auto bias_of = [&](int m) { return (MODE == MODE_FWD && p.bias != nullptr && m < p.Mdim) ? __ldg(p.bias + m) : 0.0f; };
+                if (p.fast_epi) {
+                    const int g = lane >> 2, tq = lane & 3;
+                    float b4[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    b4[i] = (MODE == MODE_FWD && p.bias != nullptr && m0w + g + 8 * i < p.Mdim) ? __ldg(p.bias + m0w + g + 8 * i) : 0.0f;
-                bool stored = false;
-#pragma unroll 1
-                for (int col = 16 * helper; col < TN; col += 16 * kPfHelpers) {
-                    if (t0 + col >= p.n || m0w >= p.Mdim) break;  // uniform in the warp
-                    if (stored && lane == 0) ptx::bulk_wait_group_read<0>();
-                    __syncwarp();
-                    const int ta = t0 + col + 2 * tq, tb = ta + 8;
-                    const float s0x = (ta < p.n) ? winv * __ldg(p.tok_inv_scale + ta) : 0.0f;
-                    const float s0y = (ta + 1 < p.n) ? winv * __ldg(p.tok_inv_scale + ta + 1) : 0.0f;
-                    const float s1x = (tb < p.n) ? winv * __ldg(p.tok_inv_scale + tb) : 0.0f;
-                    const float s1y = (tb + 1 < p.n) ? winv * __ldg(p.tok_inv_scale + tb + 1) : 0.0f;
-                    store_box(t_row, col, buf, s0x, s0y, s1x, s1y, b4, m0w, t0 + col);
-                    stored = true;
+                    for (int i = 0; i < 4; ++i) b4[i] = bias_of(m0w + g + 8 * i);
+                    bool stored = false;
+                    drain(res, m0w, t0, t_row, quarter, helper, kPfHelpers, [&](int col) {
+                        if (stored && lane == 0) ptx::bulk_wait_group_read<0>();
+                        __syncwarp();
+                        const int ta = t0 + col + 2 * tq, tb = ta + 8;
+                        store_box(t_row, col, buf, scale_of(ta), scale_of(ta + 1), scale_of(tb), scale_of(tb + 1), b4, m0w, t0 + col);
+                        stored = true;
+                    });
+                    if (lane == 0) ptx::bulk_wait_group<0>();
+                } else {
+                    const float bias = bias_of(m0w + lane);
+                    drain(res, m0w, t0, t_row, quarter, helper, kPfHelpers, [&](int col) {
+                        float sc[16];
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) sc[c] = scale_of(t0 + col + c);
+                        store_box_any(t_row, col, buf, sc, bias, m0w, t0);
+                    });
                 }
-                if (lane == 0) ptx::bulk_wait_group<0>();
             }
         }
     } else if (pf_epilogue_index(warp) >= 0) {
@@ -1087,17 +1226,12 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
         const int et = ew * 32 + lane;      // 0..127
         const float winv = pow2f(-weight_shift(p.hdr, p.q));
         const uint32_t stg = staging_base + ew * 1024;  // this warp's staging: [tokens][32 rows], 1 KiB (a second one kPfStagingBuf further)
-        const int esz = (p.splits > 1 || !p.out_bf16) ? 4 : 2;  // bytes per stored element
-        uint8_t* out_base = (p.splits > 1) ? reinterpret_cast<uint8_t*>(p.partial) : reinterpret_cast<uint8_t*>(p.out);
-        const long long out_ld = (p.splits > 1) ? (long long)p.Mdim : p.ldo;
-        // 16-byte stores need an aligned base and pitch
-        const bool vec_ok = ((reinterpret_cast<uintptr_t>(out_base) & 15u) == 0) && ((out_ld * esz) % 16 == 0);
         bool ok = true;
         int lt = 0;
         uint32_t chunks = 0;  // output boxes stored so far (fast path): selects the staging buffer
-        for (int tile = pair0; tile < num_tiles && ok; tile += num_pairs, ++lt) {
-            int m0, t0, z, kb_begin, iters;
-            tile_coords(tile, m0, t0, z, kb_begin, iters);
+        for (; lt < nseg && ok; ++lt) {
+            int m0, t0, res, kb_begin, iters;
+            tile_coords(lt, m0, t0, res, kb_begin, iters);
             const int acc = lt & 1;
             const uint32_t acc_ph = (lt >> 1) & 1;
             for (int i = et; i < TN; i += kPfEpiWarps * 32)
@@ -1108,96 +1242,34 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
             asm volatile("bar.sync 2, %0;" ::"n"(kPfEpiWarps * 32) : "memory");
             if (*ctl.abort_flag) { ok = false; break; }
             ptx::tc_fence_after_sync();
-            // accumulator row `lane` of this warp's quarter is output column m0w + lrow
             const int m0w = m0 + quarter * 32;
-            const int lrow = lane;
-            const float bias = (MODE == MODE_FWD && p.bias != nullptr && p.splits == 1 && m0w + lrow < p.Mdim)
-                                   ? __ldg(p.bias + m0w + lrow) : 0.0f;
-            uint8_t* tile_out = out_base + ((p.splits > 1) ? (long long)z * p.n * p.Mdim * 4 : 0);
             const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)acc * kAccCols;
-            const bool full_rows = vec_ok && (m0w + 32 <= p.Mdim);
+            auto bias_of = [&](int m) { return (MODE == MODE_FWD && p.bias != nullptr && m < p.Mdim) ? __ldg(p.bias + m) : 0.0f; };
+            const int step = (p.helpers && lt == nseg - 1) ? kPfHelpers : 1;  // the workers take the other boxes
             if (p.fast_epi) {
                 const int g = lane >> 2, tq = lane & 3;
                 float b4[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    b4[i] = (MODE == MODE_FWD && p.bias != nullptr && m0w + g + 8 * i < p.Mdim) ? __ldg(p.bias + m0w + g + 8 * i) : 0.0f;
-                const int cstep = (p.helpers && is_last_tile(tile)) ? 16 * kPfHelpers : 16;  // the workers take the other boxes
-#pragma unroll 1
-                for (int col = 0; col < TN; col += cstep) {
-                    if (t0 + col >= p.n || m0w >= p.Mdim) break;  // uniform in the warp
+                for (int i = 0; i < 4; ++i) b4[i] = bias_of(m0w + g + 8 * i);
+                drain(res, m0w, t0, t_row, quarter, 0, step, [&](int col) {
                     // the store that last read this buffer has to be done with it
-                    if (p.epi_bufs == 2) {
-                        if (chunks >= 2 && lane == 0) ptx::bulk_wait_group_read<1>();
-                    } else {
-                        if (chunks >= 1 && lane == 0) ptx::bulk_wait_group_read<0>();
-                    }
+                    if (chunks >= 2 && lane == 0) ptx::bulk_wait_group_read<1>();
                     __syncwarp();
-                    const uint32_t buf = stg + ((p.epi_bufs == 2) ? (chunks & 1u) * kPfStagingBuf : 0u);
+                    const uint32_t buf = stg + (chunks & 1u) * kPfStagingBuf;
                     float s0x, s0y, s1x, s1y;
                     asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(s0x), "=f"(s0y) : "r"(scale_addr + (col + 2 * tq) * 4) : "memory");
                     asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(s1x), "=f"(s1y) : "r"(scale_addr + (col + 8 + 2 * tq) * 4) : "memory");
                     store_box(t_row, col, buf, s0x, s0y, s1x, s1y, b4, m0w, t0 + col);
                     ++chunks;
-                }
-            }
-            // one token's 32 rows are 64 (bf16) or 128 (fp32) bytes: `pieces` 16-byte vectors
-            const int pieces = 2 * esz;
-            const int toks = 1024 / (32 * esz);  // tokens per staging round: 16 (bf16) or 8 (fp32)
-#pragma unroll 1
-            for (int col = 0; col < TN && !p.fast_epi; col += 16) {
-                if (t0 + col >= p.n) break;  // uniform in the warp
-                uint32_t v[16];
-                ptx::tmem_ld_x16(t_row + (uint32_t)col, v);
-                ptx::tmem_ld_wait();
-                // transpose through shared memory: staging[token][row], then 16-byte pieces of one
-                // token's 32 rows go out as coalesced vector stores
+                });
+            } else {
+                const float bias = bias_of(m0w + lane);
+                drain(res, m0w, t0, t_row, quarter, 0, step, [&](int col) {
+                    float sc[16];
 #pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    if (esz == 2) {
-                        if (half == 1) break;
-#pragma unroll
-                        for (int c = 0; c < 16; ++c) {
-                            const __nv_bfloat16 h = __float2bfloat16_rn(__uint_as_float(v[c]) * scale[col + c] + bias);
-                            asm volatile("st.shared.b16 [%0], %1;" ::"r"(stg + c * 64 + lrow * 2),
-                                         "h"(*reinterpret_cast<const unsigned short*>(&h)) : "memory");
-                        }
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < 8; ++c) {
-                            const float f = __uint_as_float(v[8 * half + c]) * scale[col + 8 * half + c] + bias;
-                            asm volatile("st.shared.b32 [%0], %1;" ::"r"(stg + c * 128 + lrow * 4), "f"(f) : "memory");
-                        }
-                    }
-                    __syncwarp();
-                    const int tbase = t0 + col + ((esz == 4) ? 8 * half : 0);
-                    for (int pc = lane; pc < toks * pieces; pc += 32) {
-                        const int c = pc / pieces, seg = pc - c * pieces;
-                        const int t = tbase + c;
-                        if (t >= p.n) continue;
-                        uint32_t r0, r1, r2, r3;
-                        asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-                                     : "r"(stg + pc * 16) : "memory");
-                        uint8_t* dst = tile_out + ((long long)t * out_ld + m0w) * esz + seg * 16;
-                        if (full_rows) {
-                            *reinterpret_cast<uint4*>(dst) = make_uint4(r0, r1, r2, r3);
-                        } else {
-                            const uint32_t rr[4] = {r0, r1, r2, r3};
-                            const int per = 16 / esz;  // elements in this piece
-#pragma unroll
-                            for (int e2 = 0; e2 < 8; ++e2) {
-                                if (e2 < per && m0w + seg * per + e2 < p.Mdim) {
-                                    if (esz == 2)
-                                        reinterpret_cast<unsigned short*>(dst)[e2] =
-                                            (unsigned short)(rr[e2 >> 1] >> ((e2 & 1) * 16));
-                                    else
-                                        reinterpret_cast<uint32_t*>(dst)[e2] = rr[e2 & 3];
-                                }
-                            }
-                        }
-                    }
-                    __syncwarp();
-                }
+                    for (int c = 0; c < 16; ++c) sc[c] = scale[col + c];
+                    store_box_any(t_row, col, stg, sc, bias, m0w, t0);
+                });
             }
             // the accumulator (and this tile's scale row) may be reused
             ptx::tc_fence_before_sync();
@@ -1513,16 +1585,18 @@ decode_kernel(const __grid_constant__ CUtensorMap tmap_bits, const DecodeParams 
 // ------------------------------------------------------------------------------------------
 
 struct ExpandPlan {
-    int TN, splits, kb_per_split, num_kb, m_tiles, m_pairs, n_tiles;
-    int a_slots, b_slots, epi_bufs;
+    int TN, num_kb, m_tiles, m_pairs, n_tiles;
+    int full_tiles, res_tiles, pieces, piece_len, pairs;                 // see ExpandParams
+    int a_slots, b_slots;
     uint32_t bits_bytes, alpha_bytes;                                    // one stage's chunk of the planes; the scales of one (row block, group)
     size_t planes_bytes;                                                 // the regrouped planes (codes for q <= 4)
     size_t smem;                                                         // dynamic shared memory of the GEMM kernel
-    size_t off_tok, off_act, off_alpha, off_bits, off_partial, total;  // workspace layout (bytes)
+    size_t off_tok, off_act, off_alpha, off_bits, off_counters, off_partial, total;  // workspace layout (bytes)
     int ld_act;                                                          // pitch of the fp16 activations (elements)
 };
 
-constexpr int kPfStageFixed = 224;                                     // fixed cost of a pipeline stage, in token-tile columns
+constexpr int kPfMinPiece = 4;
+constexpr int kPfBoxClasses = 1 + kPfWorkerWarps / 4;                  // counters per shared tile, CTA and lane quarter
 constexpr size_t kPfFixedBytes = 1024 + kPfCtlBytes + kPfScaleBytes;   // alignment slack, barriers, output scales
 
 // Tile width over tokens, the K split and the pipeline geometry.  Wide token tiles amortise the
@@ -1537,40 +1611,45 @@ ExpandPlan plan_expand(int mode, int d_out, int d_in, int q, int g, int n) {
     pl.m_tiles = ceil_div(Mdim, kBlockM);
     pl.m_pairs = ceil_div(pl.m_tiles, 2);
     pl.num_kb = ceil_div(Kdim, kBlockK);
-    int tn;
-    if (n <= 32) tn = 32;
-    else if (n <= 64) tn = 64;
-    else if (n <= 128) tn = 128;
-    else {
-        // Any multiple of 16 up to 256 is a legal UMMA width.  A stage of the kernel takes a fixed
-        // time (barriers, UMMA issue, the expansion of one weight tile whatever the width) plus a
-        // time in proportion to the width (the UMMAs themselves); measured, the fixed part is worth
-        // about kPfStageFixed columns.  The kernel is persistent with ceil(tiles / SMs) tiles per
-        // CTA, so a narrower tile can shorten the call (fewer tiles per CTA, less padding past n)
-        // but costs SM time that kernels running beside this one would have used.  The width
-        // that minimises call time x SM time wins; ties go to the wider tile.
-        long long best = -1;
-        tn = 256;
-        for (int c = 256; c >= 128; c -= 16) {
-            const long long tiles = (long long)pl.m_pairs * ceil_div(n, c);
-            const long long per_cta = (tiles + pairs - 1) / pairs;
-            const long long stage = c + kPfStageFixed;
-            const long long cost = (per_cta * stage) * (tiles * stage);
-            if (best < 0 || cost < best) { best = cost; tn = c; }
+    // Token tiles and K pieces, by the time a call is expected to take.  All in stages of a pair (about
+    // 0.33 us, set by the expansion of the weight tiles and hence nearly the same at every width; 140
+    // tiles of 208 tokens take 2 % longer than 112 of 256, two waves both):
+    //   * whole waves of tiles, then the ragged last wave (or all of a problem with fewer tiles than
+    //     pairs), whole or cut into d pieces;
+    //   * pieces that end the call are added by all 20 output warps of a CTA, each ceil(TN / 80) boxes
+    //     of 16 tokens at 0.8 us per piece, plus 3 us for the way through memory;
+    //   * pieces before whole tiles are added by four warps under the main loop of those, so they
+    //     cost nothing if that is much longer (measured: 5120 -> 20480 dX with 2048 tokens, 12 of 172
+    //     tiles in pieces, 429 -> 359 us; 1600 -> 6400, whose tiles are 25 stages, 79 -> 92 us);
+    //   * the last output, TN / 64 stages.
+    const int nt0 = ceil_div(n, 256), nt1 = std::min(ceil_div(n, 32), 8 * nt0);
+    double best = -1.0;
+    for (int nt = nt0; nt <= nt1; ++nt) {
+        const int tn = std::max(32, ceil_div(ceil_div(n, nt), 16) * 16);
+        if (ceil_div(n, tn) != nt) continue;
+        const int tiles = pl.m_pairs * nt;
+        const int waves = tiles / pairs, ragged = tiles % pairs;
+        const double stage = 1.1 - 0.1 * tn / 256.0, out = 1.0 + tn / 64.0;
+        const int dmax = ragged > 0 ? std::min(pairs / ragged, pl.num_kb / kPfMinPiece) : 1;
+        for (int d = 1; d <= std::max(1, dmax); ++d) {
+            const int len = ceil_div(pl.num_kb, d);
+            double add = 0.0;
+            if (d > 1 && waves == 0) add = 9.0 + 2.4 * ceil_div(tn, 80) * d;
+            if (d > 1 && waves > 0 && waves * pl.num_kb < 3 * 40 * d) break;  // would not stay hidden
+            const double cost = (waves * pl.num_kb + (ragged > 0 ? len : 0)) * stage + add + out;
+            if (best >= 0.0 && cost >= best) continue;
+            best = cost;
+            pl.TN = tn;
+            pl.n_tiles = nt;
+            pl.pieces = ceil_div(pl.num_kb, len);
+            pl.piece_len = len;
+            pl.res_tiles = pl.pieces > 1 ? ragged : 0;
+            pl.full_tiles = tiles - pl.res_tiles;
+            pl.pairs = waves > 0 ? (pl.res_tiles > 0 ? pairs : ceil_div(tiles, waves + (ragged > 0 ? 1 : 0)))
+                                 : tiles * pl.pieces;
         }
     }
-    pl.TN = tn;
-    pl.n_tiles = ceil_div(n, tn);
-    const int tiles = pl.m_pairs * pl.n_tiles;
-    // The K split goes through fp32 partials, a slower epilogue and a second kernel: only for
-    // problems that would otherwise leave most of the SMs idle.
-    int splits = (4 * tiles <= pairs) ? pairs / tiles : 1;
-    if (splits < 1) splits = 1;
-    const int max_splits = (pl.num_kb + 3) / 4;  // at least 4 K blocks per CTA
-    if (splits > max_splits) splits = max_splits;
-    if (splits > 32) splits = 32;
-    pl.kb_per_split = ceil_div(pl.num_kb, splits);
-    pl.splits = ceil_div(pl.num_kb, pl.kb_per_split);
+    const int tn = pl.TN;
 
     const int rows = (mode == MODE_FWD) ? 128 : 64;
     pl.bits_bytes = (q <= 3 ? 3u : (uint32_t)q) * 1024u;  // q <= 4: selector codes (3 or 4 words per 32 weights)
@@ -1578,11 +1657,10 @@ ExpandPlan plan_expand(int mode, int d_out, int d_in, int q, int g, int n) {
     // Shared memory.  A worker group takes about a microsecond from "the tensor core is done with my
     // slot" to "the slot holds the next tile", and a TMA load as long to land; both rings must be deep
     // enough to cover that at one stage per ~0.3 us.  These fit at every token-tile width.
-    pl.epi_bufs = 2;
     pl.a_slots = 6;
     pl.b_slots = 6;
     pl.smem = pl.a_slots * (size_t)kABytes + pl.b_slots * (size_t)(tn / 2) * kBlockK * 2 +
-              pl.epi_bufs * (size_t)kPfStagingBuf + kPfFixedBytes;
+              2 * (size_t)kPfStagingBuf + kPfFixedBytes;
 
     const size_t chunks_bits = (size_t)pl.m_tiles * pl.num_kb;                       // [m_tile][kb] or [u][jb]
     const size_t blocks_alpha = (size_t)((mode == MODE_FWD) ? pl.m_tiles : pl.num_kb) * G;  // [m_tile][G] or [jb][G]
@@ -1592,8 +1670,9 @@ ExpandPlan plan_expand(int mode, int d_out, int d_in, int q, int g, int n) {
     pl.off_alpha = align_up(pl.off_act + (size_t)n * pl.ld_act * 2, 128);
     pl.off_bits = align_up(pl.off_alpha + blocks_alpha * pl.alpha_bytes, 128);
     pl.planes_bytes = chunks_bits * pl.bits_bytes;
-    pl.off_partial = align_up(pl.off_bits + pl.planes_bytes, 128);
-    pl.total = pl.off_partial + (pl.splits > 1 ? (size_t)pl.splits * n * Mdim * sizeof(float) : 0);
+    pl.off_counters = align_up(pl.off_bits + pl.planes_bytes, 128);
+    pl.off_partial = align_up(pl.off_counters + (size_t)pl.res_tiles * 8 * kPfBoxClasses * sizeof(uint32_t), 128);
+    pl.total = pl.off_partial + (size_t)(pl.res_tiles * pl.pieces) * tn * 256 * sizeof(float);
     return pl;
 }
 
@@ -1631,13 +1710,8 @@ bcq_status launch_expand(const CUtensorMap& tm, const CUtensorMap& tmo, const Ex
     auto kern = expand_gemm_kernel<MODE, QM>;
     bcq_status st0 = ensure_dynamic_smem(kern, pl.smem);
     if (st0 != BCQ_OK) return st0;
-    const int tiles = pl.m_pairs * pl.n_tiles * pl.splits;
-    // persistent, at most one CTA per SM; with more tiles than pairs every pair gets the same number of
-    // tiles (as many as the busiest would get anyway): fewer CTAs pay the prologue, more epilogues
-    // overlap the next tile's main loop, and the SMs left over can run other kernels
-    const int per_pair = ceil_div(tiles, std::max(1, sm_count() / 2));
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2u * (unsigned)ceil_div(tiles, per_pair));
+    cfg.gridDim = dim3(2u * (unsigned)pl.pairs);
     cfg.blockDim = dim3(kPfThreads);
     cfg.dynamicSmemBytes = pl.smem;
     cfg.stream = stream;
@@ -1708,7 +1782,7 @@ bcq_status run_expand(int d_out, int d_in, int q, int g, int n, const void* act,
 
     // everything that can fail is done before the first launch: the output tensor map and the
     // shared-memory limits of the kernels this call may run
-    const bool fast_epi = (out_dtype == BCQ_BF16 && pl.splits == 1 && aligned16(out) && (ldo * 2) % 16 == 0 &&
+    const bool fast_epi = (out_dtype == BCQ_BF16 && aligned16(out) && (ldo * 2) % 16 == 0 &&
                            ldo >= (size_t)Mdim);
     CUtensorMap tmo = tm;
     if (fast_epi) {
@@ -1737,6 +1811,8 @@ bcq_status run_expand(int d_out, int d_in, int q, int g, int n, const void* act,
     pp.bits = bits;
     pp.alpha_t = reinterpret_cast<float*>(wsb + pl.off_alpha);
     pp.bits_t = reinterpret_cast<uint32_t*>(wsb + pl.off_bits);
+    pp.counters = reinterpret_cast<uint32_t*>(wsb + pl.off_counters);
+    pp.num_counters = pl.res_tiles * 8 * kPfBoxClasses;
     if (coded && prepared == nullptr) {
         if ((st = launch_code_planes(MODE, d_out, d_in, q, pl, bits, pp.bits_t, s)) != BCQ_OK) return st;
     }
@@ -1757,33 +1833,28 @@ bcq_status run_expand(int d_out, int d_in, int q, int g, int n, const void* act,
     p.d_out = d_out; p.d_in = d_in; p.q = q; p.g = g;
     p.G = (int)bcq_num_groups(d_in, g);
     p.pitch = pitch;
-    p.n = n; p.Mdim = Mdim; p.num_kb = pl.num_kb; p.kb_per_split = pl.kb_per_split; p.splits = pl.splits;
+    p.n = n; p.Mdim = Mdim; p.num_kb = pl.num_kb;
+    p.full_tiles = pl.full_tiles; p.res_tiles = pl.res_tiles; p.pieces = pl.pieces; p.piece_len = pl.piece_len;
     p.m_tiles = pl.m_tiles; p.m_pairs = pl.m_pairs; p.n_tiles = pl.n_tiles;
     p.tn = pl.TN;
     p.acc_cols = 32;
     while ((int)p.acc_cols < pl.TN) p.acc_cols *= 2;
-    p.a_slots = pl.a_slots; p.b_slots = pl.b_slots; p.epi_bufs = pl.epi_bufs; p.chunk_words = pl.bits_bytes / 4;
+    p.a_slots = pl.a_slots; p.b_slots = pl.b_slots; p.chunk_words = pl.bits_bytes / 4;
     p.bits_t = (coded && prepared != nullptr) ? reinterpret_cast<const uint32_t*>(prepared) : pp.bits_t;
     p.alpha_t = pp.alpha_t; p.bias = bias; p.hdr = hdr; p.tok_inv_scale = tok;
     p.out = out; p.ldo = (long long)ldo; p.out_bf16 = (out_dtype == BCQ_BF16);
     p.partial = reinterpret_cast<float*>(wsb + pl.off_partial);
-    // bf16 output with an aligned base and pitch and no K split goes out through TMA stores
+    p.counters = pp.counters;
+    // bf16 output with an aligned base and pitch goes out through TMA stores
     p.fast_epi = fast_epi ? 1 : 0;
-    // The workers find the last tile's accumulator by barrier parity alone.  They run at most
-    // `a_slots` pipeline stages ahead of the tensor core, so the parity is unambiguous only if
-    // two tiles are longer than that: then the accumulator's previous use (two tiles back) is
-    // certain to be complete when a worker has finished the last tile's stages.
-    p.helpers = (p.fast_epi && 2 * pl.num_kb >= pl.a_slots + 2) ? 1 : 0;
-    st = launch_expand_q<MODE>(tm, tmo, p, pl, s);
-    if (st != BCQ_OK) return st;
-    if (pl.splits > 1) {
-        const long long total = (long long)n * Mdim;
-        splitk_reduce_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(
-            n, Mdim, pl.splits, p.partial, bias, out, (long long)ldo, p.out_bf16);
-    bcq::count_launch();
-        BCQ_CUDA_TRY(cudaGetLastError());
-    }
-    return BCQ_OK;
+    // The workers find the last segment's accumulator by barrier parity alone.  They run at most
+    // `a_slots` pipeline stages ahead of the tensor core, so the parity is unambiguous only if the last
+    // two segments are longer than that: then the accumulator's previous use (two segments back) is
+    // certain to be complete when a worker has finished the last segment's stages (always so where a
+    // pair has no more than two segments).
+    const int len2 = pl.num_kb + (pl.res_tiles > 0 ? pl.piece_len : pl.num_kb);  // at least, of the last two of three
+    p.helpers = (pl.full_tiles <= pl.pairs || len2 >= pl.a_slots + 2) ? 1 : 0;
+    return launch_expand_q<MODE>(tm, tmo, p, pl, s);
 }
 
 template <int QM>

@@ -324,6 +324,32 @@ def test_many_tiles_per_cta_with_short_k(d_in):
     assert rel_err(bcq.linear_fwd(Xd, bd, ad, d_in, g).cpu().numpy(), ref) <= TOL
 
 
+@pytest.mark.parametrize("n,d_in,d_out,q,g", [(40, 8192, 200, 2, 128), (64, 2112, 264, 4, 64), (17, 1056, 1032, 5, 96),
+                                              (5100, 15400, 1000, 3, 15400)])
+def test_tiles_cut_along_k(n, d_in, d_out, q, g):
+    # Few tiles: every tile in several pieces, one per CTA pair (last pieces shorter).  The last case has 80
+    # tiles for 74 pairs: pieces of six tiles first, then a whole tile per pair.  Against a dense fp64
+    # product with the dequantized weights (dequantize has its own test against the oracle).
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    W = torch.randn((d_out, d_in), generator=gen, device="cuda") * 0.02
+    bits, alpha, _ = bcq.quantize(W, q, g)
+    X = torch.randn((n, d_in), generator=gen, device="cuda").bfloat16()
+    bias = torch.randn(d_out, generator=gen, device="cuda")
+    ref = (X.double() @ bcq.dequantize(bits, alpha, d_in, g).double().t()).cpu().numpy()
+    for dt, tol in ((torch.float32, TOL), (torch.bfloat16, TOL + 2.0 ** -8)):
+        Y = bcq.linear_fwd(X, bits, alpha, d_in, g, bias=bias, out_dtype=dt)
+        assert torch.equal(Y, bcq.linear_fwd(X, bits, alpha, d_in, g, bias=bias, out_dtype=dt)), "two runs differ"
+        assert rel_err(Y.float().cpu().numpy(), ref + bias.double().cpu().numpy()) <= tol
+    # the same contraction as an input gradient: the transposed matrix
+    bits, alpha, _ = bcq.quantize(W.t().contiguous(), q, 32 if d_out % 32 == 0 else d_out)
+    gt = 32 if d_out % 32 == 0 else d_out
+    ref = (X.double() @ bcq.dequantize(bits, alpha, d_out, gt).double()).cpu().numpy()
+    for dt, tol in ((torch.float32, TOL), (torch.bfloat16, TOL + 2.0 ** -8)):
+        dX = bcq.linear_bwd_x(X, bits, alpha, d_out, gt, out_dtype=dt)
+        assert torch.equal(dX, bcq.linear_bwd_x(X, bits, alpha, d_out, gt, out_dtype=dt)), "two runs differ"
+        assert rel_err(dX.float().cpu().numpy(), ref) <= tol
+
+
 def test_bwd_x_many_tiles_per_cta_with_short_k():
     n, d_in, d_out, q, g = 4096, 2560, 64, 4, 128
     _, X, dY, bits, alpha, _, _ = make_case(811, n, d_in, d_out, q, g)
