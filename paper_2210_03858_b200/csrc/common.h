@@ -1,8 +1,10 @@
-// Host-side helpers shared by the translation units of the library (no device code here).
+// Helpers shared by the translation units of the library.
 #pragma once
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
+
+#include <utility>
 
 #include "../../include/bcq.h"
 
@@ -50,6 +52,40 @@ inline int sm_count() {
     }
     return cached;
 }
+
+// Launches a kernel so that it may start while the kernel before it in the stream is finishing
+// (programmatic dependent launch): its blocks are scheduled and run up to their pdl_wait() early, which
+// takes 2 - 3 us of launch latency and set-up off every kernel of a chain.  Every kernel launched this way
+// calls pdl_wait() in all threads before it touches global memory.  cluster: CTAs per cluster.
+template <typename... Params, typename... Args>
+inline cudaError_t launch_pdl(void (*kern)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t stream, unsigned cluster,
+                              Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+    if (e != cudaSuccess) return e;
+    count_launch();
+    return cudaGetLastError();
+}
+
+#ifdef __CUDACC__
+// Until the kernel before this one in the stream has finished and its writes are visible.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The kernel after this one may be scheduled once every CTA of this one has said so (or ended).
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 

@@ -130,6 +130,7 @@ dalpha_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant
     __syncthreads();
     ptx::cluster_sync();  // the peer's barriers exist
     ptx::tc_fence_after_sync();
+    pdl_wait();
     const uint32_t tmem_base = *tmem_holder;
 
     if (warp == 0) {
@@ -158,6 +159,7 @@ dalpha_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant
                     if (++s == kStages) { s = 0; ph ^= 1u; }
                 }
             }
+            if (!p.direct) pdl_trigger();  // the reduction follows; other kernels gain nothing (see expand.cu)
             // giving up: the copies in flight are counted on the leader's barriers, which may never
             // complete; they land within microseconds, so wait a thousand times as long
             if (!ok) for (int i = 0; i < 1000; ++i) __nanosleep(2000);
@@ -313,6 +315,8 @@ dalpha_reduce_kernel(int d_out, int d_in, int q, int g, int G, int HN, int split
                      uint32_t plane_mask, float scale, int accumulate, const float* __restrict__ partial,
                      float* __restrict__ dalpha) {
     __shared__ float sums[8][32];
+    pdl_trigger();
+    pdl_wait();
     const int jx = threadIdx.x & 31, part = threadIdx.x >> 5;
     const int jblocks = (d_out + 31) / 32;
     const int jb = blockIdx.x % jblocks;
@@ -431,27 +435,10 @@ extern "C" bcq_status bcq_linear_bwd_alpha(int d_out, int d_in, int q, int g, in
     const int tiles = pl.m_tiles * pl.n_tiles * pl.splits;
     const int per_pair = ceil_div(tiles, std::max(1, sm_count() / 2));
     if ((st = ensure_dynamic_smem(dalpha_kernel, kDalphaSmem)) != BCQ_OK) return st;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2u * (unsigned)ceil_div(tiles, per_pair));
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kDalphaSmem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    BCQ_CUDA_TRY(cudaLaunchKernelEx(&cfg, dalpha_kernel, tm_dy, tm_x, p));
-    bcq::count_launch();
-    BCQ_CUDA_TRY(cudaGetLastError());
+    BCQ_CUDA_TRY(launch_pdl(dalpha_kernel, dim3(2u * (unsigned)ceil_div(tiles, per_pair)), kThreads, kDalphaSmem, s, 2, tm_dy, tm_x, p));
     if (p.direct) return BCQ_OK;
     const long long rblocks = (long long)q * p.G * ((d_out + 31) / 32);
-    dalpha_reduce_kernel<<<(unsigned)rblocks, 256, 0, s>>>(
-        d_out, d_in, q, g, p.G, kHN, pl.splits, pl.n_subtiles, pl.slots, plane_mask, scale, accumulate,
-        p.partial, dalpha);
-    bcq::count_launch();
-    BCQ_CUDA_TRY(cudaGetLastError());
+    BCQ_CUDA_TRY(launch_pdl(dalpha_reduce_kernel, dim3((unsigned)rblocks), 256, 0, s, 1, d_out, d_in, q, g, p.G, kHN, pl.splits,
+                            pl.n_subtiles, pl.slots, plane_mask, scale, accumulate, (const float*)p.partial, dalpha));
     return BCQ_OK;
 }

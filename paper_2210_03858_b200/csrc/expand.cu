@@ -340,6 +340,8 @@ template <int VPL>
 __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
     __shared__ uint32_t red[8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    pdl_trigger();
+    pdl_wait();
     // roles by block id: tokens, then max|alpha|, then the regrouping blocks.  The hardware starts
     // blocks in index order, and the short, latency-bound regrouping blocks should not queue
     // behind the register-heavy token blocks, so the ids run backwards.
@@ -516,6 +518,8 @@ template <int NW>
 __global__ void __launch_bounds__(256) code_planes_kernel(int mode, int d_out, int pitch, int q, int rows_padded,
                                                            int words_padded, int num_kb, const uint32_t* __restrict__ bits,
                                                            uint32_t* __restrict__ codes) {
+    pdl_trigger();
+    pdl_wait();
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (long long)rows_padded * words_padded) return;
     const int wd = (int)(idx % words_padded);
@@ -707,6 +711,7 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
     __syncthreads();
     ptx::cluster_sync();  // the peer's barriers exist
     ptx::tc_fence_after_sync();
+    pdl_wait();
     const uint32_t tmem_base = *tmem_holder;
 
     // every role walks the same sequence of tiles and pipeline stages
@@ -903,6 +908,9 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
                     if (++s == NB) { s = 0; ph ^= 1u; }
                 }
             }
+            // (no pdl_trigger here: blocks of the next call's pre-pass that start under this kernel crowd
+            // onto the few SMs it leaves free, and the pre-pass then lacks the others' bandwidth; measured
+            // on a training step of a layer of width 1600: 872 us without, 914 with)
             // giving up: the copies in flight are counted on the leader's barriers, which may never
             // complete; they land within microseconds, so wait a thousand times as long
             if (!ok) for (int i = 0; i < 1000; ++i) __nanosleep(2000);
@@ -1292,6 +1300,8 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
 __global__ void splitk_reduce_kernel(int n, int Mdim, int splits, const float* __restrict__ partial,
                                      const float* __restrict__ bias, void* out, long long ldo,
                                      int out_bf16) {
+    pdl_trigger();
+    pdl_wait();
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long total = (long long)n * Mdim;
     if (idx >= total) return;
@@ -1394,6 +1404,8 @@ decode_kernel(const __grid_constant__ CUtensorMap tmap_bits, const DecodeParams 
     __syncthreads();
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_holder;
+    pdl_trigger();
+    pdl_wait();
 
     if (warp == 0) {
         // ---------------- TMA producer: plane words only
@@ -1710,21 +1722,7 @@ bcq_status launch_expand(const CUtensorMap& tm, const CUtensorMap& tmo, const Ex
     auto kern = expand_gemm_kernel<MODE, QM>;
     bcq_status st0 = ensure_dynamic_smem(kern, pl.smem);
     if (st0 != BCQ_OK) return st0;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2u * (unsigned)pl.pairs);
-    cfg.blockDim = dim3(kPfThreads);
-    cfg.dynamicSmemBytes = pl.smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    BCQ_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, tm, tmo, p));
-    bcq::count_launch();
-    BCQ_CUDA_TRY(cudaGetLastError());
+    BCQ_CUDA_TRY(launch_pdl(kern, dim3(2u * (unsigned)pl.pairs), kPfThreads, pl.smem, stream, 2, tm, tmo, p));
     return BCQ_OK;
 }
 
@@ -1745,12 +1743,8 @@ bcq_status launch_code_planes(int mode, int d_out, int d_in, int q, const Expand
     const int words_padded = (mode == MODE_FWD) ? pl.num_kb * 2 : pl.m_tiles * 4;
     const long long total = (long long)rows_padded * words_padded;
     const unsigned grid = (unsigned)((total + 255) / 256);
-    if (q == 4)
-        code_planes_kernel<4><<<grid, 256, 0, s>>>(mode, d_out, pitch, q, rows_padded, words_padded, pl.num_kb, bits, codes);
-    else
-        code_planes_kernel<3><<<grid, 256, 0, s>>>(mode, d_out, pitch, q, rows_padded, words_padded, pl.num_kb, bits, codes);
-    bcq::count_launch();
-    BCQ_CUDA_TRY(cudaGetLastError());
+    BCQ_CUDA_TRY(launch_pdl(q == 4 ? code_planes_kernel<4> : code_planes_kernel<3>, dim3(grid), 256, 0, s, 1, mode, d_out, pitch, q,
+                            rows_padded, words_padded, pl.num_kb, bits, codes));
     return BCQ_OK;
 }
 
@@ -1824,10 +1818,7 @@ bcq_status run_expand(int d_out, int d_in, int q, int g, int n, const void* act,
     // rows are read twice instead (the second time from L2), four loads of a lane at a time:
     // holding them costs so many registers that the blocks resident on an SM are too few to
     // cover the memory latency (measured: 14.8 us against 11.3 us for 4096 rows of 1600).
-    if (nvec <= 32 * 4) prepare_kernel<4><<<pgrid, 256, 0, s>>>(pp);
-    else prepare_kernel<0><<<pgrid, 256, 0, s>>>(pp);
-    bcq::count_launch();
-    BCQ_CUDA_TRY(cudaGetLastError());
+    BCQ_CUDA_TRY(launch_pdl(nvec <= 32 * 4 ? prepare_kernel<4> : prepare_kernel<0>, dim3(pgrid), 256, 0, s, 1, pp));
 
     ExpandParams p;
     p.d_out = d_out; p.d_in = d_in; p.q = q; p.g = g;
@@ -1865,9 +1856,7 @@ bcq_status launch_decode(const CUtensorMap& tm_bits, const DecodeParams& p, cons
     bcq_status st0 = ensure_dynamic_smem(kern, smem);
     if (st0 != BCQ_OK) return st0;
     dim3 grid((unsigned)pl.m_tiles, (unsigned)pl.splits);
-    kern<<<grid, kThreads, smem, s>>>(tm_bits, p);
-    bcq::count_launch();
-    BCQ_CUDA_TRY(cudaGetLastError());
+    BCQ_CUDA_TRY(launch_pdl(kern, grid, kThreads, smem, s, 1, tm_bits, p));
     return BCQ_OK;
 }
 
@@ -1899,10 +1888,8 @@ bcq_status run_decode(int d_out, int d_in, int q, int g, int n, const void* X, s
     if (st != BCQ_OK) return st;
     if (pl.splits > 1) {
         const long long total = (long long)n * d_out;
-        splitk_reduce_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(
-            n, d_out, pl.splits, p.partial, bias, Y, (long long)ldy, p.out_bf16);
-    bcq::count_launch();
-        BCQ_CUDA_TRY(cudaGetLastError());
+        BCQ_CUDA_TRY(launch_pdl(splitk_reduce_kernel, dim3((unsigned)((total + 255) / 256)), 256, 0, s, 1, n, d_out, pl.splits,
+                                (const float*)p.partial, bias, Y, (long long)ldy, p.out_bf16));
     }
     return BCQ_OK;
 }

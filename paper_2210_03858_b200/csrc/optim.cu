@@ -42,6 +42,8 @@ struct AdamParams {
 __global__ void __launch_bounds__(256)
 alpha_adamw_kernel(long long count, Segments sg, AdamParams h, float* __restrict__ alpha,
                    const float* __restrict__ grad, float* __restrict__ m, float* __restrict__ v) {
+    bcq::pdl_trigger();
+    bcq::pdl_wait();
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += stride) {
         long long idx = e;
@@ -65,6 +67,8 @@ alpha_adamw_kernel(long long count, Segments sg, AdamParams h, float* __restrict
 __global__ void __launch_bounds__(256)
 alpha_gather_kernel(long long count, Segments sg, int to_compact, float* __restrict__ flat,
                     float* __restrict__ compact) {
+    bcq::pdl_trigger();
+    bcq::pdl_wait();
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += stride) {
         const int s = find_segment(sg.prefix, sg.nseg, e);
@@ -109,9 +113,8 @@ extern "C" bcq_status bcq_alpha_adamw(long long count, int nseg, const long long
     h.step_size = (float)((double)lr / (1.0 - pow((double)beta1, (double)step)));
     h.inv_sqrt_bc2 = (float)(1.0 / sqrt(1.0 - pow((double)beta2, (double)step)));
     h.grad_scale = grad_scale;
-    alpha_adamw_kernel<<<grid_for(count), 256, 0, (cudaStream_t)stream>>>(count, sg, h, alpha, dalpha, m, v);
-    bcq::count_launch();
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = bcq::launch_pdl(alpha_adamw_kernel, dim3(grid_for(count)), 256, 0, (cudaStream_t)stream, 1, count, sg, h,
+                                          alpha, dalpha, m, v);
     if (e != cudaSuccess) return bcq::cuda_fail(e);
     return BCQ_OK;
 }
@@ -122,9 +125,8 @@ static bcq_status gather_common(long long count, int nseg, const long long* seg_
     if (!seg_begin || !seg_prefix || !flat || !compact) return BCQ_ERR_NULL;
     if (count == 0) return BCQ_OK;
     Segments sg{nseg, seg_begin, seg_prefix, nullptr};
-    alpha_gather_kernel<<<grid_for(count), 256, 0, (cudaStream_t)stream>>>(count, sg, to_compact, flat, compact);
-    bcq::count_launch();
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = bcq::launch_pdl(alpha_gather_kernel, dim3(grid_for(count)), 256, 0, (cudaStream_t)stream, 1, count, sg,
+                                          to_compact, flat, compact);
     if (e != cudaSuccess) return bcq::cuda_fail(e);
     return BCQ_OK;
 }

@@ -162,6 +162,8 @@ quantize_kernel(const QuantParams p) {
     constexpr int NT = TW * 32;
     constexpr int TEAMS = (TW == 1) ? 4 : 1;
     __shared__ double red_scratch[32];
+    bcq::pdl_trigger();
+    bcq::pdl_wait();
     __shared__ double level_smem[TEAMS][1 << BCQ_MAX_Q];
 
     const int lane = threadIdx.x & 31;
@@ -459,6 +461,8 @@ team_quantize_kernel(const QuantParams p) {
     constexpr int NT = L * TW;                       // threads of a team
     constexpr int TEAMS = TW == 1 ? 128 / L : 1;     // per CTA
     __shared__ double scratch[TW == 1 ? 1 : 32];
+    bcq::pdl_trigger();
+    bcq::pdl_wait();
     const int tl = TW == 1 ? (int)(threadIdx.x & (L - 1)) : (int)threadIdx.x;
     const long long item0 = (long long)blockIdx.x * TEAMS + (TW == 1 ? threadIdx.x / L : 0);
     // teams past the last item repeat it (the shuffles need every lane) and store nothing
@@ -753,9 +757,7 @@ cudaError_t launch_team(const QuantParams& p, cudaStream_t stream) {
     constexpr int TEAMS = TW == 1 ? 128 / L : 1;
     const int threads = TW == 1 ? 128 : TW * 32;
     const unsigned blocks = (unsigned)((p.items + TEAMS - 1) / TEAMS);
-    team_quantize_kernel<NI, L, TW, Q><<<blocks, threads, 0, stream>>>(p);
-    bcq::count_launch();
-    return cudaGetLastError();
+    return bcq::launch_pdl(team_quantize_kernel<NI, L, TW, Q>, dim3(blocks), threads, 0, stream, 1, p);
 }
 
 // The smallest team that holds a group at 32 weights a thread (8 or 16 for groups of 32 or 64).
@@ -782,9 +784,7 @@ cudaError_t launch_quantize(const QuantParams& p, cudaStream_t stream) {
     long long blocks = (p.items + TEAMS - 1) / TEAMS;
     const long long cap = (long long)bcq::sm_count() * 64;  // grid-stride beyond this
     if (blocks > cap) blocks = cap;
-    quantize_kernel<EPT, TW><<<(unsigned)blocks, threads, 0, stream>>>(p);
-    bcq::count_launch();
-    return cudaGetLastError();
+    return bcq::launch_pdl(quantize_kernel<EPT, TW>, dim3((unsigned)blocks), threads, 0, stream, 1, p);
 }
 
 __global__ void dequantize_kernel(int d_out, int d_in, int q, int g, int G, int pitch,
