@@ -289,10 +289,13 @@ struct PrepParams {
     int num_counters;
 };
 
-// One warp per token row; VPL = 16-byte vectors a lane keeps in registers between finding the
-// row's largest magnitude and writing the scaled fp16 row (VPL = 0: the row is read twice).
+// WPT warps per token row.  A lane keeps up to four 16-byte vectors of the row in registers between finding
+// the row's largest magnitude and writing the scaled fp16 row, so rows of up to 1024 WPT elements are
+// read once; longer rows (WPT = 8, more than 8192 elements) are read again from L2.  Four loads of a lane
+// in flight and few registers: the token blocks are bound by memory (n x K x 4 bytes; with a warp per
+// token and two reads, 4096 x 6400 took 21 us and 4096 x 1600 8.5 us).
 // Blocks past the activation blocks scan alpha instead.
-constexpr int kPrepTokensPerBlock = 8;
+constexpr int kPrepWarps = 8;
 
 __device__ __forceinline__ uint32_t max_mag_bf16x8(const uint4& x, int k0, int K) {
     if (k0 + 8 <= K) {
@@ -336,7 +339,7 @@ __device__ __forceinline__ uint4 scale_to_fp16x8(const uint4& x, int k0, int K, 
     return o;
 }
 
-template <int VPL>
+template <int WPT>
 __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
     __shared__ uint32_t red[8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -457,52 +460,55 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
         }
         return;
     }
-    const int t = bid * kPrepTokensPerBlock + warp;
-    if (t >= p.n) return;
-    const uint4* src = reinterpret_cast<const uint4*>(p.in + (long long)t * p.ld_in);
+    const int slot = warp / WPT;                        // of the block's kPrepWarps / WPT tokens
+    const int t = bid * (kPrepWarps / WPT) + slot;
+    const int tl = (warp % WPT) * 32 + lane;            // thread of the token
+    constexpr int kThreadsPerToken = WPT * 32;
+    const bool live = t < p.n;
+    const uint4* src = reinterpret_cast<const uint4*>(p.in + (long long)(live ? t : 0) * p.ld_in);
     uint4* dst = reinterpret_cast<uint4*>(p.out + (long long)t * p.ld_out);
-    const int nvec = (p.K + 7) / 8;
+    const int nvec = live ? (p.K + 7) / 8 : 0;
     uint32_t m = 0u;
-    uint4 held[VPL > 0 ? VPL : 1];
-    if (VPL > 0) {
+    uint4 held[4];
+    int v0 = tl;
+    do {
 #pragma unroll
-        for (int i = 0; i < VPL; ++i) {
-            const int v = lane + 32 * i;
+        for (int i = 0; i < 4; ++i) {
+            const int v = v0 + kThreadsPerToken * i;
             held[i] = (v < nvec) ? __ldg(src + v) : make_uint4(0u, 0u, 0u, 0u);
         }
 #pragma unroll
-        for (int i = 0; i < VPL; ++i) m = max(m, max_mag_bf16x8(held[i], (lane + 32 * i) * 8, p.K));
-    } else {
-        // long rows: four loads of a lane in flight at a time
-        for (int v0 = lane; v0 < nvec; v0 += 128) {
-            uint4 x[4];
+        for (int i = 0; i < 4; ++i) m = max(m, max_mag_bf16x8(held[i], (v0 + kThreadsPerToken * i) * 8, p.K));
+        v0 += 4 * kThreadsPerToken;
+    } while (v0 - tl < nvec);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (WPT > 1) {
+        if (lane == 0) red[warp] = m;
+        __syncthreads();
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-                x[u] = (v0 + 32 * u < nvec) ? __ldg(src + v0 + 32 * u) : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) m = max(m, max_mag_bf16x8(x[u], (v0 + 32 * u) * 8, p.K));
-        }
+        for (int w = 0; w < WPT; ++w) m = max(m, red[slot * WPT + w]);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     const int sh = shift_for(exponent_of_bits(m << 16), 14);
     const float scale = pow2f(sh);
-    if (lane == 0) p.tok_inv_scale[t] = pow2f(-sh);
-    if (VPL > 0) {
+    if (live && tl == 0) p.tok_inv_scale[t] = pow2f(-sh);
+    if (nvec <= 4 * kThreadsPerToken) {
 #pragma unroll
-        for (int i = 0; i < VPL; ++i) {
-            const int v = lane + 32 * i;
+        for (int i = 0; i < 4; ++i) {
+            const int v = tl + kThreadsPerToken * i;
             if (v < nvec) dst[v] = scale_to_fp16x8(held[i], v * 8, p.K, scale);
         }
     } else {
-        for (int v0 = lane; v0 < nvec; v0 += 128) {
-            uint4 x[4];
+        for (v0 = tl; v0 < nvec; v0 += 4 * kThreadsPerToken) {
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-                x[u] = (v0 + 32 * u < nvec) ? __ldg(src + v0 + 32 * u) : make_uint4(0u, 0u, 0u, 0u);
+            for (int i = 0; i < 4; ++i) {
+                const int v = v0 + kThreadsPerToken * i;
+                held[i] = (v < nvec) ? __ldg(src + v) : make_uint4(0u, 0u, 0u, 0u);
+            }
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (v0 + 32 * u < nvec) dst[v0 + 32 * u] = scale_to_fp16x8(x[u], (v0 + 32 * u) * 8, p.K, scale);
+            for (int i = 0; i < 4; ++i) {
+                const int v = v0 + kThreadsPerToken * i;
+                if (v < nvec) dst[v] = scale_to_fp16x8(held[i], v * 8, p.K, scale);
+            }
         }
     }
 }
@@ -1810,15 +1816,14 @@ bcq_status run_expand(int d_out, int d_in, int q, int g, int n, const void* act,
     if (coded && prepared == nullptr) {
         if ((st = launch_code_planes(MODE, d_out, d_in, q, pl, bits, pp.bits_t, s)) != BCQ_OK) return st;
     }
-    const int tok_blocks = ceil_div(n, kPrepTokensPerBlock);
+    const int nvec = (Kdim + 7) / 8;
+    int wpt = 1;  // warps per token (see prepare_kernel)
+    while (wpt < kPrepWarps && nvec > wpt * 128) wpt *= 2;
+    const int tok_blocks = ceil_div(n, kPrepWarps / wpt);
     pp.act_blocks = tok_blocks;
     const unsigned pgrid = (unsigned)(tok_blocks + ablocks + pp.bits_blocks + alpha_tr_blocks);
-    const int nvec = (Kdim + 7) / 8;
-    // Rows of up to 1024 elements stay in registers between the two passes over them.  Longer
-    // rows are read twice instead (the second time from L2), four loads of a lane at a time:
-    // holding them costs so many registers that the blocks resident on an SM are too few to
-    // cover the memory latency (measured: 14.8 us against 11.3 us for 4096 rows of 1600).
-    BCQ_CUDA_TRY(launch_pdl(nvec <= 32 * 4 ? prepare_kernel<4> : prepare_kernel<0>, dim3(pgrid), 256, 0, s, 1, pp));
+    auto prep = wpt == 1 ? prepare_kernel<1> : wpt == 2 ? prepare_kernel<2> : wpt == 4 ? prepare_kernel<4> : prepare_kernel<8>;
+    BCQ_CUDA_TRY(launch_pdl(prep, dim3(pgrid), 256, 0, s, 1, pp));
 
     ExpandParams p;
     p.d_out = d_out; p.d_in = d_in; p.q = q; p.g = g;
