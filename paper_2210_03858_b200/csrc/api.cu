@@ -70,14 +70,12 @@ extern "C" int bcq_last_cuda_error(void) { return bcq::t_last_cuda_error; }
 extern "C" bcq_status bcq_device_timeout_flag(int* flag_out, int reset) {
     if (flag_out == nullptr) return BCQ_ERR_NULL;
     BCQ_CUDA_TRY(cudaDeviceSynchronize());
-    int a = 0, b = 0, c = 0;
+    int a = 0, b = 0;
     bcq_status st = bcq::expand_timeout_flag(&a, reset);
     if (st != BCQ_OK) return st;
     st = bcq::dalpha_timeout_flag(&b, reset);
     if (st != BCQ_OK) return st;
-    st = bcq::decode_timeout_flag(&c, reset);
-    if (st != BCQ_OK) return st;
-    *flag_out = a != 0 ? a : (b != 0 ? b : c);
+    *flag_out = a != 0 ? a : b;
     return BCQ_OK;
 }
 

@@ -184,7 +184,6 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // per-TU device timeout flags
 bcq_status expand_timeout_flag(int* flag_out, int reset);
 bcq_status dalpha_timeout_flag(int* flag_out, int reset);
-bcq_status decode_timeout_flag(int* flag_out, int reset);
 
 // workspace sizes (defined next to the kernels that use them)
 size_t fwd_workspace_bytes(int d_out, int d_in, int q, int g, int n);
