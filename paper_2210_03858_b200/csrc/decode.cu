@@ -18,11 +18,14 @@
 // left per weight is 1.6 (q = 4) or 1.2 (q = 3) instructions of the logic pipe (64 lanes per clock and SM),
 // 39 - 53 weights per clock and SM where HBM delivers 37 - 46.
 //
-// Work split: a unit is 16 rows x 128 k.  The 16-row tiles are dealt to the CTAs (two per SM), the steps
-// of 128 k to the warps of a CTA; a warp takes its steps one after the other and, within a step, all
-// tiles, so a step's activations are converted once (bf16 -> fp16 times a power of two per token and
+// Work split: a unit is 16 rows x 128 k.  The 16-row tiles are dealt to the CTAs (one per SM).  The
+// units of a CTA, numbered step by step with all tiles of a step together, are dealt to its warps, so a step's activations are converted once (bf16 -> fp16 times a power of two per token and
 // step) and stay in registers as B fragments.  Its sums wait in a private slot of shared memory per
 // tile; the slots of a tile are added at the end, in order.  No CTA needs another.
+//
+// One CTA of 16 warps an SM: with two of 8 warps, each CTA had half as many tiles to use a step's activations
+// for (OPT-6.7B layer, q = 4, one token: 68 us against 53); 20 or 24 warps with fewer registers each
+// were no faster (54 us) and slower for 16 tokens (73 and 92 us against 66).
 //
 // Weights go from global memory to registers two units ahead of their use.  The kernel may start
 // while the previous kernel of the stream is finishing (programmatic dependent launch): the pack is
@@ -37,9 +40,8 @@ namespace {
 
 using namespace bcq;
 
-constexpr int kDpWarps = 8;
+constexpr int kDpWarps = 16;
 constexpr int kDpThreads = kDpWarps * 32;
-constexpr int kDpCtasPerSm = 2;
 constexpr int kDpStepK = 128;      // weights of a row per unit: eight K = 16 MMAs
 constexpr int kDpRows = 16;        // rows of a unit: the M of the MMA
 constexpr uint32_t kDpTableBytes = kDpRows * 16;  // tables of one (tile, group)
@@ -167,8 +169,7 @@ struct DecPackedParams {
     int d_out, d_in, g, G, n;
     int steps;
     int per, rem;            // row tiles per CTA and remainder
-    int kw, tw;              // warps that share the steps of a tile; tiles at a time
-    int round, slots;        // tiles between two additions; of them, slots of one warp
+    int round;               // tiles between two additions
     uint32_t g_magic;        // ceil(2^32 / g) where k / g = hi32(k g_magic) for every k < d_in, else 0
     const __nv_bfloat16* X;
     long long ldx;
@@ -218,29 +219,29 @@ struct UnitWords {
 };
 
 template <int Q, int NT, int PARTS>
-__global__ void __launch_bounds__(kDpThreads, kDpCtasPerSm)
+__global__ void __launch_bounds__(kDpThreads, 1)
 decode_packed_kernel(const DecPackedParams p) {
     extern __shared__ float4 sums[];  // [warp][slot][NT][32 lanes]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int gr = lane >> 2, tq = lane & 3;
     const int tile0 = (int)blockIdx.x * p.per + min((int)blockIdx.x, p.rem);
     const int ntiles = p.per + ((int)blockIdx.x < p.rem ? 1 : 0);
-    const int twi = warp / p.kw, kwi = warp - twi * p.kw;
-    const int cnt = twi < p.tw ? (p.steps - kwi + p.kw - 1) / p.kw : 0;  // the warp's steps: kwi, kwi + kw, ...
-    float4* mine = sums + (size_t)warp * p.slots * (NT * 32) + lane;
+    float4* mine = sums + (size_t)warp * p.round * (NT * 32) + lane;
 
     pdl_trigger();
     for (int first = 0; first < ntiles; first += p.round) {
         const int round_n = min(p.round, ntiles - first);
-        const int nmy = twi < round_n ? (round_n - twi + p.tw - 1) / p.tw : 0;  // the warp's tiles: twi, twi + tw, ...
-        const int units = cnt * nmy;
+        // the warp's units: an equal, contiguous share of the round's, numbered step by step
+        const int all = round_n * p.steps;
+        const int u0 = all * warp / kDpWarps, u1 = all * (warp + 1) / kDpWarps;
+        const int st0 = u0 / round_n, i0 = u0 - st0 * round_n;
 
         // ---- loading: unit (step, tile) pairs in the order of use
         const uint8_t* lp_codes = p.codes;
         const uint8_t* lp_tables[PARTS];
-        int l_st = kwi, l_i = 0, l_left = units;
-        auto seek = [&]() {  // to the first tile of step l_st
-            const size_t tile = (size_t)(tile0 + first + twi);
+        int l_st = st0, l_i = i0, l_left = u1 - u0;
+        auto seek = [&]() {  // to tile l_i of step l_st
+            const size_t tile = (size_t)(tile0 + first + l_i);
             lp_codes = p.codes + (tile * p.steps + l_st) * (Q * 256) + lane * 16;
 #pragma unroll
             for (int a = 0; a < PARTS; ++a) {
@@ -249,7 +250,7 @@ decode_packed_kernel(const DecPackedParams p) {
                 lp_tables[a] = p.tables + (tile * p.G + c) * kDpTableBytes + gr * 16;
             }
         };
-        const size_t codes_stride = (size_t)p.tw * p.steps * (Q * 256), tables_stride = (size_t)p.tw * p.G * kDpTableBytes;
+        const size_t codes_stride = (size_t)p.steps * (Q * 256), tables_stride = (size_t)p.G * kDpTableBytes;
         auto load = [&](UnitWords<Q, PARTS>& u) {
             if (l_left == 0) return;
             --l_left;
@@ -267,9 +268,9 @@ decode_packed_kernel(const DecPackedParams p) {
                 u.ta[a] = ptx::ldg_nc_v4(lp_tables[a]);
                 u.tb[a] = ptx::ldg_nc_v4(lp_tables[a] + 128);
             }
-            if (++l_i == nmy) {
+            if (++l_i == round_n) {
                 l_i = 0;
-                l_st += p.kw;
+                ++l_st;
                 seek();
             } else {
                 lp_codes += codes_stride;
@@ -281,12 +282,13 @@ decode_packed_kernel(const DecPackedParams p) {
         seek();
         load(ua);
         load(ub);
+        for (int i = 0; i < round_n * NT; ++i) mine[i * 32] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (first == 0) {
             pdl_wait();
             // the activations of the warp's later steps: into L1 while the first step is at work
             // (32 lanes: 16 tokens x two 128-byte lines of a step)
-            for (int s = 1; s < (nmy > 0 ? cnt : 0); ++s) {
-                const int k = (kwi + s * p.kw) * kDpStepK + (lane & 1) * 64;
+            for (int s = st0 + 1; s * round_n < u1; ++s) {
+                const int k = s * kDpStepK + (lane & 1) * 64;
                 if ((lane >> 1) < p.n && k < p.d_in)
                     asm volatile("prefetch.global.L1 [%0];" ::"l"(p.X + (long long)(lane >> 1) * p.ldx + k));
             }
@@ -341,9 +343,10 @@ decode_packed_kernel(const DecPackedParams p) {
             }
         };
 
-        int u_st = kwi, u_i = 0;
+        int u_st = st0, u_i = i0;
+        bool fresh = true;
         auto unit = [&](const UnitWords<Q, PARTS>& u) {
-            if (u_i == 0) load_x(u_st);
+            if (fresh) load_x(u_st);
             float d[NT][4];
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt) d[nt][0] = d[nt][1] = d[nt][2] = d[nt][3] = 0.f;
@@ -366,35 +369,34 @@ decode_packed_kernel(const DecPackedParams p) {
             float4* slot = mine + u_i * (NT * 32);
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt) {
-                float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (u_st != kwi) s = slot[nt * 32];
+                float4 s = slot[nt * 32];
                 s.x = fmaf(f0[nt], d[nt][0], s.x);
                 s.y = fmaf(f1[nt], d[nt][1], s.y);
                 s.z = fmaf(f0[nt], d[nt][2], s.z);
                 s.w = fmaf(f1[nt], d[nt][3], s.w);
                 slot[nt * 32] = s;
             }
-            if (++u_i == nmy) { u_i = 0; u_st += p.kw; }
+            fresh = (++u_i == round_n);
+            if (fresh) { u_i = 0; ++u_st; }
         };
 #pragma unroll 1
-        for (int u = 0; u < units; u += 2) {
+        for (int u = u0; u < u1; u += 2) {
             unit(ua);
             load(ua);
-            if (u + 1 < units) {
+            if (u + 1 < u1) {
                 unit(ub);
                 load(ub);
             }
         }
 
-        // ---- the tiles' sums: over the warps of a tile, in order
+        // ---- the tiles' sums: over the warps, in order
         __syncthreads();
         for (int e = threadIdx.x; e < round_n * NT * 32; e += kDpThreads) {
             const int ti = e / (NT * 32), ln = e & 31, nt = (e >> 5) % NT;
-            const int slot = ti / p.tw, w0 = (ti - slot * p.tw) * p.kw;
-            const float4* src = sums + ((size_t)w0 * p.slots + slot) * (NT * 32) + nt * 32 + ln;
+            const float4* src = sums + (size_t)(ti * NT + nt) * 32 + ln;
             float4 s = src[0];
-            for (int w = 1; w < p.kw; ++w) {
-                const float4 x = src[(size_t)w * p.slots * (NT * 32)];
+            for (int w = 1; w < kDpWarps; ++w) {
+                const float4 x = src[(size_t)w * p.round * (NT * 32)];
                 s.x += x.x; s.y += x.y; s.z += x.z; s.w += x.w;
             }
             const int tok = nt * 8 + 2 * (ln & 3);
@@ -425,16 +427,12 @@ decode_packed_kernel(const DecPackedParams p) {
 
 template <int Q, int NT, int PARTS>
 bcq_status launch_decode_packed(DecPackedParams p, int tiles, cudaStream_t s) {
-    const int ctas = std::min(tiles, kDpCtasPerSm * sm_count());
+    const int ctas = std::min(tiles, sm_count());
     p.per = tiles / ctas;
     p.rem = tiles % ctas;
     const int most = p.per + (p.rem > 0 ? 1 : 0);
-    // all warps on the steps of one tile when there are enough, else several tiles at a time
-    p.kw = std::min(kDpWarps, p.steps);
-    p.tw = std::max(1, std::min(kDpWarps / p.kw, most));
-    p.round = std::min(most, kDpMaxRound / NT * p.tw);
-    p.slots = ceil_div(p.round, p.tw);
-    const size_t smem = (size_t)kDpWarps * p.slots * NT * 512;  // at most 96 KiB
+    p.round = std::min(most, kDpMaxRound / NT);
+    const size_t smem = (size_t)kDpWarps * p.round * NT * 512;  // at most 192 KiB
     auto kern = decode_packed_kernel<Q, NT, PARTS>;
     const bcq_status st = ensure_dynamic_smem(kern, smem);
     if (st != BCQ_OK) return st;
