@@ -112,6 +112,24 @@ def lib() -> C.CDLL:
     return _lib
 
 
+_call = None
+
+
+def _fn():
+    """The native entry points of the frequent calls (csrc/binding.c), bound to the loaded library."""
+    global _call
+    if _call is None:
+        lib()
+        import importlib
+        try:
+            mod = importlib.import_module(__name__ + "._bcq_call")
+        except ImportError as e:
+            raise RuntimeError("binding not built: run paper_2210_03858_b200/build.py (%s)" % e) from e
+        mod.load(LIB_PATH)
+        _call = mod
+    return _call
+
+
 def status_string(status: int) -> str:
     return lib().bcq_status_string(status).decode()
 
@@ -144,10 +162,10 @@ def workspace_bytes(op: int, d_out: int, d_in: int, q: int, g: int, n: int = 0) 
 
 # ---------------------------------------------------------------------------- helpers
 
-# The small calls of the library take a few microseconds on the GPU, so the marshalling counts: plain
-# integers instead of ctypes objects, the raw stream handle instead of a Stream object, and no size
+# The small calls of the library take a few microseconds on the GPU, so the marshalling counts: the
+# frequent calls go through csrc/binding.c instead of ctypes, with the raw stream handle instead of a Stream object, and no size
 # query where the caller brought the workspace (the library checks its size anyway).  Measured on the
-# optimiser step plus checkpoint (two calls): 24 -> 15 us.
+# optimiser step plus checkpoint (two calls): 24 -> 12 us.
 
 _torch_module = None
 
@@ -205,7 +223,7 @@ def quantize(W, q: int, g: int, alt_iters: int = 0, want_sq_err: bool = False):
     bits = torch.empty((q, d_out, 4 * ((d_in + 127) // 128)), dtype=torch.int32, device=dev)
     alpha = torch.empty((q, d_out, G), dtype=torch.float32, device=dev)
     sq_err = torch.empty((d_out, G), dtype=torch.float64, device=dev) if want_sq_err else None
-    _check(lib().bcq_quantize(d_out, d_in, q, g, _ptr(W), W.stride(0), alt_iters, _ptr(bits),
+    _check(_fn().quantize(d_out, d_in, q, g, _ptr(W), W.stride(0), alt_iters, _ptr(bits),
                               _ptr(alpha), _ptr(sq_err), _stream()), "bcq_quantize")
     return bits, alpha, sq_err
 
@@ -248,7 +266,7 @@ def _fwd(fn, op, name, X, bits, alpha, d_in, g, bias, out, out_dtype, ws):
     assert X.is_cuda and X.dtype == torch.bfloat16 and X.dim() == 2 and X.stride(1) == 1
     if isinstance(bits, PreparedPlanes):
         assert bits.op == OP_FWD and op == OP_FWD
-        fn, name = lib().bcq_linear_fwd_prepared, "bcq_linear_fwd_prepared"
+        fn, name = _fn().fwd_prepared, "bcq_linear_fwd_prepared"
     q, d_out, _ = bits.shape
     n = X.shape[0]
     if out is None:
@@ -261,13 +279,13 @@ def _fwd(fn, op, name, X, bits, alpha, d_in, g, bias, out, out_dtype, ws):
 
 def linear_fwd(X, bits, alpha, d_in: int, g: int, bias=None, out=None, out_dtype=None, ws=None):
     """bcq_linear_fwd: X bf16 [n][d_in] -> Y [n][d_out] (Eq. 2)."""
-    return _fwd(lib().bcq_linear_fwd, OP_FWD, "bcq_linear_fwd", X, bits, alpha, d_in, g, bias, out,
+    return _fwd(_fn().fwd, OP_FWD, "bcq_linear_fwd", X, bits, alpha, d_in, g, bias, out,
                 out_dtype, ws)
 
 
 def linear_decode(X, bits, alpha, d_in: int, g: int, bias=None, out=None, out_dtype=None, ws=None):
     """bcq_linear_decode: same as linear_fwd for 1..16 tokens."""
-    return _fwd(lib().bcq_linear_decode, OP_DECODE, "bcq_linear_decode", X, bits, alpha, d_in, g,
+    return _fwd(_fn().decode, OP_DECODE, "bcq_linear_decode", X, bits, alpha, d_in, g,
                 bias, out, out_dtype, ws)
 
 
@@ -294,7 +312,7 @@ def linear_decode_packed(X, pack, d_out: int, d_in: int, q: int, g: int, bias=No
     if out is None:
         out = torch.empty((n, d_out), dtype=out_dtype or torch.float32, device=X.device)
     ws, ws_bytes = _ws(OP_DECODE_PACKED, d_out, d_in, q, g, n, ws, X.device)
-    _check(lib().bcq_linear_decode_packed(d_out, d_in, q, g, n, _ptr(X), X.stride(0), _ptr(pack),
+    _check(_fn().packed(d_out, d_in, q, g, n, _ptr(X), X.stride(0), _ptr(pack),
                                           _ptr(bias), _ptr(out), out.stride(0), _dtype_code(out),
                                           _ptr(ws), ws_bytes, _stream()), "bcq_linear_decode_packed")
     return out
@@ -329,10 +347,10 @@ def linear_bwd_x(dY, bits, alpha, d_in: int, g: int, out=None, out_dtype=None, w
     if out is None:
         out = torch.empty((n, d_in), dtype=out_dtype or torch.float32, device=dY.device)
     ws, ws_bytes = _ws(OP_BWD_X, d_out, d_in, q, g, n, ws, dY.device)
-    fn, name = lib().bcq_linear_bwd_x, "bcq_linear_bwd_x"
+    fn, name = _fn().bwd_x, "bcq_linear_bwd_x"
     if isinstance(bits, PreparedPlanes):
         assert bits.op == OP_BWD_X
-        fn, name = lib().bcq_linear_bwd_x_prepared, "bcq_linear_bwd_x_prepared"
+        fn, name = _fn().bwd_x_prepared, "bcq_linear_bwd_x_prepared"
     _check(fn(d_out, d_in, q, g, n, _ptr(dY), dY.stride(0), _ptr(bits), _ptr(alpha), _ptr(out),
               out.stride(0), _dtype_code(out), _ptr(ws), ws_bytes, _stream()), name)
     return out
@@ -351,7 +369,7 @@ def linear_bwd_alpha(dY, X, bits, d_in: int, g: int, plane_mask=None, scale: flo
     if out is None:
         out = torch.zeros((q, d_out, num_groups(d_in, g)), dtype=torch.float32, device=X.device)
     ws, ws_bytes = _ws(OP_BWD_ALPHA, d_out, d_in, q, g, n, ws, X.device)
-    _check(lib().bcq_linear_bwd_alpha(d_out, d_in, q, g, n, _ptr(dY), dY.stride(0), _ptr(X),
+    _check(_fn().bwd_alpha(d_out, d_in, q, g, n, _ptr(dY), dY.stride(0), _ptr(X),
                                       X.stride(0), _ptr(bits), plane_mask, scale,
                                       1 if accumulate else 0, _ptr(out), _ptr(ws), ws_bytes,
                                       _stream()), "bcq_linear_bwd_alpha")
@@ -391,7 +409,7 @@ def alpha_adamw(alpha, dalpha, m, v, step: int, lr: float, beta1: float = 0.9, b
         count, nseg, b, pfx, sc = alpha.numel(), 0, None, None, None
     else:
         count, nseg, b, pfx, sc = segments.count, segments.nseg, segments.begin, segments.prefix, segments.scale
-    _check(lib().bcq_alpha_adamw(count, nseg, _ptr(b), _ptr(pfx), _ptr(sc), _ptr(alpha), _ptr(dalpha), _ptr(m),
+    _check(_fn().adamw(count, nseg, _ptr(b), _ptr(pfx), _ptr(sc), _ptr(alpha), _ptr(dalpha), _ptr(m),
                                  _ptr(v), step, lr, beta1, beta2, eps, weight_decay, grad_scale, _stream()),
            "bcq_alpha_adamw")
 
@@ -400,7 +418,7 @@ def alpha_pack(alpha_flat, segments: Segments):
     """bcq_alpha_pack: the trained scales as one compact fp32 tensor (the per-task checkpoint)."""
     torch = _torch()
     out = torch.empty(segments.count, dtype=torch.float32, device=alpha_flat.device)
-    _check(lib().bcq_alpha_pack(segments.count, segments.nseg, _ptr(segments.begin), _ptr(segments.prefix),
+    _check(_fn().pack(segments.count, segments.nseg, _ptr(segments.begin), _ptr(segments.prefix),
                                 _ptr(alpha_flat), _ptr(out), _stream()), "bcq_alpha_pack")
     return out
 
@@ -408,7 +426,7 @@ def alpha_pack(alpha_flat, segments: Segments):
 def alpha_unpack(packed, alpha_flat, segments: Segments):
     """bcq_alpha_unpack: writes a checkpoint's scales back into the flat array."""
     assert packed.numel() == segments.count
-    _check(lib().bcq_alpha_unpack(segments.count, segments.nseg, _ptr(segments.begin), _ptr(segments.prefix),
+    _check(_fn().unpack(segments.count, segments.nseg, _ptr(segments.begin), _ptr(segments.prefix),
                                   _ptr(packed), _ptr(alpha_flat), _stream()), "bcq_alpha_unpack")
 
 

@@ -1,15 +1,17 @@
-"""Builds the CUDA library in-tree: csrc/*.cu -> libbcq_b200.so (sm_100a only)."""
+"""Builds the library in-tree: csrc/*.cu -> libbcq_b200.so (sm_100a only), csrc/binding.c -> _bcq_call.so."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libbcq_b200.so")
+CALL = os.path.join(HERE, "_bcq_call.so")
 OBJ_DIR = os.path.join(HERE, "_build")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -22,14 +24,23 @@ def _sources():
 
 def _deps():
     return _sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + \
-        [os.path.join(os.path.dirname(HERE), "include", "bcq.h")]
+        [os.path.join(CSRC, "binding.c"), os.path.join(os.path.dirname(HERE), "include", "bcq.h")]
 
 
 def is_stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(CALL):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(CALL))
     return any(os.path.getmtime(p) > t for p in _deps())
+
+
+def _build_binding():
+    cmd = [os.environ.get("CC", "gcc"), "-O2", "-fPIC", "-shared", "-I" + sysconfig.get_paths()["include"],
+           os.path.join(CSRC, "binding.c"), "-o", CALL + ".tmp", "-ldl"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError("gcc failed for binding.c:\n" + r.stderr)
+    os.replace(CALL + ".tmp", CALL)
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:
@@ -55,6 +66,7 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
     if r.returncode != 0:
         raise RuntimeError("link failed:\n" + r.stderr)
     os.replace(LIB + ".tmp", LIB)
+    _build_binding()
     return LIB
 
 
