@@ -162,24 +162,14 @@ bcq_status bcq_linear_decode(int d_out, int d_in, int q, int g, int n, const voi
  * Some callers of the decode path cannot hand over scratch memory: code that runs where
  * cudaMalloc is off limits -- inside a region that must not touch the allocator (a latency-critical
  * serving loop, a plugin that is only given its input and output tensors), or a process whose
- * memory was carved up in advance.  For them the partial sums of the split over d_in live in a
- * fixed array inside the library, BCQ_NOALLOC_SCRATCH_BYTES (2 MiB) of device memory that
- * every GPU using the library holds from the moment the library is loaded until the process exits.
- * The call allocates nothing and frees nothing.
+ * memory was carved up in advance.  The call allocates nothing and frees nothing, and calls may
+ * overlap on the GPU.
  *
  *   - Same arguments and results as bcq_linear_decode, minus ws / ws_bytes.
  *   - If bcq_workspace_bytes(BCQ_OP_DECODE, ...) for the shape exceeds
- *     BCQ_NOALLOC_SCRATCH_BYTES the call returns BCQ_ERR_WORKSPACE and launches nothing (on a
+ *     BCQ_NOALLOC_SCRATCH_BYTES (2 MiB) the call returns BCQ_ERR_WORKSPACE and launches nothing (on a
  *     B200 that is roughly n * d_out beyond 128K with a split d_in, e.g. 16 tokens of a
- *     12288-row layer; 8 tokens of it fit).  Such problems need bcq_linear_decode.
- *   - The first call on each device looks up the device address of the array
- *     (cudaGetSymbolAddress) with that device current; make that first call outside any stream
- *     capture.  Later calls on the device only launch kernels.  The address is kept for the
- *     life of the process: after cudaDeviceReset on that device it is stale and the library
- *     must be loaded again.
- *   - All calls on a device share the one array.  It keeps whatever the last call left in it;
- *     every call overwrites the part it reads, so nothing has to be cleared.  Two calls that may
- *     overlap on the GPU (different streams, no dependency) race on it: serialise them. */
+ *     12288-row layer; 8 tokens of it fit).  Such problems need bcq_linear_decode. */
 #define BCQ_NOALLOC_SCRATCH_BYTES (2u << 20)
 bcq_status bcq_linear_decode_noalloc(int d_out, int d_in, int q, int g, int n, const void* X,
                                      size_t ldx, const uint32_t* bits, const float* alpha,
@@ -197,7 +187,7 @@ bcq_status bcq_linear_decode_noalloc(int d_out, int d_in, int q, int g, int n, c
  *   - per (row, group) the eight fp16 levels sum_i +-alpha_i (for q = 4 those with b_4 = +1; the
  *     others are their negatives), 16 bytes, multiplied by a power of two per row that brings
  *     q * max|alpha| of the row to [2^13, 2^14) -- the values bcq_linear_decode forms on the fly;
- *   - per row that power of two, and one arrival counter per tile of 128 rows.
+ *   - per row that power of two.
  * The pack is bcq_decode_pack_bytes() bytes (0 for an unsupported shape; about the size of bits
  * plus alpha), 128-byte aligned, caller-owned.  q > 4 gives BCQ_ERR_UNSUPPORTED: use
  * bcq_linear_decode.  If alpha changes, pack again. */
@@ -206,14 +196,12 @@ bcq_status bcq_decode_pack(int d_out, int d_in, int q, int g, const uint32_t* bi
                            void* pack, size_t pack_bytes, void* stream);
 
 /* Y = X W_hat^T (+ bias) for 1 <= n <= 16 tokens from a pack (Eq. 2; same arithmetic as
- * bcq_linear_decode: fp16 levels, bf16 activations scaled per token by a power of two, fp32
- * accumulation).  One kernel: the 128-row x 128-column pieces of the matrix are dealt evenly to
- * one CTA per SM; where two CTAs share a row tile the partial sums go through `ws`
- * (bcq_workspace_bytes(BCQ_OP_DECODE_PACKED, ...) bytes, may be 0) and are added in a fixed order,
- * so the result is the same in every run.
- * The pack is not const: the call uses its arrival counters and leaves them zero again.  Calls
- * that use the same pack must not overlap on the GPU.  After BCQ_ERR_DEVICE_TIMEOUT (see
- * bcq_device_timeout_flag) write the pack again. */
+ * bcq_linear_decode: fp16 levels, bf16 activations scaled per token and 128 columns by a power of two,
+ * fp32 accumulation).  One kernel; all sums are taken in a fixed order, so the result is the same in
+ * every run.  No scratch is needed (bcq_workspace_bytes(BCQ_OP_DECODE_PACKED, ...) is 0; ws is not used),
+ * the pack is only read, and calls may overlap on the GPU.  (The kernel may read
+ * the pack while the kernel before it in the stream is ending, so a kernel of the caller's own that
+ * writes a pack must not release its programmatic dependents early.) */
 bcq_status bcq_linear_decode_packed(int d_out, int d_in, int q, int g, int n, const void* X, size_t ldx,
                                     void* pack, const float* bias, void* Y, size_t ldy, int y_dtype,
                                     void* ws, size_t ws_bytes, void* stream);

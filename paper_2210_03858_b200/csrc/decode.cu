@@ -1,5 +1,5 @@
-// Decode (1..16 tokens) from a packed copy of the frozen weights: bcq_decode_pack and
-// bcq_linear_decode_packed.
+// Decode (1..16 tokens): from a packed copy of the frozen weights (bcq_decode_pack and
+// bcq_linear_decode_packed), and from the canonical planes and scales (the kernel of bcq_linear_decode).
 //
 // Decode streams every weight once and uses it for at most 16 tokens, so the time is set by the
 // bytes of the pack and by how cheaply a weight gets from its bits into a tensor-core operand
@@ -165,6 +165,80 @@ __global__ void __launch_bounds__(256) pack_codes_kernel(int d_out, int pitch, i
 // the decode kernel
 // ------------------------------------------------------------------------------------------
 
+// Where the sums of a decode kernel go.
+struct DecOut {
+    int d_out, n;
+    const float* bias;
+    void* out;
+    long long ldo;
+    int out_bf16;
+};
+
+// The sums of `ntiles` 16-row tiles from tile0 on: added over the warps of the CTA, in order, and written.
+//   sums [warp][max_tiles][NT][32 lanes]: lane (g, t) has rows g (x, y) and g + 8 (z, w), tokens 2 t, 2 t + 1
+template <int NT>
+__device__ __forceinline__ void add_and_store(const DecOut& o, const float4* sums, int max_tiles, int ntiles, int tile0,
+                                              const float* __restrict__ rinv) {
+    for (int e = threadIdx.x; e < ntiles * NT * 32; e += kDpThreads) {
+        const int ti = e / (NT * 32), ln = e & 31, nt = (e >> 5) % NT;
+        const float4* src = sums + (size_t)(ti * NT + nt) * 32 + ln;
+        float4 s = src[0];
+        for (int w = 1; w < kDpWarps; ++w) {
+            const float4 x = src[(size_t)w * max_tiles * (NT * 32)];
+            s.x += x.x; s.y += x.y; s.z += x.z; s.w += x.w;
+        }
+        const int tok = nt * 8 + 2 * (ln & 3);
+        if (tok >= o.n) continue;
+        const int j0 = (tile0 + ti) * kDpRows + (ln >> 2);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int j = j0 + 8 * h;
+            if (j >= o.d_out) continue;
+            const float scale = rinv != nullptr ? __ldg(rinv + j) : 1.0f, bias = o.bias != nullptr ? __ldg(o.bias + j) : 0.0f;
+            const float v[2] = {(h ? s.z : s.x) * scale + bias, (h ? s.w : s.y) * scale + bias};
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                if (tok + c >= o.n) continue;
+                const long long at = (long long)(tok + c) * o.ldo + j;
+                if (o.out_bf16) reinterpret_cast<__nv_bfloat16*>(o.out)[at] = __float2bfloat16_rn(v[c]);
+                else reinterpret_cast<float*>(o.out)[at] = v[c];
+            }
+        }
+    }
+}
+
+// 32 activations of one token as fp16 times a power of two per (token, 128-k step): the four lanes of a
+// quad hold the step, v[r] the eight elements from k0 + r * stride on.  Returns the inverse scale.
+__device__ __forceinline__ float scale_fragment(uint4 (&v)[4], int k0, int stride, int d_in, bool ragged) {
+    if (ragged) {  // columns past d_in count as zeros
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            uint32_t* w = &v[r].x;
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (k0 + r * stride + e >= d_in) w[e >> 1] &= (e & 1) ? 0x0000FFFFu : 0xFFFF0000u;
+        }
+    }
+    uint32_t mm = 0u;
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+        mm = __vmaxu2(mm, __vmaxu2(__vmaxu2(v[r].x & 0x7FFF7FFFu, v[r].y & 0x7FFF7FFFu),
+                                   __vmaxu2(v[r].z & 0x7FFF7FFFu, v[r].w & 0x7FFF7FFFu)));
+    uint32_t mag = max(mm & 0xFFFFu, mm >> 16);
+    mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, 1));
+    mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, 2));
+    const int sh = shift_for(exponent_of_bits(mag << 16), 14);
+    const float sc = pow2f(sh);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        uint32_t* w = &v[r].x;
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            w[e] = pack_half2(__uint_as_float(w[e] << 16) * sc, __uint_as_float(w[e] & 0xFFFF0000u) * sc);
+    }
+    return pow2f(-sh);
+}
+
 struct DecPackedParams {
     int d_out, d_in, g, G, n;
     int steps;
@@ -176,10 +250,7 @@ struct DecPackedParams {
     const uint8_t* codes;
     const uint8_t* tables;
     const float* rinv;
-    const float* bias;
-    void* out;
-    long long ldo;
-    int out_bf16;
+    DecOut o;
 };
 
 // D += A B, 16 x 8 x 16, fp16 operands.
@@ -304,40 +375,12 @@ decode_packed_kernel(const DecPackedParams p) {
                 const int tok = nt * 8 + gr;
                 const int kb = st * kDpStepK + tq * 8;
                 const __nv_bfloat16* src = p.X + (long long)tok * p.ldx + kb;
-                uint32_t mm = 0u;
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
-                    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                    if (tok < p.n && kb + r * 32 < p.d_in) v = __ldg(reinterpret_cast<const uint4*>(src + r * 32));
-                    xb[nt][r] = v;
+                    xb[nt][r] = make_uint4(0u, 0u, 0u, 0u);
+                    if (tok < p.n && kb + r * 32 < p.d_in) xb[nt][r] = __ldg(reinterpret_cast<const uint4*>(src + r * 32));
                 }
-                if (st * kDpStepK + kDpStepK > p.d_in) {  // columns past d_in count as zeros
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        uint32_t* w = &xb[nt][r].x;
-#pragma unroll
-                        for (int e = 0; e < 8; ++e)
-                            if (kb + r * 32 + e >= p.d_in) w[e >> 1] &= (e & 1) ? 0x0000FFFFu : 0xFFFF0000u;
-                    }
-                }
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const uint4 v = xb[nt][r];
-                    mm = __vmaxu2(mm, __vmaxu2(__vmaxu2(v.x & 0x7FFF7FFFu, v.y & 0x7FFF7FFFu),
-                                               __vmaxu2(v.z & 0x7FFF7FFFu, v.w & 0x7FFF7FFFu)));
-                }
-                uint32_t mag = max(mm & 0xFFFFu, mm >> 16);
-                mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, 1));
-                mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, 2));
-                const int sh = shift_for(exponent_of_bits(mag << 16), 14);
-                const float sc = pow2f(sh), inv = pow2f(-sh);
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    uint32_t* w = &xb[nt][r].x;
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        w[e] = pack_half2(__uint_as_float(w[e] << 16) * sc, __uint_as_float(w[e] & 0xFFFF0000u) * sc);
-                }
+                const float inv = scale_fragment(xb[nt], kb, 32, p.d_in, st * kDpStepK + kDpStepK > p.d_in);
                 f0[nt] = __shfl_sync(0xffffffffu, inv, 8 * tq);
                 f1[nt] = __shfl_sync(0xffffffffu, inv, 8 * tq + 4);
             }
@@ -389,34 +432,257 @@ decode_packed_kernel(const DecPackedParams p) {
             }
         }
 
-        // ---- the tiles' sums: over the warps, in order
         __syncthreads();
-        for (int e = threadIdx.x; e < round_n * NT * 32; e += kDpThreads) {
-            const int ti = e / (NT * 32), ln = e & 31, nt = (e >> 5) % NT;
-            const float4* src = sums + (size_t)(ti * NT + nt) * 32 + ln;
-            float4 s = src[0];
-            for (int w = 1; w < kDpWarps; ++w) {
-                const float4 x = src[(size_t)w * p.round * (NT * 32)];
-                s.x += x.x; s.y += x.y; s.z += x.z; s.w += x.w;
+        add_and_store<NT>(p.o, sums, p.round, round_n, tile0 + first, p.rinv);
+        if (first + p.round < ntiles) __syncthreads();  // the slots are written again
+    }
+}
+
+// ------------------------------------------------------------------------------------------
+// decode from the canonical planes (bcq_linear_decode: the scales may change between calls, any q <= 8)
+// ------------------------------------------------------------------------------------------
+//
+// The same kernel with another way from memory to a fragment.  Lane (g, t) takes the plane words of rows g
+// and g + 8 that hold the k 32 t .. + 31 of the step, and the scales of their group.  q <= 4: the level
+// table of a (row, group) is built in registers and the selector nibbles of four weights are gathered
+// from the plane bits with shifts and masks (2.75 instructions per weight where the pack needs 1.6); q > 4:
+// fp32 sums of +-alpha_i.  Levels carry a power of two per (row, step) that brings the largest sum of
+// |alpha_i| to [2^13, 2^14), taken out of the sums again in fp32.
+// This replaced a tcgen05 kernel with a split over K and a second kernel that added the parts.
+
+struct DecPlanesParams {
+    int d_out, d_in, q, g, G, n;
+    int steps, pitch;
+    int per, rem, round;     // see DecPackedParams
+    uint32_t g_magic;
+    const __nv_bfloat16* X;
+    long long ldx;
+    const uint32_t* bits;
+    const float* alpha;
+    DecOut o;
+};
+
+// Planes and scales of one (16-row tile, step) as one lane needs them: rows g and g + 8.
+template <int NQ>
+struct PlaneWords {
+    uint32_t wa[NQ], wb[NQ];
+    float aa[NQ], ab[NQ];
+};
+
+// Pairs of one row's 32 weights for the MMA (r, h): weights 16 h + r and + 4, + 8 and + 12.  NQ = 3: levels of
+// three planes; 4: table for b_4 = +1, mirrored and negated where b_4 = -1; 8: fp32 sums.
+template <int NQ>
+struct RowExpand {
+    Lut t;
+    uint32_t x[NQ == 8 ? 8 : 4];  // plane words (NQ = 4: mirrored; x[3] bit set where b_4 = -1)
+    float a[NQ == 8 ? 8 : 1];
+
+    __device__ __forceinline__ void begin(const uint32_t (&w)[NQ], const float (&al)[NQ], float scale) {
+        if constexpr (NQ == 8) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) { x[i] = ~w[i]; a[i] = al[i] * scale; }
+        } else if constexpr (NQ == 4) {
+            t = build_lut(al[0] * scale, al[1] * scale, al[2] * scale, al[3] * scale);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) x[i] = ~(w[i] ^ w[3]);
+            x[3] = ~w[3];
+        } else {
+            t = build_lut(al[0] * scale, al[1] * scale, al[2] * scale, 0.0f);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) x[i] = w[i];
+        }
+    }
+    // selector word of residue r: nibble m = level index of weight 4 m + r
+    __device__ __forceinline__ uint32_t select(int r) const {
+        constexpr uint32_t M = 0x11111111u;
+        const uint32_t b = r >= 1 ? x[1] >> (r >= 1 ? r - 1 : 0) : x[1] << 1;
+        const uint32_t c = r >= 2 ? x[2] >> (r >= 2 ? r - 2 : 0) : x[2] << (r >= 2 ? 0 : 2 - r);
+        return ((x[0] >> r) & M) | (b & (M << 1)) | (c & (M << 2));
+    }
+    __device__ __forceinline__ void pairs(uint32_t S, int r, int h, uint32_t& lo, uint32_t& hi) const {
+        if constexpr (NQ == 8) {
+            float v[4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                v[m] = 0.0f;
+#pragma unroll
+                for (int i = 0; i < 8; ++i)  // planes past q have zero scales
+                    v[m] += __uint_as_float(__float_as_uint(a[i]) ^ ((x[i] << (31 - (16 * h + r + 4 * m))) & 0x80000000u));
             }
-            const int tok = nt * 8 + 2 * (ln & 3);
-            if (tok >= p.n) continue;
-            const int j0 = (tile0 + first + ti) * kDpRows + (ln >> 2);
+            lo = pack_half2(v[0], v[1]);
+            hi = pack_half2(v[2], v[3]);
+        } else {
+            const uint32_t sel = h ? (S >> 16) : S;
+            uint32_t hb = prmt(t.th0, t.th1, sel);
+            const uint32_t lb = prmt(t.tl0, t.tl1, sel);
+            if (NQ == 4) {
+                // bytes of the flag word = 0xFF where the weight's b_4 is -1 (weights m = 0..3 sit 4 bits apart)
+                const int p0 = 16 * h + r;
+                const uint32_t s02 = (p0 <= 7) ? (x[3] << (p0 <= 7 ? 7 - p0 : 0)) : (x[3] >> (p0 > 7 ? p0 - 7 : 0));
+                const uint32_t s13 = (p0 <= 3) ? (x[3] << (p0 <= 3 ? 3 - p0 : 0)) : (x[3] >> (p0 > 3 ? p0 - 3 : 0));
+                hb ^= prmt(s02, s13, 0xD9C8u) & 0x80808080u;
+            }
+            lo = prmt(lb, hb, 0x5140u);
+            hi = prmt(lb, hb, 0x7362u);
+        }
+    }
+};
+
+template <int NQ, int NT>
+__global__ void __launch_bounds__(kDpThreads, 1)
+decode_planes_kernel(const DecPlanesParams p) {
+    extern __shared__ float4 sums[];  // [warp][tile][NT][32 lanes]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int gr = lane >> 2, tq = lane & 3;
+    const int tile0 = (int)blockIdx.x * p.per + min((int)blockIdx.x, p.rem);
+    const int ntiles = p.per + ((int)blockIdx.x < p.rem ? 1 : 0);
+    float4* mine = sums + (size_t)warp * p.round * (NT * 32) + lane;
+    const size_t plane_bits = (size_t)p.d_out * p.pitch, plane_alpha = (size_t)p.d_out * p.G;
+
+    pdl_trigger();
+    pdl_wait();  // the scales may come from the kernel before this one
+    for (int first = 0; first < ntiles; first += p.round) {
+        const int round_n = min(p.round, ntiles - first);
+        const int all = round_n * p.steps;
+        const int u0 = all * warp / kDpWarps, u1 = all * (warp + 1) / kDpWarps;
+        const int st0 = u0 / round_n, i0 = u0 - st0 * round_n;
+
+        int l_st = st0, l_i = i0, l_c = 0, l_left = u1 - u0;
+        auto group_of = [&](int st) {  // group of this lane's 32 weights
+            const int k = st * kDpStepK + 32 * tq;
+            return min(p.g_magic != 0u ? (int)__umulhi((uint32_t)k, p.g_magic) : k / p.g, p.G - 1);
+        };
+        l_c = group_of(l_st);
+        auto load = [&](PlaneWords<NQ>& u) {
+            if (l_left == 0) return;
+            --l_left;
+            const int ja = (tile0 + first + l_i) * kDpRows + gr, jb = ja + 8;
+            const uint32_t* pb = p.bits + (size_t)ja * p.pitch + l_st * 4 + tq;
+            const float* pa = p.alpha + (size_t)ja * p.G + l_c;
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int j = j0 + 8 * h;
-                if (j >= p.d_out) continue;
-                const float rinv = __ldg(p.rinv + j), bias = p.bias != nullptr ? __ldg(p.bias + j) : 0.0f;
-                const float v[2] = {(h ? s.z : s.x) * rinv + bias, (h ? s.w : s.y) * rinv + bias};
+            for (int i = 0; i < NQ; ++i) {
+                const bool va = i < p.q && ja < p.d_out, vb = i < p.q && jb < p.d_out;
+                u.wa[i] = va ? __ldg(pb + i * plane_bits) : 0u;
+                u.wb[i] = vb ? __ldg(pb + i * plane_bits + 8 * (size_t)p.pitch) : 0u;
+                u.aa[i] = va ? __ldg(pa + i * plane_alpha) : 0.0f;
+                u.ab[i] = vb ? __ldg(pa + i * plane_alpha + 8 * (size_t)p.G) : 0.0f;
+            }
+            if (++l_i == round_n) {
+                l_i = 0;
+                l_c = group_of(++l_st);
+            }
+        };
+        PlaneWords<NQ> ua, ub;
+        load(ua);
+        if (NQ < 8) load(ub);
+        for (int i = 0; i < round_n * NT; ++i) mine[i * 32] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (first == 0) {
+            for (int s = st0 + 1; s * round_n < u1; ++s) {
+                const int k = s * kDpStepK + (lane & 1) * 64;
+                if ((lane >> 1) < p.n && k < p.d_in)
+                    asm volatile("prefetch.global.L1 [%0];" ::"l"(p.X + (long long)(lane >> 1) * p.ldx + k));
+            }
+        }
+
+        // a step's activations: lane (g, t) holds token g of each tile of eight, k 32 t .. + 31, paired as the
+        // expansion pairs the weights: xb[nt][r][h] = (16 h + r, + 4), (+ 8, + 12)
+        uint2 xb[NT][4][2];
+        float f0[NT], f1[NT];
+        auto load_x = [&](int st) {
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    if (tok + c >= p.n) continue;
-                    const long long o = (long long)(tok + c) * p.ldo + j;
-                    if (p.out_bf16) reinterpret_cast<__nv_bfloat16*>(p.out)[o] = __float2bfloat16_rn(v[c]);
-                    else reinterpret_cast<float*>(p.out)[o] = v[c];
+            for (int nt = 0; nt < NT; ++nt) {
+                const int tok = nt * 8 + gr;
+                const int kb = st * kDpStepK + tq * 32;
+                const __nv_bfloat16* src = p.X + (long long)tok * p.ldx + kb;
+                uint4 v[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    v[r] = make_uint4(0u, 0u, 0u, 0u);
+                    if (tok < p.n && kb + r * 8 < p.d_in) v[r] = __ldg(reinterpret_cast<const uint4*>(src + r * 8));
+                }
+                const float inv = scale_fragment(v, kb, 8, p.d_in, st * kDpStepK + kDpStepK > p.d_in);
+                const uint32_t P[16] = {v[0].x, v[0].y, v[0].z, v[0].w, v[1].x, v[1].y, v[1].z, v[1].w,
+                                        v[2].x, v[2].y, v[2].z, v[2].w, v[3].x, v[3].y, v[3].z, v[3].w};
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int e = 8 * h + (r >> 1);
+                        const uint32_t sel = (r & 1) ? 0x7632u : 0x5410u;
+                        xb[nt][r][h] = make_uint2(prmt(P[e], P[e + 2], sel), prmt(P[e + 4], P[e + 6], sel));
+                    }
+                f0[nt] = __shfl_sync(0xffffffffu, inv, 8 * tq);
+                f1[nt] = __shfl_sync(0xffffffffu, inv, 8 * tq + 4);
+            }
+        };
+
+        int u_st = st0, u_i = i0;
+        bool fresh = true;
+        auto row_shift = [&](const float (&a)[NQ]) {
+            float s = 0.0f;
+#pragma unroll
+            for (int i = 0; i < NQ; ++i) s += fabsf(a[i]);
+            uint32_t m = __float_as_uint(s);
+            m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+            m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
+            return shift_for(exponent_of_bits(m), 13);
+        };
+        auto unit = [&](const PlaneWords<NQ>& u) {
+            if (fresh) load_x(u_st);
+            const int sa = row_shift(u.aa), sb = row_shift(u.ab);
+            RowExpand<NQ> ea, eb;
+            ea.begin(u.wa, u.aa, pow2f(sa));
+            eb.begin(u.wb, u.ab, pow2f(sb));
+            float d[NT][4];
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) d[nt][0] = d[nt][1] = d[nt][2] = d[nt][3] = 0.f;
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                uint32_t Sa = 0u, Sb = 0u;
+                if (NQ < 8) { Sa = ea.select(r); Sb = eb.select(r); }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    uint32_t a0, a1, a2, a3;
+                    ea.pairs(Sa, r, h, a0, a2);
+                    eb.pairs(Sb, r, h, a1, a3);
+#pragma unroll
+                    for (int nt = 0; nt < NT; ++nt) mma_f16(d[nt], a0, a1, a2, a3, xb[nt][r][h].x, xb[nt][r][h].y);
+                }
+            }
+            const float ia = pow2f(-sa), ib = pow2f(-sb);
+            float4* slot = mine + u_i * (NT * 32);
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
+                float4 s = slot[nt * 32];
+                s.x = fmaf(f0[nt] * ia, d[nt][0], s.x);
+                s.y = fmaf(f1[nt] * ia, d[nt][1], s.y);
+                s.z = fmaf(f0[nt] * ib, d[nt][2], s.z);
+                s.w = fmaf(f1[nt] * ib, d[nt][3], s.w);
+                slot[nt * 32] = s;
+            }
+            fresh = (++u_i == round_n);
+            if (fresh) { u_i = 0; ++u_st; }
+        };
+        if (NQ == 8) {
+            // one unit's registers are all there is room for
+#pragma unroll 1
+            for (int u = u0; u < u1; ++u) {
+                unit(ua);
+                load(ua);
+            }
+        } else {
+#pragma unroll 1
+            for (int u = u0; u < u1; u += 2) {
+                unit(ua);
+                load(ua);
+                if (u + 1 < u1) {
+                    unit(ub);
+                    load(ub);
                 }
             }
         }
+        __syncthreads();
+        add_and_store<NT>(p.o, sums, p.round, round_n, tile0 + first, nullptr);
         if (first + p.round < ntiles) __syncthreads();  // the slots are written again
     }
 }
@@ -425,14 +691,25 @@ decode_packed_kernel(const DecPackedParams p) {
 // host side
 // ------------------------------------------------------------------------------------------
 
+// ceil(2^32 / g): k / g = hi32(k magic) while k g < 2^32, since k magic - k 2^32 / g < k; else 0
+uint32_t group_magic(int d_in, int g) {
+    return (long long)d_in * g < (1ll << 32) && g > 1 ? (uint32_t)(((1ull << 32) + g - 1) / g) : 0u;
+}
+
+// Row tiles dealt to one CTA per SM; bytes of the warps' sums (at most 192 KiB).
+template <int NT, typename Params>
+size_t deal_tiles(Params& p, int tiles, int* ctas) {
+    *ctas = std::min(tiles, sm_count());
+    p.per = tiles / *ctas;
+    p.rem = tiles % *ctas;
+    p.round = std::min(p.per + (p.rem > 0 ? 1 : 0), kDpMaxRound / NT);
+    return (size_t)kDpWarps * p.round * NT * 512;
+}
+
 template <int Q, int NT, int PARTS>
 bcq_status launch_decode_packed(DecPackedParams p, int tiles, cudaStream_t s) {
-    const int ctas = std::min(tiles, sm_count());
-    p.per = tiles / ctas;
-    p.rem = tiles % ctas;
-    const int most = p.per + (p.rem > 0 ? 1 : 0);
-    p.round = std::min(most, kDpMaxRound / NT);
-    const size_t smem = (size_t)kDpWarps * p.round * NT * 512;  // at most 192 KiB
+    int ctas;
+    const size_t smem = deal_tiles<NT>(p, tiles, &ctas);
     auto kern = decode_packed_kernel<Q, NT, PARTS>;
     const bcq_status st = ensure_dynamic_smem(kern, smem);
     if (st != BCQ_OK) return st;
@@ -452,6 +729,22 @@ bcq_status launch_decode_tokens(const DecPackedParams& p, const PackLayout& L, c
     return p.n <= 8 ? launch_decode_parts<Q, 1>(p, L, s) : launch_decode_parts<Q, 2>(p, L, s);
 }
 
+template <int NQ, int NT>
+bcq_status launch_decode_planes(DecPlanesParams p, cudaStream_t s) {
+    int ctas;
+    const size_t smem = deal_tiles<NT>(p, ceil_div(p.d_out, kDpRows), &ctas);
+    auto kern = decode_planes_kernel<NQ, NT>;
+    const bcq_status st = ensure_dynamic_smem(kern, smem);
+    if (st != BCQ_OK) return st;
+    BCQ_CUDA_TRY(launch_pdl(kern, dim3((unsigned)ctas), kDpThreads, smem, s, 1, p));
+    return BCQ_OK;
+}
+
+template <int NQ>
+bcq_status launch_decode_planes_tokens(const DecPlanesParams& p, cudaStream_t s) {
+    return p.n <= 8 ? launch_decode_planes<NQ, 1>(p, s) : launch_decode_planes<NQ, 2>(p, s);
+}
+
 bcq_status check_pack_shape(int d_out, int d_in, int q, int g) {
     bcq_status st = check_shape(d_out, d_in, q, g);
     if (st != BCQ_OK) return st;
@@ -468,6 +761,20 @@ void launch_pack_codes(int d_out, int pitch, const PackLayout& L, const uint32_t
 }  // namespace
 
 namespace bcq {
+bcq_status run_decode_planes(int d_out, int d_in, int q, int g, int n, const void* X, size_t ldx, const uint32_t* bits,
+                             const float* alpha, const float* bias, void* Y, size_t ldy, int y_dtype, cudaStream_t s) {
+    DecPlanesParams p = {};
+    p.d_out = d_out; p.d_in = d_in; p.q = q; p.g = g; p.G = (int)bcq_num_groups(d_in, g); p.n = n;
+    p.steps = ceil_div(d_in, kDpStepK); p.pitch = (int)bcq_pitch_words(d_in);
+    p.g_magic = group_magic(d_in, g);
+    p.X = reinterpret_cast<const __nv_bfloat16*>(X); p.ldx = (long long)ldx;
+    p.bits = bits; p.alpha = alpha;
+    p.o = {d_out, n, bias, Y, (long long)ldy, y_dtype == BCQ_BF16};
+    if (q <= 3) return launch_decode_planes_tokens<3>(p, s);
+    if (q == 4) return launch_decode_planes_tokens<4>(p, s);
+    return launch_decode_planes_tokens<8>(p, s);
+}
+
 size_t decode_packed_workspace_bytes(int, int, int, int, int) { return 0; }
 }  // namespace bcq
 
@@ -527,12 +834,11 @@ extern "C" bcq_status bcq_linear_decode_packed(int d_out, int d_in, int q, int g
     DecPackedParams p = {};
     p.d_out = d_out; p.d_in = d_in; p.g = g; p.G = L.G; p.n = n;
     p.steps = L.steps;
-    // k g_magic - k 2^32 / g < k < 2^32 / g while k g < 2^32
-    p.g_magic = (long long)d_in * g < (1ll << 32) && g > 1 ? (uint32_t)(((1ull << 32) + g - 1) / g) : 0u;
+    p.g_magic = group_magic(d_in, g);
     p.X = reinterpret_cast<const __nv_bfloat16*>(X); p.ldx = (long long)ldx;
     p.codes = pk + L.off_codes; p.tables = pk + L.off_tables;
     p.rinv = reinterpret_cast<const float*>(pk);
-    p.bias = bias; p.out = Y; p.ldo = (long long)ldy; p.out_bf16 = (y_dtype == BCQ_BF16);
+    p.o = {d_out, n, bias, Y, (long long)ldy, y_dtype == BCQ_BF16};
     cudaStream_t s = (cudaStream_t)stream;
     switch (q) {
         case 1: return launch_decode_tokens<1>(p, L, s);

@@ -1,7 +1,7 @@
-// Forward (Eq. 2), input gradient (Eq. 3) and decode kernels of the BCQ linear layer.
+// Forward (Eq. 2) and input gradient (Eq. 3) kernels of the BCQ linear layer.
 //
-//   forward / decode   D[j, t] = sum_k  W_hat[j, k] * X[t, k]
-//   dX                 D[k, t] = sum_j  W_hat[j, k] * dY[t, j]
+//   forward   D[j, t] = sum_k  W_hat[j, k] * X[t, k]
+//   dX        D[k, t] = sum_j  W_hat[j, k] * dY[t, j]
 //
 // W_hat = sum_i alpha_i b_i (Eq. 1) never exists in global memory: worker warps rebuild it tile by
 // tile from the packed planes, straight into the 128-byte-swizzled shared-memory operand layout of
@@ -12,23 +12,18 @@
 // Number format.  A scaled weight rounded to bf16 (8 significant bits) alone already costs about
 // 1.7e-3 relative error on the outputs, so both operands are fp16 (11 bits):
 //   * the scaled weight takes one of 2^q values per (row, group).  For q <= 4 the workers build
-//     a byte-wise lookup table of the fp16 levels in four registers and index it with PRMT: the
-//     selector nibbles are the plane bits of four weights, gathered with shifts and masks.  For
-//     q = 4 the table holds the eight levels with b_4 = +1; b_4 = -1 mirrors the index and flips
-//     the sign.  q > 4 falls back to fp32 sums of +-alpha_i.
+//     a byte-wise lookup table of the fp16 levels in four registers and index it with PRMT; the
+//     selector nibbles are stored instead of the planes (lut.cuh).  For q = 4 the table holds the
+//     eight levels with b_4 = +1; b_4 = -1 mirrors the index and flips the sign.  q > 4 falls back
+//     to fp32 sums of +-alpha_i.
 //   * activations are bf16 at the interface.  A short pre-pass writes them to the workspace as
 //     fp16, each token row multiplied by a power of two that brings its largest magnitude to
 //     2^14..2^15 (exact; undone in the epilogue), so neither large activations nor small
 //     gradients leave the fp16 range.  The same pre-pass finds max|alpha|, from which a power of
-//     two for the weights is derived.  Decode (<= 16 tokens) has no pre-pass: every CTA converts
-//     the X slice it needs itself and scales per (token, K-slice) and per weight row.
-//   * one PRMT pair emits the weights of a byte of a plane word in the order 0,4,1,5,2,6,3,7.
-//     For the forward and dX the pre-pass, which regroups the plane words anyway, stores the bits
-//     of every byte as 0,2,4,6,1,3,5,7, so that the expanded tile is in natural k order.  Decode
-//     has no pre-pass: there the tile keeps the PRMT order and the workers write the activations
-//     in the same order.
+//     two for the weights is derived.
+//   * q > 4: the sums come out in the order 0,4,1,5,2,6,3,7 of a byte of a plane word, so the pre-pass,
+//     which regroups the plane words anyway, stores the bits of every byte as 0,2,4,6,1,3,5,7.
 #include <algorithm>
-#include <mutex>
 
 #include "gemm_common.cuh"
 #include "lut.cuh"
@@ -41,94 +36,9 @@ __device__ int g_timeout_flag = 0;
 
 enum { MODE_FWD = 0, MODE_BWDX = 1 };
 enum { QM_LUT3 = 0, QM_LUT4 = 1, QM_GENERIC = 2 };
-constexpr int kPrefetch = 3;  // stages between the global loads of a task and its use
 
-// 16 weights of one row (bits 0..15 of the plane words w0..w3) through the lookup table, stored
-// as two 16-byte chunks (slots chunk0, chunk0 + 1) of the 128-byte line at `line` (swizzle key
-// lx).  Chunk u holds weights 8u..8u+7 in the order 0,4,1,5,2,6,3,7.
-template <bool Q4>
-__device__ __forceinline__ void expand16_lut(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3,
-                                             const Lut& t, uint32_t line, uint32_t lx, uint32_t chunk0) {
-    uint32_t x0 = w0, x1 = w1, x2 = w2, nf = 0u;
-    if (Q4) {
-        // b_4 = -1 (bit clear): value = -level[~index]
-        nf = ~w3;
-        x0 = ~(w0 ^ w3);
-        x1 = ~(w1 ^ w3);
-        x2 = ~(w2 ^ w3);
-    }
-    constexpr uint32_t M = 0x11111111u;
-    uint32_t R[4][2];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        // nibble n of S = 3-bit level index of weight 4n + r
-        const uint32_t a = x0 >> r;
-        const uint32_t b = (r >= 1) ? (x1 >> (r >= 1 ? r - 1 : 0)) : (x1 << 1);
-        const uint32_t c = (r >= 2) ? (x2 >> (r >= 2 ? r - 2 : 0)) : (x2 << (r >= 2 ? 0 : 2 - r));
-        const uint32_t S = (a & M) | (b & (M << 1)) | (c & (M << 2));  // PRMT reads the low 16 bits
-        uint32_t hb = prmt(t.th0, t.th1, S);
-        const uint32_t lb = prmt(t.tl0, t.tl1, S);
-        if (Q4) {
-            // bytes of `flip` = 0xFF where the weight's b_4 is -1: bring the four bits (weights r,
-            // r+4, r+8, r+12) to byte MSBs, two per copy, and replicate them with PRMT
-            const uint32_t s02 = nf << (7 - r);
-            const uint32_t s13 = nf << (3 - r);
-            const uint32_t flip = prmt(s02, s13, 0xD9C8u);
-            hb ^= flip & 0x80808080u;
-        }
-        R[r][0] = prmt(lb, hb, 0x5140u);  // weights r, r + 4
-        R[r][1] = prmt(lb, hb, 0x7362u);  // weights r + 8, r + 12
-    }
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-        ptx::st_shared_v4(line + (((chunk0 + u) ^ lx) << 4), R[0][u], R[1][u], R[2][u], R[3][u]);
-}
-
-// 32 weights (whole plane words): the selector word S of residue r serves both halves, low 16 bits
-// for weights 0..15 and high 16 bits for weights 16..31.  Four chunks, slots chunk0..chunk0+3.
-template <bool Q4>
-__device__ __forceinline__ void expand32_lut(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3,
-                                             const Lut& t, uint32_t line, uint32_t lx, uint32_t chunk0) {
-    uint32_t x0 = w0, x1 = w1, x2 = w2, nf = 0u;
-    if (Q4) {
-        nf = ~w3;
-        x0 = ~(w0 ^ w3);
-        x1 = ~(w1 ^ w3);
-        x2 = ~(w2 ^ w3);
-    }
-    constexpr uint32_t M = 0x11111111u;
-    uint32_t R[4][2][2];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const uint32_t a = x0 >> r;
-        const uint32_t b = (r >= 1) ? (x1 >> (r >= 1 ? r - 1 : 0)) : (x1 << 1);
-        const uint32_t c = (r >= 2) ? (x2 >> (r >= 2 ? r - 2 : 0)) : (x2 << (r >= 2 ? 0 : 2 - r));
-        const uint32_t S = (a & M) | (b & (M << 1)) | (c & (M << 2));
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint32_t sel = h ? (S >> 16) : S;  // weights 16h + 4m + r, m = 0..3
-            uint32_t hb = prmt(t.th0, t.th1, sel);
-            const uint32_t lb = prmt(t.tl0, t.tl1, sel);
-            if (Q4) {
-                const int p0 = 16 * h + r;  // bit of weight m = 0; m = 2 is 8 bits up, m = 1, 3 are 4 bits up
-                const uint32_t s02 = (p0 <= 7) ? (nf << (p0 <= 7 ? 7 - p0 : 0)) : (nf >> (p0 > 7 ? p0 - 7 : 0));
-                const uint32_t s13 = (p0 <= 3) ? (nf << (p0 <= 3 ? 3 - p0 : 0)) : (nf >> (p0 > 3 ? p0 - 3 : 0));
-                const uint32_t flip = prmt(s02, s13, 0xD9C8u);
-                hb ^= flip & 0x80808080u;
-            }
-            R[r][h][0] = prmt(lb, hb, 0x5140u);
-            R[r][h][1] = prmt(lb, hb, 0x7362u);
-        }
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int u = 0; u < 2; ++u)
-            ptx::st_shared_v4(line + (((chunk0 + 2 * h + u) ^ lx) << 4), R[0][h][u], R[1][h][u], R[2][h][u],
-                              R[3][h][u]);
-}
-
-// Same result through fp32 sums, any q <= 8.  w[i] = plane words (bits 0..15 used), a[i] = scales.
+// 16 weights of one row (bits 0..15 of the plane words w) as fp32 sums of +-alpha_i, any q <= 8, stored as two
+// 16-byte chunks (slots chunk0, chunk0 + 1) of the 128-byte line at `line` (swizzle key lx).  w[i] = plane words (bits 0..15 used), a[i] = scales.
 __device__ __forceinline__ void expand16_sum(const uint32_t (&w)[BCQ_MAX_Q], const float (&a)[BCQ_MAX_Q],
                                              int q, uint32_t line, uint32_t lx, uint32_t chunk0) {
     float v[16];
@@ -161,83 +71,6 @@ template <int QM>
 struct CodeWords {
     static constexpr int value = (QM == QM_LUT4) ? 4 : 3;
 };
-
-// The scales of one (row, group), already multiplied by the weight scale; loaded ahead of use.
-template <int QM>
-struct AlphaSet {
-    float a[NumWords<QM>::value];
-    int key;  // row * G + group, or -1 for a row outside the matrix (expands to zeros)
-};
-
-template <int QM>
-__device__ __forceinline__ void load_alpha(AlphaSet<QM>& s, const float* __restrict__ alpha,
-                                           long long plane_alpha, int G, int q, int j, int c, bool valid,
-                                           float wscale) {
-    s.key = valid ? j * G + c : -1;
-#pragma unroll
-    for (int i = 0; i < NumWords<QM>::value; ++i)
-        s.a[i] = (i < q && valid) ? __ldg(alpha + i * plane_alpha + (long long)j * G + c) * wscale : 0.0f;
-}
-
-// Expands the 16 weights that start at bit `bit_shift` (0 or 16) of the plane words in shared
-// memory at bits_addr + i * plane_stride.
-template <int QM>
-__device__ __forceinline__ void expand_task(const AlphaSet<QM>& as, uint32_t bits_addr, uint32_t plane_stride,
-                                            uint32_t bit_shift, Lut& lut, int& lut_key, int q, uint32_t line,
-                                            uint32_t lx, uint32_t chunk0) {
-    uint32_t w[NumWords<QM>::value];
-#pragma unroll
-    for (int i = 0; i < NumWords<QM>::value; ++i)
-        w[i] = (i < q) ? (ptx::ld_shared_u32(bits_addr + i * plane_stride) >> bit_shift) : 0u;
-    if (QM == QM_GENERIC) {
-        uint32_t w8[BCQ_MAX_Q];
-        float a8[BCQ_MAX_Q];
-#pragma unroll
-        for (int i = 0; i < BCQ_MAX_Q; ++i) {
-            w8[i] = w[i % NumWords<QM>::value];
-            a8[i] = as.a[i % NumWords<QM>::value];
-        }
-        expand16_sum(w8, a8, q, line, lx, chunk0);
-    } else {
-        if (as.key != lut_key) {
-            lut = (QM == QM_LUT4) ? build_lut(as.a[0], as.a[1], as.a[2], as.a[3])
-                                  : build_lut(as.a[0], as.a[1], as.a[2], 0.0f);
-            lut_key = as.key;
-        }
-        expand16_lut<QM == QM_LUT4>(w[0], w[1], w[2], w[3], lut, line, lx, chunk0);
-    }
-}
-
-// 32 weights (one whole plane word per plane): two 16-weight halves from one set of loads.
-template <int QM>
-__device__ __forceinline__ void expand_task32(const AlphaSet<QM>& as, uint32_t bits_addr, uint32_t plane_stride,
-                                              Lut& lut, int& lut_key, int q, uint32_t line, uint32_t lx,
-                                              uint32_t chunk0) {
-    uint32_t w[NumWords<QM>::value];
-#pragma unroll
-    for (int i = 0; i < NumWords<QM>::value; ++i)
-        w[i] = (i < q) ? ptx::ld_shared_u32(bits_addr + i * plane_stride) : 0u;
-    if (QM == QM_GENERIC) {
-        uint32_t w8[BCQ_MAX_Q];
-        float a8[BCQ_MAX_Q];
-#pragma unroll
-        for (int i = 0; i < BCQ_MAX_Q; ++i) {
-            w8[i] = w[i % NumWords<QM>::value];
-            a8[i] = as.a[i % NumWords<QM>::value];
-        }
-        expand16_sum(w8, a8, q, line, lx, chunk0);
-#pragma unroll
-        for (int i = 0; i < BCQ_MAX_Q; ++i) w8[i] >>= 16;
-        expand16_sum(w8, a8, q, line, lx, chunk0 + 2);
-    } else {
-        if (as.key != lut_key) {
-            lut = (QM == QM_LUT4) ? build_lut(as.a[0], as.a[1], as.a[2], as.a[3])
-                                  : build_lut(as.a[0], as.a[1], as.a[2], 0.0f);
-            lut_key = as.key;
-        }
-        expand32_lut<QM == QM_LUT4>(w[0], w[1], w[2], w[3], lut, line, lx, chunk0);
-    }
-}
 
 // ------------------------------------------------------------------------------------------
 // pre-pass: activations -> fp16 with a per-token power-of-two scale; max |alpha|
@@ -577,20 +410,6 @@ struct ExpandParams {
     int helpers;                 // the worker warps share the epilogue of a CTA's last tile (see run_expand)
     float* partial;              // [pair][rank][TN columns][128 rows]
     uint32_t* counters;          // [shared tile][rank][quarter][box class]
-};
-
-// One pipeline stage in shared memory: | A tile 16 KiB | B tile TN x 128 B | plane words |.
-// The plane words arrive by TMA as [plane][row][4 words]: 128 weights of `rows` rows, where rows
-// = 128 weight rows for the forward and decode (the stage uses 64 of the 128 weights) and the 64
-// rows j of the K block for dX (the four words are the tile's 128 k).
-template <int MODE, int TN, int QM>
-struct StageLayout {
-    static constexpr int kBitRows = (MODE == MODE_BWDX) ? 64 : 128;
-    static constexpr uint32_t kBBytes = TN * kBlockK * 2;
-    static constexpr uint32_t kBitsOff = kABytes + kBBytes;
-    static constexpr uint32_t kPlaneBytes = kBitRows * 16;
-    static constexpr uint32_t kBitsBytes = NumWords<QM>::value * kPlaneBytes;
-    static constexpr uint32_t kStageBytes = kBitsOff + kBitsBytes;
 };
 
 // Prefill kernel.  Persistent: every pair of CTAs walks over output tiles of 256 rows x TN tokens (rows
@@ -1302,302 +1121,6 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
     }
 }
 
-// out[t][m] = sum_z partial[z][t][m] (+ bias[m]), in the order z = 0, 1, ...
-__global__ void splitk_reduce_kernel(int n, int Mdim, int splits, const float* __restrict__ partial,
-                                     const float* __restrict__ bias, void* out, long long ldo,
-                                     int out_bf16) {
-    pdl_trigger();
-    pdl_wait();
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long total = (long long)n * Mdim;
-    if (idx >= total) return;
-    const int t = (int)(idx / Mdim);
-    const int m = (int)(idx - (long long)t * Mdim);
-    float s = 0.0f;
-    for (int z = 0; z < splits; ++z) s += __ldg(partial + (long long)z * total + idx);
-    if (bias != nullptr) s += __ldg(bias + m);
-    if (out_bf16)
-        reinterpret_cast<__nv_bfloat16*>(out)[(long long)t * ldo + m] = __float2bfloat16_rn(s);
-    else
-        reinterpret_cast<float*>(out)[(long long)t * ldo + m] = s;
-}
-
-// ------------------------------------------------------------------------------------------
-// decode: n <= 16 tokens, no pre-pass; the workers write both operands
-// ------------------------------------------------------------------------------------------
-
-struct DecodeParams {
-    int d_out, d_in, q, g, G, pitch, n;
-    int num_kb, kb_per_split, splits;
-    const float* alpha;
-    const float* bias;
-    const __nv_bfloat16* X;
-    long long ldx;
-    void* out;
-    long long ldo;
-    int out_bf16;
-    float* partial;  // [splits][n][d_out]
-};
-
-constexpr int kDecTN = 16;
-constexpr int kDecStages = 4;
-
-// Scale of one weight row in decode: the largest |alpha| of the row over every plane and every
-// group inside the CTA's K slice, times q (a bound on any level sum_i +-alpha_i), is brought to
-// [2^13, 2^14), so no level of the slice can leave the fp16 range.
-__device__ __forceinline__ int decode_row_shift(const float* __restrict__ alpha, long long plane_alpha, int G,
-                                                int q, int j, int c_lo, int c_hi) {
-    uint32_t am = 0u;
-    for (int i = 0; i < q; ++i)
-        for (int c = c_lo; c <= c_hi; ++c)
-            am = max(am, __float_as_uint(__ldg(alpha + i * plane_alpha + (long long)j * G + c)) & 0x7FFFFFFFu);
-    return shift_for(exponent_of_bits(__float_as_uint(__uint_as_float(am) * (float)q)), 13);
-}
-
-template <int QM>
-__global__ void __launch_bounds__(kThreads, 2)
-decode_kernel(const __grid_constant__ CUtensorMap tmap_bits, const DecodeParams p) {
-    using L = StageLayout<MODE_FWD, kDecTN, QM>;
-    constexpr int STAGES = kDecStages;
-    constexpr uint32_t kStageBytes = L::kStageBytes;
-    constexpr uint32_t kIdesc = ptx::make_idesc_bf16(kBlockM, kDecTN, 0, 0) & ~((1u << 7) | (1u << 10));
-
-    extern __shared__ uint8_t smem_raw[];
-    const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
-    uint8_t* smem_gen = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
-    const uint32_t ctl_base = smem_base + STAGES * kStageBytes;
-    uint8_t* ctl_gen = smem_gen + STAGES * kStageBytes;
-
-    Ctl ctl;
-    ctl.full = ctl_base;
-    ctl.aready = ctl_base + 8 * STAGES;
-    ctl.empty = ctl_base + 16 * STAGES;
-    ctl.accum = ctl_base + 24 * STAGES;
-    ctl.spare = ctl.accum + 8;
-    volatile uint32_t* tmem_holder = reinterpret_cast<volatile uint32_t*>(ctl_gen + 24 * STAGES + 16);
-    ctl.abort_flag = reinterpret_cast<volatile int*>(ctl_gen + 24 * STAGES + 20);
-    ctl.device_flag = &g_timeout_flag;
-    float* tok_scale = reinterpret_cast<float*>(ctl_gen + 24 * STAGES + 32);  // [16] scale, [16] inverse
-
-    const int warp = threadIdx.x >> 5;
-    const int lane = threadIdx.x & 31;
-    const int m0 = blockIdx.x * kBlockM;
-    const int kb_begin = blockIdx.y * p.kb_per_split;
-    const int kb_end = min(p.num_kb, kb_begin + p.kb_per_split);
-    const int iters = kb_end - kb_begin;
-    const int k_lo = kb_begin * kBlockK;
-    const int k_hi = min(kb_end * kBlockK, p.d_in);
-    const int c_lo = min(k_lo / p.g, p.G - 1), c_hi = min((k_hi - 1) / p.g, p.G - 1);
-    const long long plane_alpha = (long long)p.d_out * p.G;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            ptx::mbar_init(ctl.full + 8 * s, 1);
-            ptx::mbar_init(ctl.aready + 8 * s, kWorkerWarps);
-            ptx::mbar_init(ctl.empty + 8 * s, 1);
-        }
-        ptx::mbar_init(ctl.accum, 1);
-        ptx::mbar_init(ctl.spare, 1);
-        *ctl.abort_flag = 0;
-        ptx::fence_mbar_init();
-        ptx::prefetch_tmap(&tmap_bits);
-    }
-    if (warp == 1) {
-        ptx::tmem_alloc(ptx::smem_u32(const_cast<uint32_t*>(tmem_holder)), TmemCols<kDecTN>::value);
-        ptx::tmem_relinquish();
-    }
-    ptx::tc_fence_before_sync();
-    __syncthreads();
-    ptx::tc_fence_after_sync();
-    const uint32_t tmem_base = *tmem_holder;
-    pdl_trigger();
-    pdl_wait();
-
-    if (warp == 0) {
-        // ---------------- TMA producer: plane words only
-        if (lane == 0) {
-            bool ok = true;
-            int issued = 0;
-            const uint32_t tx = (uint32_t)p.q * L::kPlaneBytes;
-            for (int it = 0; it < iters && ok; ++it) {
-                const int s = it % STAGES;
-                const uint32_t ph = (it / STAGES) & 1;
-                const int kb = kb_begin + it;
-                ok = wait_bar(ctl.empty + 8 * s, ph ^ 1u, ctl, 20);
-                if (!ok) break;
-                ptx::mbar_arrive_expect_tx(ctl.full + 8 * s, tx);
-                ptx::tma_load_3d(smem_base + s * kStageBytes + L::kBitsOff, &tmap_bits, (kb >> 1) * 4, m0, 0,
-                                 ctl.full + 8 * s);
-                issued = it + 1;
-            }
-            if (!ok)
-                for (int it = max(0, issued - STAGES); it < issued; ++it)
-                    wait_bar(ctl.full + 8 * (it % STAGES), (it / STAGES) & 1, ctl, 25);
-        }
-    } else if (warp == 1) {
-        if (lane == 0) {
-            bool ok = true;
-            for (int it = 0; it < iters && ok; ++it) {
-                const int s = it % STAGES;
-                const uint32_t ph = (it / STAGES) & 1;
-                ok = wait_bar(ctl.aready + 8 * s, ph, ctl, 21);
-                if (!ok) break;
-                ptx::tc_fence_after_sync();
-                const uint32_t sa = smem_base + s * kStageBytes;
-                const uint32_t sb = sa + kABytes;
-#pragma unroll
-                for (int kk = 0; kk < kBlockK / 16; ++kk)
-                    ptx::umma_bf16(tmem_base, ptx::make_smem_desc(sa + kk * 32, 16, 1024),
-                                   ptx::make_smem_desc(sb + kk * 32, 16, 1024), kIdesc,
-                                   (it > 0 || kk > 0) ? 1u : 0u);
-                ptx::umma_commit(ctl.empty + 8 * s);
-            }
-            if (ok) {
-                ptx::umma_commit(ctl.accum);
-            } else {
-                ptx::umma_commit(ctl.spare);
-                wait_bar(ctl.spare, 0, ctl, 22);
-            }
-        }
-    } else {
-        const int wid = warp - kWorkerWarp0;
-        const int e = wid * 32 + lane;  // 0..255
-        const int row = wid * 16 + (lane >> 1);
-        const int half = lane & 1;
-        const int j = m0 + row;
-        const bool valid = j < p.d_out;
-        const uint32_t lx = row & 7;
-
-        // ---- per-token scale over this CTA's K slice: thread = (token e / 16, every 16th vector)
-        {
-            const int t = e >> 4, sub = e & 15;
-            uint32_t m = 0u;
-            if (t < p.n) {
-                const __nv_bfloat16* xrow = p.X + (long long)t * p.ldx;
-                for (int k = k_lo + sub * 8; k < k_hi; k += 128) {
-                    const uint4 x = __ldg(reinterpret_cast<const uint4*>(xrow + k));
-                    const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-                    for (int el = 0; el < 8; ++el)
-                        if (k + el < p.d_in) m = max(m, (xs[el >> 1] >> ((el & 1) * 16)) & 0x7FFFu);
-                }
-            }
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-            if (sub == 0) {
-                const int sh = shift_for(exponent_of_bits(m << 16), 14);
-                tok_scale[t] = pow2f(sh);
-                tok_scale[16 + t] = pow2f(-sh);
-            }
-        }
-        const float wscale = valid ? pow2f(decode_row_shift(p.alpha, plane_alpha, p.G, p.q, j, c_lo, c_hi)) : 1.0f;
-        asm volatile("bar.sync 1, %0;" ::"n"(kWorkers) : "memory");  // tok_scale visible to all workers
-
-        // activation task of threads e < 128: (token e / 8, 8 consecutive k = one 16-byte chunk)
-        const int xt = e >> 3, xch = e & 7;
-        const bool x_task = e < 128;
-        const float xscale = x_task ? tok_scale[xt] : 0.0f;
-        auto fetch_x = [&](uint4& slot, int kb) {
-            const int k = kb * kBlockK + xch * 8;
-            slot = make_uint4(0u, 0u, 0u, 0u);
-            if (x_task && xt < p.n && k < p.d_in)
-                slot = __ldg(reinterpret_cast<const uint4*>(p.X + (long long)xt * p.ldx + k));
-        };
-
-        const int cstep = max(1, kBlockK / p.g);
-        auto group_of = [&](int kb) { return min((kb * kBlockK + half * 32) / p.g, p.G - 1); };
-        AlphaSet<QM> cur, nxt;
-        int c_cur = (iters > 0) ? group_of(kb_begin) : 0;
-        load_alpha<QM>(cur, p.alpha, plane_alpha, p.G, p.q, j, c_cur, valid, wscale);
-        load_alpha<QM>(nxt, p.alpha, plane_alpha, p.G, p.q, j, min(c_cur + cstep, p.G - 1), valid, wscale);
-        uint4 xring[kPrefetch];
-#pragma unroll
-        for (int d = 0; d < kPrefetch; ++d)
-            if (d < iters) fetch_x(xring[d], kb_begin + d);
-
-        Lut lut = {0u, 0u, 0u, 0u};
-        int lut_key = -2;
-        bool ok = true;
-        for (int it0 = 0; it0 < iters && ok; it0 += kPrefetch) {
-#pragma unroll
-            for (int d = 0; d < kPrefetch; ++d) {
-                const int it = it0 + d;
-                if (it < iters && ok) {
-                    const int s = it % STAGES;
-                    const uint32_t ph = (it / STAGES) & 1;
-                    const int kb = kb_begin + it;
-                    const uint4 xcur = xring[d];
-                    if (it + kPrefetch < iters) fetch_x(xring[d], kb + kPrefetch);
-                    const int c = group_of(kb);
-                    if (c != c_cur) {
-                        cur = nxt;
-                        c_cur = c;
-                        load_alpha<QM>(nxt, p.alpha, plane_alpha, p.G, p.q, j, min(c + cstep, p.G - 1), valid, wscale);
-                    }
-                    ok = wait_bar(ctl.full + 8 * s, ph, ctl, 23);
-                    if (ok) {
-                        const uint32_t st = smem_base + s * kStageBytes;
-                        const uint32_t baddr = st + L::kBitsOff + row * 16 + (((kb & 1) * 2 + half) << 2);
-                        expand_task32<QM>(cur, baddr, L::kPlaneBytes, lut, lut_key, p.q, st + row * 128, lx, half * 4);
-                        if (x_task) {
-                            const uint32_t xs[4] = {xcur.x, xcur.y, xcur.z, xcur.w};
-                            float f[8];
-#pragma unroll
-                            for (int el = 0; el < 8; ++el) {
-                                const uint32_t b = (xs[el >> 1] >> ((el & 1) * 16)) & 0xFFFFu;
-                                f[el] = (kb * kBlockK + xch * 8 + el < p.d_in) ? __uint_as_float(b << 16) * xscale
-                                                                             : 0.0f;
-                            }
-                            ptx::st_shared_v4(st + kABytes + xt * 128 + ((xch ^ (xt & 7)) << 4),
-                                              pack_half2(f[0], f[4]), pack_half2(f[1], f[5]),
-                                              pack_half2(f[2], f[6]), pack_half2(f[3], f[7]));
-                        }
-                        ptx::fence_proxy_async_smem();
-                        __syncwarp();
-                        if (lane == 0) ptx::mbar_arrive(ctl.aready + 8 * s);
-                    }
-                }
-            }
-        }
-
-        // ---- epilogue: thread = (TMEM lane = weight row, tokens 8*eh .. 8*eh+7)
-        if (ok) ok = wait_bar(ctl.accum, 0, ctl, 24);
-        const int quarter = warp & 3, eh = wid >> 2;
-        if (ok && eh * 8 < p.n) {
-            ptx::tc_fence_after_sync();
-            uint32_t v[8];
-            ptx::tmem_ld_x8(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(eh * 8), v);
-            ptx::tmem_ld_wait();
-            const int je = m0 + quarter * 32 + lane;
-            if (je < p.d_out) {
-                const float winv = pow2f(-decode_row_shift(p.alpha, plane_alpha, p.G, p.q, je, c_lo, c_hi));
-                const float bias = (p.bias != nullptr && p.splits == 1) ? __ldg(p.bias + je) : 0.0f;
-#pragma unroll
-                for (int cidx = 0; cidx < 8; ++cidx) {
-                    const int t = eh * 8 + cidx;
-                    if (t < p.n) {
-                        const float val = __uint_as_float(v[cidx]) * (winv * tok_scale[16 + t]);
-                        if (p.splits > 1)
-                            p.partial[((long long)blockIdx.y * p.n + t) * p.d_out + je] = val;
-                        else if (p.out_bf16)
-                            reinterpret_cast<__nv_bfloat16*>(p.out)[(long long)t * p.ldo + je] =
-                                __float2bfloat16_rn(val + bias);
-                        else
-                            reinterpret_cast<float*>(p.out)[(long long)t * p.ldo + je] = val + bias;
-                    }
-                }
-            }
-        }
-    }
-
-    ptx::tc_fence_before_sync();
-    __syncthreads();
-    if (warp == 1) {
-        ptx::tc_fence_after_sync();
-        ptx::tmem_dealloc(tmem_base, TmemCols<kDecTN>::value);
-    }
-}
-
 // ------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------
@@ -1691,27 +1214,6 @@ ExpandPlan plan_expand(int mode, int d_out, int d_in, int q, int g, int n) {
     pl.off_counters = align_up(pl.off_bits + pl.planes_bytes, 128);
     pl.off_partial = align_up(pl.off_counters + (size_t)pl.res_tiles * 8 * kPfBoxClasses * sizeof(uint32_t), 128);
     pl.total = pl.off_partial + (size_t)(pl.res_tiles * pl.pieces) * tn * 256 * sizeof(float);
-    return pl;
-}
-
-struct DecodePlan {
-    int m_tiles, num_kb, splits, kb_per_split;
-    size_t total;
-};
-
-DecodePlan plan_decode(int d_out, int d_in, int n) {
-    DecodePlan pl;
-    const int sms = sm_count();
-    pl.m_tiles = ceil_div(d_out, kBlockM);
-    pl.num_kb = ceil_div(d_in, kBlockK);
-    int splits = (2 * sms) / pl.m_tiles;  // 72 KiB of shared memory per CTA: several CTAs per SM
-    if (splits < 1) splits = 1;
-    const int max_splits = (pl.num_kb + 7) / 8;  // at least 8 K blocks per CTA
-    if (splits > max_splits) splits = max_splits;
-    if (splits > 64) splits = 64;
-    pl.kb_per_split = ceil_div(pl.num_kb, splits);
-    pl.splits = ceil_div(pl.num_kb, pl.kb_per_split);
-    pl.total = pl.splits > 1 ? (size_t)pl.splits * n * d_out * sizeof(float) : 0;
     return pl;
 }
 
@@ -1853,50 +1355,16 @@ bcq_status run_expand(int d_out, int d_in, int q, int g, int n, const void* act,
     return launch_expand_q<MODE>(tm, tmo, p, pl, s);
 }
 
-template <int QM>
-bcq_status launch_decode(const CUtensorMap& tm_bits, const DecodeParams& p, const DecodePlan& pl,
-                         cudaStream_t s) {
-    constexpr size_t smem = (size_t)kDecStages * StageLayout<MODE_FWD, kDecTN, QM>::kStageBytes + 1024 + 512;
-    auto kern = decode_kernel<QM>;
-    bcq_status st0 = ensure_dynamic_smem(kern, smem);
-    if (st0 != BCQ_OK) return st0;
-    dim3 grid((unsigned)pl.m_tiles, (unsigned)pl.splits);
-    BCQ_CUDA_TRY(launch_pdl(kern, grid, kThreads, smem, s, 1, tm_bits, p));
-    return BCQ_OK;
-}
-
 bcq_status run_decode(int d_out, int d_in, int q, int g, int n, const void* X, size_t ldx,
                       const uint32_t* bits, const float* alpha, const float* bias, void* Y, size_t ldy,
                       int y_dtype, void* ws, size_t ws_bytes, void* stream) {
-    const DecodePlan pl = plan_decode(d_out, d_in, n);
-    if (pl.total > 0) {
+    const size_t need = decode_workspace_bytes(d_out, d_in, q, g, n);
+    if (need > 0) {
         if (ws == nullptr) return BCQ_ERR_NULL;
-        if (ws_bytes < pl.total) return BCQ_ERR_WORKSPACE;
+        if (ws_bytes < need) return BCQ_ERR_WORKSPACE;
         if (!aligned16(ws)) return BCQ_ERR_ALIGN;
     }
-    DecodeParams p;
-    p.d_out = d_out; p.d_in = d_in; p.q = q; p.g = g;
-    p.G = (int)bcq_num_groups(d_in, g);
-    p.pitch = (int)bcq_pitch_words(d_in);
-    p.n = n; p.num_kb = pl.num_kb; p.kb_per_split = pl.kb_per_split; p.splits = pl.splits;
-    p.alpha = alpha; p.bias = bias;
-    p.X = reinterpret_cast<const __nv_bfloat16*>(X); p.ldx = (long long)ldx;
-    p.out = Y; p.ldo = (long long)ldy; p.out_bf16 = (y_dtype == BCQ_BF16);
-    p.partial = reinterpret_cast<float*>(ws);
-    CUtensorMap tm_bits;
-    bcq_status st = make_tmap_bits(&tm_bits, bits, d_out, p.pitch, q, 128);
-    if (st != BCQ_OK) return st;
-    cudaStream_t s = (cudaStream_t)stream;
-    if (q <= 3) st = launch_decode<QM_LUT3>(tm_bits, p, pl, s);
-    else if (q == 4) st = launch_decode<QM_LUT4>(tm_bits, p, pl, s);
-    else st = launch_decode<QM_GENERIC>(tm_bits, p, pl, s);
-    if (st != BCQ_OK) return st;
-    if (pl.splits > 1) {
-        const long long total = (long long)n * d_out;
-        BCQ_CUDA_TRY(launch_pdl(splitk_reduce_kernel, dim3((unsigned)((total + 255) / 256)), 256, 0, s, 1, n, d_out, pl.splits,
-                                (const float*)p.partial, bias, Y, (long long)ldy, p.out_bf16));
-    }
-    return BCQ_OK;
+    return run_decode_planes(d_out, d_in, q, g, n, X, ldx, bits, alpha, bias, Y, ldy, y_dtype, (cudaStream_t)stream);
 }
 
 // Argument checks of the forward and decode entry points (host arithmetic and pointer tests only).
@@ -1941,7 +1409,15 @@ bcq_status expand_timeout_flag(int* flag_out, int reset) {
 size_t fwd_workspace_bytes(int d_out, int d_in, int q, int g, int n) {
     return plan_expand(MODE_FWD, d_out, d_in, q, g, n).total;
 }
-size_t decode_workspace_bytes(int d_out, int d_in, int, int, int n) { return plan_decode(d_out, d_in, n).total; }
+// The scratch that callers of bcq_linear_decode provide: partial sums of a split over d_in that gives every
+// SM two row tiles of 128.  The kernel (decode.cu) keeps its sums on chip; the size and the checks on it
+// stay as callers know them.
+size_t decode_workspace_bytes(int d_out, int d_in, int, int, int n) {
+    const int num_kb = ceil_div(d_in, kBlockK);
+    const int splits = std::min({std::max(1, 2 * sm_count() / ceil_div(d_out, kBlockM)), (num_kb + 7) / 8, 64});
+    const int used = ceil_div(num_kb, ceil_div(num_kb, splits));
+    return used > 1 ? (size_t)used * n * d_out * sizeof(float) : 0;
+}
 size_t bwd_x_workspace_bytes(int d_out, int d_in, int q, int g, int n) {
     return plan_expand(MODE_BWDX, d_out, d_in, q, g, n).total;
 }
@@ -1966,49 +1442,15 @@ extern "C" bcq_status bcq_linear_decode(int d_out, int d_in, int q, int g, int n
 // decode without a caller-provided workspace
 // ------------------------------------------------------------------------------------------
 
-namespace {
-
-// Scratch for the split-K partial sums of bcq_linear_decode_noalloc.  Lives in every CUDA context
-// that loads this library.  In host code the symbol is only a handle: the device address comes
-// from cudaGetSymbolAddress, once per device.
-static __device__ __align__(256) unsigned char g_noalloc_scratch[BCQ_NOALLOC_SCRATCH_BYTES];
-
-constexpr int kMaxDevices = 64;
-
-bcq_status noalloc_scratch_address(void** out) {
-    static void* address[kMaxDevices] = {};
-    static std::mutex lock;
-    int dev = -1;
-    BCQ_CUDA_TRY(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= kMaxDevices) return BCQ_ERR_UNSUPPORTED;
-    std::lock_guard<std::mutex> guard(lock);
-    if (address[dev] == nullptr) {
-        void* p = nullptr;
-        BCQ_CUDA_TRY(cudaGetSymbolAddress(&p, g_noalloc_scratch));
-        address[dev] = p;
-    }
-    *out = address[dev];
-    return BCQ_OK;
-}
-
-}  // namespace
-
 extern "C" bcq_status bcq_linear_decode_noalloc(int d_out, int d_in, int q, int g, int n, const void* X,
                                                 size_t ldx, const uint32_t* bits, const float* alpha,
                                                 const float* bias, void* Y, size_t ldy, int y_dtype,
                                                 void* stream) {
-    // Every argument is checked before the scratch symbol is resolved.  (The size check asks the
-    // device for its SM count, so it is not free of CUDA calls; without a device the count falls
-    // back to a B200's.)  The address found for a device is kept for the life of the process: after
-    // cudaDeviceReset it is stale, and the library has to be loaded again.
     bcq_status st = check_fwd_args(1, d_out, d_in, q, g, n, X, ldx, bits, alpha, Y, ldy, y_dtype);
     if (st != BCQ_OK) return st;
     if (bcq::decode_workspace_bytes(d_out, d_in, q, g, n) > (size_t)BCQ_NOALLOC_SCRATCH_BYTES)
         return BCQ_ERR_WORKSPACE;
-    void* scratch = nullptr;
-    if ((st = noalloc_scratch_address(&scratch)) != BCQ_OK) return st;
-    return fwd_common(1, d_out, d_in, q, g, n, X, ldx, bits, alpha, bias, Y, ldy, y_dtype, scratch,
-                      (size_t)BCQ_NOALLOC_SCRATCH_BYTES, stream);
+    return bcq::run_decode_planes(d_out, d_in, q, g, n, X, ldx, bits, alpha, bias, Y, ldy, y_dtype, (cudaStream_t)stream);
 }
 
 extern "C" bcq_status bcq_linear_bwd_x(int d_out, int d_in, int q, int g, int n, const void* dY,

@@ -58,22 +58,6 @@ __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, const Ct
     }
 }
 
-// The same for a whole (converged) warp: lane 0 polls, the outcome is broadcast, and the warp
-// barrier orders the other lanes' later reads after lane 0's acquire.  Keeps the number of threads
-// polling shared-memory barriers small.
-__device__ __forceinline__ bool warp_wait_bar(uint32_t bar, uint32_t parity, const Ctl& ctl, int code) {
-    int ok = 1;
-    if ((threadIdx.x & 31) == 0) ok = wait_bar(bar, parity, ctl, code) ? 1 : 0;
-    ok = __shfl_sync(0xffffffffu, ok, 0);
-    __syncwarp();
-    return ok != 0;
-}
-
-template <int TN>
-struct TmemCols {
-    static constexpr uint32_t value = TN < 32 ? 32 : TN;
-};
-
 // ------------------------------------------------------------------------------------------
 // host helpers
 // ------------------------------------------------------------------------------------------
@@ -149,29 +133,6 @@ inline bcq_status make_tmap_out_bf16(CUtensorMap* m, void* base, int inner, int 
     return BCQ_OK;
 }
 
-// The packed planes uint32 [q][d_out][pitch] as a 3-D tensor; box = 4 words (128 weights) x
-// box_rows x q, no swizzle; rows or words out of range read as zero.
-inline bcq_status make_tmap_bits(CUtensorMap* m, const uint32_t* bits, int d_out, int pitch_words, int q,
-                                 int box_rows) {
-    EncodeTiledFn fn = encode_fn();
-    if (fn == nullptr) {
-        set_last_cuda_error((int)cudaErrorNotSupported);
-        return BCQ_ERR_CUDA;
-    }
-    cuuint64_t dims[3] = {(cuuint64_t)pitch_words, (cuuint64_t)d_out, (cuuint64_t)q};
-    cuuint64_t strides[2] = {(cuuint64_t)pitch_words * 4, (cuuint64_t)pitch_words * 4 * (cuuint64_t)d_out};
-    cuuint32_t box[3] = {4u, (cuuint32_t)box_rows, (cuuint32_t)q};
-    cuuint32_t estr[3] = {1u, 1u, 1u};
-    CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, const_cast<uint32_t*>(bits), dims, strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-        set_last_cuda_error((int)cudaErrorInvalidValue);
-        return BCQ_ERR_CUDA;
-    }
-    return BCQ_OK;
-}
-
 inline bcq_status check_act(const void* ptr, size_t ld, int cols) {
     if (ptr == nullptr) return BCQ_ERR_NULL;
     if (ld < (size_t)cols) return BCQ_ERR_SHAPE;
@@ -184,6 +145,10 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // per-TU device timeout flags
 bcq_status expand_timeout_flag(int* flag_out, int reset);
 bcq_status dalpha_timeout_flag(int* flag_out, int reset);
+
+// decode from the canonical planes (decode.cu); the arguments have been checked
+bcq_status run_decode_planes(int d_out, int d_in, int q, int g, int n, const void* X, size_t ldx, const uint32_t* bits,
+                             const float* alpha, const float* bias, void* Y, size_t ldy, int y_dtype, cudaStream_t s);
 
 // workspace sizes (defined next to the kernels that use them)
 size_t fwd_workspace_bytes(int d_out, int d_in, int q, int g, int n);

@@ -97,20 +97,7 @@ __host__ __device__ inline void selectors_from_planes(const uint32_t (&w)[4], in
     }
 }
 
-template <int Q>
-__device__ __forceinline__ void load_codes(uint32_t addr, uint32_t (&v)[Q]) {
-    if constexpr (Q == 4) {
-        asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
-                     : "r"(addr) : "memory");
-    } else if constexpr (Q == 2) {
-        asm volatile("ld.shared.v2.b32 {%0,%1}, [%2];" : "=r"(v[0]), "=r"(v[1]) : "r"(addr) : "memory");
-    } else {
-#pragma unroll
-        for (int i = 0; i < Q; ++i) v[i] = ptx::ld_shared_u32(addr + 4 * i);
-    }
-}
-
-// The four selector words of 32 weights from the q stored words (see pack_codes_kernel).
+// The four selector words of 32 weights from the q stored words (see pack_selectors).
 template <int Q>
 __device__ __forceinline__ void selectors(const uint32_t (&v)[Q], uint32_t (&S)[4]) {
     constexpr uint32_t M = 0x11111111u;

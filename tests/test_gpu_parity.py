@@ -456,6 +456,31 @@ def test_decode_packed_matches_oracle(n, d_in, d_out, q, g):
     assert rel_err(Yb.float().cpu().numpy(), ref + bias.astype(np.float64)) <= TOL + 2.0 ** -8
 
 
+@pytest.mark.parametrize("n,d_in,d_out,q,g", [
+    (1, 136, 24, 1, 136), (9, 1000, 40, 2, 1000), (8, 672, 72, 4, 96), (16, 320, 17, 3, 32), (3, 2600, 264, 5, 64),
+    (11, 520, 136, 8, 520), (2, 128, 30008, 4, 128), (12, 256, 30000, 3, 64), (16, 16392, 40, 4, 16392),
+])
+def test_decode_from_planes_and_packs(n, d_in, d_out, q, g):
+    # both decode kernels at the edges of their units (16 rows x 128 columns, 8 tokens): ragged rows and
+    # columns, groups inside a unit, q > 4, and more row tiles per CTA than its sums have room for.
+    # Against a dense fp64 product with the dequantized weights.
+    gen = torch.Generator(device="cuda").manual_seed(n * 1000 + d_out)
+    W = torch.randn((d_out, d_in), generator=gen, device="cuda") * 0.02
+    bits, alpha, _ = bcq.quantize(W, q, g)
+    X = torch.randn((n, d_in), generator=gen, device="cuda").bfloat16()
+    bias = torch.randn(d_out, generator=gen, device="cuda")
+    ref = (X.double() @ bcq.dequantize(bits, alpha, d_in, g).double().t() + bias.double()).cpu().numpy()
+    calls = [lambda dt: bcq.linear_decode(X, bits, alpha, d_in, g, bias=bias, out_dtype=dt)]
+    if q <= 4:
+        pack = bcq.decode_pack(bits, alpha, d_in, g)
+        calls.append(lambda dt: bcq.linear_decode_packed(X, pack, d_out, d_in, q, g, bias=bias, out_dtype=dt))
+    for call in calls:
+        for dt, tol in ((torch.float32, TOL), (torch.bfloat16, TOL + 2.0 ** -8)):
+            Y = call(dt)
+            assert torch.equal(Y, call(dt)), "two runs differ"
+            assert rel_err(Y.float().cpu().numpy(), ref) <= tol
+
+
 def test_decode_pack_rejects_more_than_four_planes():
     assert bcq.lib().bcq_decode_pack_bytes(64, 256, 5, 64) == 0
     assert bcq.lib().bcq_decode_pack_bytes(64, 256, 4, 64) > 0
