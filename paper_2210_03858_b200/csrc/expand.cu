@@ -24,6 +24,7 @@
 //   * q > 4: the sums come out in the order 0,4,1,5,2,6,3,7 of a byte of a plane word, so the pre-pass,
 //     which regroups the plane words anyway, stores the bits of every byte as 0,2,4,6,1,3,5,7.
 #include <algorithm>
+#include <cmath>
 
 #include "gemm_common.cuh"
 #include "lut.cuh"
@@ -1163,6 +1164,13 @@ ExpandPlan plan_expand(int mode, int d_out, int d_in, int q, int g, int n) {
     //     cost nothing if that is much longer (measured: 5120 -> 20480 dX with 2048 tokens, 12 of 172
     //     tiles in pieces, 429 -> 359 us; 1600 -> 6400, whose tiles are 25 stages, 79 -> 92 us);
     //   * the last output, TN / 64 stages.
+    // That is the time of a call with the chip to itself.  A layer stack that runs on several streams
+    // pays for the pair stages a plan occupies instead (narrow tiles expand the same weights again for
+    // each), so these weigh in with a small exponent: it turns down a plan that is a few per cent
+    // faster alone and takes twice the stages.  Forward and backward of gpt2-medium's
+    // linears (2048 tokens, q = 3): one block on one stream 285 -> 291 us, the stack on nine streams
+    // 684 -> 750 TFLOP/s; one 1024 x 1024 layer on three streams 85 -> 146 TFLOP/s; 1000 x 1528 at
+    // 777 tokens on one stream 63 -> 65 us.
     const int nt0 = ceil_div(n, 256), nt1 = std::min(ceil_div(n, 32), 8 * nt0);
     double best = -1.0;
     for (int nt = nt0; nt <= nt1; ++nt) {
@@ -1178,8 +1186,10 @@ ExpandPlan plan_expand(int mode, int d_out, int d_in, int q, int g, int n) {
             if (d > 1 && waves == 0) add = 9.0 + 2.4 * ceil_div(tn, 80) * d;
             if (d > 1 && waves > 0 && waves * pl.num_kb < 3 * 40 * d) break;  // would not stay hidden
             const double cost = (waves * pl.num_kb + (ragged > 0 ? len : 0)) * stage + add + out;
-            if (best >= 0.0 && cost >= best) continue;
-            best = cost;
+            const double stages = (waves > 0 ? tiles : tiles * ceil_div(pl.num_kb, len)) * (double)len;
+            const double score = cost * std::pow(stages, 0.2);
+            if (best >= 0.0 && score >= best) continue;
+            best = score;
             pl.TN = tn;
             pl.n_tiles = nt;
             pl.pieces = ceil_div(pl.num_kb, len);
