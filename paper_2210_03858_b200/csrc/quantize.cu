@@ -3,16 +3,16 @@
 // One "team" of threads owns one (row, group) problem and keeps its weights in registers.
 //
 // team_quantize_kernel (greedy for every q, alternating for q <= 4): a thread holds up to 32 weights, so
-// a group of 128 is four lanes and a warp works on eight groups; a team is up to a warp for g <= 1024
-// and a whole CTA above that.  Four lanes share 128 consecutive weights, lane l taking the 16-byte
+// a group of 128 is four lanes and a warp works on eight groups (greedy; alternating takes 8 or 16
+// lanes, see launch_team_size); a team is up to a warp for g <= 1024 and a whole CTA above that.  Four lanes share 128 consecutive weights, lane l taking the 16-byte
 // pieces l, l + 4, ...: full 32-byte sectors from memory, and the four lanes' sign bits make four
 // container words with one 4 x 4 byte transpose.  With a warp per group (four weights a lane), as
 // this kernel worked before, a plane of 128 weights cost five rounds of 64-bit shuffles and a
 // ballot per 32 weights; now two rounds, and per weight and plane two fp64 additions and one shift
 // that collects the sign.  Measured, before and after: greedy q = 4, g = 128, the four linears of a
 // layer of width 1600 (30.7 M weights) 162 -> 69 us (2.1 TB/s; the logic pipe is 55 % busy, the fp64
-// pipe 21 %); five alternating rounds, q = 3, g = 128, 5120 x 5120: 1119 -> 373 us (instruction fetch of
-// the unrolled rounds and fp64 latency at 2.6 warps per scheduler bound it).
+// pipe 21 %); five alternating rounds, q = 3, g = 128, 5120 x 5120: 1119 -> 350 us (instruction fetch of
+// the unrolled rounds and fp64 latency at five warps per scheduler bound it).
 //
 // Sums are fp64 and are reduced in a fixed order, so a result never depends on scheduling.
 //
@@ -454,7 +454,8 @@ struct LevelSearch {
 // Q = 0: greedy, p.q planes; Q > 0: alternating with Q planes.  A thread holds 4 NI weights, a team is L
 // lanes (TW = 1) or TW warps.
 template <int NI, int L, int TW, int Q>
-__global__ void __launch_bounds__(TW == 1 ? 128 : TW * 32, TW == 1 ? (Q == 0 ? 5 : 3) : TW <= 4 ? 12 / TW : 1)
+__global__ void __launch_bounds__(TW == 1 ? 128 : TW * 32,
+                                  TW == 1 ? (Q == 0 || NI == 4 ? 5 : NI == 2 ? 6 : 3) : TW <= 4 ? (NI == 4 ? 20 : 12) / TW : 1)
 team_quantize_kernel(const QuantParams p) {
     constexpr bool ALT = Q > 0;
     constexpr int EPT = 4 * NI;
@@ -760,15 +761,35 @@ cudaError_t launch_team(const QuantParams& p, cudaStream_t stream) {
     return bcq::launch_pdl(team_quantize_kernel<NI, L, TW, Q>, dim3(blocks), threads, 0, stream, 1, p);
 }
 
-// The smallest team that holds a group at 32 weights a thread (8 or 16 for groups of 32 or 64).
+// Greedy: the smallest team that holds a group at 32 weights a thread (8 or 16 for groups of 32 or 64).
+// Alternating: a thread goes through its weights one after the other in every round, so a problem that
+// is over in a few waves takes as long as one thread does, and fewer weights a thread are better;
+// more lanes mean more shuffles and more copies of the solve, which a long one pays for.  Measured, five
+// rounds, at 32 / 16 / 8 weights a thread:
+//   g = 128, q = 4   512 x 512 56 / 37 / 28 us   2048 x 1536 209 / 138 / 118   3000 x 4096 401 / 333 / 401
+//                    5120 x 5120 711 / 653 / 851
+//   g = 128, q = 3   512 x 512 31 / 20 / 21 us   1406 x 1582 93 / 55 / 58   5120 x 5120 357 / 345 / 468
+//   g = 256, q = 3   1406 x 1582 106 / 57 us     5120 x 5120 355 / 346
+//   a row, q = 3     1024 x 1024 80 / 53 us      2048 x 1536 128 / 98       3000 x 4096 231 / 288
+// The line between "few waves" and "long" is 30720 weights per SM (4.5 M on 148, three waves of the
+// 16-weight teams).
 template <int Q>
 cudaError_t launch_team_size(const QuantParams& p, cudaStream_t s) {
     const int g = p.g;
+    const bool few = Q > 0 && p.items * g <= 30720ll * bcq::sm_count();
     if (g <= 32) return launch_team<2, 4, 1, Q>(p, s);
     if (g <= 64) return launch_team<4, 4, 1, Q>(p, s);
-    if (g <= 128) return launch_team<8, 4, 1, Q>(p, s);
-    if (g <= 256) return launch_team<8, 8, 1, Q>(p, s);
-    if (g <= 512) return launch_team<8, 16, 1, Q>(p, s);
+    if constexpr (Q > 0) {
+        if (g <= 128) return few ? launch_team<2, 16, 1, Q>(p, s) : launch_team<4, 8, 1, Q>(p, s);
+        if (g <= 256) return launch_team<4, 16, 1, Q>(p, s);
+        if (g <= 512) return launch_team<4, 32, 1, Q>(p, s);
+        if (g <= 1024 && few) return launch_team<4, 32, 2, Q>(p, s);
+        if (g <= 2048 && few) return launch_team<4, 32, 4, Q>(p, s);
+    } else {
+        if (g <= 128) return launch_team<8, 4, 1, Q>(p, s);
+        if (g <= 256) return launch_team<8, 8, 1, Q>(p, s);
+        if (g <= 512) return launch_team<8, 16, 1, Q>(p, s);
+    }
     if (g <= 1024) return launch_team<8, 32, 1, Q>(p, s);
     if (g <= 2048) return launch_team<8, 32, 2, Q>(p, s);
     if (g <= 4096) return launch_team<8, 32, 4, Q>(p, s);

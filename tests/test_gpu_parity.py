@@ -134,6 +134,26 @@ def test_quantize_team_sizes_with_exact_ties(d_in, g, alt):
             np.testing.assert_allclose(sq.cpu().numpy(), sq_ref, rtol=1e-6, atol=1e-12)
 
 
+@pytest.mark.parametrize("d_in,g", [(420, 96), (260, 128), (1023, 1023), (1582, 1582)])
+def test_quantize_alternating_short_and_long_problems(d_in, g):
+    # The size of the team depends on how much there is to do: the same five rows alone and repeated past
+    # the line (30720 weights per SM).  Values as in the test above, so the bits are the oracle's exactly.
+    rng = np.random.default_rng(d_in)
+    W = (rng.integers(-6, 7, size=(5, d_in)) / 64.0).astype(np.float32)
+    W[0, ::3] = -0.0
+    W[2, : d_in // 2] = 0.25
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    reps = 30720 * sms // (5 * -(-d_in // g) * g) + 1
+    Wd = torch.from_numpy(W).cuda()
+    for q in (1, 2, 3, 4):
+        bits_ref, alpha_ref, sq_ref, _ = oracle.quantize(W, q, g, alt_iters=3)
+        for r in (1, reps):
+            bits, alpha, sq = bcq.quantize(Wd.repeat(r, 1), q, g, 3, want_sq_err=True)
+            np.testing.assert_array_equal(host_bits(bits), np.tile(bits_ref, (1, r, 1)))
+            np.testing.assert_allclose(alpha.cpu().numpy(), np.tile(alpha_ref, (1, r, 1)), rtol=1e-6, atol=1e-9)
+            np.testing.assert_allclose(sq.cpu().numpy(), np.tile(sq_ref, (r, 1)), rtol=1e-6, atol=1e-12)
+
+
 def test_quantize_strided_input_and_determinism():
     W = synth.weights(48, 384, (101, 0, 0))
     Wp = np.zeros((48, 400), dtype=np.float32)
