@@ -26,6 +26,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "expand_rules.h"
 #include "gemm_common.cuh"
 #include "lut.cuh"
 
@@ -444,7 +445,6 @@ struct ExpandParams {
 // first.  It writes its fp32 sums to the workspace, and for each box of the output the warp that arrives
 // last (a counter) adds the pieces in order and writes the result, so no warp waits for another and the
 // result does not depend on which one is last.
-constexpr int kPfGroups = 4;
 constexpr int kPfGroupWarps = 4;
 constexpr int kPfWorkerWarps = kPfGroups * kPfGroupWarps;  // 16
 constexpr int kPfEpiWarp0 = kPfWorkerWarps;
@@ -1208,7 +1208,7 @@ ExpandPlan plan_expand(int mode, int d_out, int d_in, int q, int g, int n) {
     // Shared memory.  A worker group takes about a microsecond from "the tensor core is done with my
     // slot" to "the slot holds the next tile", and a TMA load as long to land; both rings must be deep
     // enough to cover that at one stage per ~0.3 us.  These fit at every token-tile width.
-    pl.a_slots = 6;
+    pl.a_slots = kPfWeightSlots;
     pl.b_slots = 6;
     pl.smem = pl.a_slots * (size_t)kABytes + pl.b_slots * (size_t)(tn / 2) * kBlockK * 2 +
               2 * (size_t)kPfStagingBuf + kPfFixedBytes;
@@ -1355,13 +1355,7 @@ bcq_status run_expand(int d_out, int d_in, int q, int g, int n, const void* act,
     p.counters = pp.counters;
     // bf16 output with an aligned base and pitch goes out through TMA stores
     p.fast_epi = fast_epi ? 1 : 0;
-    // The workers find the last segment's accumulator by barrier parity alone.  They run at most
-    // `a_slots` pipeline stages ahead of the tensor core, so the parity is unambiguous only if the last
-    // two segments are longer than that: then the accumulator's previous use (two segments back) is
-    // certain to be complete when a worker has finished the last segment's stages (always so where a
-    // pair has no more than two segments).
-    const int len2 = pl.num_kb + (pl.res_tiles > 0 ? pl.piece_len : pl.num_kb);  // at least, of the last two of three
-    p.helpers = (pl.full_tiles <= pl.pairs || len2 >= pl.a_slots + 2) ? 1 : 0;
+    p.helpers = helpers_may_share(pl.full_tiles, pl.pairs, pl.num_kb) ? 1 : 0;
     return launch_expand_q<MODE>(tm, tmo, p, pl, s);
 }
 
