@@ -199,9 +199,7 @@ bcq_status bcq_decode_pack(int d_out, int d_in, int q, int g, const uint32_t* bi
  * bcq_linear_decode: fp16 levels, bf16 activations scaled per token and 128 columns by a power of two,
  * fp32 accumulation).  One kernel; all sums are taken in a fixed order, so the result is the same in
  * every run.  No scratch is needed (bcq_workspace_bytes(BCQ_OP_DECODE_PACKED, ...) is 0; ws is not used),
- * the pack is only read, and calls may overlap on the GPU.  (The kernel may read
- * the pack while the kernel before it in the stream is ending, so a kernel of the caller's own that
- * writes a pack must not release its programmatic dependents early.) */
+ * the pack is only read, and calls may overlap on the GPU. */
 bcq_status bcq_linear_decode_packed(int d_out, int d_in, int q, int g, int n, const void* X, size_t ldx,
                                     void* pack, const float* bias, void* Y, size_t ldy, int y_dtype,
                                     void* ws, size_t ws_bytes, void* stream);

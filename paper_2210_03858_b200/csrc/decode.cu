@@ -28,9 +28,9 @@
 // were no faster (54 us) and slower for 16 tokens (73 and 92 us against 66).
 //
 // Weights go from global memory to registers two units ahead of their use.  The kernel may start
-// while the previous kernel of the stream is finishing (programmatic dependent launch): the pack is
-// frozen, so the first two units are requested before the grid dependency wait; the activations are
-// read after it.
+// while the previous kernel of the stream is finishing (programmatic dependent launch).  That may be the
+// kernel that writes the pack, and only the grid dependency wait makes its writes visible, so nothing
+// is read before it; the first two units are merely brought into L2.
 #include <algorithm>
 
 #include "gemm_common.cuh"
@@ -322,6 +322,18 @@ decode_packed_kernel(const DecPackedParams p) {
             }
         };
         const size_t codes_stride = (size_t)p.steps * (Q * 256), tables_stride = (size_t)p.G * kDpTableBytes;
+        auto touch = [&]() {  // into L2: the first unit and the next one of the step
+            for (int u = 0; u < min(2, l_left); ++u) {
+                if (u > 0 && l_i + u >= round_n) break;
+#pragma unroll
+                for (int v = 0; v < (Q + 1) / 2; ++v) ptx::prefetch_l2(lp_codes + u * codes_stride + v * 512 - (2 * v + 1 == Q ? lane * 8 : 0));
+#pragma unroll
+                for (int a = 0; a < PARTS; ++a) {
+                    ptx::prefetch_l2(lp_tables[a] + u * tables_stride);
+                    ptx::prefetch_l2(lp_tables[a] + u * tables_stride + 128);
+                }
+            }
+        };
         auto load = [&](UnitWords<Q, PARTS>& u) {
             if (l_left == 0) return;
             --l_left;
@@ -351,11 +363,12 @@ decode_packed_kernel(const DecPackedParams p) {
         };
         UnitWords<Q, PARTS> ua, ub;
         seek();
+        if (first == 0) touch();
+        for (int i = 0; i < round_n * NT; ++i) mine[i * 32] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (first == 0) pdl_wait();
         load(ua);
         load(ub);
-        for (int i = 0; i < round_n * NT; ++i) mine[i * 32] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (first == 0) {
-            pdl_wait();
             // the activations of the warp's later steps: into L1 while the first step is at work
             // (32 lanes: 16 tokens x two 128-byte lines of a step)
             for (int s = st0 + 1; s * round_n < u1; ++s) {
@@ -783,8 +796,6 @@ extern "C" size_t bcq_decode_pack_bytes(int d_out, int d_in, int q, int g) {
     return pack_layout(d_out, d_in, q, g).total;
 }
 
-// (The three kernels are launched the ordinary way: the decode kernel reads the pack before its grid
-// dependency wait, so it must not start before they have finished.)
 extern "C" bcq_status bcq_decode_pack(int d_out, int d_in, int q, int g, const uint32_t* bits,
                                       const float* alpha, void* pack, size_t pack_bytes, void* stream) {
     bcq_status st = check_pack_shape(d_out, d_in, q, g);

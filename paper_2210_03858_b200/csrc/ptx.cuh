@@ -94,6 +94,9 @@ __device__ __forceinline__ uint32_t ldg_nc_u32(const void* p) {
     return v;
 }
 
+// Brings the 128-byte line of `p` into L2.  Reads nothing, so it needs no ordering with the line's writer.
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // Makes this thread's generic-proxy writes to shared memory visible to the async proxy
 // (TMA and the tensor core read shared memory through it).
 __device__ __forceinline__ void fence_proxy_async_smem() {

@@ -521,6 +521,34 @@ def test_decode_from_planes_and_packs(n, d_in, d_out, q, g):
             assert rel_err(Y.float().cpu().numpy(), ref) <= tol
 
 
+@pytest.mark.parametrize("d_in,d_out,q,g,n", [(1024, 264, 4, 128, 1), (4096, 1000, 3, 64, 3), (512, 2400, 2, 512, 16)])
+def test_decode_right_after_packing_into_a_used_buffer(d_in, d_out, q, g, n):
+    # the decode kernel may start while the kernels that write its pack are still running: two matrices are
+    # packed in turn into one buffer, each decoded at once, and must give what they give from packs of
+    # their own
+    lib = bcq.lib()
+    gen = torch.Generator(device="cuda").manual_seed(d_in)
+    X = torch.randn((n, d_in), generator=gen, device="cuda").bfloat16()
+    mats, ref = [], []
+    for _ in range(2):
+        bits, alpha, _ = bcq.quantize(torch.randn((d_out, d_in), generator=gen, device="cuda") * 0.02, q, g)
+        mats.append((bits, alpha))
+        own = bcq.decode_pack(bits, alpha, d_in, g)
+        torch.cuda.synchronize()
+        ref.append(bcq.linear_decode_packed(X, own, d_out, d_in, q, g))
+    pack = torch.empty(lib.bcq_decode_pack_bytes(d_out, d_in, q, g), dtype=torch.uint8, device="cuda")
+    outs = [torch.empty((n, d_out), device="cuda") for _ in range(60)]
+    torch.cuda.synchronize()
+    stream = torch.cuda.current_stream().cuda_stream
+    for i, out in enumerate(outs):
+        bits, alpha = mats[i % 2]
+        assert lib.bcq_decode_pack(d_out, d_in, q, g, bits.data_ptr(), alpha.data_ptr(), pack.data_ptr(), pack.numel(),
+                                   stream) == 0
+        bcq.linear_decode_packed(X, pack, d_out, d_in, q, g, out=out)
+    for i, out in enumerate(outs):
+        assert torch.equal(out, ref[i % 2]), i
+
+
 def test_decode_pack_rejects_more_than_four_planes():
     assert bcq.lib().bcq_decode_pack_bytes(64, 256, 5, 64) == 0
     assert bcq.lib().bcq_decode_pack_bytes(64, 256, 4, 64) > 0
