@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
+#include <string.h>
 
 #include <utility>
 
@@ -81,6 +82,37 @@ inline cudaError_t launch_pdl(void (*kern)(Params...), dim3 grid, int threads, s
 }
 
 #ifdef __CUDACC__
+// Loads from global memory.  A kernel launched by launch_pdl is alive while the kernel before it still
+// writes, and what that kernel writes are its inputs.  So its loads may not take the non-coherent path
+// (ld.global.nc, __ldg, what the compiler makes of const __restrict__), which is defined only for memory
+// that nobody writes while the kernel lives, and they must stay behind pdl_wait(): these are ordinary loads
+// in volatile asm, which keeps its place.  ld_stream stays out of L1 (data that an SM reads once).
+// Measured over the calls of a layer: no difference to the non-coherent loads.
+#define BCQ_DEFINE_LOAD(name, how)                                                                             \
+    template <typename T>                                                                                      \
+    __device__ __forceinline__ T name(const T* p) {                                                            \
+        static_assert(sizeof(T) == 4 || sizeof(T) == 8 || sizeof(T) == 16, "4, 8 or 16 bytes");                \
+        T v;                                                                                                   \
+        if constexpr (sizeof(T) == 4) {                                                                        \
+            uint32_t r;                                                                                        \
+            asm volatile("ld.global" how ".b32 %0, [%1];" : "=r"(r) : "l"(p));                                 \
+            memcpy(&v, &r, 4);                                                                                 \
+        } else if constexpr (sizeof(T) == 8) {                                                                 \
+            uint2 r;                                                                                           \
+            asm volatile("ld.global" how ".v2.b32 {%0,%1}, [%2];" : "=r"(r.x), "=r"(r.y) : "l"(p));            \
+            memcpy(&v, &r, 8);                                                                                 \
+        } else {                                                                                               \
+            uint4 r;                                                                                           \
+            asm volatile("ld.global" how ".v4.b32 {%0,%1,%2,%3}, [%4];"                                        \
+                         : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));                               \
+            memcpy(&v, &r, 16);                                                                                \
+        }                                                                                                      \
+        return v;                                                                                              \
+    }
+BCQ_DEFINE_LOAD(ld, "")
+BCQ_DEFINE_LOAD(ld_stream, ".L1::no_allocate")
+#undef BCQ_DEFINE_LOAD
+
 // Until the kernel before this one in the stream has finished and its writes are visible.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // The kernel after this one may be scheduled once every CTA of this one has said so (or ended).

@@ -231,7 +231,7 @@ dalpha_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant
 #pragma unroll
                 for (int i = 0; i < BCQ_MAX_Q; ++i) {
                     const bool act = (i < p.q) && ((p.plane_mask >> i) & 1u) && j_ok && (kw < p.pitch);
-                    nw[ch][i] = act ? ~__ldg(p.bits + i * plane_words + (long long)j * p.pitch + kw) : 0u;
+                    nw[ch][i] = act ? ~ld(p.bits + i * plane_words + (long long)j * p.pitch + kw) : 0u;
                 }
             }
 
@@ -312,8 +312,8 @@ dalpha_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant
 // eight loads per output are in flight at once), then the eight sums are added in order 0..7.
 __global__ void __launch_bounds__(256)
 dalpha_reduce_kernel(int d_out, int d_in, int q, int g, int G, int HN, int splits, int n_subtiles, int slots,
-                     uint32_t plane_mask, float scale, int accumulate, const float* __restrict__ partial,
-                     float* __restrict__ dalpha) {
+                     uint32_t plane_mask, float scale, int accumulate, const float* partial,
+                     float* dalpha) {
     __shared__ float sums[8][32];
     pdl_trigger();
     pdl_wait();
@@ -334,7 +334,7 @@ dalpha_reduce_kernel(int d_out, int d_in, int q, int g, int G, int HN, int split
         for (int e = part; e < total; e += 8) {
             const int z = e / st_n, st = st_lo + (e - z * st_n);
             const int slot = c - min((st * HN) / g, G - 1);
-            s += __ldg(partial + ((((long long)z * n_subtiles + st) * q + i) * slots + slot) * d_out + j);
+            s += ld(partial + ((((long long)z * n_subtiles + st) * q + i) * slots + slot) * d_out + j);
         }
     }
     sums[part][jx] = s;

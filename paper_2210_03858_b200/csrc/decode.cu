@@ -93,8 +93,8 @@ __device__ __forceinline__ uint32_t code_pos(int w, int lane) {
 // ------------------------------------------------------------------------------------------
 
 // One thread per weight row: the power of two of the row and its inverse.
-__global__ void pack_rowscale_kernel(int d_out, int q, int G, int rows_padded, const float* __restrict__ alpha,
-                                     float* __restrict__ rinv) {
+__global__ void pack_rowscale_kernel(int d_out, int q, int G, int rows_padded, const float* alpha,
+                                     float* rinv) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= rows_padded) return;
     float inv = 1.0f;
@@ -102,26 +102,26 @@ __global__ void pack_rowscale_kernel(int d_out, int q, int G, int rows_padded, c
         uint32_t am = 0u;
         for (int i = 0; i < q; ++i)
             for (int c = 0; c < G; ++c)
-                am = max(am, __float_as_uint(__ldg(alpha + ((long long)i * d_out + j) * G + c)) & 0x7FFFFFFFu);
+                am = max(am, __float_as_uint(ld(alpha + ((long long)i * d_out + j) * G + c)) & 0x7FFFFFFFu);
         inv = pow2f(-shift_for(exponent_of_bits(__float_as_uint(__uint_as_float(am) * (float)q)), 13));
     }
     rinv[j] = inv;
 }
 
 // One thread per (tile, group, row): the lookup table of the row's levels in that group.
-__global__ void pack_tables_kernel(int d_out, int q, int G, long long total, const float* __restrict__ alpha,
-                                   const float* __restrict__ rinv, uint4* __restrict__ tables) {
+__global__ void pack_tables_kernel(int d_out, int q, int G, long long total, const float* alpha,
+                                   const float* rinv, uint4* tables) {
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= total) return;
     const int c = (int)((idx >> 4) % G);
     const int j = (int)((idx >> 4) / G) * kDpRows + (int)(idx & 15);
     uint4 out = make_uint4(0u, 0u, 0u, 0u);  // rows past d_out expand to zeros
     if (j < d_out) {
-        const float wscale = 1.0f / __ldg(rinv + j);  // a power of two
+        const float wscale = 1.0f / ld(rinv + j);  // a power of two
         float a[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-            a[i] = (i < q) ? __ldg(alpha + ((long long)i * d_out + j) * G + c) * wscale : 0.0f;
+            a[i] = (i < q) ? ld(alpha + ((long long)i * d_out + j) * G + c) * wscale : 0.0f;
         const Lut t = build_lut(a[0], a[1], a[2], a[3]);  // q <= 3: a[3] = 0 is the base
         out = make_uint4(t.tl0, t.tl1, t.th0, t.th1);
     }
@@ -131,7 +131,7 @@ __global__ void pack_tables_kernel(int d_out, int q, int G, long long total, con
 // One warp per unit.
 template <int Q>
 __global__ void __launch_bounds__(256) pack_codes_kernel(int d_out, int pitch, int tiles, int steps,
-                                                         const uint32_t* __restrict__ bits, uint32_t* __restrict__ codes) {
+                                                         const uint32_t* bits, uint32_t* codes) {
     const long long unit = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (unit >= (long long)tiles * steps) return;
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(256) pack_codes_kernel(int d_out, int pitch, i
             uint32_t w[4] = {0u, 0u, 0u, 0u}, S[4];
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
-                const uint4 src = __ldg(reinterpret_cast<const uint4*>(bits + ((long long)i * d_out + j) * pitch) + st);
+                const uint4 src = ld(reinterpret_cast<const uint4*>(bits + ((long long)i * d_out + j) * pitch) + st);
                 w[i] = ((src.x >> (8 * t)) & 0xFFu) | (((src.y >> (8 * t)) & 0xFFu) << 8) |
                        (((src.z >> (8 * t)) & 0xFFu) << 16) | (((src.w >> (8 * t)) & 0xFFu) << 24);
             }
@@ -178,7 +178,7 @@ struct DecOut {
 //   sums [warp][max_tiles][NT][32 lanes]: lane (g, t) has rows g (x, y) and g + 8 (z, w), tokens 2 t, 2 t + 1
 template <int NT>
 __device__ __forceinline__ void add_and_store(const DecOut& o, const float4* sums, int max_tiles, int ntiles, int tile0,
-                                              const float* __restrict__ rinv) {
+                                              const float* rinv) {
     for (int e = threadIdx.x; e < ntiles * NT * 32; e += kDpThreads) {
         const int ti = e / (NT * 32), ln = e & 31, nt = (e >> 5) % NT;
         const float4* src = sums + (size_t)(ti * NT + nt) * 32 + ln;
@@ -194,7 +194,7 @@ __device__ __forceinline__ void add_and_store(const DecOut& o, const float4* sum
         for (int h = 0; h < 2; ++h) {
             const int j = j0 + 8 * h;
             if (j >= o.d_out) continue;
-            const float scale = rinv != nullptr ? __ldg(rinv + j) : 1.0f, bias = o.bias != nullptr ? __ldg(o.bias + j) : 0.0f;
+            const float scale = rinv != nullptr ? ld(rinv + j) : 1.0f, bias = o.bias != nullptr ? ld(o.bias + j) : 0.0f;
             const float v[2] = {(h ? s.z : s.x) * scale + bias, (h ? s.w : s.y) * scale + bias};
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
@@ -339,17 +339,17 @@ decode_packed_kernel(const DecPackedParams p) {
             --l_left;
 #pragma unroll
             for (int v = 0; v < Q / 2; ++v) {
-                const uint4 x = ptx::ldg_nc_v4(lp_codes + v * 512);
+                const uint4 x = ld_stream(reinterpret_cast<const uint4*>(lp_codes + v * 512));
                 u.c[4 * v] = x.x; u.c[4 * v + 1] = x.y; u.c[4 * v + 2] = x.z; u.c[4 * v + 3] = x.w;
             }
             if (Q & 1) {
-                const uint2 x = ptx::ldg_nc_v2(lp_codes + (Q / 2) * 512 - lane * 8);
+                const uint2 x = ld_stream(reinterpret_cast<const uint2*>(lp_codes + (Q / 2) * 512 - lane * 8));
                 u.c[2 * Q - 2] = x.x; u.c[2 * Q - 1] = x.y;
             }
 #pragma unroll
             for (int a = 0; a < PARTS; ++a) {
-                u.ta[a] = ptx::ldg_nc_v4(lp_tables[a]);
-                u.tb[a] = ptx::ldg_nc_v4(lp_tables[a] + 128);
+                u.ta[a] = ld_stream(reinterpret_cast<const uint4*>(lp_tables[a]));
+                u.tb[a] = ld_stream(reinterpret_cast<const uint4*>(lp_tables[a] + 128));
             }
             if (++l_i == round_n) {
                 l_i = 0;
@@ -391,7 +391,7 @@ decode_packed_kernel(const DecPackedParams p) {
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
                     xb[nt][r] = make_uint4(0u, 0u, 0u, 0u);
-                    if (tok < p.n && kb + r * 32 < p.d_in) xb[nt][r] = __ldg(reinterpret_cast<const uint4*>(src + r * 32));
+                    if (tok < p.n && kb + r * 32 < p.d_in) xb[nt][r] = ld(reinterpret_cast<const uint4*>(src + r * 32));
                 }
                 const float inv = scale_fragment(xb[nt], kb, 32, p.d_in, st * kDpStepK + kDpStepK > p.d_in);
                 f0[nt] = __shfl_sync(0xffffffffu, inv, 8 * tq);
@@ -575,10 +575,10 @@ decode_planes_kernel(const DecPlanesParams p) {
 #pragma unroll
             for (int i = 0; i < NQ; ++i) {
                 const bool va = i < p.q && ja < p.d_out, vb = i < p.q && jb < p.d_out;
-                u.wa[i] = va ? __ldg(pb + i * plane_bits) : 0u;
-                u.wb[i] = vb ? __ldg(pb + i * plane_bits + 8 * (size_t)p.pitch) : 0u;
-                u.aa[i] = va ? __ldg(pa + i * plane_alpha) : 0.0f;
-                u.ab[i] = vb ? __ldg(pa + i * plane_alpha + 8 * (size_t)p.G) : 0.0f;
+                u.wa[i] = va ? ld(pb + i * plane_bits) : 0u;
+                u.wb[i] = vb ? ld(pb + i * plane_bits + 8 * (size_t)p.pitch) : 0u;
+                u.aa[i] = va ? ld(pa + i * plane_alpha) : 0.0f;
+                u.ab[i] = vb ? ld(pa + i * plane_alpha + 8 * (size_t)p.G) : 0.0f;
             }
             if (++l_i == round_n) {
                 l_i = 0;
@@ -611,7 +611,7 @@ decode_planes_kernel(const DecPlanesParams p) {
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
                     v[r] = make_uint4(0u, 0u, 0u, 0u);
-                    if (tok < p.n && kb + r * 8 < p.d_in) v[r] = __ldg(reinterpret_cast<const uint4*>(src + r * 8));
+                    if (tok < p.n && kb + r * 8 < p.d_in) v[r] = ld(reinterpret_cast<const uint4*>(src + r * 8));
                 }
                 const float inv = scale_fragment(v, kb, 8, p.d_in, st * kDpStepK + kDpStepK > p.d_in);
                 const uint32_t P[16] = {v[0].x, v[0].y, v[0].z, v[0].w, v[1].x, v[1].y, v[1].z, v[1].w,

@@ -90,9 +90,9 @@ struct WsHeader {
 
 // Power of two for the weights: q * max|alpha| lands in [2^13, 2^14).  Called by whole warps.
 __device__ __forceinline__ int weight_shift(const WsHeader* hdr, int q) {
-    const int nb = (int)min(__ldg(&hdr->nblocks), (uint32_t)kMaxAlphaBlocks);  // never past the header
+    const int nb = (int)min(ld(&hdr->nblocks), (uint32_t)kMaxAlphaBlocks);  // never past the header
     uint32_t m = 0u;
-    for (int b = threadIdx.x & 31; b < nb; b += 32) m = max(m, __ldg(&hdr->block_max[b]));
+    for (int b = threadIdx.x & 31; b < nb; b += 32) m = max(m, ld(&hdr->block_max[b]));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     return shift_for(exponent_of_bits(__float_as_uint(__uint_as_float(m) * (float)q)), 13);
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
             const int rows_left = p.d_out - rt * 128;
             for (int e = threadIdx.x; e < count; e += 256) {
                 const int r = e / p.G, c = e - r * p.G;
-                const float v = (r < rows_left) ? __ldg(src + e) : 0.0f;
+                const float v = (r < rows_left) ? ld(src + e) : 0.0f;
                 long long o;
                 if (p.mode == MODE_FWD) {
                     o = (((long long)rt * p.G + c) * p.q + i) * 128 + r;
@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
 #pragma unroll
         for (int pass = 0; pass < 16; ++pass) {
             const int j = rt * 128 + pass * 8 + warp;
-            held[pass] = (j < p.d_out && col_l < ncols) ? __ldg(src + (long long)j * ncols + col_l) : 0u;
+            held[pass] = (j < p.d_out && col_l < ncols) ? ld(src + (long long)j * ncols + col_l) : 0u;
         }
 #pragma unroll
         for (int pass = 0; pass < 16; ++pass) {
@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
         uint32_t m = 0u;
         for (long long o = ((long long)bid - p.act_blocks) * 256 + threadIdx.x; o < p.alpha_count;
              o += nb * 256)
-            m = max(m, __float_as_uint(__ldg(p.alpha + o)) & 0x7FFFFFFFu);
+            m = max(m, __float_as_uint(ld(p.alpha + o)) & 0x7FFFFFFFu);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
         if (lane == 0) red[warp] = m;
@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int v = v0 + kThreadsPerToken * i;
-            held[i] = (v < nvec) ? __ldg(src + v) : make_uint4(0u, 0u, 0u, 0u);
+            held[i] = (v < nvec) ? ld(src + v) : make_uint4(0u, 0u, 0u, 0u);
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) m = max(m, max_mag_bf16x8(held[i], (v0 + kThreadsPerToken * i) * 8, p.K));
@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int v = v0 + kThreadsPerToken * i;
-                held[i] = (v < nvec) ? __ldg(src + v) : make_uint4(0u, 0u, 0u, 0u);
+                held[i] = (v < nvec) ? ld(src + v) : make_uint4(0u, 0u, 0u, 0u);
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -357,8 +357,8 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
 // meet zero activations).
 template <int NW>
 __global__ void __launch_bounds__(256) code_planes_kernel(int mode, int d_out, int pitch, int q, int rows_padded,
-                                                           int words_padded, int num_kb, const uint32_t* __restrict__ bits,
-                                                           uint32_t* __restrict__ codes) {
+                                                           int words_padded, int num_kb, const uint32_t* bits,
+                                                           uint32_t* codes) {
     pdl_trigger();
     pdl_wait();
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(256) code_planes_kernel(int mode, int d_out, i
     uint32_t w[4] = {0u, 0u, 0u, 0u};
     const bool valid = (j < d_out) && (wd < pitch);
     for (int i = 0; i < q; ++i)
-        if (valid) w[i] = __ldg(bits + ((long long)i * d_out + j) * pitch + wd);
+        if (valid) w[i] = ld(bits + ((long long)i * d_out + j) * pitch + wd);
     uint32_t S[4];
     selectors_from_planes(w, q, S);
     if (!valid)
@@ -887,19 +887,19 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
 #pragma unroll
                 for (int i = 0; i < NL; ++i) {
                     if (i < p.q) {
-                        const uint2 v = ptx::ldg_nc_v2(src + i * (kRows * kUnit));
+                        const uint2 v = ld_stream(reinterpret_cast<const uint2*>(src + i * (kRows * kUnit)));
                         cv[0][i] = v.x; cv[1][i] = v.y;
                     } else {
                         cv[0][i] = 0u; cv[1][i] = 0u;
                     }
                 }
             } else if (NWC == 4) {
-                const uint4 v0 = ptx::ldg_nc_v4(src), v1 = ptx::ldg_nc_v4(src + 4);
+                const uint4 v0 = ld_stream(reinterpret_cast<const uint4*>(src)), v1 = ld_stream(reinterpret_cast<const uint4*>(src + 4));
                 cv[0][0] = v0.x; cv[0][1] = v0.y; cv[0][2] = v0.z; cv[0][NL - 1] = v0.w;
                 cv[1][0] = v1.x; cv[1][1] = v1.y; cv[1][2] = v1.z; cv[1][NL - 1] = v1.w;
             } else {
                 // six words, 8-byte aligned
-                const uint2 v0 = ptx::ldg_nc_v2(src), v1 = ptx::ldg_nc_v2(src + 2), v2 = ptx::ldg_nc_v2(src + 4);
+                const uint2 v0 = ld_stream(reinterpret_cast<const uint2*>(src)), v1 = ld_stream(reinterpret_cast<const uint2*>(src + 2)), v2 = ld_stream(reinterpret_cast<const uint2*>(src + 4));
                 cv[0][0] = v0.x; cv[0][1] = v0.y; cv[0][2] = v1.x;
                 cv[1][0] = v1.y; cv[1][1] = v2.x; cv[1][2] = v2.y;
             }
@@ -907,7 +907,7 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
                 const float* ap = p.alpha_t + x.alpha_idx;
 #pragma unroll
                 for (int i = 0; i < NSC; ++i)
-                    av[i] = (i < p.q) ? __uint_as_float(ptx::ldg_nc_u32(ap + i * kRows)) : 0.0f;
+                    av[i] = (i < p.q) ? ld_stream(ap + i * kRows) : 0.0f;
             }
         };
 
@@ -928,7 +928,7 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
                 const float* ap = p.alpha_t + x.alpha_idx + alpha_block;  // group c + 1
 #pragma unroll
                 for (int i = 0; i < NSC; ++i)
-                    a2[i] = (i < p.q) ? __uint_as_float(ptx::ldg_nc_u32(ap + i * kRows)) : 0.0f;
+                    a2[i] = (i < p.q) ? ld_stream(ap + i * kRows) : 0.0f;
             }
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
@@ -1026,8 +1026,8 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
                 const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)acc * kAccCols;
                 const uint32_t buf = smem_base + (uint32_t)warp * 1024u;
                 const float winv = 1.0f / wscale;  // a power of two
-                auto scale_of = [&](int t) { return (t < p.n) ? winv * __ldg(p.tok_inv_scale + t) : 0.0f; };
-                auto bias_of = [&](int m) { return (MODE == MODE_FWD && p.bias != nullptr && m < p.Mdim) ? __ldg(p.bias + m) : 0.0f; };
+                auto scale_of = [&](int t) { return (t < p.n) ? winv * ld(p.tok_inv_scale + t) : 0.0f; };
+                auto bias_of = [&](int m) { return (MODE == MODE_FWD && p.bias != nullptr && m < p.Mdim) ? ld(p.bias + m) : 0.0f; };
                 if (p.fast_epi) {
                     const int g = lane >> 2, tq = lane & 3;
                     float b4[4];
@@ -1069,7 +1069,7 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
             const int acc = lt & 1;
             const uint32_t acc_ph = (lt >> 1) & 1;
             for (int i = et; i < TN; i += kPfEpiWarps * 32)
-                scale[i] = (t0 + i < p.n) ? winv * __ldg(p.tok_inv_scale + t0 + i) : 0.0f;
+                scale[i] = (t0 + i < p.n) ? winv * ld(p.tok_inv_scale + t0 + i) : 0.0f;
             // one warp polls the accumulator's barrier (a whole tile away), the others park on the
             // hardware barrier that also publishes the scale row; a timeout shows in the abort flag
             if (ew == 0) wait_bar(ctl.accum + 8 * acc, acc_ph, ctl, 7, 1000u);
@@ -1078,7 +1078,7 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
             ptx::tc_fence_after_sync();
             const int m0w = m0 + quarter * 32;
             const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)acc * kAccCols;
-            auto bias_of = [&](int m) { return (MODE == MODE_FWD && p.bias != nullptr && m < p.Mdim) ? __ldg(p.bias + m) : 0.0f; };
+            auto bias_of = [&](int m) { return (MODE == MODE_FWD && p.bias != nullptr && m < p.Mdim) ? ld(p.bias + m) : 0.0f; };
             const int step = (p.helpers && lt == nseg - 1) ? kPfHelpers : 1;  // the workers take the other boxes
             if (p.fast_epi) {
                 const int g = lane >> 2, tq = lane & 3;

@@ -21,11 +21,11 @@ struct Segments {
 };
 
 // Segment that holds compact index e (prefix[s] <= e < prefix[s + 1]).
-__device__ __forceinline__ int find_segment(const long long* __restrict__ prefix, int nseg, long long e) {
+__device__ __forceinline__ int find_segment(const long long* prefix, int nseg, long long e) {
     int lo = 0, hi = nseg - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(prefix + mid) <= e) lo = mid; else hi = mid - 1;
+        if (bcq::ld(prefix + mid) <= e) lo = mid; else hi = mid - 1;
     }
     return lo;
 }
@@ -40,8 +40,8 @@ struct AdamParams {
 };
 
 __global__ void __launch_bounds__(256)
-alpha_adamw_kernel(long long count, Segments sg, AdamParams h, float* __restrict__ alpha,
-                   const float* __restrict__ grad, float* __restrict__ m, float* __restrict__ v) {
+alpha_adamw_kernel(long long count, Segments sg, AdamParams h, float* alpha,
+                   const float* grad, float* m, float* v) {
     bcq::pdl_trigger();
     bcq::pdl_wait();
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -50,8 +50,8 @@ alpha_adamw_kernel(long long count, Segments sg, AdamParams h, float* __restrict
         float gs = h.grad_scale;
         if (sg.nseg > 0) {
             const int s = find_segment(sg.prefix, sg.nseg, e);
-            idx = __ldg(sg.begin + s) + (e - __ldg(sg.prefix + s));
-            if (sg.scale != nullptr) gs *= __ldg(sg.scale + s);
+            idx = bcq::ld(sg.begin + s) + (e - bcq::ld(sg.prefix + s));
+            if (sg.scale != nullptr) gs *= bcq::ld(sg.scale + s);
         }
         const float g = gs * grad[idx];
         const float mm = h.beta1 * m[idx] + h.om_beta1 * g;
@@ -65,14 +65,14 @@ alpha_adamw_kernel(long long count, Segments sg, AdamParams h, float* __restrict
 
 // to_compact != 0: compact[e] = flat[...]; else flat[...] = compact[e].
 __global__ void __launch_bounds__(256)
-alpha_gather_kernel(long long count, Segments sg, int to_compact, float* __restrict__ flat,
-                    float* __restrict__ compact) {
+alpha_gather_kernel(long long count, Segments sg, int to_compact, float* flat,
+                    float* compact) {
     bcq::pdl_trigger();
     bcq::pdl_wait();
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += stride) {
         const int s = find_segment(sg.prefix, sg.nseg, e);
-        const long long idx = __ldg(sg.begin + s) + (e - __ldg(sg.prefix + s));
+        const long long idx = bcq::ld(sg.begin + s) + (e - bcq::ld(sg.prefix + s));
         if (to_compact) compact[e] = flat[idx]; else flat[idx] = compact[e];
     }
 }

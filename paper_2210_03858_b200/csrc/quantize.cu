@@ -192,7 +192,7 @@ quantize_kernel(const QuantParams p) {
 #pragma unroll
         for (int e = 0; e < EPT; ++e) {
             const int kl = e * NT + tid;
-            const float v = (kl < m) ? __ldg(wrow + kl) : 0.0f;
+            const float v = (kl < m) ? bcq::ld(wrow + kl) : 0.0f;
             r[e] = (double)v;
             w[e] = v;
             code[e] = 0u;
@@ -493,7 +493,7 @@ team_quantize_kernel(const QuantParams p) {
     if (m == EPT * NT && p.vec) {
 #pragma unroll
         for (int i = 0; i < NI; ++i) {
-            const float4 v = __ldg(reinterpret_cast<const float4*>(src + 16 * i));
+            const float4 v = bcq::ld(reinterpret_cast<const float4*>(src + 16 * i));
             w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
         }
     } else {
@@ -502,11 +502,11 @@ team_quantize_kernel(const QuantParams p) {
         for (int i = 0; i < NI; ++i) {
             const int left = m - (kt + 16 * i);
             if (p.vec && left >= 4) {
-                const float4 v = __ldg(reinterpret_cast<const float4*>(src + 16 * i));
+                const float4 v = bcq::ld(reinterpret_cast<const float4*>(src + 16 * i));
                 w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
             } else {
 #pragma unroll
-                for (int e = 0; e < 4; ++e) w[4 * i + e] = (e < left) ? __ldg(src + 16 * i + e) : 0.0f;
+                for (int e = 0; e < 4; ++e) w[4 * i + e] = (e < left) ? bcq::ld(src + 16 * i + e) : 0.0f;
             }
             valid |= (left >= 4 ? 0xFu : left > 0 ? (1u << left) - 1u : 0u) << (4 * i);
         }
@@ -809,8 +809,8 @@ cudaError_t launch_quantize(const QuantParams& p, cudaStream_t stream) {
 }
 
 __global__ void dequantize_kernel(int d_out, int d_in, int q, int g, int G, int pitch,
-                                  const uint32_t* __restrict__ bits,
-                                  const float* __restrict__ alpha, float* __restrict__ W_hat,
+                                  const uint32_t* bits,
+                                  const float* alpha, float* W_hat,
                                   long long ldw) {
     const int j = blockIdx.y;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -818,8 +818,8 @@ __global__ void dequantize_kernel(int d_out, int d_in, int q, int g, int G, int 
     const int c = k / g;
     float s = 0.0f;
     for (int i = 0; i < q; ++i) {
-        const uint32_t word = __ldg(bits + ((long long)i * d_out + j) * pitch + (k >> 5));
-        const float a = __ldg(alpha + ((long long)i * d_out + j) * G + c);
+        const uint32_t word = bcq::ld(bits + ((long long)i * d_out + j) * pitch + (k >> 5));
+        const float a = bcq::ld(alpha + ((long long)i * d_out + j) * G + c);
         s += ((word >> (k & 31)) & 1u) ? a : -a;
     }
     W_hat[(long long)j * ldw + k] = s;
