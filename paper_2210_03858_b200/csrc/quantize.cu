@@ -451,11 +451,80 @@ struct LevelSearch {
     }
 };
 
+// Groups with an infinite or NaN weight.  The team kernel keeps residuals as magnitudes and signs, and the sign of a
+// NaN says nothing: r >= 0 is false for it.  The first scale a1 of such a group is infinite or NaN, so the
+// residuals of the second plane are w -+ a1 and everything after it is NaN.
+__device__ __forceinline__ bool greedy_sign_not_finite(float w, float a1, int plane) {
+    if (plane == 0) return w >= 0.f;
+    return plane == 1 && (w >= 0.f ? (double)w - (double)a1 : (double)w + (double)a1) >= 0.0;
+}
+
+// Container word `wi` of such a group in the greedy planes.
+__device__ __noinline__ void greedy_word_not_finite(const QuantParams p, long long item, int wi, float a1) {
+    const int j = (int)(item / p.G), k0 = (int)(item % p.G) * p.g + 32 * wi, m = min(min(p.g - 32 * wi, p.d_in - k0), 32);
+    if (m <= 0) return;
+    const float* w = p.W + (long long)j * p.ldw + k0;
+#pragma unroll 1
+    for (int i = 0; i < p.q; ++i) {
+        uint32_t word = 0u;
+#pragma unroll 1
+        for (int e = 0; e < m; ++e)
+            if (greedy_sign_not_finite(bcq::ld(w + e), a1, i)) word |= 1u << e;
+        p.bits[((long long)i * p.d_out + j) * p.pitch + (k0 >> 5)] = word;
+    }
+}
+
+// The scales (and the squared error) of such a group after alternating rounds, by the definition.  The right-hand
+// sides of a fit are not finite, so no level is nearer than another: after the first round every weight
+// has the largest code, and for q > 1 the fit is singular from then on.
+__device__ __noinline__ void fit_not_finite(const QuantParams p, long long item, float a1) {
+    const int j = (int)(item / p.G), k0 = (int)(item % p.G) * p.g, m = min(p.g, p.d_in - k0), q = p.q;
+    const float* w = p.W + (long long)j * p.ldw + k0;
+    double A[BCQ_MAX_Q][BCQ_MAX_Q + 1], plain = 0.0;
+    float a[BCQ_MAX_Q];
+    a[0] = a1;
+#pragma unroll 1
+    for (int i = 1; i < q; ++i) a[i] = __int_as_float(0x7FFFFFFF);
+#pragma unroll 1
+    for (int i = 0; i < q; ++i) {
+        A[i][q] = 0.0;
+#pragma unroll 1
+        for (int l = 0; l < q; ++l) A[i][l] = (double)m;
+    }
+#pragma unroll 1
+    for (int k = 0; k < m; ++k) {
+        const float x = bcq::ld(w + k);
+        plain += (double)x;
+#pragma unroll 1
+        for (int i = 0; i < q; ++i) {
+            const bool pos = greedy_sign_not_finite(x, a1, i);
+            A[i][q] += pos ? (double)x : -(double)x;
+#pragma unroll 1
+            for (int l = 0; l < q; ++l) A[i][l] -= pos != greedy_sign_not_finite(x, a1, l) ? 2.0 : 0.0;
+        }
+    }
+    solve_ls(q, (double)m, A, a);
+    if (q == 1) a[0] = (float)__ddiv_rn(plain, (double)m);
+#pragma unroll 1
+    for (int i = 0; i < q; ++i) p.alpha[i * p.items + item] = a[i];
+    if (p.sq_err != nullptr) {
+        double E = 0.0, wh = 0.0;
+#pragma unroll 1
+        for (int i = 0; i < q; ++i) wh += (double)a[i];
+#pragma unroll 1
+        for (int k = 0; k < m; ++k) {
+            const double d = (double)bcq::ld(w + k) - wh;
+            E += d * d;
+        }
+        p.sq_err[item] = E;
+    }
+}
+
 // Q = 0: greedy, p.q planes; Q > 0: alternating with Q planes.  A thread holds 4 NI weights, a team is L
 // lanes (TW = 1) or TW warps.
 template <int NI, int L, int TW, int Q>
 __global__ void __launch_bounds__(TW == 1 ? 128 : TW * 32,
-                                  TW == 1 ? (Q == 0 || NI == 4 ? 5 : NI == 2 ? 6 : 3) : TW <= 4 ? (NI == 4 ? 20 : 12) / TW : 1)
+                                  TW == 1 ? (NI == 2 || (Q == 0 && NI == 4) ? 6 : Q == 0 || NI == 4 ? 5 : 3) : TW <= 4 ? (NI == 4 ? 20 : 12) / TW : 1)
 team_quantize_kernel(const QuantParams p) {
     constexpr bool ALT = Q > 0;
     constexpr int EPT = 4 * NI;
@@ -586,9 +655,11 @@ team_quantize_kernel(const QuantParams p) {
                 if (t[e] == 0.0 && ((valid >> e) & 1u)) negs &= ~(1u << e);
         }
     };
+    float a1 = 0.f;  // first scale: not finite if a weight of the group is not
     if constexpr (!ALT) {
         for (int i = 0; i < q; ++i) {
             const float ai = scale_of();
+            if (i == 0) a1 = ai;
             const uint32_t word = transpose_bits(~negs);
             if (writes) dst[i * plane_words] = word & word_mask;
             if (live && tl == 0) adst[i * plane_alpha] = ai;
@@ -601,6 +672,7 @@ team_quantize_kernel(const QuantParams p) {
             neg[i] = negs;
             if (i + 1 < Q) next_residual(a[i]);
         }
+        a1 = a[0];
 
         // ---- alternating rounds.  From here on only magnitudes count: b_i w = (b_i sign(w)) |w|, so the
         // sums run over |w| with the signs `neg` relative to sign(w), and so do the mismatch counts.
@@ -750,6 +822,15 @@ team_quantize_kernel(const QuantParams p) {
         for (int e = 0; e < EPT; ++e) local += t[e] * t[e];
         const double E = lanes_sum<L, TW>(local, scratch);
         if (live && tl == 0) p.sq_err[(long long)j * p.G + c] = E;
+    }
+    if (!(fabsf(a1) <= 3.402823466e38f)) {
+        // rare: everything is formed again, so that nothing of it is kept for the sake of these calls
+        uint32_t block;
+        asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(block));
+        const long long again = (long long)block * TEAMS + (TW == 1 ? threadIdx.x / L : 0);
+        const int t = TW == 1 ? (int)(threadIdx.x & (L - 1)) : (int)threadIdx.x;
+        if (!ALT && again < p.items && (t & 3) < NI / 2) greedy_word_not_finite(p, again, (t >> 2) * (NI / 2) + (t & 3), a1);
+        if (ALT && again < p.items && t == 0) fit_not_finite(p, again, a1);
     }
 }
 

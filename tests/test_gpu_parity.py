@@ -154,6 +154,23 @@ def test_quantize_alternating_short_and_long_problems(d_in, g):
             np.testing.assert_allclose(sq.cpu().numpy(), np.tile(sq_ref, (r, 1)), rtol=1e-6, atol=1e-12)
 
 
+@pytest.mark.parametrize("alt", [0, 2])
+@pytest.mark.parametrize("d_in,g", [(64, 32), (130, 64), (420, 128), (1000, 1000), (3000, 3000)])
+def test_quantize_weights_that_are_not_finite(d_in, g, alt):
+    # r >= 0 is false for a NaN whatever its sign bit, and a group with an infinity has NaN residuals from its
+    # second plane on: the bits of such groups (and of their neighbours) are the oracle's all the same
+    rng = np.random.default_rng(d_in)
+    W = (rng.integers(-6, 7, size=(7, d_in)) / 64.0).astype(np.float32)
+    W[0, 3], W[1, 5], W[2, 7], W[3, d_in - 1] = np.nan, np.inf, -np.inf, np.float32(-np.nan)
+    W[4, 9], W[4, 11], W[5, :] = np.inf, -np.inf, np.nan
+    for q in (1, 2, 3, 4):
+        bits_ref, alpha_ref, sq_ref, _ = oracle.quantize(W, q, g, alt_iters=alt)
+        bits, alpha, sq = bcq.quantize(torch.from_numpy(W).cuda(), q, g, alt, want_sq_err=True)
+        np.testing.assert_array_equal(host_bits(bits), bits_ref)
+        np.testing.assert_allclose(alpha.cpu().numpy(), alpha_ref, rtol=1e-6, atol=1e-9, equal_nan=True)
+        np.testing.assert_allclose(sq.cpu().numpy(), sq_ref, rtol=1e-6, atol=1e-12, equal_nan=True)
+
+
 def test_quantize_strided_input_and_determinism():
     W = synth.weights(48, 384, (101, 0, 0))
     Wp = np.zeros((48, 400), dtype=np.float32)
