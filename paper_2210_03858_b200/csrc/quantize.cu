@@ -308,12 +308,22 @@ quantize_kernel(const QuantParams p) {
 // the team kernel
 // ------------------------------------------------------------------------------------------
 
-// Sum over a team of L lanes (TW = 1) or TW warps.
-template <int L, int TW>
-__device__ __forceinline__ double lanes_sum(double v, double* scratch) {
-#pragma unroll
-    for (int o = L / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (TW == 1) return v;
+// A sum over a group is a tree whose shape depends on the group size alone, so a row gets the same scales whichever
+// team takes it, and hence whatever else is in the call.  Where a group may be taken by teams of different
+// size (alternating, up to 2048 weights) its leaves are two neighbouring 16-byte pieces of one lane of a
+// quad, 8 weights.  Over them, neighbours first: the leaves of a lane (tree_of_leaves), the quads of a
+// warp, the warps; the four lanes of a quad come last.
+template <int N>
+__device__ __forceinline__ double tree_of_leaves(const double (&p)[N]) {
+    static_assert(N == 1 || N == 2 || N == 4, "leaves of a thread");
+    if constexpr (N == 1) return p[0];
+    else if constexpr (N == 2) return p[0] + p[1];
+    else return (p[0] + p[1]) + (p[2] + p[3]);
+}
+
+// A value of each warp, uniform in the warp: added over the CTA, in order.
+template <int TW>
+__device__ __forceinline__ double warps_sum(double v, double* scratch) {
     __syncthreads();
     if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = v;
     __syncthreads();
@@ -321,6 +331,30 @@ __device__ __forceinline__ double lanes_sum(double v, double* scratch) {
 #pragma unroll 1
     for (int w = 0; w < TW; ++w) t += scratch[w];
     return t;
+}
+
+// Sum over a team of L lanes (TW = 1) or TW warps of the lanes' leaves.
+template <int L, int TW>
+__device__ __forceinline__ double lanes_sum(double v, double* scratch) {
+#pragma unroll
+    for (int o = 4; o < L; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if constexpr (TW == 2 || TW == 4) {
+        __syncthreads();
+        if ((threadIdx.x & 31) < 4) scratch[(threadIdx.x >> 5) * 4 + (threadIdx.x & 3)] = v;
+        __syncthreads();
+        double t[4];
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {
+            t[l] = scratch[l] + scratch[4 + l];
+            if (TW == 4) t[l] += scratch[8 + l] + scratch[12 + l];
+        }
+        return (t[0] + t[1]) + (t[2] + t[3]);
+    } else {
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        v += __shfl_xor_sync(0xffffffffu, v, 2);
+        if constexpr (TW == 1) return v;
+        else return warps_sum<TW>(v, scratch);
+    }
 }
 
 // Four lanes hold the bits of 128 consecutive weights: bit 4 i + e of a lane's word is weight
@@ -529,6 +563,8 @@ team_quantize_kernel(const QuantParams p) {
     constexpr bool ALT = Q > 0;
     constexpr int EPT = 4 * NI;
     constexpr int NT = L * TW;                       // threads of a team
+    constexpr int LEAVES = !ALT || (NI == 8 && TW >= 4) ? 1 : NI / 2;  // see lanes_sum
+    constexpr int LEAF = EPT / LEAVES;
     constexpr int TEAMS = TW == 1 ? 128 / L : 1;     // per CTA
     __shared__ double scratch[TW == 1 ? 1 : 32];
     bcq::pdl_trigger();
@@ -608,15 +644,20 @@ team_quantize_kernel(const QuantParams p) {
     float* adst = p.alpha + (long long)j * p.G + c;
     // scale of the next plane; `negs` are its signs
     auto scale_of = [&]() {
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+        double leaf[LEAVES];
 #pragma unroll
-        for (int e = 0; e < EPT; e += 4) {
-            s0 += fabs(t[e]);
-            s1 += fabs(t[e + 1]);
-            s2 += fabs(t[e + 2]);
-            s3 += fabs(t[e + 3]);
+        for (int k = 0; k < LEAVES; ++k) {
+            double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+#pragma unroll
+            for (int e = k * LEAF; e < (k + 1) * LEAF; e += 4) {
+                s0 += fabs(t[e]);
+                s1 += fabs(t[e + 1]);
+                s2 += fabs(t[e + 2]);
+                s3 += fabs(t[e + 3]);
+            }
+            leaf[k] = (s0 + s1) + (s2 + s3);
         }
-        const double S = lanes_sum<L, TW>((s0 + s1) + (s2 + s3), scratch);
+        const double S = lanes_sum<L, TW>(tree_of_leaves(leaf), scratch);
         // a power-of-two group size divides exactly by multiplying with its reciprocal
         return (float)(inv_m != 0.0 ? __dmul_rn(S, inv_m) : __ddiv_rn(S, md));
     };
@@ -689,21 +730,35 @@ team_quantize_kernel(const QuantParams p) {
         zero &= valid;
 #pragma unroll
         for (int o = L / 2; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-        if (TW > 1) amax = (float)lanes_sum<1, TW>((double)amax, scratch);  // a bound: the sum over the warps
+        if constexpr (TW > 1) amax = (float)warps_sum<TW>((double)amax, scratch);  // a bound: the sum over the warps
 #pragma unroll
         for (int i = 0; i < Q; ++i) neg[i] ^= sgn;
 
-        double S[Q];
+        double S[Q];  // this thread's part of B^T w; a leaf is added from its last weight to its first
+        double leaf[Q], odd[Q], upper[Q];
+        auto end_leaf = [&](int k) {  // leaves come from the last to the first
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                if (LEAVES == 1) S[i] = leaf[i];
+                else if (k & 1) odd[i] = leaf[i];
+                else if (LEAVES == 4 && k == 2) upper[i] = leaf[i] + odd[i];
+                else S[i] = LEAVES == 4 ? (leaf[i] + odd[i]) + upper[i] : leaf[i] + odd[i];
+            }
+        };
         auto sums_from_signs = [&]() {
 #pragma unroll
-            for (int i = 0; i < Q; ++i) S[i] = 0.0;
+            for (int k = LEAVES - 1; k >= 0; --k) {
 #pragma unroll
-            for (int e = 0; e < EPT; ++e) {
-                const double x = (double)w[e];
-                const int hi = __double2hiint(x), lo = __double2loint(x);
+                for (int i = 0; i < Q; ++i) leaf[i] = 0.0;
 #pragma unroll
-                for (int i = 0; i < Q; ++i)
-                    S[i] += __hiloint2double(hi ^ (int)((neg[i] << (31 - e)) & 0x80000000u), lo);
+                for (int e = (k + 1) * LEAF - 1; e >= k * LEAF; --e) {
+                    const double x = (double)w[e];
+                    const int hi = __double2hiint(x), lo = __double2loint(x);
+#pragma unroll
+                    for (int i = 0; i < Q; ++i)
+                        leaf[i] += __hiloint2double(hi ^ (int)((neg[i] << (31 - e)) & 0x80000000u), lo);
+                }
+                end_leaf(k);
             }
         };
         sums_from_signs();
@@ -739,7 +794,7 @@ team_quantize_kernel(const QuantParams p) {
 #pragma unroll
                     for (int l = i + 1; l < Q; ++l, ++n) {
                         double mism = (double)((cnt[n / 2] >> (16 * (n & 1))) & 0xFFFFu);
-                        if (TW > 1) mism = lanes_sum<1, TW>(mism, scratch);
+                        if constexpr (TW > 1) mism = warps_sum<TW>(mism, scratch);
                         A[i][l] = md - 2.0 * mism;
                         A[l][i] = A[i][l];
                     }
@@ -755,21 +810,24 @@ team_quantize_kernel(const QuantParams p) {
             flip0 = (ls.codes >> (Q - 1)) & 1u;
             float near = tiny;
 #pragma unroll
-            for (int i = 0; i < Q; ++i) {
-                S[i] = 0.0;
-                neg[i] = 0u;
-            }
+            for (int i = 0; i < Q; ++i) neg[i] = 0u;
 #pragma unroll
-            for (int e = EPT - 1; e >= 0; --e) {
-                const uint32_t y = ls.find(w[e], near);
-                const double x = (double)w[e];
-                const int hi = __double2hiint(x), lo = __double2loint(x);
+            for (int k = LEAVES - 1; k >= 0; --k) {
 #pragma unroll
-                for (int i = 0; i < Q; ++i) {
-                    const uint32_t b = y << (31 - i);
-                    neg[i] = __funnelshift_l(b, neg[i], 1);
-                    S[i] += __hiloint2double(hi ^ (int)(b & 0x80000000u), lo);
+                for (int i = 0; i < Q; ++i) leaf[i] = 0.0;
+#pragma unroll
+                for (int e = (k + 1) * LEAF - 1; e >= k * LEAF; --e) {
+                    const uint32_t y = ls.find(w[e], near);
+                    const double x = (double)w[e];
+                    const int hi = __double2hiint(x), lo = __double2loint(x);
+#pragma unroll
+                    for (int i = 0; i < Q; ++i) {
+                        const uint32_t b = y << (31 - i);
+                        neg[i] = __funnelshift_l(b, neg[i], 1);
+                        leaf[i] += __hiloint2double(hi ^ (int)(b & 0x80000000u), lo);
+                    }
                 }
+                end_leaf(k);
             }
             if (!(near > ls.delta)) {
                 // some weight of this thread is too close to call in fp32
@@ -817,10 +875,14 @@ team_quantize_kernel(const QuantParams p) {
         }
     }
     if (p.sq_err != nullptr) {
-        double local = 0.0;
+        double leaf[LEAVES];
 #pragma unroll
-        for (int e = 0; e < EPT; ++e) local += t[e] * t[e];
-        const double E = lanes_sum<L, TW>(local, scratch);
+        for (int k = 0; k < LEAVES; ++k) {
+            leaf[k] = 0.0;
+#pragma unroll
+            for (int e = k * LEAF; e < (k + 1) * LEAF; ++e) leaf[k] += t[e] * t[e];
+        }
+        const double E = lanes_sum<L, TW>(tree_of_leaves(leaf), scratch);
         if (live && tl == 0) p.sq_err[(long long)j * p.G + c] = E;
     }
     if (!(fabsf(a1) <= 3.402823466e38f)) {
@@ -850,6 +912,8 @@ cudaError_t launch_team(const QuantParams& p, cudaStream_t stream) {
 //   g = 128, q = 4   512 x 512 56 / 37 / 28 us   2048 x 1536 209 / 138 / 118   3000 x 4096 401 / 333 / 401
 //                    5120 x 5120 711 / 653 / 851
 //   g = 128, q = 3   512 x 512 31 / 20 / 21 us   1406 x 1582 93 / 55 / 58   5120 x 5120 357 / 345 / 468
+//   g = 128, 1600 x 1600, 16 / 8 a thread: q = 1 18.6 / 15.5 us, q = 2 37.9 / 33.4, q = 3 72.7 / 63.8;
+//                    64 x 512, q = 3 13.0 / 10.1 (so for every q, though two problems of q = 3 above lose 5 %)
 //   g = 256, q = 3   1406 x 1582 106 / 57 us     5120 x 5120 355 / 346
 //   a row, q = 3     1024 x 1024 80 / 53 us      2048 x 1536 128 / 98       3000 x 4096 231 / 288
 // The line between "few waves" and "long" is 30720 weights per SM (4.5 M on 148, three waves of the

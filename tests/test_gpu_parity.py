@@ -171,6 +171,21 @@ def test_quantize_weights_that_are_not_finite(d_in, g, alt):
         np.testing.assert_allclose(sq.cpu().numpy(), sq_ref, rtol=1e-6, atol=1e-12, equal_nan=True)
 
 
+@pytest.mark.parametrize("d_in,g", [(64, 32), (256, 64), (640, 128), (1000, 256), (700, 700), (1500, 1500)])
+def test_quantize_a_row_alone_and_among_many(d_in, g):
+    # Every (row, group) is a problem of its own: what a row becomes must not depend on how many others are
+    # in the call, to the last bit, though the teams that share a group differ in size.
+    gen = torch.Generator(device="cuda").manual_seed(d_in)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rows = 30720 * sms // (-(-d_in // g) * g) + 1                    # past the line between the team sizes
+    W = torch.randn((rows, d_in), generator=gen, device="cuda") * 0.02
+    pick = slice(rows // 2, rows // 2 + 600)
+    for q, alt in ((1, 3), (2, 3), (3, 3), (4, 3), (4, 0)):
+        bits, alpha, sq = bcq.quantize(W, q, g, alt, want_sq_err=True)
+        b, a, s = bcq.quantize(W[pick].contiguous(), q, g, alt, want_sq_err=True)
+        assert torch.equal(b, bits[:, pick]) and torch.equal(a, alpha[:, pick]) and torch.equal(s, sq[pick])
+
+
 def test_quantize_strided_input_and_determinism():
     W = synth.weights(48, 384, (101, 0, 0))
     Wp = np.zeros((48, 400), dtype=np.float32)
