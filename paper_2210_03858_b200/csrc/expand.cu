@@ -1355,7 +1355,7 @@ bcq_status run_expand(int d_out, int d_in, int q, int g, int n, const void* act,
     p.counters = pp.counters;
     // bf16 output with an aligned base and pitch goes out through TMA stores
     p.fast_epi = fast_epi ? 1 : 0;
-    p.helpers = helpers_may_share(pl.full_tiles, pl.pairs, pl.num_kb) ? 1 : 0;
+    p.helpers = helpers_may_share(pl.full_tiles, pl.res_tiles > 0, pl.pairs, pl.num_kb) ? 1 : 0;
     return launch_expand_q<MODE>(tm, tmo, p, pl, s);
 }
 

@@ -13,7 +13,9 @@ PROGRAM = r"""
 int main() {
     std::printf("%d %d\n", bcq::kPfGroups, bcq::kPfWeightSlots);
     for (int full = 1; full <= 40; ++full)
-        for (int kb = 1; kb <= 12; ++kb) std::printf("%d %d %d\n", full, kb, (int)bcq::helpers_may_share(full, 8, kb));
+        for (int kb = 1; kb <= 12; ++kb)
+            for (int parts = 0; parts < 2; ++parts)
+                std::printf("%d %d %d %d\n", full, kb, parts, (int)bcq::helpers_may_share(full, parts, 8, kb));
 }
 """
 
@@ -26,12 +28,13 @@ def rule(tmp_path_factory):
     subprocess.run(["g++", "-std=c++17", "-I", CSRC, str(src), "-o", str(exe)], check=True)
     lines = subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.splitlines()
     groups, slots = map(int, lines[0].split())
-    return groups, slots, {tuple(map(int, l.split()[:2])): l.split()[2] == "1" for l in lines[1:]}
+    return groups, slots, {tuple(map(int, l.split()[:3])): l.split()[3] == "1" for l in lines[1:]}
 
 
 def worst_case_is_safe(groups, slots, segments, kb):
     """Whether every group, as far ahead as its waits allow, finds the accumulator's use before last
-    complete when it starts to wait for the last one."""
+    complete when it starts to wait for the last one.  (A part in front is counted as long as a tile: what
+    comes before the last two segments does not matter.)"""
     total = segments * kb
     if segments < 3:
         return True
@@ -49,10 +52,11 @@ def worst_case_is_safe(groups, slots, segments, kb):
 
 def test_workers_share_the_last_output_only_where_the_parity_is_unambiguous(rule):
     groups, slots, allowed = rule
-    for (full, kb), ok in allowed.items():
-        # 8 pairs; a pair walks full / 8 tiles, rounded up or down, and perhaps one part of a shared tile
-        for segments in {full // 8, -(-full // 8)}:
+    for (full, kb, parts), ok in allowed.items():
+        # 8 pairs; a pair walks full / 8 tiles, rounded up or down, after perhaps one part of a shared tile
+        for tiles in {full // 8, -(-full // 8)}:
             if ok:
-                assert worst_case_is_safe(groups, slots, segments, kb), (full, kb, segments)
-    # ... and wherever the K loop is not short they do
-    assert all(ok for (full, kb), ok in allowed.items() if full <= 8 or 2 * kb >= groups + slots)
+                assert worst_case_is_safe(groups, slots, tiles + parts, kb), (full, kb, parts)
+    # ... and wherever there is no earlier use, or the K loop is not short, they do
+    assert all(ok for (full, kb, parts), ok in allowed.items()
+               if -(-full // 8) + parts <= 2 or 2 * kb >= groups + slots)
