@@ -159,7 +159,8 @@ dalpha_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant
                     if (++s == kStages) { s = 0; ph ^= 1u; }
                 }
             }
-            if (!p.direct) pdl_trigger();  // the reduction follows; other kernels gain nothing (see expand.cu)
+            // (no pdl_trigger here: the reduction's blocks would crowd onto the SMs that this kernel leaves
+            // free, see launch_pdl; 1528 x 1000 at 777 tokens, four planes, 16.4 us with it and 13.7 without)
             // giving up: the copies in flight are counted on the leader's barriers, which may never
             // complete; they land within microseconds, so wait a thousand times as long
             if (!ok) for (int i = 0; i < 1000; ++i) __nanosleep(2000);

@@ -357,9 +357,9 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
 // meet zero activations).
 template <int NW>
 __global__ void __launch_bounds__(256) code_planes_kernel(int mode, int d_out, int pitch, int q, int rows_padded,
-                                                           int words_padded, int num_kb, const uint32_t* bits,
+                                                           int words_padded, int num_kb, int early, const uint32_t* bits,
                                                            uint32_t* codes) {
-    pdl_trigger();
+    if (early) pdl_trigger();
     pdl_wait();
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (long long)rows_padded * words_padded) return;
@@ -1261,8 +1261,11 @@ bcq_status launch_code_planes(int mode, int d_out, int d_in, int q, const Expand
     const int words_padded = (mode == MODE_FWD) ? pl.num_kb * 2 : pl.m_tiles * 4;
     const long long total = (long long)rows_padded * words_padded;
     const unsigned grid = (unsigned)((total + 255) / 256);
+    // the pre-pass may come in early where this kernel's blocks leave room on every SM (see launch_pdl):
+    // 1024 x 1024 at 64 tokens, q = 1, 128 blocks, 14.2 us a call with it and 15.4 without
+    const int early = grid <= (unsigned)sm_count() ? 1 : 0;
     BCQ_CUDA_TRY(launch_pdl(q == 4 ? code_planes_kernel<4> : code_planes_kernel<3>, dim3(grid), 256, 0, s, 1, mode, d_out, pitch, q,
-                            rows_padded, words_padded, pl.num_kb, bits, codes));
+                            rows_padded, words_padded, pl.num_kb, early, bits, codes));
     return BCQ_OK;
 }
 

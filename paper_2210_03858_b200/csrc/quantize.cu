@@ -162,8 +162,7 @@ quantize_kernel(const QuantParams p) {
     constexpr int NT = TW * 32;
     constexpr int TEAMS = (TW == 1) ? 4 : 1;
     __shared__ double red_scratch[32];
-    bcq::pdl_trigger();
-    bcq::pdl_wait();
+    bcq::pdl_wait();  // (and no pdl_trigger, see launch_pdl)
     __shared__ double level_smem[TEAMS][1 << BCQ_MAX_Q];
 
     const int lane = threadIdx.x & 31;
