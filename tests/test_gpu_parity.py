@@ -292,6 +292,24 @@ def test_bwd_alpha_partial_tiles_of_a_cta_pair(n, d_in, d_out, q, g):
     assert rel_err(bcq.linear_bwd_alpha(dYd, Xd, bd, d_in, g).cpu().numpy(), ref) <= TOL
 
 
+@pytest.mark.parametrize("mask", [0b1, 0b10, 0b1010, 0b10000000, 0b11010110, 0b11111111])
+@pytest.mark.parametrize("n,d_in,d_out,g", [(130, 200, 72, 200), (70, 320, 136, 32)])
+def test_bwd_alpha_of_some_planes(n, d_in, d_out, g, mask):
+    # planes of the mask are written, the others keep what they held
+    q = 8
+    _, X, dY, bits, alpha, _, _ = make_case(60 + n, n, d_in, d_out, q, g)
+    Xd, dYd, bd, ad = _upload(X, dY, bits, alpha)
+    ref = oracle.bwd_alpha(dY, X, bits, d_in, g)
+    out = torch.full_like(ad, 7.0)
+    bcq.linear_bwd_alpha(dYd, Xd, bd, d_in, g, plane_mask=mask, out=out)
+    o = out.cpu().numpy()
+    for i in range(q):
+        if (mask >> i) & 1:
+            assert np.abs(o[i] - ref[i]).max() <= TOL * np.abs(ref).max()
+        else:
+            assert (o[i] == 7.0).all()
+
+
 @pytest.mark.parametrize("n", [1, 4, 16, 5])
 @pytest.mark.parametrize("d_in,d_out,q,g", [(4096, 1536, 3, 128), (1024, 520, 4, 128), (2048, 256, 3, 2048)])
 def test_decode_matches_oracle(n, d_in, d_out, q, g):
