@@ -24,7 +24,6 @@
 //   * q > 4: the sums come out in the order 0,4,1,5,2,6,3,7 of a byte of a plane word, so the pre-pass,
 //     which regroups the plane words anyway, stores the bits of every byte as 0,2,4,6,1,3,5,7.
 #include <algorithm>
-#include <cmath>
 
 #include "expand_rules.h"
 #include "gemm_common.cuh"
@@ -1153,24 +1152,26 @@ ExpandPlan plan_expand(int mode, int d_out, int d_in, int q, int g, int n) {
     pl.m_tiles = ceil_div(Mdim, kBlockM);
     pl.m_pairs = ceil_div(pl.m_tiles, 2);
     pl.num_kb = ceil_div(Kdim, kBlockK);
-    // Token tiles and K pieces, by the time a call is expected to take.  All in stages of a pair (about
-    // 0.33 us, set by the expansion of the weight tiles and hence nearly the same at every width; 140
-    // tiles of 208 tokens take 2 % longer than 112 of 256, two waves both):
+    // Token tiles and K pieces, by the time a call is expected to take.  All in stages of a pair at q <= 4 (about
+    // 0.3 us, set by the expansion of the weight tiles and hence nearly the same at every width; 140
+    // tiles of 208 tokens take 2 % longer than 112 of 256, two waves both; q > 4 adds +-alpha_i weight by
+    // weight, four times as long):
     //   * whole waves of tiles, then the ragged last wave (or all of a problem with fewer tiles than
     //     pairs), whole or cut into d pieces;
-    //   * pieces that end the call are added by all 20 output warps of a CTA, each ceil(TN / 80) boxes
-    //     of 16 tokens at 0.8 us per piece, plus 3 us for the way through memory;
+    //   * pieces that end the call are added by all 20 output warps of a CTA: 2.4 us for the way through
+    //     memory, 0.33 us per piece for each of a warp's boxes of 16 tokens, and their bytes written and read
+    //     at 11 TB/s.  Measured, 4096 -> 256, q = 3, 64 tokens, 1 / 2 / 4 / 8 / 16 pieces: 33.0 / 27.0 / 23.2 /
+    //     22.2 / 23.2 us, 16 tokens 33.3 / 26.3 / 22.2 / 20.8 / 22.2; 64 tokens, q = 8: 86.7 / 52.2 / 34.1 / 26.6 /
+    //     23.6; 4096 -> 1024 at 2048 tokens, one piece (32 tiles of 256) or two (36 of 240) 31.7 / 30.0;
     //   * pieces before whole tiles are added by four warps under the main loop of those, so they
-    //     cost nothing if that is much longer (measured: 5120 -> 20480 dX with 2048 tokens, 12 of 172
+    //     cost nothing if that is much longer (measured: 5120 -> 20480 dX with 2048 tokens, 12 of 160
     //     tiles in pieces, 429 -> 359 us; 1600 -> 6400, whose tiles are 25 stages, 79 -> 92 us);
     //   * the last output, TN / 64 stages.
-    // That is the time of a call with the chip to itself.  A layer stack that runs on several streams
-    // pays for the pair stages a plan occupies instead (narrow tiles expand the same weights again for
-    // each), so these weigh in with a small exponent: it turns down a plan that is a few per cent
-    // faster alone and takes twice the stages.  Forward and backward of gpt2-medium's
-    // linears (2048 tokens, q = 3): one block on one stream 285 -> 291 us, the stack on nine streams
-    // 684 -> 750 TFLOP/s; one 1024 x 1024 layer on three streams 85 -> 146 TFLOP/s; 1000 x 1528 at
-    // 777 tokens on one stream 63 -> 65 us.
+    // That is the time of a call with the chip to itself.  A layer stack that runs on several streams pays for the
+    // pairs that a plan holds and for how long, so a whole chip's time counts for a quarter on top of it.
+    // (The rule before counted stages, not the time that pieces take to be added, and cut 4096 -> 1024 in two
+    // on 72 pairs where 32 take 6 % longer: GPT-2-medium stack, 24 layers at 2048 tokens, forward, dalpha and
+    // dX on nine streams 732 TFLOP/s, 792 now.)
     const int nt0 = ceil_div(n, 256), nt1 = std::min(ceil_div(n, 32), 8 * nt0);
     double best = -1.0;
     for (int nt = nt0; nt <= nt1; ++nt) {
@@ -1178,26 +1179,26 @@ ExpandPlan plan_expand(int mode, int d_out, int d_in, int q, int g, int n) {
         if (ceil_div(n, tn) != nt) continue;
         const int tiles = pl.m_pairs * nt;
         const int waves = tiles / pairs, ragged = tiles % pairs;
-        const double stage = 1.1 - 0.1 * tn / 256.0, out = 1.0 + tn / 64.0;
+        const double stage = (q <= 4 ? 1.0 : 4.0) * (1.1 - 0.1 * tn / 256.0), out = 1.0 + tn / 64.0;
         const int dmax = ragged > 0 ? std::min(pairs / ragged, pl.num_kb / kPfMinPiece) : 1;
         for (int d = 1; d <= std::max(1, dmax); ++d) {
-            const int len = ceil_div(pl.num_kb, d);
+            const int len = ceil_div(pl.num_kb, d), pieces = ceil_div(pl.num_kb, len);
             double add = 0.0;
-            if (d > 1 && waves == 0) add = 9.0 + 2.4 * ceil_div(tn, 80) * d;
+            if (d > 1 && waves == 0)
+                add = 8.0 + 1.1 * ceil_div(tn, 80) * pieces + 0.62e-6 * tiles * pieces * (double)(tn * 256 * 4);
             if (d > 1 && waves > 0 && waves * pl.num_kb < 3 * 40 * d) break;  // would not stay hidden
             const double cost = (waves * pl.num_kb + (ragged > 0 ? len : 0)) * stage + add + out;
-            const double stages = (waves > 0 ? tiles : tiles * ceil_div(pl.num_kb, len)) * (double)len;
-            const double score = cost * std::pow(stages, 0.2);
+            const int used = waves == 0 ? tiles * pieces : pieces > 1 ? pairs : ceil_div(tiles, waves + (ragged > 0 ? 1 : 0));
+            const double score = cost + 0.25 * used * cost / pairs;
             if (best >= 0.0 && score >= best) continue;
             best = score;
             pl.TN = tn;
             pl.n_tiles = nt;
-            pl.pieces = ceil_div(pl.num_kb, len);
+            pl.pieces = pieces;
             pl.piece_len = len;
-            pl.res_tiles = pl.pieces > 1 ? ragged : 0;
+            pl.res_tiles = pieces > 1 ? ragged : 0;
             pl.full_tiles = tiles - pl.res_tiles;
-            pl.pairs = waves > 0 ? (pl.res_tiles > 0 ? pairs : ceil_div(tiles, waves + (ragged > 0 ? 1 : 0)))
-                                 : tiles * pl.pieces;
+            pl.pairs = used;
         }
     }
     const int tn = pl.TN;
