@@ -19,9 +19,11 @@
 // 39 - 53 weights per clock and SM where HBM delivers 37 - 46.
 //
 // Work split: a unit is 16 rows x 128 k.  The 16-row tiles are dealt to the CTAs (one per SM).  The
-// units of a CTA, numbered step by step with all tiles of a step together, are dealt to its warps, so a step's activations are converted once (bf16 -> fp16 times a power of two per token and
-// step) and stay in registers as B fragments.  Its sums wait in a private slot of shared memory per
-// tile; the slots of a tile are added at the end, in order.  No CTA needs another.
+// units of a CTA, numbered step by step with all tiles of a step together, are dealt to its warps, so a
+// step's activations are converted once (bf16 -> fp16 times a power of two per token and step) and stay in
+// registers as B fragments.  Its sums wait in a private slot of shared memory per tile; the slots of a
+// tile are added at the end, in order.  Where there are too few tiles for the SMs, the CTAs of a cluster
+// share the steps of a tile (deal_tiles); otherwise no CTA needs another.
 //
 // One CTA of 16 warps an SM: with two of 8 warps, each CTA had half as many tiles to use a step's activations
 // for (OPT-6.7B layer, q = 4, one token: 68 us against 53); 20 or 24 warps with fewer registers each
@@ -176,15 +178,32 @@ struct DecOut {
 
 // The sums of `ntiles` 16-row tiles from tile0 on: added over the warps of the CTA, in order, and written.
 //   sums [warp][max_tiles][NT][32 lanes]: lane (g, t) has rows g (x, y) and g + 8 (z, w), tokens 2 t, 2 t + 1
-template <int NT>
-__device__ __forceinline__ void add_and_store(const DecOut& o, const float4* sums, int max_tiles, int ntiles, int tile0,
-                                              const float* rinv) {
-    for (int e = threadIdx.x; e < ntiles * NT * 32; e += kDpThreads) {
-        const int ti = e / (NT * 32), ln = e & 31, nt = (e >> 5) % NT;
-        const float4* src = sums + (size_t)(ti * NT + nt) * 32 + ln;
+// SPLIT: the `split` CTAs of a cluster hold parts of the same sums; the first one adds them, in order of rank.
+template <int NT, bool SPLIT>
+__device__ __forceinline__ void add_and_store(const DecOut& o, float4* sums, int max_tiles, int ntiles, int tile0,
+                                              const float* rinv, int split) {
+    const int items = ntiles * NT * 32;
+    auto over_warps = [&](int e) {
+        const float4* src = sums + e;
         float4 s = src[0];
         for (int w = 1; w < kDpWarps; ++w) {
             const float4 x = src[(size_t)w * max_tiles * (NT * 32)];
+            s.x += x.x; s.y += x.y; s.z += x.z; s.w += x.w;
+        }
+        return s;
+    };
+    const int rank = SPLIT ? (int)ptx::cluster_rank() : 0;
+    if (SPLIT) {
+        if (rank > 0)
+            for (int e = threadIdx.x; e < items; e += kDpThreads) sums[e] = over_warps(e);
+        __syncthreads();
+        ptx::cluster_sync();
+    }
+    for (int e = threadIdx.x; rank == 0 && e < items; e += kDpThreads) {
+        const int ti = e / (NT * 32), ln = e & 31, nt = (e >> 5) % NT;
+        float4 s = over_warps(e);
+        for (int r = 1; SPLIT && r < split; ++r) {
+            const float4 x = ptx::ld_cluster_v4(ptx::cluster_addr(ptx::smem_u32(sums + e), (uint32_t)r));
             s.x += x.x; s.y += x.y; s.z += x.z; s.w += x.w;
         }
         const int tok = nt * 8 + 2 * (ln & 3);
@@ -204,6 +223,10 @@ __device__ __forceinline__ void add_and_store(const DecOut& o, const float4* sum
                 else reinterpret_cast<float*>(o.out)[at] = v[c];
             }
         }
+    }
+    if (SPLIT) {  // the sums have been read
+        __syncthreads();
+        ptx::cluster_sync();
     }
 }
 
@@ -244,6 +267,7 @@ struct DecPackedParams {
     int steps;
     int per, rem;            // row tiles per CTA and remainder
     int round;               // tiles between two additions
+    int split;               // CTAs of a cluster that share the steps of their tiles
     uint32_t g_magic;        // ceil(2^32 / g) where k / g = hi32(k g_magic) for every k < d_in, else 0
     const __nv_bfloat16* X;
     long long ldx;
@@ -289,23 +313,28 @@ struct UnitWords {
     uint4 ta[PARTS], tb[PARTS];  // tables of rows g and g + 8
 };
 
-template <int Q, int NT, int PARTS>
+template <int Q, int NT, int PARTS, bool SPLIT>
 __global__ void __launch_bounds__(kDpThreads, 1)
 decode_packed_kernel(const DecPackedParams p) {
     extern __shared__ float4 sums[];  // [warp][slot][NT][32 lanes]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int gr = lane >> 2, tq = lane & 3;
-    const int tile0 = (int)blockIdx.x * p.per + min((int)blockIdx.x, p.rem);
-    const int ntiles = p.per + ((int)blockIdx.x < p.rem ? 1 : 0);
+    const int cta = SPLIT ? (int)blockIdx.x / p.split : (int)blockIdx.x;
+    const int tile0 = cta * p.per + min(cta, p.rem);
+    const int ntiles = p.per + (cta < p.rem ? 1 : 0);
+    // the CTA's steps: all of them, or its rank's share
+    const int part = SPLIT ? (int)blockIdx.x - cta * p.split : 0;
+    const int step0 = SPLIT ? (int)((long long)p.steps * part / p.split) : 0;
+    const int nsteps = SPLIT ? (int)((long long)p.steps * (part + 1) / p.split) - step0 : p.steps;
     float4* mine = sums + (size_t)warp * p.round * (NT * 32) + lane;
 
     pdl_trigger();
     for (int first = 0; first < ntiles; first += p.round) {
         const int round_n = min(p.round, ntiles - first);
         // the warp's units: an equal, contiguous share of the round's, numbered step by step
-        const int all = round_n * p.steps;
+        const int all = round_n * nsteps;
         const int u0 = all * warp / kDpWarps, u1 = all * (warp + 1) / kDpWarps;
-        const int st0 = u0 / round_n, i0 = u0 - st0 * round_n;
+        const int st0 = step0 + u0 / round_n, i0 = u0 - (st0 - step0) * round_n;
 
         // ---- loading: unit (step, tile) pairs in the order of use
         const uint8_t* lp_codes = p.codes;
@@ -371,7 +400,7 @@ decode_packed_kernel(const DecPackedParams p) {
         if (first == 0) {
             // the activations of the warp's later steps: into L1 while the first step is at work
             // (32 lanes: 16 tokens x two 128-byte lines of a step)
-            for (int s = st0 + 1; s * round_n < u1; ++s) {
+            for (int s = st0 + 1; (s - step0) * round_n < u1; ++s) {
                 const int k = s * kDpStepK + (lane & 1) * 64;
                 if ((lane >> 1) < p.n && k < p.d_in)
                     asm volatile("prefetch.global.L1 [%0];" ::"l"(p.X + (long long)(lane >> 1) * p.ldx + k));
@@ -446,7 +475,7 @@ decode_packed_kernel(const DecPackedParams p) {
         }
 
         __syncthreads();
-        add_and_store<NT>(p.o, sums, p.round, round_n, tile0 + first, p.rinv);
+        add_and_store<NT, SPLIT>(p.o, sums, p.round, round_n, tile0 + first, p.rinv, p.split);
         if (first + p.round < ntiles) __syncthreads();  // the slots are written again
     }
 }
@@ -466,7 +495,7 @@ decode_packed_kernel(const DecPackedParams p) {
 struct DecPlanesParams {
     int d_out, d_in, q, g, G, n;
     int steps, pitch;
-    int per, rem, round;     // see DecPackedParams
+    int per, rem, round, split;  // see DecPackedParams
     uint32_t g_magic;
     const __nv_bfloat16* X;
     long long ldx;
@@ -541,14 +570,19 @@ struct RowExpand {
     }
 };
 
-template <int NQ, int NT>
+template <int NQ, int NT, bool SPLIT>
 __global__ void __launch_bounds__(kDpThreads, 1)
 decode_planes_kernel(const DecPlanesParams p) {
     extern __shared__ float4 sums[];  // [warp][tile][NT][32 lanes]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int gr = lane >> 2, tq = lane & 3;
-    const int tile0 = (int)blockIdx.x * p.per + min((int)blockIdx.x, p.rem);
-    const int ntiles = p.per + ((int)blockIdx.x < p.rem ? 1 : 0);
+    const int cta = SPLIT ? (int)blockIdx.x / p.split : (int)blockIdx.x;
+    const int tile0 = cta * p.per + min(cta, p.rem);
+    const int ntiles = p.per + (cta < p.rem ? 1 : 0);
+    // the CTA's steps: all of them, or its rank's share
+    const int part = SPLIT ? (int)blockIdx.x - cta * p.split : 0;
+    const int step0 = SPLIT ? (int)((long long)p.steps * part / p.split) : 0;
+    const int nsteps = SPLIT ? (int)((long long)p.steps * (part + 1) / p.split) - step0 : p.steps;
     float4* mine = sums + (size_t)warp * p.round * (NT * 32) + lane;
     const size_t plane_bits = (size_t)p.d_out * p.pitch, plane_alpha = (size_t)p.d_out * p.G;
 
@@ -556,9 +590,9 @@ decode_planes_kernel(const DecPlanesParams p) {
     pdl_wait();  // the scales may come from the kernel before this one
     for (int first = 0; first < ntiles; first += p.round) {
         const int round_n = min(p.round, ntiles - first);
-        const int all = round_n * p.steps;
+        const int all = round_n * nsteps;
         const int u0 = all * warp / kDpWarps, u1 = all * (warp + 1) / kDpWarps;
-        const int st0 = u0 / round_n, i0 = u0 - st0 * round_n;
+        const int st0 = step0 + u0 / round_n, i0 = u0 - (st0 - step0) * round_n;
 
         int l_st = st0, l_i = i0, l_c = 0, l_left = u1 - u0;
         auto group_of = [&](int st) {  // group of this lane's 32 weights
@@ -590,7 +624,7 @@ decode_planes_kernel(const DecPlanesParams p) {
         if (NQ < 8) load(ub);
         for (int i = 0; i < round_n * NT; ++i) mine[i * 32] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (first == 0) {
-            for (int s = st0 + 1; s * round_n < u1; ++s) {
+            for (int s = st0 + 1; (s - step0) * round_n < u1; ++s) {
                 const int k = s * kDpStepK + (lane & 1) * 64;
                 if ((lane >> 1) < p.n && k < p.d_in)
                     asm volatile("prefetch.global.L1 [%0];" ::"l"(p.X + (long long)(lane >> 1) * p.ldx + k));
@@ -695,7 +729,7 @@ decode_planes_kernel(const DecPlanesParams p) {
             }
         }
         __syncthreads();
-        add_and_store<NT>(p.o, sums, p.round, round_n, tile0 + first, nullptr);
+        add_and_store<NT, SPLIT>(p.o, sums, p.round, round_n, tile0 + first, nullptr, p.split);
         if (first + p.round < ntiles) __syncthreads();  // the slots are written again
     }
 }
@@ -709,12 +743,23 @@ uint32_t group_magic(int d_in, int g) {
     return (long long)d_in * g < (1ll << 32) && g > 1 ? (uint32_t)(((1ull << 32) + g - 1) / g) : 0u;
 }
 
-// Row tiles dealt to one CTA per SM; bytes of the warps' sums (at most 192 KiB).
+// Row tiles dealt to one CTA per SM; bytes of the warps' sums (at most 192 KiB).  A matrix with few row tiles
+// gives each to a cluster of 2, 4 or 8 CTAs that share its steps, as long as a CTA keeps a step for every
+// warp (fewer: 2048 -> 256, q = 4, one token 4.6 us without a cluster, 5.5 in pairs) and the clusters find
+// their places at once (on 148 SMs at most 65, 32 and 16 of them).  Measured, one CTA a tile, now, and the
+// kernels with the columns dealt over all SMs that these replaced, 16 tokens:
+//   planes, q = 4   16384 -> 512 32.4 / 12.0 / 18.8 us   16384 -> 128 32.0 / 8.0 / 18.3   4096 -> 512 10.4 / 7.7 / 17.2
+//   planes, q = 6   16384 -> 512 61.6 / 19.1 / 32.3      32768 -> 32 113 / 18.3 / 27.7
+//   packed, q = 4   16384 -> 512 20.1 / 9.2 / 26.3       65536 -> 16 70.5 / 12.6 / 63.7
 template <int NT, typename Params>
 size_t deal_tiles(Params& p, int tiles, int* ctas) {
-    *ctas = std::min(tiles, sm_count());
-    p.per = tiles / *ctas;
-    p.rem = tiles % *ctas;
+    const int sms = sm_count();
+    p.split = 1;
+    while (p.split < 8 && p.steps >= 2 * kDpWarps * p.split && 2 * p.split * tiles <= sms - sms / 8) p.split *= 2;
+    const int clusters = std::min(tiles, sms);
+    *ctas = clusters * p.split;
+    p.per = tiles / clusters;
+    p.rem = tiles % clusters;
     p.round = std::min(p.per + (p.rem > 0 ? 1 : 0), kDpMaxRound / NT);
     return (size_t)kDpWarps * p.round * NT * 512;
 }
@@ -723,10 +768,10 @@ template <int Q, int NT, int PARTS>
 bcq_status launch_decode_packed(DecPackedParams p, int tiles, cudaStream_t s) {
     int ctas;
     const size_t smem = deal_tiles<NT>(p, tiles, &ctas);
-    auto kern = decode_packed_kernel<Q, NT, PARTS>;
+    auto kern = p.split > 1 ? decode_packed_kernel<Q, NT, PARTS, true> : decode_packed_kernel<Q, NT, PARTS, false>;
     const bcq_status st = ensure_dynamic_smem(kern, smem);
     if (st != BCQ_OK) return st;
-    BCQ_CUDA_TRY(launch_pdl(kern, dim3((unsigned)ctas), kDpThreads, smem, s, 1, p));
+    BCQ_CUDA_TRY(launch_pdl(kern, dim3((unsigned)ctas), kDpThreads, smem, s, (unsigned)p.split, p));
     return BCQ_OK;
 }
 
@@ -746,10 +791,10 @@ template <int NQ, int NT>
 bcq_status launch_decode_planes(DecPlanesParams p, cudaStream_t s) {
     int ctas;
     const size_t smem = deal_tiles<NT>(p, ceil_div(p.d_out, kDpRows), &ctas);
-    auto kern = decode_planes_kernel<NQ, NT>;
+    auto kern = p.split > 1 ? decode_planes_kernel<NQ, NT, true> : decode_planes_kernel<NQ, NT, false>;
     const bcq_status st = ensure_dynamic_smem(kern, smem);
     if (st != BCQ_OK) return st;
-    BCQ_CUDA_TRY(launch_pdl(kern, dim3((unsigned)ctas), kDpThreads, smem, s, 1, p));
+    BCQ_CUDA_TRY(launch_pdl(kern, dim3((unsigned)ctas), kDpThreads, smem, s, (unsigned)p.split, p));
     return BCQ_OK;
 }
 

@@ -158,6 +158,19 @@ __device__ __forceinline__ uint32_t leader_addr(uint32_t addr) {
     return r;
 }
 
+// Address, in the cluster's shared window, of the same variable of the CTA of the given rank; and a load from it.
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ float4 ld_cluster_v4(uint32_t cluster_addr) {
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(cluster_addr) : "memory");
+    return v;
+}
+
 // Arrives on a barrier of either CTA (an address in the shared window of the cluster).  What it orders
 // here are this CTA's own writes to its own shared memory (made visible to the tensor core by the proxy
 // fence before it) and its reads of tensor memory, so the release needs no wider scope than the CTA: a

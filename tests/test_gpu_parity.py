@@ -599,6 +599,27 @@ def test_decode_right_after_packing_into_a_used_buffer(d_in, d_out, q, g, n):
         assert torch.equal(out, ref[i % 2]), i
 
 
+@pytest.mark.parametrize("n", [1, 9])
+@pytest.mark.parametrize("d_in,d_out,q,g", [(4096, 1040, 4, 128), (4224, 1030, 3, 96), (8200, 512, 2, 8200),
+                                            (16384, 250, 4, 64), (8192, 16, 6, 128), (4100, 17, 1, 4100)])
+def test_decode_of_few_rows_by_clusters(n, d_in, d_out, q, g):
+    # few row tiles and a long row: 2, 4 or 8 CTAs share a tile's steps, evenly or not (4224: 33 steps, 8200: 65);
+    # 4096 and 1040 rows lie on the lines of the rule.  Against a dense fp64 product.
+    gen = torch.Generator(device="cuda").manual_seed(d_in + d_out)
+    W = torch.randn((d_out, d_in), generator=gen, device="cuda") * 0.02
+    bits, alpha, _ = bcq.quantize(W, q, g)
+    X = torch.randn((n, (d_in + 7) // 8 * 8), generator=gen, device="cuda").bfloat16()[:, :d_in]
+    bias = torch.randn(d_out, generator=gen, device="cuda")
+    ref = (X.double() @ bcq.dequantize(bits, alpha, d_in, g).double().t() + bias.double()).cpu().numpy()
+    outs = [[bcq.linear_decode(X, bits, alpha, d_in, g, bias=bias) for _ in range(3)]]
+    if q <= 4:
+        pack = bcq.decode_pack(bits, alpha, d_in, g)
+        outs.append([bcq.linear_decode_packed(X, pack, d_out, d_in, q, g, bias=bias) for _ in range(3)])
+    for ys in outs:
+        assert torch.equal(ys[0], ys[1]) and torch.equal(ys[0], ys[2]), "runs differ"
+        assert rel_err(ys[0].cpu().numpy(), ref) <= TOL
+
+
 def test_decode_pack_rejects_more_than_four_planes():
     assert bcq.lib().bcq_decode_pack_bytes(64, 256, 5, 64) == 0
     assert bcq.lib().bcq_decode_pack_bytes(64, 256, 4, 64) > 0
