@@ -1,4 +1,5 @@
-"""Builds the library in-tree: csrc/*.cu -> libbcq_b200.so (sm_100a only), csrc/binding.c -> _bcq_call.so."""
+"""Builds the library in-tree: csrc/*.cu -> libbcq_b200.so (sm_100a only), csrc/binding.c -> the extension
+module _bcq_call, whose file name carries the interpreter's ABI tag."""
 from __future__ import annotations
 
 import glob
@@ -11,7 +12,8 @@ from concurrent.futures import ThreadPoolExecutor
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libbcq_b200.so")
-CALL = os.path.join(HERE, "_bcq_call.so")
+# the tag keeps another interpreter version from importing an extension that was not built for it
+CALL = os.path.join(HERE, "_bcq_call" + sysconfig.get_config_var("EXT_SUFFIX"))
 OBJ_DIR = os.path.join(HERE, "_build")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -41,6 +43,9 @@ def _build_binding():
     if r.returncode != 0:
         raise RuntimeError("gcc failed for binding.c:\n" + r.stderr)
     os.replace(CALL + ".tmp", CALL)
+    untagged = os.path.join(HERE, "_bcq_call.so")  # of an older tree: any interpreter would import it
+    if os.path.exists(untagged):
+        os.remove(untagged)
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:
