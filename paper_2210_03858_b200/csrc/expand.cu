@@ -39,7 +39,7 @@ enum { MODE_FWD = 0, MODE_BWDX = 1 };
 enum { QM_LUT3 = 0, QM_LUT4 = 1, QM_GENERIC = 2 };
 
 // 16 weights of one row (bits 0..15 of the plane words w) as fp32 sums of +-alpha_i, any q <= 8, stored as two
-// 16-byte chunks (slots chunk0, chunk0 + 1) of the 128-byte line at `line` (swizzle key lx).  w[i] = plane words (bits 0..15 used), a[i] = scales.
+// 16-byte chunks (slots chunk0, chunk0 + 1) of the 128-byte line at `line` (swizzle key lx); a[i] = scales.
 __device__ __forceinline__ void expand16_sum(const uint32_t (&w)[BCQ_MAX_Q], const float (&a)[BCQ_MAX_Q],
                                              int q, uint32_t line, uint32_t lx, uint32_t chunk0) {
     float v[16];
@@ -115,7 +115,6 @@ struct PrepParams {
     int mode, d_out, q, G, pitch, num_kb, amax_blocks, bits_blocks;
     int row_tiles;   // ceil(d_out / 128)
     int bits_cblk;   // ceil(pitch / 32): 32-word column blocks of the plane words
-    int alpha_cblk;  // ceil(G / 32)
     const uint32_t* bits;
     float* alpha_t;
     uint32_t* bits_t;
@@ -184,13 +183,10 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
     // behind the register-heavy token blocks, so the ids run backwards.
     const int bid = (int)gridDim.x - 1 - (int)blockIdx.x;
     if (bid >= p.act_blocks + p.amax_blocks) {
-        // ---- regroup a block of 128 rows x 32 columns (plane words or scales) of one plane:
-        // coalesced reads into shared memory, then coalesced writes of the stage chunks
         __shared__ uint32_t tile[128][33];
         int b = bid - p.act_blocks - p.amax_blocks;
-        const bool is_alpha = b >= p.bits_blocks;
-        if (is_alpha) b -= p.bits_blocks;
-        if (is_alpha) {
+        if (b >= p.bits_blocks) {
+            b -= p.bits_blocks;
             // ---- scales of one plane and one tile of 128 rows: alpha[i][j][c] is contiguous over
             // (j, c), so the block reads it as one coalesced run and scatters the values to their
             // places in the regrouped array (rows past d_out become zeros)
@@ -214,62 +210,52 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
             }
             return;
         }
-        const int cblks = is_alpha ? p.alpha_cblk : p.bits_cblk;
-        const int cb = b % cblks;
-        const int rt = (b / cblks) % p.row_tiles;
-        const int i = b / (cblks * p.row_tiles);
-        const int ncols = is_alpha ? p.G : p.pitch;
-        const uint32_t* src = is_alpha ? reinterpret_cast<const uint32_t*>(p.alpha) : p.bits;
-        src += (long long)i * p.d_out * ncols;
+        // ---- plane words (q > 4), 128 rows x 32 words of one plane: coalesced reads into shared memory,
+        // then coalesced writes of the stage chunks
+        const int cb = b % p.bits_cblk;
+        const int rt = (b / p.bits_cblk) % p.row_tiles;
+        const int i = b / (p.bits_cblk * p.row_tiles);
+        const uint32_t* src = p.bits + (long long)i * p.d_out * p.pitch;
         // all sixteen loads of a thread in flight at once: the block's time is one memory latency
         uint32_t held[16];
         const int col_l = cb * 32 + lane;
 #pragma unroll
         for (int pass = 0; pass < 16; ++pass) {
             const int j = rt * 128 + pass * 8 + warp;
-            held[pass] = (j < p.d_out && col_l < ncols) ? ld(src + (long long)j * ncols + col_l) : 0u;
+            held[pass] = (j < p.d_out && col_l < p.pitch) ? ld(src + (long long)j * p.pitch + col_l) : 0u;
         }
 #pragma unroll
         for (int pass = 0; pass < 16; ++pass) {
+            // even bits of every byte to its low nibble, odd bits to the high nibble: one PRMT
+            // pair of the expansion emits weights 0,4,1,5,2,6,3,7 of a byte, so with the bits
+            // stored as 0,2,4,6,1,3,5,7 the expanded tile comes out in natural k order
             uint32_t v = held[pass];
-            if (!is_alpha) {
-                // even bits of every byte to its low nibble, odd bits to the high nibble: one PRMT
-                // pair of the expansion emits weights 0,4,1,5,2,6,3,7 of a byte, so with the bits
-                // stored as 0,2,4,6,1,3,5,7 the expanded tile comes out in natural k order
-                uint32_t t = (v ^ (v >> 1)) & 0x22222222u;
-                v ^= t ^ (t << 1);
-                t = (v ^ (v >> 2)) & 0x0C0C0C0Cu;
-                v ^= t ^ (t << 2);
-            }
+            uint32_t t = (v ^ (v >> 1)) & 0x22222222u;
+            v ^= t ^ (t << 1);
+            t = (v ^ (v >> 2)) & 0x0C0C0C0Cu;
+            v ^= t ^ (t << 2);
             tile[pass * 8 + warp][lane] = v;
         }
         __syncthreads();
         const int t = threadIdx.x;
-        uint32_t* dst = is_alpha ? reinterpret_cast<uint32_t*>(p.alpha_t) : p.bits_t;
 #pragma unroll 4
         for (int pass = 0; pass < 16; ++pass) {
             int r, cl;
-            if (is_alpha) { r = t & 127; cl = pass * 2 + (t >> 7); }
-            else if (p.mode == MODE_FWD) { r = t >> 1; cl = pass * 2 + (t & 1); }
+            if (p.mode == MODE_FWD) { r = t >> 1; cl = pass * 2 + (t & 1); }
             else { r = (pass & 1) * 64 + (t >> 2); cl = (pass >> 1) * 4 + (t & 3); }
             const int col = cb * 32 + cl;
-            if (col >= ncols) continue;
+            if (col >= p.pitch) continue;
             long long o;
             if (p.mode == MODE_FWD) {
-                if (is_alpha) {
-                    o = (((long long)rt * p.G + col) * p.q + i) * 128 + r;
-                } else {
-                    const int kb = col >> 1;
-                    if (kb >= p.num_kb) continue;
-                    o = ((((long long)rt * p.num_kb + kb) * p.q + i) * 128 + r) * 2 + (col & 1);
-                }
+                const int kb = col >> 1;
+                if (kb >= p.num_kb) continue;
+                o = ((((long long)rt * p.num_kb + kb) * p.q + i) * 128 + r) * 2 + (col & 1);
             } else {
                 const int jb = rt * 2 + (r >> 6), rr = r & 63;
                 if (jb >= p.num_kb) continue;
-                if (is_alpha) o = (((long long)jb * p.G + col) * p.q + i) * 64 + rr;
-                else o = ((((long long)(col >> 2) * p.num_kb + jb) * p.q + i) * 64 + rr) * 4 + (col & 3);
+                o = ((((long long)(col >> 2) * p.num_kb + jb) * p.q + i) * 64 + rr) * 4 + (col & 3);
             }
-            dst[o] = tile[r][cl];
+            p.bits_t[o] = tile[r][cl];
         }
         return;
     }
@@ -385,14 +371,14 @@ __global__ void __launch_bounds__(256) code_planes_kernel(int mode, int d_out, i
 // ------------------------------------------------------------------------------------------
 
 struct ExpandParams {
-    int d_out, d_in, q, g, G, pitch, n;
+    int q, g, G, n;
     int Mdim;          // d_out (fwd) or d_in (dX)
     int num_kb;        // K blocks of 64 over d_in (fwd) or d_out (dX)
     // The first full_tiles output tiles go whole to the pairs in turn; the res_tiles tiles after them
     // are cut into `pieces` pieces of piece_len stages, one for each of the first res_tiles * pieces pairs
     int full_tiles, res_tiles, pieces, piece_len;
     int m_tiles;           // row tiles of 128 of the regrouped planes
-    int m_pairs, n_tiles;  // output tiles: pairs of row tiles, token tiles
+    int m_pairs;           // output tiles of a token tile: pairs of row tiles
     int tn;                // token tile width
     uint32_t acc_cols;     // tensor-memory columns per accumulator
     // pipeline geometry (chosen on the host)
@@ -460,7 +446,8 @@ constexpr int kPfMaxSlots = 8;                                // per ring
 constexpr uint32_t kPfGroupBar0 = 4;                           // named barriers 4..7: one per worker group
 constexpr uint32_t kPfCtlBytes = 384;                          // barriers, TMEM handle, abort flag
 constexpr uint32_t kPfScaleBytes = 256 * 4;                    // [TN] output scales of the tile being drained
-constexpr uint32_t kPfStagingBuf = kPfEpiWarps * 1024;         // per epilogue warp one 1 KiB buffer of 32 rows x 16 bf16 (8 fp32) tokens; two such sets
+// per epilogue warp one 1 KiB buffer of 32 rows x 16 bf16 (8 fp32) tokens; two such sets
+constexpr uint32_t kPfStagingBuf = kPfEpiWarps * 1024;
 
 template <int MODE, int QM>
 __global__ void __launch_bounds__(kPfThreads, 1)
@@ -539,7 +526,6 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
     pdl_wait();
     const uint32_t tmem_base = *tmem_holder;
 
-    // every role walks the same sequence of tiles and pipeline stages
     // every role walks the same sequence of segments (a tile, or this pair's part of one) and pipeline
     // stages
     const int nres = pair0 < p.res_tiles * p.pieces ? 1 : 0;
@@ -1058,7 +1044,8 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
         const int quarter = warp & 3;       // TMEM lanes 32 * quarter .. + 31
         const int et = ew * 32 + lane;      // 0..127
         const float winv = pow2f(-weight_shift(p.hdr, p.q));
-        const uint32_t stg = staging_base + ew * 1024;  // this warp's staging: [tokens][32 rows], 1 KiB (a second one kPfStagingBuf further)
+        // this warp's staging: [tokens][32 rows], 1 KiB (a second one kPfStagingBuf further)
+        const uint32_t stg = staging_base + ew * 1024;
         bool ok = true;
         int lt = 0;
         uint32_t chunks = 0;  // output boxes stored so far (fast path): selects the staging buffer
@@ -1253,7 +1240,6 @@ bcq_status launch_expand_q(const CUtensorMap& tm, const CUtensorMap& tmo, const 
     return launch_expand<MODE, QM_GENERIC>(tm, tmo, p, pl, stream);
 }
 
-// act: bf16 [n][ldact] with Kdim valid columns (X for the forward, dY for dX).
 // Writes the selector codes of the planes (q <= 4) in the chunk order of mode `mode`.
 bcq_status launch_code_planes(int mode, int d_out, int d_in, int q, const ExpandPlan& pl, const uint32_t* bits,
                               uint32_t* codes, cudaStream_t s) {
@@ -1320,7 +1306,6 @@ bcq_status run_expand(int d_out, int d_in, int q, int g, int n, const void* act,
     pp.amax_blocks = (int)ablocks;
     pp.row_tiles = ceil_div(d_out, 128);
     pp.bits_cblk = ceil_div(pitch, 32);
-    pp.alpha_cblk = ceil_div(pp.G, 32);
     const bool coded = q <= 4;  // selector codes (written once, or by the launch below); q > 4: plane words
     pp.bits_blocks = coded ? 0 : q * pp.row_tiles * pp.bits_cblk;
     const int alpha_tr_blocks = q * pp.row_tiles;  // one block per (plane, tile of 128 rows)
@@ -1342,12 +1327,11 @@ bcq_status run_expand(int d_out, int d_in, int q, int g, int n, const void* act,
     BCQ_CUDA_TRY(launch_pdl(prep, dim3(pgrid), 256, 0, s, 1, pp));
 
     ExpandParams p;
-    p.d_out = d_out; p.d_in = d_in; p.q = q; p.g = g;
+    p.q = q; p.g = g;
     p.G = (int)bcq_num_groups(d_in, g);
-    p.pitch = pitch;
     p.n = n; p.Mdim = Mdim; p.num_kb = pl.num_kb;
     p.full_tiles = pl.full_tiles; p.res_tiles = pl.res_tiles; p.pieces = pl.pieces; p.piece_len = pl.piece_len;
-    p.m_tiles = pl.m_tiles; p.m_pairs = pl.m_pairs; p.n_tiles = pl.n_tiles;
+    p.m_tiles = pl.m_tiles; p.m_pairs = pl.m_pairs;
     p.tn = pl.TN;
     p.acc_cols = 32;
     while ((int)p.acc_cols < pl.TN) p.acc_cols *= 2;

@@ -13,7 +13,6 @@ namespace bcq {
 constexpr int kThreads = 320;       // warp 0: TMA, warp 1: UMMA + TMEM, warps 2..9: workers
 constexpr int kWorkerWarp0 = 2;
 constexpr int kWorkerWarps = 8;
-constexpr int kWorkers = kWorkerWarps * 32;
 constexpr int kBlockM = 128;
 constexpr int kBlockK = 64;
 constexpr uint32_t kABytes = kBlockM * kBlockK * 2;  // one 16-bit A tile: 16 KiB
