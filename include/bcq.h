@@ -94,7 +94,8 @@ size_t bcq_workspace_bytes(int op, int d_out, int d_in, int q, int g, int n);
  *   last least-squares fit.  A group whose planes make B^T B singular keeps its previous
  *   alpha in that round.
  * Sums, residuals and the q x q solve are carried in fp64; every alpha is rounded to fp32 as
- * soon as it is computed and the rounded value is used from then on.
+ * soon as it is computed and the rounded value is used from then on.  What a (row, group) becomes depends
+ * on its weights alone, to the last bit: the order of its sums is a function of g.
  *
  *   W      in : float [d_out][ldw], ldw >= d_in
  *   bits   out: container format above (padding bits are written as 0)
@@ -123,7 +124,7 @@ bcq_status bcq_dequantize(int d_out, int d_in, int q, int g, const uint32_t* bit
  * Arithmetic: the scaled weight sum_i alpha_i b_i is formed in fp32 and rounded once to fp16;
  * the bf16 activations are converted exactly to fp16 after a per-token power-of-two scaling
  * that is undone on output; products are accumulated in fp32 in the tensor core.  The same
- * holds for bcq_linear_decode and bcq_linear_bwd_x. */
+ * holds for bcq_linear_bwd_x; bcq_linear_decode scales in smaller blocks (see there). */
 bcq_status bcq_linear_fwd(int d_out, int d_in, int q, int g, int n, const void* X, size_t ldx,
                           const uint32_t* bits, const float* alpha, const float* bias, void* Y,
                           size_t ldy, int y_dtype, void* ws, size_t ws_bytes, void* stream);
@@ -149,8 +150,11 @@ bcq_status bcq_linear_bwd_x_prepared(int d_out, int d_in, int q, int g, int n, c
                                      int dx_dtype, void* ws, size_t ws_bytes, void* stream);
 
 /* Same computation for the decode regime, 1 <= n <= 16 tokens, where the cost is streaming
- * the packed planes from memory once (Section "Inference Speed").  Workspace op is
- * BCQ_OP_DECODE.  n > 16 gives BCQ_ERR_SHAPE. */
+ * the packed planes from memory once (Section "Inference Speed").  The powers of two that bring
+ * weights and activations into the fp16 range are taken per row and 128 columns and per token and 128
+ * columns; the sums over 128 columns are added in fp32, in a fixed order.  Workspace op is BCQ_OP_DECODE:
+ * the sums stay on chip and ws is not written, but its size is checked as it always was.  n > 16 gives
+ * BCQ_ERR_SHAPE. */
 bcq_status bcq_linear_decode(int d_out, int d_in, int q, int g, int n, const void* X, size_t ldx,
                              const uint32_t* bits, const float* alpha, const float* bias,
                              void* Y, size_t ldy, int y_dtype, void* ws, size_t ws_bytes,
@@ -186,7 +190,7 @@ bcq_status bcq_linear_decode_noalloc(int d_out, int d_in, int q, int g, int n, c
  *     (row, group), q bits per weight as in `bits`;
  *   - per (row, group) the eight fp16 levels sum_i +-alpha_i (for q = 4 those with b_4 = +1; the
  *     others are their negatives), 16 bytes, multiplied by a power of two per row that brings
- *     q * max|alpha| of the row to [2^13, 2^14) -- the values bcq_linear_decode forms on the fly;
+ *     q * max|alpha| of the row to [2^13, 2^14) -- what bcq_linear_decode forms on the fly;
  *   - per row that power of two.
  * The pack is bcq_decode_pack_bytes() bytes (0 for an unsupported shape; about the size of bits
  * plus alpha), 128-byte aligned, caller-owned.  q > 4 gives BCQ_ERR_UNSUPPORTED: use

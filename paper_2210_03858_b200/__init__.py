@@ -163,9 +163,9 @@ def workspace_bytes(op: int, d_out: int, d_in: int, q: int, g: int, n: int = 0) 
 # ---------------------------------------------------------------------------- helpers
 
 # The small calls of the library take a few microseconds on the GPU, so the marshalling counts: the
-# frequent calls go through csrc/binding.c instead of ctypes, with the raw stream handle instead of a Stream object, and no size
-# query where the caller brought the workspace (the library checks its size anyway).  Measured on the
-# optimiser step plus checkpoint (two calls): 24 -> 12 us.
+# frequent calls go through csrc/binding.c instead of ctypes, with the raw stream handle instead of a
+# Stream object, and no size query where the caller brought the workspace (the library checks its size
+# anyway).  Measured on the optimiser step plus checkpoint (two calls): 24 -> 12 us.
 
 _torch_module = None
 
@@ -323,9 +323,8 @@ NOALLOC_SCRATCH_BYTES = 2 << 20
 
 def linear_decode_noalloc(X, bits, alpha, d_in: int, g: int, bias=None, out=None):
     """bcq_linear_decode_noalloc: decode for callers that cannot provide scratch memory -- the
-    library call itself allocates nothing (its partial sums go to a fixed 2 MiB array inside the
-    library).  ``out`` must be given by such a caller; it is created here only as a convenience
-    for tests."""
+    library call itself allocates nothing (its sums stay on chip).  ``out`` must be given by such a
+    caller; it is created here only as a convenience for tests."""
     torch = _torch()
     assert X.is_cuda and X.dtype == torch.bfloat16 and X.dim() == 2 and X.stride(1) == 1
     q, d_out, _ = bits.shape

@@ -94,7 +94,6 @@ extern "C" size_t bcq_workspace_bytes(int op, int d_out, int d_in, int q, int g,
         case BCQ_OP_DECODE: return n > 16 ? 0 : bcq::decode_workspace_bytes(d_out, d_in, q, g, n);
         case BCQ_OP_BWD_X: return bcq::bwd_x_workspace_bytes(d_out, d_in, q, g, n);
         case BCQ_OP_BWD_ALPHA: return bcq::bwd_alpha_workspace_bytes(d_out, d_in, q, g, n);
-        case BCQ_OP_DECODE_PACKED: return n > 16 ? 0 : bcq::decode_packed_workspace_bytes(d_out, d_in, q, g, n);
-        default: return 0;
+        default: return 0;  // BCQ_OP_QUANTIZE, BCQ_OP_DECODE_PACKED: sums stay on chip
     }
 }

@@ -7,8 +7,8 @@
 // 128 x 256 tile of a CTA alone takes 48 KiB into shared memory and reads 48 KiB back, 192 bytes a
 // cycle against the 128 of shared memory; in a pair each CTA holds half of the columns, 128 bytes a
 // cycle.  Measured, CTA alone and pair: 1600 -> 6400 with 4096 tokens 75.5 and 68.5 us, 5120 -> 20480
-// with 2048 tokens 326 and 276 us (1558 TFLOP/s).  The epilogue never writes D: thread = (row j, half of the tile's columns) reads
-// its accumulator row from tensor memory 32 columns at a time, applies the signs of every
+// with 2048 tokens 326 and 276 us (1558 TFLOP/s).  The epilogue never writes D: thread = (row j, half of
+// the tile's columns) reads its accumulator row from tensor memory 32 columns at a time, applies the signs of every
 // requested plane from one 32-bit word of the packed planes, and sums per group.  Partial sums
 // (one per split over tokens, column sub-tile and group piece) go to the workspace and a second
 // kernel adds them in a fixed order, so the result does not depend on scheduling.  When every

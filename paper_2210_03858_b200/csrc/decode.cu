@@ -832,8 +832,6 @@ bcq_status run_decode_planes(int d_out, int d_in, int q, int g, int n, const voi
     if (q == 4) return launch_decode_planes_tokens<4>(p, s);
     return launch_decode_planes_tokens<8>(p, s);
 }
-
-size_t decode_packed_workspace_bytes(int, int, int, int, int) { return 0; }
 }  // namespace bcq
 
 extern "C" size_t bcq_decode_pack_bytes(int d_out, int d_in, int q, int g) {

@@ -154,6 +154,5 @@ size_t fwd_workspace_bytes(int d_out, int d_in, int q, int g, int n);
 size_t decode_workspace_bytes(int d_out, int d_in, int q, int g, int n);
 size_t bwd_x_workspace_bytes(int d_out, int d_in, int q, int g, int n);
 size_t bwd_alpha_workspace_bytes(int d_out, int d_in, int q, int g, int n);
-size_t decode_packed_workspace_bytes(int d_out, int d_in, int q, int g, int n);
 
 }  // namespace bcq

@@ -4,14 +4,15 @@
 //
 // team_quantize_kernel (greedy for every q, alternating for q <= 4): a thread holds up to 32 weights, so
 // a group of 128 is four lanes and a warp works on eight groups (greedy; alternating takes 8 or 16
-// lanes, see launch_team_size); a team is up to a warp for g <= 1024 and a whole CTA above that.  Four lanes share 128 consecutive weights, lane l taking the 16-byte
+// lanes, see launch_team_size); a team is up to a warp for g <= 1024 (two warps for short alternating
+// problems) and a whole CTA above that.  Four lanes share 128 consecutive weights, lane l taking the 16-byte
 // pieces l, l + 4, ...: full 32-byte sectors from memory, and the four lanes' sign bits make four
 // container words with one 4 x 4 byte transpose.  With a warp per group (four weights a lane), as
 // this kernel worked before, a plane of 128 weights cost five rounds of 64-bit shuffles and a
 // ballot per 32 weights; now two rounds, and per weight and plane two fp64 additions and one shift
 // that collects the sign.  Measured, before and after: greedy q = 4, g = 128, the four linears of a
-// layer of width 1600 (30.7 M weights) 162 -> 69 us (2.1 TB/s; the logic pipe is 55 % busy, the fp64
-// pipe 21 %); five alternating rounds, q = 3, g = 128, 5120 x 5120: 1119 -> 350 us (instruction fetch of
+// layer of width 1600 (30.7 M weights) 162 -> 59 us (2.5 TB/s; the logic pipe is 55 % busy, the fp64
+// pipe 21 %); five alternating rounds, q = 3, g = 128, 5120 x 5120: 1119 -> 360 us (instruction fetch of
 // the unrolled rounds and fp64 latency at five warps per scheduler bound it).
 //
 // Sums are fp64 and are reduced in a fixed order, so a result never depends on scheduling.
@@ -557,7 +558,9 @@ __device__ __noinline__ void fit_not_finite(const QuantParams p, long long item,
 // lanes (TW = 1) or TW warps.
 template <int NI, int L, int TW, int Q>
 __global__ void __launch_bounds__(TW == 1 ? 128 : TW * 32,
-                                  TW == 1 ? (NI == 2 || (Q == 0 && NI == 4) ? 6 : Q == 0 || NI == 4 ? 5 : 3) : TW <= 4 ? (NI == 4 ? 20 : 12) / TW : 1)
+                                  TW == 1   ? (NI == 2 || (Q == 0 && NI == 4) ? 6 : Q == 0 || NI == 4 ? 5 : 3)
+                                  : TW <= 4 ? (NI == 4 ? 20 : 12) / TW
+                                            : 1)
 team_quantize_kernel(const QuantParams p) {
     constexpr bool ALT = Q > 0;
     constexpr int EPT = 4 * NI;

@@ -536,7 +536,7 @@ def test_decode_packed_matches_oracle(n, d_in, d_out, q, g):
     ref = oracle.fwd(X, bits, alpha, d_in, g)
     pack = bcq.decode_pack(bd, ad, d_in, g)
     Y = bcq.linear_decode_packed(Xd, pack, d_out, d_in, q, g)
-    Y2 = bcq.linear_decode_packed(Xd, pack, d_out, d_in, q, g)   # the pack's counters are back at zero
+    Y2 = bcq.linear_decode_packed(Xd, pack, d_out, d_in, q, g)
     torch.cuda.synchronize()
     assert torch.equal(Y, Y2)
     assert rel_err(Y.cpu().numpy(), ref) <= TOL

@@ -2,10 +2,9 @@
 
 A caller that may not call cudaMalloc (it runs where the allocator is off limits, or it was only
 handed its inputs and outputs) cannot give bcq_linear_decode a workspace.  The no-alloc entry
-point keeps the split-K partial sums in a fixed array inside the library instead.  This file
-checks, through the C ABI, that it gives the same result as bcq_linear_decode -- twice in a row,
-since the array is shared by all calls and keeps the previous call's contents -- and that a shape
-whose partial sums do not fit is refused before anything is launched.
+point needs none.  This file checks, through the C ABI, that it gives the same result as
+bcq_linear_decode -- twice in a row, since nothing may be left over from the call before -- and that a
+shape beyond the documented limit is refused before anything is launched.
 
 The file name sorts last on purpose: a run that stops at the first failure has then already run
 every other test.
@@ -46,7 +45,7 @@ def test_noalloc_decode_matches_decode_twice_in_a_row():
         out1 = torch.full((n, d_out), float("nan"), device="cuda")
         out2 = torch.full((n, d_out), float("nan"), device="cuda")
         bcq.linear_decode_noalloc(Xd, bd, ad, d_in, g, out=out1)
-        bcq.linear_decode_noalloc(Xd, bd, ad, d_in, g, out=out2)   # scratch still holds call 1's sums
+        bcq.linear_decode_noalloc(Xd, bd, ad, d_in, g, out=out2)
         torch.cuda.synchronize()
         scale = float(expect.abs().max())
         for out in (out1, out2):
@@ -56,8 +55,8 @@ def test_noalloc_decode_matches_decode_twice_in_a_row():
 
 
 def test_noalloc_decode_refuses_what_does_not_fit():
-    # the arguments are checked on the host before the scratch symbol is resolved or anything is
-    # launched, so the (16-byte aligned, never dereferenced) fake pointers are safe to pass
+    # the arguments are checked on the host before anything is launched, so the (16-byte aligned,
+    # never dereferenced) fake pointers are safe to pass
     lib = bcq.lib()
     p, null = C.c_void_p(256), C.c_void_p(0)
     d_out, d_in, q, g, n = 12288, 4096, 4, 128, 16       # 3 splits x 16 x 12288 floats > 2 MiB
