@@ -493,11 +493,20 @@ __device__ __forceinline__ bool greedy_sign_not_finite(float w, float a1, int pl
     return plane == 1 && (w >= 0.f ? (double)w - (double)a1 : (double)w + (double)a1) >= 0.0;
 }
 
+// First scale of a group: the mean of |w|.
+__device__ __noinline__ float first_scale(const float* w, int m) {
+    double S = 0.0;
+#pragma unroll 1
+    for (int k = 0; k < m; ++k) S += fabs((double)bcq::ld(w + k));
+    return (float)__ddiv_rn(S, (double)m);
+}
+
 // Container word `wi` of such a group in the greedy planes.
-__device__ __noinline__ void greedy_word_not_finite(const QuantParams p, long long item, int wi, float a1) {
+__device__ __noinline__ void greedy_word_not_finite(const QuantParams p, long long item, int wi) {
     const int j = (int)(item / p.G), k0 = (int)(item % p.G) * p.g + 32 * wi, m = min(min(p.g - 32 * wi, p.d_in - k0), 32);
     if (m <= 0) return;
     const float* w = p.W + (long long)j * p.ldw + k0;
+    const float a1 = first_scale(w - 32 * wi, min(p.g, p.d_in - k0 + 32 * wi));
 #pragma unroll 1
     for (int i = 0; i < p.q; ++i) {
         uint32_t word = 0u;
@@ -511,9 +520,11 @@ __device__ __noinline__ void greedy_word_not_finite(const QuantParams p, long lo
 // The scales (and the squared error) of such a group after alternating rounds, by the definition.  The right-hand
 // sides of a fit are not finite, so no level is nearer than another: after the first round every weight
 // has the largest code, and for q > 1 the fit is singular from then on.
-__device__ __noinline__ void fit_not_finite(const QuantParams p, long long item, float a1) {
+__device__ __noinline__ void fit_not_finite(const QuantParams p, long long item) {
     const int j = (int)(item / p.G), k0 = (int)(item % p.G) * p.g, m = min(p.g, p.d_in - k0), q = p.q;
     const float* w = p.W + (long long)j * p.ldw + k0;
+    const float a1 = first_scale(w, m);
+    if (fabsf(a1) <= 3.402823466e38f) return;  // finite weights, a scale that a fit took out of range
     double A[BCQ_MAX_Q][BCQ_MAX_Q + 1], plain = 0.0;
     float a[BCQ_MAX_Q];
     a[0] = a1;
@@ -698,11 +709,10 @@ team_quantize_kernel(const QuantParams p) {
                 if (t[e] == 0.0 && ((valid >> e) & 1u)) negs &= ~(1u << e);
         }
     };
-    float a1 = 0.f;  // first scale: not finite if a weight of the group is not
+    float last = 0.f;  // a scale that is not finite if a weight of the group is not
     if constexpr (!ALT) {
         for (int i = 0; i < q; ++i) {
-            const float ai = scale_of();
-            if (i == 0) a1 = ai;
+            const float ai = last = scale_of();
             const uint32_t word = transpose_bits(~negs);
             if (writes) dst[i * plane_words] = word & word_mask;
             if (live && tl == 0) adst[i * plane_alpha] = ai;
@@ -715,7 +725,6 @@ team_quantize_kernel(const QuantParams p) {
             neg[i] = negs;
             if (i + 1 < Q) next_residual(a[i]);
         }
-        a1 = a[0];
 
         // ---- alternating rounds.  From here on only magnitudes count: b_i w = (b_i sign(w)) |w|, so the
         // sums run over |w| with the signs `neg` relative to sign(w), and so do the mismatch counts.
@@ -847,6 +856,7 @@ team_quantize_kernel(const QuantParams p) {
                 sums_from_signs();
             }
         }
+        last = a[0];
         // ---- write the planes
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
@@ -887,14 +897,14 @@ team_quantize_kernel(const QuantParams p) {
         const double E = lanes_sum<L, TW>(tree_of_leaves(leaf), scratch);
         if (live && tl == 0) p.sq_err[(long long)j * p.G + c] = E;
     }
-    if (!(fabsf(a1) <= 3.402823466e38f)) {
+    if (!(fabsf(last) <= 3.402823466e38f)) {
         // rare: everything is formed again, so that nothing of it is kept for the sake of these calls
         uint32_t block;
         asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(block));
         const long long again = (long long)block * TEAMS + (TW == 1 ? threadIdx.x / L : 0);
         const int t = TW == 1 ? (int)(threadIdx.x & (L - 1)) : (int)threadIdx.x;
-        if (!ALT && again < p.items && (t & 3) < NI / 2) greedy_word_not_finite(p, again, (t >> 2) * (NI / 2) + (t & 3), a1);
-        if (ALT && again < p.items && t == 0) fit_not_finite(p, again, a1);
+        if (!ALT && again < p.items && (t & 3) < NI / 2) greedy_word_not_finite(p, again, (t >> 2) * (NI / 2) + (t & 3));
+        if (ALT && again < p.items && t == 0) fit_not_finite(p, again);
     }
 }
 
