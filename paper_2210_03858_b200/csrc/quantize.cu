@@ -17,11 +17,15 @@
 //
 // Sums are fp64 and are reduced in a fixed order, so a result never depends on scheduling.
 //
+// sorted_quantize_kernel (alternating, q = 2 .. 4, groups of up to 256, three rounds or more): see there.
+//
 // quantize_kernel (alternating, q > 4): one warp per group up to 1024 weights, a CTA above.
 //
 // Appendix "Details on BCQ Format": Eq. ap:1-ap:3 (greedy), Eq. ap:4 and the following
 // paragraph (alternating).
-#include "common.h"
+#include <algorithm>
+
+#include "gemm_common.cuh"
 
 namespace {
 
@@ -908,6 +912,643 @@ team_quantize_kernel(const QuantParams p) {
     }
 }
 
+// ------------------------------------------------------------------------------------------
+// alternating, groups of up to 256 weights: rounds on sorted magnitudes
+// ------------------------------------------------------------------------------------------
+//
+// In a round a weight's code depends on its magnitude alone, and does not decrease with it: the levels cut the
+// sorted magnitudes of a group into 2^(Q-1) runs.  So a group is sorted once, with the running sums of its
+// magnitudes beside it, and a round is Q = 3: three searches and as many differences of running sums,
+// whatever the group's size.  The greedy start is a tree of such cuts too.
+//
+// A warp takes up to 32 groups.  (1) In teams of L lanes it loads 32 / L groups at a time, sorts them in registers
+// (a network in each lane, then merges across the lanes) and puts keys and running sums into shared memory.
+// (2) Lane k does all rounds of group k, so a least-squares solve is done once per group and not by every lane
+// of a team.  (3) In teams again, the weights are read once more (from L2), find their levels and are
+// written as planes.  Warps are blocks of their own, so that some sort while others wait for the chains of fp64
+// divisions of (2); ten fit an SM (20 KiB each at groups of 128).
+//
+// The team kernel keeps a group in registers and goes through its weights in every round, and all lanes of a team solve.
+// Measured, that and this: 5120 x 5120, g = 128, q = 3: five rounds 364 and 169 us, fifteen 905 and 270; q = 4 689
+// and 297.  What bounds it now: min and max of the sort run at half rate (the logic pipe), and the code, 15 to 30 KiB for
+// a pass, comes slowly to eight warps an SM (stall no_instruction; 4.2 an issue with everything unrolled, 250 us).
+//
+// Key of a weight: its magnitude's bits shifted left by one, below them 1 where it is not negative: integers in the
+// order of the magnitudes, of equal ones the negative first.  That is the order in which sign(0) = +1 decides
+// a residual of exactly zero (a negative weight with |w| = a gets b = +1, that is, against its own sign, like
+// the smaller magnitudes; a positive one like the larger).
+constexpr uint32_t kNoKey = 0xFFFFFFFFu;  // behind every weight
+constexpr int kRun = 4;                   // keys between two running sums
+
+template <int N>
+__device__ __forceinline__ void sort_keys(uint32_t (&v)[N]) {  // Batcher's odd-even merge sort
+#pragma unroll
+    for (int p = 1; p < N; p *= 2)
+#pragma unroll
+        for (int k = p; k >= 1; k /= 2)
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const int at = i - k % p;  // pairs (i, i + k) inside blocks of 2 k from k mod p on
+                if (at >= 0 && at % (2 * k) < k && i + k < N && i / (2 * p) == (i + k) / (2 * p)) {
+                    const uint32_t a = v[i], b = v[i + k];
+                    v[i] = min(a, b);
+                    v[i + k] = max(a, b);
+                }
+            }
+}
+
+// N keys a lane, ascending in each lane, to ascending over the L lanes of a team (lane l: N l .. N l + N - 1).
+template <int N, int L>
+__device__ __forceinline__ void merge_lanes(uint32_t (&v)[N], int tl) {
+    // (loops: unrolled, the code of the kernel would not fit the instruction caches)
+#pragma unroll 1
+    for (int w = 2; w <= L; w *= 2) {
+        // the smaller half of two neighbouring sequences to the lower lanes ...
+        const bool upper = (tl & (w / 2)) != 0;
+#pragma unroll
+        for (int i = 0; i < N / 2; ++i) {
+            const uint32_t a = __shfl_xor_sync(0xffffffffu, v[N - 1 - i], w - 1), b = __shfl_xor_sync(0xffffffffu, v[i], w - 1);
+            v[i] = upper ? max(v[i], a) : min(v[i], a);
+            v[N - 1 - i] = upper ? max(v[N - 1 - i], b) : min(v[N - 1 - i], b);
+        }
+        // ... and each half, which rises and falls once, into order
+#pragma unroll 1
+        for (int d = w / 4; d >= 1; d /= 2) {
+            const bool up = (tl & d) != 0;
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const uint32_t a = __shfl_xor_sync(0xffffffffu, v[i], d);
+                v[i] = up ? max(v[i], a) : min(v[i], a);
+            }
+        }
+#pragma unroll
+        for (int d = N / 2; d >= 1; d /= 2)
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+                if ((i & d) == 0) {
+                    const uint32_t a = v[i], b = v[i + d];
+                    v[i] = min(a, b);
+                    v[i + d] = max(a, b);
+                }
+    }
+}
+
+// Keys of weights below the cut t of a greedy plane: magnitudes under t, and of those equal to t the negative ones.
+__device__ __forceinline__ uint32_t key_below(double t) {
+    if (!(t > 0.0)) return 0u;  // a zero counts as positive
+    const float f = __double2float_rd(t);
+    return (__float_as_uint(f) << 1) + ((double)f == t ? 1u : 2u);
+}
+
+__device__ __forceinline__ float key_magnitude(uint32_t key) { return __uint_as_float(key >> 1); }
+
+template <int NI, int L>
+struct SortedShape {
+    static_assert(L >= 4, "four lanes share 128 weights");
+    static constexpr int EPT = 4 * NI, C = EPT * L, TEAMS = 32 / L, RUNS = C / kRun;
+    static constexpr int GROUPS = C > 128 ? 16 : 32;  // of a warp: what leaves room for eight warps on an SM
+    static constexpr size_t bytes = (size_t)C * GROUPS * 4 + (size_t)(RUNS + 1) * GROUPS * 8;
+};
+
+constexpr int kSortWarps = 4;  // of a block, at most
+
+template <int NI, int L, int Q>
+__global__ void __launch_bounds__(32 * kSortWarps, 2)
+sorted_quantize_kernel(const QuantParams p, int batch) {
+    using Sh = SortedShape<NI, L>;
+    constexpr int EPT = Sh::EPT, C = Sh::C, TEAMS = Sh::TEAMS, RUNS = Sh::RUNS, GROUPS = Sh::GROUPS;
+    constexpr int N = 1 << (Q - 1);
+    constexpr int LEAF = 8, LEAVES = EPT / LEAF;  // see lanes_sum
+    constexpr uint32_t kMask = (1u << Q) - 1u;
+    extern __shared__ double sorted_smem[];
+    const int warp = threadIdx.x >> 5;
+    double* sums = sorted_smem + warp * (Sh::bytes / 8);                       // [RUNS + 1][GROUPS], the last row: of all
+    uint32_t* keys = reinterpret_cast<uint32_t*>(sums + (RUNS + 1) * GROUPS);  // [C][GROUPS]
+    const int lane = threadIdx.x & 31;
+    const int tl = lane & (L - 1);
+    // the column of a group is turned by the lane that holds the position, so that the lanes of a team store to
+    // different banks
+    auto key_at = [&](int pos, int grp) { return pos * GROUPS + (grp ^ ((pos / EPT) * TEAMS & (GROUPS - 1))); };
+    auto sum_at = [&](int run, int grp) { return run * GROUPS + (grp ^ ((run * kRun / EPT) * TEAMS & (GROUPS - 1))); };
+
+    bcq::pdl_wait();  // (and no pdl_trigger: a long kernel, see launch_pdl)
+    // (warps past the last group do it again)
+    const long long first = min(((long long)blockIdx.x * (blockDim.x >> 5) + warp) * batch, p.items - 1);
+    const int count = (int)min((long long)batch, p.items - first);  // groups of this warp
+
+    struct Place { int j, c, m; };
+    auto place = [&](long long item) {
+        Place x;
+        if (p.g_magic != 0u) {
+            x.j = (int)(__umulhi((uint32_t)item, p.g_magic) >> p.g_shift);
+            x.c = (int)((uint32_t)item - (uint32_t)x.j * (uint32_t)p.G);
+        } else {
+            x.j = (int)(item / p.G);
+            x.c = (int)(item - (long long)x.j * p.G);
+        }
+        x.m = min(p.g, p.d_in - x.c * p.g);
+        return x;
+    };
+    // Weight 4 i + e of a lane: 16 i + e after its first.
+    const int kt = (tl >> 2) * (16 * NI) + (tl & 3) * 4;
+    // pieces 4 from .. of a lane
+    auto load = [&](const Place& x, int from, auto& w) {
+        constexpr int COUNT = sizeof(w) / sizeof(float);
+        const float* src = p.W + (long long)x.j * p.ldw + x.c * p.g + kt + 16 * from;
+        if (x.m == C && p.vec) {
+#pragma unroll
+            for (int i = 0; i < COUNT / 4; ++i) {
+                const float4 v = bcq::ld(reinterpret_cast<const float4*>(src + 16 * i));
+                w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
+            }
+        } else {
+            const int left = x.m - kt - 16 * from;
+#pragma unroll
+            for (int e = 0; e < COUNT; ++e) w[e] = 16 * (e / 4) + e % 4 < left ? bcq::ld(src + 16 * (e / 4) + e % 4) : 0.0f;
+        }
+    };
+    // teams past the last group repeat it (the shuffles need every lane) and store nothing
+    auto group_of = [&](int pass) { return min(pass * TEAMS + lane / L, count - 1); };
+    const int passes = (batch + TEAMS - 1) / TEAMS;
+
+    // ---- (1) sort
+    {
+        Place at = place(first + group_of(0)), next = at;
+        float w[EPT];
+        load(at, 0, w);
+#pragma unroll 1
+        for (int pass = 0; pass < passes; ++pass) {
+            __syncthreads();
+            uint32_t v[EPT];
+#pragma unroll
+            for (int e = 0; e < EPT; ++e) {
+                const uint32_t b = __float_as_uint(__fmul_rn(w[e], -1.0f));
+                v[e] = __funnelshift_l(b, b, 1);
+            }
+            if (at.m < C) {
+#pragma unroll
+                for (int e = 0; e < EPT; ++e)
+                    v[e] = kt + 16 * (e / 4) + e % 4 >= at.m ? kNoKey : min(v[e], kNoKey - 1u);  // (a NaN has these bits)
+            }
+            if (pass + 1 < passes) {
+                next = place(first + group_of(pass + 1));
+                load(next, 0, w);
+            }
+            sort_keys<EPT>(v);
+            merge_lanes<EPT, L>(v, tl);
+            // running sums: in blocks of 16 keys from the left, the blocks in a scan over their numbers: an order that the
+            // lanes' share of a group does not show in
+            constexpr int BLOCK = EPT < 16 ? EPT : 16, BLOCKS = EPT / BLOCK;
+            double before[EPT / kRun], upto[BLOCKS];
+            auto add_blocks = [&](bool all) {
+#pragma unroll
+                for (int b = 0; b < BLOCKS; ++b) {
+                    double s = 0.0;
+#pragma unroll
+                    for (int e = b * BLOCK; e < (b + 1) * BLOCK; ++e) {
+                        if (e % kRun == 0) before[e / kRun] = s;
+                        if (all || v[e] != kNoKey) s += (double)key_magnitude(v[e]);
+                    }
+                    upto[b] = s;
+                }
+            };
+            if (at.m == C) add_blocks(true);
+            else add_blocks(false);
+#pragma unroll
+            for (int o = 1; o < C / BLOCK; o <<= 1) {
+                double from[BLOCKS];
+#pragma unroll
+                for (int b = 0; b < BLOCKS; ++b)  // block o before this one
+                    from[b] = o < BLOCKS && b >= o ? upto[b - o]
+                                                   : __shfl_up_sync(0xffffffffu, upto[(b - o) & (BLOCKS - 1)], o < BLOCKS ? 1 : o / BLOCKS, L);
+#pragma unroll
+                for (int b = 0; b < BLOCKS; ++b)
+                    if (tl * BLOCKS + b >= o) upto[b] = from[b] + upto[b];
+            }
+            double base[BLOCKS];
+            base[0] = __shfl_up_sync(0xffffffffu, upto[BLOCKS - 1], 1, L);
+            if (tl == 0) base[0] = 0.0;
+#pragma unroll
+            for (int b = 1; b < BLOCKS; ++b) base[b] = upto[b - 1];
+            const int grp = pass * TEAMS + lane / L;
+            if (grp < count) {
+#pragma unroll
+                for (int e = 0; e < EPT; ++e) keys[key_at(tl * EPT + e, grp)] = v[e];
+#pragma unroll
+                for (int r = 0; r < EPT / kRun; ++r) sums[sum_at(tl * (EPT / kRun) + r, grp)] = base[r * kRun / BLOCK] + before[r];
+                if (tl == L - 1) sums[RUNS * GROUPS + grp] = upto[BLOCKS - 1];
+            }
+            at = next;
+        }
+    }
+    __syncwarp();
+
+    // ---- (2) rounds: a group per lane
+    const int grp = min(lane, count - 1);
+    const long long item = first + grp;
+    float a[Q], a_cut[Q];  // scales; the scales that the last cuts were made for
+    LevelSearch<Q> ls;
+    {
+        const int m = place(item).m;
+        const double md = (double)m;
+        const double inv_m = m == p.g ? p.inv_g : (m & (m - 1)) == 0 ? 1.0 / md : 0.0;
+        const double total = sums[RUNS * GROUPS + grp];
+        auto mean = [&](double S) { return (float)(inv_m != 0.0 ? __dmul_rn(S, inv_m) : __ddiv_rn(S, md)); };
+        auto key = [&](int pos) { return keys[key_at(pos, grp)]; };
+        // number of keys below k, and the sum of their magnitudes
+        auto cut = [&](uint32_t k, double& sum) {
+            int r = 0;
+#pragma unroll
+            for (int s = RUNS / 2; s >= 1; s /= 2)
+                if (key((r + s) * kRun) < k) r += s;
+            double t = sums[sum_at(r, grp)];
+            int n = r * kRun;
+#pragma unroll
+            for (int e = 0; e < kRun; ++e) {
+                const uint32_t x = key(r * kRun + e);
+                if (x < k) {
+                    t += (double)key_magnitude(x);
+                    ++n;
+                }
+            }
+            sum = t;
+            return n;
+        };
+        // the runs: run s is cuts[s] .. cuts[s + 1] - 1; below[s] = sum of the magnitudes before it
+        int cuts[N + 1];
+        double below[N + 1];
+        cuts[0] = 0; below[0] = 0.0;
+        cuts[N] = m; below[N] = total;
+
+        const float amax = key_magnitude(key(m - 1));
+        float tiny = __int_as_float(0x7F800000);  // smallest magnitude that is not zero
+        {
+            int zeros = 0;
+#pragma unroll 1
+            while (zeros < m && key(zeros) < 2u) ++zeros;
+            if (zeros < m) tiny = key_magnitude(key(zeros));
+        }
+        // Greedy: plane i cuts every run of the planes before it at its centre, a sum of +-a_1 .. +-a_(i-1).  Cut s of
+        // the final ones, 1 .. N - 1, comes with plane turn(s).
+        auto turn = [](int s) {
+            int i = Q - 1;
+            for (; (s & 1) == 0; s >>= 1) --i;
+            return i;
+        };
+        double centre[N];
+        uint32_t at[N];  // keys below at[s] are below cut s
+#pragma unroll
+        for (int s = 0; s < N; ++s) { centre[s] = 0.0; at[s] = 0u; }
+        a[0] = mean(total);
+        centre[N / 2] = (double)a[0];
+        // codes of the runs, a nibble each: bit i set where plane i is against the sign of the weight
+        ls.codes = 0u;
+#pragma unroll
+        for (int s = 0; s < N; ++s)
+#pragma unroll
+            for (int i = 1; i < Q; ++i) ls.codes |= (uint32_t)(~(s >> (Q - 1 - i)) & 1) << (4 * s + i);
+        ls.delta = 0.f;
+#pragma unroll
+        for (int s = 0; s < N; ++s) ls.mid[s] = 0.f;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) a_cut[i] = 0.f;
+        bool close = false;  // some weight is too close to a cut to call in fp32
+        // Rounds 1 - Q .. -1 are the greedy planes, one body for all: unrolled, it would not fit the instruction caches
+#pragma unroll 1
+        for (int it = 1 - Q;; ++it) {
+            __syncthreads();
+            if (it < 0) {
+                const int plane = it + Q;
+#pragma unroll
+                for (int s = 1; s < N; ++s)
+                    if (plane == turn(s)) at[s] = key_below(centre[s]);
+            } else {
+            // ---- B^T w and B^T B from the runs
+            double A[Q][Q + 1], S[Q];
+            int agree[Q][Q];  // weights on which planes i and l agree, less the others
+            double part[N];
+            int num[N];
+#pragma unroll
+            for (int s = 0; s < N; ++s) {
+                part[s] = below[s + 1] - below[s];
+                num[s] = cuts[s + 1] - cuts[s];
+            }
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                S[i] = 0.0;
+#pragma unroll
+                for (int s = 0; s < N; ++s) {
+                    const uint32_t b = (ls.codes << (31 - 4 * s - i)) & 0x80000000u;
+                    S[i] += __hiloint2double(__double2hiint(part[s]) ^ (int)b, __double2loint(part[s]));
+                }
+#pragma unroll
+                for (int l = i + 1; l < Q; ++l) {
+                    agree[i][l] = 0;
+#pragma unroll
+                    for (int s = 0; s < N; ++s) {
+                        const uint32_t x = (ls.codes >> (4 * s + i)) ^ (ls.codes >> (4 * s + l));
+                        agree[i][l] += (x & 1u) ? -num[s] : num[s];
+                    }
+                }
+            }
+            // those weights get the code that the definition gives: the whole warp looks through the group
+            for (uint32_t todo = __ballot_sync(0xffffffffu, close); todo != 0u; todo &= todo - 1u) {
+                const int f = __ffs(todo) - 1;
+                auto of = [&](auto v) { return __shfl_sync(0xffffffffu, v, f); };
+                const int fm = of(m);
+                const uint32_t fcodes = of(ls.codes);
+                const float fdelta = of(0.5f * ls.delta);
+                float fmid[N], fa[Q];
+                int fcut[N];
+#pragma unroll
+                for (int s = 1; s < N; ++s) { fmid[s] = of(ls.mid[s]); fcut[s] = of(cuts[s]); }
+#pragma unroll
+                for (int i = 0; i < Q; ++i) fa[i] = of(a_cut[i]);
+                double dS[Q];
+                int dagree[Q][Q];
+#pragma unroll
+                for (int i = 0; i < Q; ++i) {
+                    dS[i] = 0.0;
+#pragma unroll
+                    for (int l = i + 1; l < Q; ++l) dagree[i][l] = 0;
+                }
+#pragma unroll 1
+                for (int e = lane; e < fm; e += 32) {
+                    const uint32_t k = keys[key_at(e, f)];
+                    const float x = key_magnitude(k);
+                    float near = x == 0.f ? __int_as_float(0x7F800000) : x;
+                    int run = 0;
+#pragma unroll
+                    for (int s = 1; s < N; ++s) {
+                        near = fminf(near, fabsf(x - fmid[s]));
+                        run += e >= fcut[s] ? 4 : 0;
+                    }
+                    if (near > fdelta) continue;
+                    const bool negative = (k & 1u) == 0u;
+                    const uint32_t was = (fcodes >> run) & kMask;
+                    const uint32_t now = (~nearest_code<Q>(negative ? -(double)x : (double)x, fa) & kMask) ^ (negative ? kMask : 0u);
+#pragma unroll
+                    for (int i = 0; i < Q; ++i) {
+                        if (((was ^ now) >> i) & 1u) dS[i] += ((now >> i) & 1u) ? -2.0 * (double)x : 2.0 * (double)x;
+#pragma unroll
+                        for (int l = i + 1; l < Q; ++l)
+                            dagree[i][l] += 2 * ((int)(((was >> i) ^ (was >> l)) & 1u) - (int)(((now >> i) ^ (now >> l)) & 1u));
+                    }
+                }
+                __syncwarp();
+#pragma unroll
+                for (int i = 0; i < Q; ++i) {
+                    const double d = warp_sum(dS[i]);
+                    if (lane == f) S[i] += d;
+#pragma unroll
+                    for (int l = i + 1; l < Q; ++l) {
+                        const int n = __reduce_add_sync(0xffffffffu, dagree[i][l]);
+                        if (lane == f) agree[i][l] += n;
+                    }
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                A[i][Q] = S[i];
+                A[i][i] = md;
+#pragma unroll
+                for (int l = i + 1; l < Q; ++l) A[i][l] = A[l][i] = (double)agree[i][l];
+            }
+            // ---- least-squares alpha for the current signs
+            solve_ls_static<Q>(md, A, a);
+            if (it == p.alt_iters) break;  // the last pass is the final refit only
+            // ---- every weight moves to the nearest level
+#pragma unroll
+            for (int i = 0; i < Q; ++i) a_cut[i] = a[i];
+            ls.build(a, amax);
+#pragma unroll
+            for (int s = 1; s < N; ++s) at[s] = __float_as_uint(ls.mid[s]) << 1;
+            }
+#pragma unroll
+            for (int s = 1; s < N; ++s) cuts[s] = cut(at[s], below[s]);
+            if (it < 0) {
+                const int plane = it + Q;
+                double S = 0.0;
+#pragma unroll
+                for (int t = 1; t < Q; ++t)
+#pragma unroll
+                    for (int s = 1; s < N; ++s)
+                        if (t == turn(s) && plane >= t) {
+                            const int half = N >> t, lo = s - half, hi = s + half;
+                            if (cuts[s] <= cuts[lo]) { cuts[s] = cuts[lo]; below[s] = below[lo]; }
+                            if (cuts[s] >= cuts[hi]) { cuts[s] = cuts[hi]; below[s] = below[hi]; }
+                            if (plane == t)
+                                S += ((below[hi] - below[s]) - (double)(cuts[hi] - cuts[s]) * centre[s]) +
+                                     ((double)(cuts[s] - cuts[lo]) * centre[s] - (below[s] - below[lo]));
+                        }
+                const float ai = mean(S);
+#pragma unroll
+                for (int i = 1; i < Q; ++i)
+                    if (plane == i) a[i] = ai;
+#pragma unroll
+                for (int s = 1; s < N; ++s)
+                    if (plane == turn(s)) {
+                        const int half = (N >> turn(s)) / 2;
+                        if (half > 0) {
+                            centre[s - half] = centre[s] - (double)ai;
+                            centre[s + half] = centre[s] + (double)ai;
+                        }
+                    }
+            } else {
+                float near = tiny;
+#pragma unroll
+                for (int s = 1; s < N; ++s) {
+                    if (cuts[s] > 0) near = fminf(near, ls.mid[s] - key_magnitude(key(cuts[s] - 1)));
+                    if (cuts[s] < m) near = fminf(near, key_magnitude(key(cuts[s])) - ls.mid[s]);
+                }
+                // fp32 decides where a weight is 2^-22 of the largest level away from the midpoint, which is rounded by
+                // 2^-24 of itself; half of ls.delta keeps the neighbourhoods of two midpoints apart
+                close = lane < count && !(near > 0.5f * ls.delta);
+            }
+        }
+    }
+    __syncwarp();
+    // what (3) needs of a group, in place of its keys
+    float* hand = reinterpret_cast<float*>(keys);  // [row][GROUPS]
+    constexpr int ROW_CODES = 0, ROW_DELTA = 1, ROW_CUT = 2, ROW_MID = ROW_CUT + Q, ROW_A = ROW_MID + N;
+    static_assert(ROW_A + Q <= C, "rows of the keys");
+    if (lane < count) {
+        keys[ROW_CODES * GROUPS + lane] = ls.codes;
+        hand[ROW_DELTA * GROUPS + lane] = ls.delta;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            hand[(ROW_CUT + i) * GROUPS + lane] = a_cut[i];
+            hand[(ROW_A + i) * GROUPS + lane] = a[i];
+            p.alpha[i * p.items + item] = a[i];
+        }
+#pragma unroll
+        for (int s = 1; s < N; ++s) hand[(ROW_MID + s) * GROUPS + lane] = ls.mid[s];
+    }
+    __syncwarp();
+
+    // ---- (3) planes, 16 weights of a lane at a time
+    {
+        constexpr int PART = EPT < 16 ? EPT : 16, PARTS = EPT / PART;
+        const long long plane_words = (long long)p.d_out * p.pitch;
+        Place at = place(first + group_of(0)), next = at;
+        float wn[PART];
+        uint32_t neg[Q];
+        double leaf[LEAVES];
+        load(at, (PARTS - 1) * (PART / 4), wn);
+#pragma unroll 1
+        for (int turn = 0; turn < passes * PARTS; ++turn) {
+            __syncthreads();
+            const int pass = turn / PARTS, part = PARTS - 1 - turn % PARTS;  // the last weights first
+            const int g3 = group_of(pass);
+            float w[PART];
+#pragma unroll
+            for (int e = 0; e < PART; ++e) w[e] = wn[e] + 0.0f;
+            if (turn + 1 < passes * PARTS) {
+                if (part == 0) next = place(first + group_of(pass + 1));
+                load(next, (part == 0 ? PARTS - 1 : part - 1) * (PART / 4), wn);
+            }
+            const uint32_t codes = keys[ROW_CODES * GROUPS + g3];
+            // bit e of past[s]: weight e is below cut s; every midpoint is subtracted from every weight, which leaves the
+            // choice of the code to a few operations on whole words
+            uint32_t sgn = 0u, zero = 0u, now[Q], past[N];
+            float mid[N];
+#pragma unroll
+            for (int s = 1; s < N; ++s) {
+                mid[s] = hand[(ROW_MID + s) * GROUPS + g3];
+                past[s] = 0u;
+            }
+            float near = __int_as_float(0x7F800000), least = near;
+#pragma unroll
+            for (int e = PART - 1; e >= 0; --e) {
+                sgn = __funnelshift_l(__float_as_uint(w[e]), sgn, 1);
+                const float x = fabsf(w[e]);
+                least = fminf(least, x);
+#pragma unroll
+                for (int s = 1; s < N; ++s) {
+                    const float d = x - mid[s];
+                    near = fminf(near, fabsf(d));
+                    past[s] = __funnelshift_l(__float_as_uint(d), past[s], 1);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                now[i] = 0u - ((codes >> (4 * (N - 1) + i)) & 1u);
+#pragma unroll
+                for (int s = 1; s < N; ++s) {
+                    const uint32_t turns = ((codes >> (4 * s + i)) ^ (codes >> (4 * s - 4 + i))) & 1u;
+                    now[i] ^= past[s] & (0u - turns);
+                }
+            }
+            if (least == 0.f) {
+                least = __int_as_float(0x7F800000);
+#pragma unroll
+                for (int e = 0; e < PART; ++e) {
+                    if (w[e] == 0.f) zero |= 1u << e;
+                    else least = fminf(least, fabsf(w[e]));
+                }
+                // a zero is equidistant from +L and -L, the larger code (plane Q - 1 at +1) wins
+                if (((codes >> (Q - 1)) & 1u) == 0u) zero = 0u;
+            }
+#pragma unroll
+            for (int i = 0; i < Q; ++i) now[i] = (now[i] ^ sgn ^ zero) & ((1u << PART) - 1u);
+            const float delta = hand[ROW_DELTA * GROUPS + g3];
+            if (!(fminf(near, least) > delta)) {
+                // some weights of this lane are too close to a cut to call in fp32
+                uint32_t hits = 0u;
+#pragma unroll
+                for (int e = 0; e < PART; ++e) {
+                    float d = fabsf(w[e]);
+                    if (d == 0.f && delta < 3.0e38f) d = __int_as_float(0x7F800000);
+#pragma unroll
+                    for (int s = 1; s < N; ++s) d = fminf(d, fabsf(fabsf(w[e]) - mid[s]));
+                    if (!(d > delta)) hits |= 1u << e;
+                }
+                float ac[Q];
+#pragma unroll
+                for (int i = 0; i < Q; ++i) ac[i] = hand[(ROW_CUT + i) * GROUPS + g3];
+                const float* src = p.W + (long long)at.j * p.ldw + at.c * p.g;
+#pragma unroll 1
+                for (; hits != 0u; hits &= hits - 1u) {
+                    const int e = __ffs(hits) - 1, k = kt + 4 * PART * part + 16 * (e / 4) + e % 4;
+                    const uint32_t code = nearest_code<Q>(k < at.m ? (double)(bcq::ld(src + k) + 0.0f) : 0.0, ac);
+#pragma unroll
+                    for (int i = 0; i < Q; ++i) now[i] = (now[i] & ~(1u << e)) | ((~(code >> i) & 1u) << e);
+                }
+            }
+            const bool live = pass * TEAMS + lane / L < count;
+            if (p.sq_err != nullptr) {
+#pragma unroll
+                for (int k = 0; k < PART / LEAF; ++k) {
+                    double sum = 0.0;
+#pragma unroll
+                    for (int e = k * LEAF; e < (k + 1) * LEAF; ++e) {
+                        double wh = 0.0;
+#pragma unroll
+                        for (int i = 0; i < Q; ++i) {
+                            const double ai = (double)hand[(ROW_A + i) * GROUPS + g3];
+                            wh = ((now[i] >> e) & 1u) ? wh - ai : wh + ai;
+                        }
+                        const double d = kt + 4 * PART * part + 16 * (e / 4) + e % 4 < at.m ? (double)w[e] - wh : 0.0;
+                        sum += d * d;
+                    }
+#pragma unroll
+                    for (int h = 0; h < PARTS; ++h)
+                        if (h == part) leaf[h * (PART / LEAF) + k] = sum;
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < Q; ++i) neg[i] = part == PARTS - 1 ? now[i] : (neg[i] << (PART & 31)) | now[i];
+            if (part > 0) continue;
+            const int wi = (tl >> 2) * (NI / 2) + (tl & 3);  // container word of the group this lane writes
+            const bool writes = live && (tl & 3) < NI / 2 && 32 * wi < at.m;
+            const uint32_t word_mask = at.m - 32 * wi >= 32 ? 0xFFFFFFFFu : (1u << ((at.m - 32 * wi) & 31)) - 1u;
+            uint32_t* row = p.bits + (long long)at.j * p.pitch;
+            uint32_t* dst = row + ((at.c * p.g) >> 5) + wi;
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                const uint32_t word = transpose_bits(~neg[i]);
+                if (writes) dst[i * plane_words] = word & word_mask;
+            }
+            // zero padding words of the row, optional squared error
+            if (at.c == p.G - 1 && live) {
+                const int first_pad = (p.d_in + 31) >> 5;
+                const int npad = p.pitch - first_pad;  // 0..3
+#pragma unroll 1
+                for (int e = tl; e < npad * Q; e += L) {
+                    const int i = e / npad;
+                    row[i * plane_words + first_pad + (e - i * npad)] = 0u;
+                }
+            }
+            if (p.sq_err != nullptr) {
+                double unused[1];
+                const double E = lanes_sum<L, 1>(tree_of_leaves(leaf), unused);
+                if (live && tl == 0) p.sq_err[(long long)at.j * p.G + at.c] = E;
+            }
+            at = next;
+        }
+    }
+    __syncwarp();
+    if (lane < count && !(fabsf(a[0]) <= 3.402823466e38f)) fit_not_finite(p, item);
+}
+
+// Groups to a warp: as few as fill the chip once (a warp goes through (1) and (3) 32 / L groups at a time, so a
+// small problem is over sooner with fewer), at most the 32 that (2) has lanes for (1600 x 1600, q = 2, g = 128: 26 us with 650
+// warps of 32 groups, 20 with 1300 of 16).  Four warps to a block in lockstep where there are three waves of them: they
+// share what they fetch of the code (5120 x 5120, g = 128, with warps on their own: q = 3 186 us and 183, q = 4 415 and 381).
+template <int NI, int L, int Q>
+cudaError_t launch_sorted(const QuantParams& p, cudaStream_t stream) {
+    using Sh = SortedShape<NI, L>;
+    const auto kern = sorted_quantize_kernel<NI, L, Q>;
+    const bcq_status st = bcq::ensure_dynamic_smem(kern, kSortWarps * Sh::bytes);
+    if (st != BCQ_OK) return cudaErrorUnknown;
+    const long long places = 9ll * bcq::sm_count();
+    int batch = std::max(Sh::TEAMS, 4);
+    while (batch < Sh::GROUPS && (p.items + batch - 1) / batch > places) batch *= 2;
+    const long long warps = (p.items + batch - 1) / batch;
+    const int per_block = warps >= 24ll * bcq::sm_count() ? kSortWarps : 1;
+    return bcq::launch_pdl(kern, dim3((unsigned)((warps + per_block - 1) / per_block)), 32 * per_block, per_block * Sh::bytes, stream, 1, p, batch);
+}
+
 template <int NI, int L, int TW, int Q>
 cudaError_t launch_team(const QuantParams& p, cudaStream_t stream) {
     constexpr int TEAMS = TW == 1 ? 128 / L : 1;
@@ -928,12 +1569,25 @@ cudaError_t launch_team(const QuantParams& p, cudaStream_t stream) {
 //                    64 x 512, q = 3 13.0 / 10.1 (so for every q, though two problems of q = 3 above lose 5 %)
 //   g = 256, q = 3   1406 x 1582 106 / 57 us     5120 x 5120 355 / 346
 //   a row, q = 3     1024 x 1024 80 / 53 us      2048 x 1536 128 / 98       3000 x 4096 231 / 288
+// From three rounds on groups of up to 256 go to the sorted kernel, which takes about 110 us for 5120 x 5120 before the
+// first round and 12 (q = 3) for each, where the team kernel takes 90 and 55 (one round, q = 2 / 3 / 4: 84 / 145 / 237
+// us here, 98 / 130 / 203 there; three 140 / 258 / 461 and 108 / 147 / 245; 1600 x 1600, one round 15 / 25 / 41 and 22 / 28 / 47,
+// three 22 / 40 / 81 and 24 / 31 / 45).  Problems of a few hundred groups are chains of latencies in both and lose 1 - 5 us there
+// (64 x 512, q = 3, five rounds 12.8 and 14.1).
 // The line between "few waves" and "long" is 30720 weights per SM (4.5 M on 148, three waves of the
 // 16-weight teams).
 template <int Q>
 cudaError_t launch_team_size(const QuantParams& p, cudaStream_t s) {
     const int g = p.g;
     const bool few = Q > 0 && p.items * g <= 30720ll * bcq::sm_count();
+    // (the choice must not depend on the number of rows: the two kernels add in different orders)
+    if constexpr (Q > 1)
+        if (p.alt_iters >= 3) {
+            if (g <= 32) return launch_sorted<2, 4, Q>(p, s);
+            if (g <= 64) return launch_sorted<4, 4, Q>(p, s);
+            if (g <= 128) return launch_sorted<8, 4, Q>(p, s);
+            if (g <= 256) return launch_sorted<8, 8, Q>(p, s);
+        }
     if (g <= 32) return launch_team<2, 4, 1, Q>(p, s);
     if (g <= 64) return launch_team<4, 4, 1, Q>(p, s);
     if constexpr (Q > 0) {

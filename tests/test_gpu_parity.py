@@ -186,6 +186,30 @@ def test_quantize_a_row_alone_and_among_many(d_in, g):
         assert torch.equal(b, bits[:, pick]) and torch.equal(a, alpha[:, pick]) and torch.equal(s, sq[pick])
 
 
+@pytest.mark.parametrize("alt", [3, 15])
+@pytest.mark.parametrize("d_in,g", [(32, 32), (64, 64), (130, 64), (288, 96), (420, 128), (256, 256), (1001, 256)])
+def test_quantize_rounds_on_sorted_magnitudes(d_in, g, alt):
+    # Values whose sums are exact in fp64 (see above), so that the bits are the oracle's: ties with a scale and with a
+    # midpoint, groups of one magnitude, of zeros, with one weight far above the rest, infinities and NaNs; rows
+    # that are no multiple of a warp's share, aligned and not, alone and 150 times.
+    rng = np.random.default_rng(d_in + alt)
+    W = (rng.integers(-40, 41, size=(13, d_in)) / 64.0).astype(np.float32)
+    W[0, ::3], W[1], W[2] = -0.0, 0.0, np.where(rng.random(d_in) < 0.5, 0.25, -0.25)
+    W[3] = rng.integers(-1, 2, size=d_in) * 0.5
+    W[4, d_in // 2] = 1024.0
+    W[5, 3], W[6, 5], W[7, 7], W[8, :], W[9, [1, 9]] = np.nan, np.inf, -np.inf, np.nan, (np.inf, -np.inf)
+    W[10, 0] = np.array([0x7FFFFFFF], np.uint32).view(np.float32)[0]
+    odd = torch.zeros((13, d_in + 1), dtype=torch.float32, device="cuda")[:, 1:]
+    odd.copy_(torch.from_numpy(W))
+    for q in (2, 3, 4):
+        bits_ref, alpha_ref, sq_ref, _ = oracle.quantize(W, q, g, alt_iters=alt)
+        for src, r in ((odd, 1), (torch.from_numpy(W).cuda(), 1), (torch.from_numpy(W).cuda().repeat(150, 1), 150)):
+            bits, alpha, sq = bcq.quantize(src, q, g, alt, want_sq_err=True)
+            np.testing.assert_array_equal(host_bits(bits), np.tile(bits_ref, (1, r, 1)))
+            np.testing.assert_allclose(alpha.cpu().numpy(), np.tile(alpha_ref, (1, r, 1)), rtol=1e-6, atol=1e-9, equal_nan=True)
+            np.testing.assert_allclose(sq.cpu().numpy(), np.tile(sq_ref, (r, 1)), rtol=1e-6, atol=1e-12, equal_nan=True)
+
+
 def test_quantize_strided_input_and_determinism():
     W = synth.weights(48, 384, (101, 0, 0))
     Wp = np.zeros((48, 400), dtype=np.float32)
