@@ -398,12 +398,14 @@ __device__ __forceinline__ void sort_levels(double (&L)[N], uint32_t (&c)[N]) {
     }
 }
 
-// Nearest of the 2^Q levels, the largest code among equidistant ones: the definition.
+// Nearest of the 2^Q levels, the largest code among equidistant ones: the definition.  (Unrolled, so that the chains
+// of the levels run side by side; scales by value, which keeps the callers' out of local memory.)
 template <int Q>
-__device__ __noinline__ uint32_t nearest_code(double w, const float (&a)[Q]) {
+__device__ __noinline__ uint32_t nearest_code_of(double w, float a0, float a1, float a2, float a3) {
+    const float a[4] = {a0, a1, a2, a3};
     uint32_t best = 0u;
     double dbest = 0.0;
-#pragma unroll 1
+#pragma unroll
     for (int s = (1 << Q) - 1; s >= 0; --s) {
         double L = 0.0;
 #pragma unroll
@@ -415,6 +417,10 @@ __device__ __noinline__ uint32_t nearest_code(double w, const float (&a)[Q]) {
         }
     }
     return best;
+}
+template <int Q>
+__device__ __forceinline__ uint32_t nearest_code(double w, const float (&a)[Q]) {
+    return nearest_code_of<Q>(w, a[0], a[Q > 1 ? 1 : 0], a[Q > 2 ? 2 : 0], a[Q > 3 ? 3 : 0]);
 }
 
 // What a round of the alternating method needs to know about the levels of a group.  They come in
@@ -926,7 +932,7 @@ team_quantize_kernel(const QuantParams p) {
 // (2) Lane k does all rounds of group k, so a least-squares solve is done once per group and not by every lane
 // of a team.  (3) In teams again, the weights are read once more (from L2), find their levels and are
 // written as planes.  Warps are blocks of their own, so that some sort while others wait for the chains of fp64
-// divisions of (2); ten fit an SM (20 KiB each at groups of 128).
+// divisions of (2); eight or nine fit an SM (25 KiB each).
 //
 // The team kernel keeps a group in registers and goes through its weights in every round, and all lanes of a team solve.
 // Measured, that and this: 5120 x 5120, g = 128, q = 3: five rounds 364 and 169 us, fifteen 905 and 270; q = 4 689
@@ -1212,7 +1218,8 @@ sorted_quantize_kernel(const QuantParams p, int batch) {
         for (int s = 0; s < N; ++s) ls.mid[s] = 0.f;
 #pragma unroll
         for (int i = 0; i < Q; ++i) a_cut[i] = 0.f;
-        bool close = false;  // some weight is too close to a cut to call in fp32
+        bool close = false;    // some weight is too close to a cut to call in fp32
+        bool settled = false;  // further rounds change nothing
         // Rounds 1 - Q .. -1 are the greedy planes, one body for all: unrolled, it would not fit the instruction caches
 #pragma unroll 1
         for (int it = 1 - Q;; ++it) {
@@ -1264,6 +1271,7 @@ sorted_quantize_kernel(const QuantParams p, int batch) {
                 for (int s = 1; s < N; ++s) { fmid[s] = of(ls.mid[s]); fcut[s] = of(cuts[s]); }
 #pragma unroll
                 for (int i = 0; i < Q; ++i) fa[i] = of(a_cut[i]);
+                bool changed = false;
                 double dS[Q];
                 int dagree[Q][Q];
 #pragma unroll
@@ -1287,6 +1295,7 @@ sorted_quantize_kernel(const QuantParams p, int batch) {
                     const bool negative = (k & 1u) == 0u;
                     const uint32_t was = (fcodes >> run) & kMask;
                     const uint32_t now = (~nearest_code<Q>(negative ? -(double)x : (double)x, fa) & kMask) ^ (negative ? kMask : 0u);
+                    changed |= now != was;
 #pragma unroll
                     for (int i = 0; i < Q; ++i) {
                         if (((was ^ now) >> i) & 1u) dS[i] += ((now >> i) & 1u) ? -2.0 * (double)x : 2.0 * (double)x;
@@ -1295,7 +1304,7 @@ sorted_quantize_kernel(const QuantParams p, int batch) {
                             dagree[i][l] += 2 * ((int)(((was >> i) ^ (was >> l)) & 1u) - (int)(((now >> i) ^ (now >> l)) & 1u));
                     }
                 }
-                __syncwarp();
+                if (!__any_sync(0xffffffffu, changed)) continue;
 #pragma unroll
                 for (int i = 0; i < Q; ++i) {
                     const double d = warp_sum(dS[i]);
@@ -1315,7 +1324,19 @@ sorted_quantize_kernel(const QuantParams p, int batch) {
                 for (int l = i + 1; l < Q; ++l) A[i][l] = A[l][i] = (double)agree[i][l];
             }
             // ---- least-squares alpha for the current signs
-            solve_ls_static<Q>(md, A, a);
+            float fit[Q];
+#pragma unroll
+            for (int i = 0; i < Q; ++i) fit[i] = a[i];
+            solve_ls_static<Q>(md, A, fit);
+            // scales that come out as they went in stay so, and with them the codes (where all magnitudes are alike every
+            // weight is too close to a cut, and this spares all rounds but one of looking at each)
+            bool same = it > 0;
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                if (!settled) a[i] = fit[i];
+                same = same && a[i] == a_cut[i];
+            }
+            settled = settled || same;
             if (it == p.alt_iters) break;  // the last pass is the final refit only
             // ---- every weight moves to the nearest level
 #pragma unroll
@@ -1363,7 +1384,7 @@ sorted_quantize_kernel(const QuantParams p, int batch) {
                 }
                 // fp32 decides where a weight is 2^-22 of the largest level away from the midpoint, which is rounded by
                 // 2^-24 of itself; half of ls.delta keeps the neighbourhoods of two midpoints apart
-                close = lane < count && !(near > 0.5f * ls.delta);
+                close = lane < count && !settled && !(near > 0.5f * ls.delta);
             }
         }
     }
@@ -1371,7 +1392,8 @@ sorted_quantize_kernel(const QuantParams p, int batch) {
     // what (3) needs of a group, in place of its keys
     float* hand = reinterpret_cast<float*>(keys);  // [row][GROUPS]
     constexpr int ROW_CODES = 0, ROW_DELTA = 1, ROW_CUT = 2, ROW_MID = ROW_CUT + Q, ROW_A = ROW_MID + N;
-    static_assert(ROW_A + Q <= C, "rows of the keys");
+    constexpr int ROWS = ROW_A + Q;
+    static_assert(ROWS * GROUPS + (EPT < 16 ? EPT : 16) * 32 <= C * GROUPS, "space of the keys");
     if (lane < count) {
         keys[ROW_CODES * GROUPS + lane] = ls.codes;
         hand[ROW_DELTA * GROUPS + lane] = ls.delta;
@@ -1466,11 +1488,13 @@ sorted_quantize_kernel(const QuantParams p, int batch) {
                 float ac[Q];
 #pragma unroll
                 for (int i = 0; i < Q; ++i) ac[i] = hand[(ROW_CUT + i) * GROUPS + g3];
-                const float* src = p.W + (long long)at.j * p.ldw + at.c * p.g;
+                float* copy = hand + ROWS * GROUPS + lane;  // (by way of shared memory: registers have no index)
+#pragma unroll
+                for (int e = 0; e < PART; ++e) copy[e * 32] = w[e];
 #pragma unroll 1
                 for (; hits != 0u; hits &= hits - 1u) {
-                    const int e = __ffs(hits) - 1, k = kt + 4 * PART * part + 16 * (e / 4) + e % 4;
-                    const uint32_t code = nearest_code<Q>(k < at.m ? (double)(bcq::ld(src + k) + 0.0f) : 0.0, ac);
+                    const int e = __ffs(hits) - 1;
+                    const uint32_t code = nearest_code<Q>((double)copy[e * 32], ac);
 #pragma unroll
                     for (int i = 0; i < Q; ++i) now[i] = (now[i] & ~(1u << e)) | ((~(code >> i) & 1u) << e);
                 }
