@@ -114,6 +114,7 @@ struct PrepParams {
     //            alpha_t [jb][G][q][64 rows]
     int mode, d_out, q, G, pitch, num_kb, amax_blocks, bits_blocks;
     int row_tiles;   // ceil(d_out / 128)
+    int alpha_w;     // groups to a block of the scales' regrouping: a power of two, at most 32
     int bits_cblk;   // ceil(pitch / 32): 32-word column blocks of the plane words
     const uint32_t* bits;
     float* alpha_t;
@@ -122,9 +123,9 @@ struct PrepParams {
     int num_counters;
 };
 
-// WPT warps per token row.  A lane keeps up to four 16-byte vectors of the row in registers between finding
-// the row's largest magnitude and writing the scaled fp16 row, so rows of up to 1024 WPT elements are
-// read once; longer rows (WPT = 8, more than 8192 elements) are read again from L2.  Four loads of a lane
+// WPT warps per token row.  A lane keeps up to HELD (four or twelve) 16-byte vectors of the row in registers between finding
+// the row's largest magnitude and writing the scaled fp16 row, so rows of up to 1024 WPT (24576) elements are
+// read once; longer rows are read again from L2.  Four loads of a lane
 // in flight and few registers: the token blocks are bound by memory (n x K x 4 bytes; with a warp per
 // token and two reads, 4096 x 6400 took 21 us and 4096 x 1600 8.5 us).
 // Blocks past the activation blocks scan alpha instead.
@@ -172,7 +173,7 @@ __device__ __forceinline__ uint4 scale_to_fp16x8(const uint4& x, int k0, int K, 
     return o;
 }
 
-template <int WPT>
+template <int WPT, int HELD = 4>
 __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
     __shared__ uint32_t red[8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -187,26 +188,41 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
         int b = bid - p.act_blocks - p.amax_blocks;
         if (b >= p.bits_blocks) {
             b -= p.bits_blocks;
-            // ---- scales of one plane and one tile of 128 rows: alpha[i][j][c] is contiguous over
-            // (j, c), so the block reads it as one coalesced run and scatters the values to their
-            // places in the regrouped array (rows past d_out become zeros)
-            const int rt = b % p.row_tiles;
-            const int i = b / p.row_tiles;
-            const float* src = p.alpha + ((long long)i * p.d_out + (long long)rt * 128) * p.G;
-            const int count = 128 * p.G;
+            // ---- scales of one plane, 128 rows x alpha_w groups: coalesced reads along the groups (alpha[i][j][c] is
+            // contiguous over (j, c)), coalesced writes along the rows (rows past d_out become zeros).  All loads
+            // of a thread are in flight at once: a block for all groups of 128 rows, one load at a time, took
+            // 0.8 us for every second group (d_in = 20480, g = 128, 2048 tokens: 70 us for the pre-pass, now 27)
+            const int w = p.alpha_w, shift = __ffs(w) - 1;
+            const int cblk = (p.G + w - 1) >> shift;
+            const int c0 = (b % cblk) << shift;
+            const int rt = (b / cblk) % p.row_tiles;
+            const int i = b / (cblk * p.row_tiles);
+            const float* src = p.alpha + ((long long)i * p.d_out + (long long)rt * 128) * p.G + c0;
             const int rows_left = p.d_out - rt * 128;
-            for (int e = threadIdx.x; e < count; e += 256) {
-                const int r = e / p.G, c = e - r * p.G;
-                const float v = (r < rows_left) ? ld(src + e) : 0.0f;
+            float held[16];
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                const int e = threadIdx.x + 256 * k, r = e >> shift, c = e & (w - 1);
+                held[k] = r < 128 && r < rows_left && c0 + c < p.G ? ld(src + (long long)r * p.G + c) : 0.0f;
+            }
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                const int e = threadIdx.x + 256 * k, r = e >> shift, c = e & (w - 1);
+                if (r < 128) tile[r][c] = __float_as_uint(held[k]);
+            }
+            __syncthreads();
+            for (int e = threadIdx.x; e < 128 * w; e += 256) {
+                const int r = e & 127, c = e >> 7;
+                if (c0 + c >= p.G) break;
                 long long o;
                 if (p.mode == MODE_FWD) {
-                    o = (((long long)rt * p.G + c) * p.q + i) * 128 + r;
+                    o = (((long long)rt * p.G + c0 + c) * p.q + i) * 128 + r;
                 } else {
                     const int jb = rt * 2 + (r >> 6), rr = r & 63;
                     if (jb >= p.num_kb) continue;
-                    o = (((long long)jb * p.G + c) * p.q + i) * 64 + rr;
+                    o = (((long long)jb * p.G + c0 + c) * p.q + i) * 64 + rr;
                 }
-                p.alpha_t[o] = v;
+                p.alpha_t[o] = __uint_as_float(tile[r][c]);
             }
             return;
         }
@@ -263,11 +279,30 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
         // ---- max |alpha| of this block's share of the scales
         if (bid == p.act_blocks)
             for (int i = threadIdx.x; i < p.num_counters; i += 256) p.counters[i] = 0u;
-        const long long nb = p.amax_blocks;
+        // (eight loads in flight; 16 bytes each where the scales are aligned)
+        const long long step = (long long)p.amax_blocks * 256, at = ((long long)bid - p.act_blocks) * 256 + threadIdx.x;
         uint32_t m = 0u;
-        for (long long o = ((long long)bid - p.act_blocks) * 256 + threadIdx.x; o < p.alpha_count;
-             o += nb * 256)
-            m = max(m, __float_as_uint(ld(p.alpha + o)) & 0x7FFFFFFFu);
+        long long done = 0;
+        if ((reinterpret_cast<uintptr_t>(p.alpha) & 15u) == 0) {
+            const long long nv = p.alpha_count >> 2;
+            const uint4* v4 = reinterpret_cast<const uint4*>(p.alpha);
+            for (long long o = at; o < nv; o += 8 * step) {
+                uint4 v[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v[k] = o + k * step < nv ? ld(v4 + o + k * step) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    m = max(m, max(max(v[k].x & 0x7FFFFFFFu, v[k].y & 0x7FFFFFFFu), max(v[k].z & 0x7FFFFFFFu, v[k].w & 0x7FFFFFFFu)));
+            }
+            done = nv << 2;
+        }
+        for (long long o = done + at; o < p.alpha_count; o += 8 * step) {
+            uint32_t v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = o + k * step < p.alpha_count ? __float_as_uint(ld(p.alpha + o + k * step)) : 0u;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) m = max(m, v[k] & 0x7FFFFFFFu);
+        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
         if (lane == 0) red[warp] = m;
@@ -276,7 +311,7 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
 #pragma unroll
             for (int w = 0; w < 8; ++w) m = max(m, red[w]);
             p.hdr->block_max[bid - p.act_blocks] = m;
-            if (bid == p.act_blocks) p.hdr->nblocks = (uint32_t)nb;
+            if (bid == p.act_blocks) p.hdr->nblocks = (uint32_t)p.amax_blocks;
         }
         return;
     }
@@ -289,17 +324,17 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
     uint4* dst = reinterpret_cast<uint4*>(p.out + (long long)t * p.ld_out);
     const int nvec = live ? (p.K + 7) / 8 : 0;
     uint32_t m = 0u;
-    uint4 held[4];
+    uint4 held[HELD];
     int v0 = tl;
     do {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < HELD; ++i) {
             const int v = v0 + kThreadsPerToken * i;
             held[i] = (v < nvec) ? ld(src + v) : make_uint4(0u, 0u, 0u, 0u);
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) m = max(m, max_mag_bf16x8(held[i], (v0 + kThreadsPerToken * i) * 8, p.K));
-        v0 += 4 * kThreadsPerToken;
+        for (int i = 0; i < HELD; ++i) m = max(m, max_mag_bf16x8(held[i], (v0 + kThreadsPerToken * i) * 8, p.K));
+        v0 += HELD * kThreadsPerToken;
     } while (v0 - tl < nvec);
     m = __reduce_max_sync(0xffffffffu, m);
     if (WPT > 1) {
@@ -311,21 +346,21 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
     const int sh = shift_for(exponent_of_bits(m << 16), 14);
     const float scale = pow2f(sh);
     if (live && tl == 0) p.tok_inv_scale[t] = pow2f(-sh);
-    if (nvec <= 4 * kThreadsPerToken) {
+    if (nvec <= HELD * kThreadsPerToken) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < HELD; ++i) {
             const int v = tl + kThreadsPerToken * i;
             if (v < nvec) dst[v] = scale_to_fp16x8(held[i], v * 8, p.K, scale);
         }
     } else {
-        for (v0 = tl; v0 < nvec; v0 += 4 * kThreadsPerToken) {
+        for (v0 = tl; v0 < nvec; v0 += HELD * kThreadsPerToken) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < HELD; ++i) {
                 const int v = v0 + kThreadsPerToken * i;
                 held[i] = (v < nvec) ? ld(src + v) : make_uint4(0u, 0u, 0u, 0u);
             }
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < HELD; ++i) {
                 const int v = v0 + kThreadsPerToken * i;
                 if (v < nvec) dst[v] = scale_to_fp16x8(held[i], v * 8, p.K, scale);
             }
@@ -1308,7 +1343,9 @@ bcq_status run_expand(int d_out, int d_in, int q, int g, int n, const void* act,
     pp.bits_cblk = ceil_div(pitch, 32);
     const bool coded = q <= 4;  // selector codes (written once, or by the launch below); q > 4: plane words
     pp.bits_blocks = coded ? 0 : q * pp.row_tiles * pp.bits_cblk;
-    const int alpha_tr_blocks = q * pp.row_tiles;  // one block per (plane, tile of 128 rows)
+    pp.alpha_w = 1;
+    while (pp.alpha_w < 32 && pp.alpha_w < pp.G) pp.alpha_w *= 2;
+    const int alpha_tr_blocks = q * pp.row_tiles * ceil_div(pp.G, pp.alpha_w);
     pp.bits = bits;
     pp.alpha_t = reinterpret_cast<float*>(wsb + pl.off_alpha);
     pp.bits_t = reinterpret_cast<uint32_t*>(wsb + pl.off_bits);
@@ -1323,7 +1360,7 @@ bcq_status run_expand(int d_out, int d_in, int q, int g, int n, const void* act,
     const int tok_blocks = ceil_div(n, kPrepWarps / wpt);
     pp.act_blocks = tok_blocks;
     const unsigned pgrid = (unsigned)(tok_blocks + ablocks + pp.bits_blocks + alpha_tr_blocks);
-    auto prep = wpt == 1 ? prepare_kernel<1> : wpt == 2 ? prepare_kernel<2> : wpt == 4 ? prepare_kernel<4> : prepare_kernel<8>;
+    auto prep = wpt == 1 ? prepare_kernel<1> : wpt == 2 ? prepare_kernel<2> : wpt == 4 ? prepare_kernel<4> : nvec <= 1024 || nvec > 3072 ? prepare_kernel<8> : prepare_kernel<8, 12>;
     BCQ_CUDA_TRY(launch_pdl(prep, dim3(pgrid), 256, 0, s, 1, pp));
 
     ExpandParams p;
