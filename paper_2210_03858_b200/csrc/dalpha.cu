@@ -32,7 +32,8 @@ struct DalphaParams {
     int m_tiles, n_tiles;
     int n_subtiles;      // column sub-tiles of width kHN over d_in
     int slots;           // partial slots per sub-tile
-    uint32_t plane_mask;
+    uint32_t planes;     // nibble k: the k-th plane of the mask
+    int num_planes;
     const uint32_t* bits;
     float* partial;      // [splits][n_subtiles][q][slots][d_out]
     // direct != 0: every output has exactly one partial (no token split, one group per column
@@ -52,7 +53,10 @@ constexpr int kHN = kTN / 2;   // of an epilogue sub-tile, and of the half of B 
 constexpr int kTM = 2 * kBlockM;
 constexpr int kStages = 6;
 constexpr uint32_t kStageBytes = kABytes + kHN * kBlockK * 2;  // 32 KiB
-constexpr size_t kDalphaSmem = (size_t)kStages * kStageBytes + 1024 + 256;
+// sign words of the epilogue's threads, [column chunk of 32][plane of the mask][thread]
+constexpr uint32_t kSignBytes = (kHN / 32) * BCQ_MAX_Q * kWorkerWarps * 32 * 4;  // 32 KiB
+constexpr size_t kDalphaSmem = (size_t)kStages * kStageBytes + 1024 + 256 + kSignBytes;
+static_assert(kDalphaSmem <= 232448, "shared memory of a CTA");
 
 // Persistent: every pair of CTAs walks over (row tile, column tile, token split) tiles; two
 // accumulators in tensor memory, so the sign-and-sum epilogue of one tile runs under the main loop of
@@ -209,10 +213,17 @@ dalpha_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant
         }
         __syncwarp();
     } else {
-        // ---------------- epilogue: thread = (row j, HN columns of the tile)
+        // ---------------- epilogue: thread = (row j, HN columns of the tile).  Loops over chunks and planes, not
+        // unrolled: a CTA has one to three tiles, so the code runs from cold instruction caches, and the time is what
+        // fetching it takes (written out for all planes and chunks, 50 KiB: the last epilogue of a call took 5.1 us with
+        // one plane; 1024 x 1024, one plane, 64 tokens 8.3 us a call and 6.1 now, 2048 tokens 11.9 and 9.8)
         const int quarter = warp & 3;
         const int half = (warp - kWorkerWarp0) >> 2;
+        const int et = (int)threadIdx.x - kWorkerWarp0 * 32;
+        constexpr int ET = kWorkerWarps * 32;
+        uint32_t* words = reinterpret_cast<uint32_t*>(ctl_gen + 256) + et;  // this thread's; [chunk * num_planes + plane] * ET
         const long long plane_words = (long long)p.d_out * p.pitch;
+        const int np = p.num_planes;
         bool ok = true;
         int lt = 0;
         for (int tile = pair0; tile < num_tiles && ok; tile += num_pairs, ++lt) {
@@ -225,15 +236,12 @@ dalpha_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant
             const int subtile = (k0 / kTN) * 2 + half;
 
             // the sign words do not depend on the accumulator: fetch them while the main loop runs
-            uint32_t nw[NCH][BCQ_MAX_Q];
+#pragma unroll 1
+            for (int i = 0; i < np; ++i) {
+                const uint32_t* src = p.bits + (long long)((p.planes >> (4 * i)) & 15u) * plane_words + (long long)j * p.pitch + (kbase >> 5);
 #pragma unroll
-            for (int ch = 0; ch < NCH; ++ch) {
-                const int kw = (kbase >> 5) + ch;
-#pragma unroll
-                for (int i = 0; i < BCQ_MAX_Q; ++i) {
-                    const bool act = (i < p.q) && ((p.plane_mask >> i) & 1u) && j_ok && (kw < p.pitch);
-                    nw[ch][i] = act ? ~ld(p.bits + i * plane_words + (long long)j * p.pitch + kw) : 0u;
-                }
+                for (int ch = 0; ch < NCH; ++ch)
+                    words[(ch * np + i) * ET] = j_ok && (kbase >> 5) + ch < p.pitch ? ~ld(src + ch) : 0u;
             }
 
             ok = wait_bar(ctl.accum + 8 * acc, (uint32_t)(lt >> 1) & 1u, ctl, 16, 512u);
@@ -241,56 +249,45 @@ dalpha_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant
             ptx::tc_fence_after_sync();
             if (kbase < p.d_in) {
                 const int c_first = min(kbase / p.g, p.G - 1);
-                float accs[BCQ_MAX_Q];
-#pragma unroll
-                for (int i = 0; i < BCQ_MAX_Q; ++i) accs[i] = 0.0f;
-                int cur_c = c_first;
-                auto flush = [&](int c) {
-                    if (!j_ok) return;
-                    const int slot = c - c_first;
-#pragma unroll
-                    for (int i = 0; i < BCQ_MAX_Q; ++i) {
-                        if (i < p.q && ((p.plane_mask >> i) & 1u)) {
-                            if (p.direct) {
-                                float* dst = p.dalpha + ((long long)i * p.d_out + j) * p.G + c;
-                                *dst = p.accumulate ? (*dst + p.scale * accs[i]) : (p.scale * accs[i]);
-                            } else {
-                                const long long idx =
-                                    ((((long long)z * p.n_subtiles + subtile) * p.q + i) * p.slots + slot) * p.d_out + j;
-                                p.partial[idx] = accs[i];
-                            }
-                        }
-                    }
-                };
-#pragma unroll
+                int c = c_first, next_edge = c < p.G - 1 ? (c + 1) * p.g : p.d_in;  // first column of the next group
+                bool fresh = true;
+#pragma unroll 1
                 for (int ch = 0; ch < NCH; ++ch) {
                     const int kg = kbase + ch * 32;
-                    if (kg < p.d_in) {  // uniform in the warp
-                        const int c = min(kg / p.g, p.G - 1);
-                        if (c != cur_c) {
-                            flush(cur_c);
-                            cur_c = c;
+                    if (kg >= p.d_in) break;  // uniform in the warp
+                    uint32_t v[32];
+                    ptx::tmem_ld_x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)acc * kAccCols +
+                                         (uint32_t)(half * HN + ch * 32), v);
+                    ptx::tmem_ld_wait();
+                    const bool last = ch == NCH - 1 || kg + 32 >= next_edge;  // of this group in this sub-tile
+#pragma unroll 1
+                    for (int i = 0; i < np; ++i) {
+                        const uint32_t w = words[(ch * np + i) * ET];
+                        float sum = 0.0f;
 #pragma unroll
-                            for (int i = 0; i < BCQ_MAX_Q; ++i) accs[i] = 0.0f;
-                        }
-                        uint32_t v[32];
-                        ptx::tmem_ld_x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)acc * kAccCols +
-                                             (uint32_t)(half * HN + ch * 32), v);
-                        ptx::tmem_ld_wait();
-#pragma unroll
-                        for (int i = 0; i < BCQ_MAX_Q; ++i) {
-                            if (i < p.q && ((p.plane_mask >> i) & 1u)) {
-                                const uint32_t w = nw[ch][i];
-                                float sum = 0.0f;
-#pragma unroll
-                                for (int b = 0; b < 32; ++b)
-                                    sum += __uint_as_float(v[b] ^ ((w << (31 - b)) & 0x80000000u));
-                                accs[i] += sum;
+                        for (int b = 0; b < 32; ++b)
+                            sum += __uint_as_float(v[b] ^ ((w << (31 - b)) & 0x80000000u));
+                        // the group's sum so far waits in place of the plane's first sign word, which is used up
+                        uint32_t* so_far = words + i * ET;
+                        if (!fresh) sum = __uint_as_float(*so_far) + sum;
+                        if (!last) {
+                            *so_far = __float_as_uint(sum);
+                        } else if (j_ok) {
+                            const int plane = (int)(p.planes >> (4 * i)) & 15;
+                            if (p.direct) {
+                                float* dst = p.dalpha + ((long long)plane * p.d_out + j) * p.G + c;
+                                *dst = p.accumulate ? (*dst + p.scale * sum) : (p.scale * sum);
+                            } else {
+                                p.partial[((((long long)z * p.n_subtiles + subtile) * p.q + plane) * p.slots + (c - c_first)) * p.d_out + j] = sum;
                             }
                         }
                     }
+                    fresh = last;
+                    if (kg + 32 >= next_edge) {
+                        ++c;
+                        next_edge = c < p.G - 1 ? next_edge + p.g : p.d_in;
+                    }
                 }
-                flush(cur_c);
             }
             // the accumulator may be overwritten by the tile after next
             ptx::tc_fence_before_sync();
@@ -426,7 +423,10 @@ extern "C" bcq_status bcq_linear_bwd_alpha(int d_out, int d_in, int q, int g, in
     p.pitch = (int)bcq_pitch_words(d_in);
     p.n = n; p.num_kb = pl.num_kb; p.kb_per_split = pl.kb_per_split; p.splits = pl.splits;
     p.m_tiles = pl.m_tiles; p.n_tiles = pl.n_tiles;
-    p.n_subtiles = pl.n_subtiles; p.slots = pl.slots; p.plane_mask = plane_mask;
+    p.n_subtiles = pl.n_subtiles; p.slots = pl.slots;
+    p.planes = 0; p.num_planes = 0;
+    for (int i = 0; i < q; ++i)
+        if ((plane_mask >> i) & 1u) p.planes |= (uint32_t)i << (4 * p.num_planes++);
     p.bits = bits; p.partial = reinterpret_cast<float*>(ws);
     p.direct = (pl.splits == 1 && g == kHN) ? 1 : 0;
     p.accumulate = accumulate; p.scale = scale; p.dalpha = dalpha;
@@ -440,12 +440,8 @@ extern "C" bcq_status bcq_linear_bwd_alpha(int d_out, int d_in, int q, int g, in
     if (p.direct) return BCQ_OK;
     // (only blocks of planes in the mask: the others would wait for this kernel and leave.  q = 8, one plane,
     // 5120 x 5120, g = 64, 64 tokens: 143 us with them, 52 without)
-    uint32_t planes = 0;
-    int count = 0;
-    for (int i = 0; i < q; ++i)
-        if ((plane_mask >> i) & 1u) planes |= (uint32_t)i << (4 * count++);
-    const long long rblocks = (long long)count * p.G * ((d_out + 31) / 32);
+    const long long rblocks = (long long)p.num_planes * p.G * ((d_out + 31) / 32);
     BCQ_CUDA_TRY(launch_pdl(dalpha_reduce_kernel, dim3((unsigned)rblocks), 256, 0, s, 1, d_out, d_in, q, g, p.G, kHN, pl.splits,
-                            pl.n_subtiles, pl.slots, planes, scale, accumulate, (const float*)p.partial, dalpha));
+                            pl.n_subtiles, pl.slots, p.planes, scale, accumulate, (const float*)p.partial, dalpha));
     return BCQ_OK;
 }
