@@ -77,21 +77,18 @@ struct CodeWords {
 // pre-pass: activations -> fp16 with a per-token power-of-two scale; max |alpha|
 // ------------------------------------------------------------------------------------------
 
-constexpr int kMaxAlphaBlocks = 124;
+constexpr int kMaxAlphaBlocks = 128;
 
-// Head of the forward / dX workspace: max |alpha| of each pre-pass block that scanned alpha (bit
-// patterns; the consumer takes the maximum over the first `nblocks`).  No zero-initialisation.
+// Head of the forward / dX workspace: max |alpha| of each pre-pass block that scanned alpha (bit patterns), zeros
+// for blocks that there are not: a lane of the consumer takes four with one load, and nothing has to be read first.
 struct WsHeader {
-    uint32_t nblocks;
-    uint32_t pad[3];
     uint32_t block_max[kMaxAlphaBlocks];
 };
 
 // Power of two for the weights: q * max|alpha| lands in [2^13, 2^14).  Called by whole warps.
 __device__ __forceinline__ int weight_shift(const WsHeader* hdr, int q) {
-    const int nb = (int)min(ld(&hdr->nblocks), (uint32_t)kMaxAlphaBlocks);  // never past the header
-    uint32_t m = 0u;
-    for (int b = threadIdx.x & 31; b < nb; b += 32) m = max(m, ld(&hdr->block_max[b]));
+    const uint4 v = ld(reinterpret_cast<const uint4*>(hdr->block_max) + (threadIdx.x & 31));
+    uint32_t m = max(max(v.x, v.y), max(v.z, v.w));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     return shift_for(exponent_of_bits(__float_as_uint(__uint_as_float(m) * (float)q)), 13);
@@ -277,8 +274,10 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
     }
     if (bid >= p.act_blocks) {
         // ---- max |alpha| of this block's share of the scales
-        if (bid == p.act_blocks)
+        if (bid == p.act_blocks) {
             for (int i = threadIdx.x; i < p.num_counters; i += 256) p.counters[i] = 0u;
+            for (int i = p.amax_blocks + threadIdx.x; i < kMaxAlphaBlocks; i += 256) p.hdr->block_max[i] = 0u;
+        }
         // (eight loads in flight; 16 bytes each where the scales are aligned)
         const long long step = (long long)p.amax_blocks * 256, at = ((long long)bid - p.act_blocks) * 256 + threadIdx.x;
         uint32_t m = 0u;
@@ -311,7 +310,6 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
 #pragma unroll
             for (int w = 0; w < 8; ++w) m = max(m, red[w]);
             p.hdr->block_max[bid - p.act_blocks] = m;
-            if (bid == p.act_blocks) p.hdr->nblocks = (uint32_t)p.amax_blocks;
         }
         return;
     }
@@ -824,7 +822,7 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
         const int wid = pf_worker_index(warp);  // 0..15
         const int group = wid / kPfGroupWarps;  // takes the stages whose running index is `group` mod kPfGroups
         const int wl = wid % kPfGroupWarps;
-        const float wscale = pow2f(weight_shift(p.hdr, p.q));
+        float wscale = 0.0f;  // known once the first loads are on their way
 
         // A task is one 128-byte line of the weight tile: 64 weights of one row.
         // fwd : (weight row m0 + row, the stage's 64 k); a warp takes 32 consecutive rows
@@ -1008,6 +1006,7 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
         float avA[NSC], avB[NSC];
         if (QM == QM_GENERIC) {
             // q > 4: one set of registers, loaded at the head of the task (under the wait for the slot)
+            wscale = pow2f(weight_shift(p.hdr, p.q));
             while (cur.valid && ok) {
                 issue(cur, cvA, avA);
                 ok = process(cur, cvA, avA);
@@ -1017,6 +1016,7 @@ expand_gemm_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_cons
             // q <= 4: the loads of the next task are in flight while this one is expanded (two
             // register sets, so that nothing has to wait for a load in order to be moved)
             if (cur.valid) issue(cur, cvA, avA);
+            wscale = pow2f(weight_shift(p.hdr, p.q));
             while (cur.valid && ok) {
                 Cur nxt = cur;
                 advance(nxt);
