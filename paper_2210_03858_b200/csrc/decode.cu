@@ -29,7 +29,10 @@
 // for (OPT-6.7B layer, q = 4, one token: 68 us against 53); 20 or 24 warps with fewer registers each
 // were no faster (54 us) and slower for 16 tokens (73 and 92 us against 66).
 //
-// Weights go from global memory to registers two units ahead of their use.  The kernel may start
+// Weights go from global memory to registers a unit ahead of their use, and the code of a unit is there once: two register
+// sets in turn, two units ahead, doubled it, and a loop that fits the instruction caches gains more than the distance
+// (4096 -> 16384, q = 4, one token 15.2 us and 13.9; the same pack from L2 takes no less time than from memory, so what
+// bounds a unit is not its way here but the logic pipe).  The kernel may start
 // while the previous kernel of the stream is finishing (programmatic dependent launch).  That may be the
 // kernel that writes the pack, and only the grid dependency wait makes its writes visible, so nothing
 // is read before it; the first two units are merely brought into L2.
@@ -390,13 +393,12 @@ decode_packed_kernel(const DecPackedParams p) {
                 for (int a = 0; a < PARTS; ++a) lp_tables[a] += tables_stride;
             }
         };
-        UnitWords<Q, PARTS> ua, ub;
+        UnitWords<Q, PARTS> next;
         seek();
         if (first == 0) touch();
         for (int i = 0; i < round_n * NT; ++i) mine[i * 32] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (first == 0) pdl_wait();
-        load(ua);
-        load(ub);
+        load(next);
         if (first == 0) {
             // the activations of the warp's later steps: into L1 while the first step is at work
             // (32 lanes: 16 tokens x two 128-byte lines of a step)
@@ -431,7 +433,6 @@ decode_packed_kernel(const DecPackedParams p) {
         int u_st = st0, u_i = i0;
         bool fresh = true;
         auto unit = [&](const UnitWords<Q, PARTS>& u) {
-            if (fresh) load_x(u_st);
             float d[NT][4];
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt) d[nt][0] = d[nt][1] = d[nt][2] = d[nt][3] = 0.f;
@@ -465,13 +466,11 @@ decode_packed_kernel(const DecPackedParams p) {
             if (fresh) { u_i = 0; ++u_st; }
         };
 #pragma unroll 1
-        for (int u = u0; u < u1; u += 2) {
-            unit(ua);
-            load(ua);
-            if (u + 1 < u1) {
-                unit(ub);
-                load(ub);
-            }
+        for (int u = u0; u < u1; ++u) {
+            if (fresh) load_x(u_st);
+            const UnitWords<Q, PARTS> now = next;
+            load(next);
+            unit(now);
         }
 
         __syncthreads();
@@ -619,9 +618,8 @@ decode_planes_kernel(const DecPlanesParams p) {
                 l_c = group_of(++l_st);
             }
         };
-        PlaneWords<NQ> ua, ub;
-        load(ua);
-        if (NQ < 8) load(ub);
+        PlaneWords<NQ> next;
+        load(next);
         for (int i = 0; i < round_n * NT; ++i) mine[i * 32] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (first == 0) {
             for (int s = st0 + 1; (s - step0) * round_n < u1; ++s) {
@@ -675,7 +673,6 @@ decode_planes_kernel(const DecPlanesParams p) {
             return shift_for(exponent_of_bits(m), 13);
         };
         auto unit = [&](const PlaneWords<NQ>& u) {
-            if (fresh) load_x(u_st);
             const int sa = row_shift(u.aa), sb = row_shift(u.ab);
             RowExpand<NQ> ea, eb;
             ea.begin(u.wa, u.aa, pow2f(sa));
@@ -710,22 +707,16 @@ decode_planes_kernel(const DecPlanesParams p) {
             fresh = (++u_i == round_n);
             if (fresh) { u_i = 0; ++u_st; }
         };
-        if (NQ == 8) {
-            // one unit's registers are all there is room for
 #pragma unroll 1
-            for (int u = u0; u < u1; ++u) {
-                unit(ua);
-                load(ua);
-            }
-        } else {
-#pragma unroll 1
-            for (int u = u0; u < u1; u += 2) {
-                unit(ua);
-                load(ua);
-                if (u + 1 < u1) {
-                    unit(ub);
-                    load(ub);
-                }
+        for (int u = u0; u < u1; ++u) {
+            if (fresh) load_x(u_st);
+            if (NQ == 8) {  // one unit's registers are all there is room for
+                unit(next);
+                load(next);
+            } else {
+                const PlaneWords<NQ> now = next;
+                load(next);
+                unit(now);
             }
         }
         __syncthreads();
