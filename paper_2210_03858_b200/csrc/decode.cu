@@ -50,6 +50,7 @@ constexpr int kDpThreads = kDpWarps * 32;
 constexpr int kDpStepK = 128;      // weights of a row per unit: eight K = 16 MMAs
 constexpr int kDpRows = 16;        // rows of a unit: the M of the MMA
 constexpr uint32_t kDpTableBytes = kDpRows * 16;  // tables of one (tile, group)
+constexpr size_t kDpMaxSmem = 232448;  // of a CTA
 constexpr int kDpMaxRound = 24;    // tiles a CTA takes between two additions of its warps' sums
 
 // ------------------------------------------------------------------------------------------
@@ -271,6 +272,7 @@ struct DecPackedParams {
     int per, rem;            // row tiles per CTA and remainder
     int round;               // tiles between two additions
     int split;               // CTAs of a cluster that share the steps of their tiles
+    uint32_t x_stride;       // XS: bytes of a token's fragments in shared memory
     uint32_t g_magic;        // ceil(2^32 / g) where k / g = hi32(k g_magic) for every k < d_in, else 0
     const __nv_bfloat16* X;
     long long ldx;
@@ -316,7 +318,9 @@ struct UnitWords {
     uint4 ta[PARTS], tb[PARTS];  // tables of rows g and g + 8
 };
 
-template <int Q, int NT, int PARTS, bool SPLIT>
+// XS (few tokens, see launch_decode_packed): the CTA's activations are converted once, by all threads, into shared memory.  A
+// warp that converts a step for itself works for eight tokens whatever their number, and again for every step.
+template <int Q, int NT, int PARTS, bool SPLIT, bool XS>
 __global__ void __launch_bounds__(kDpThreads, 1)
 decode_packed_kernel(const DecPackedParams p) {
     extern __shared__ float4 sums[];  // [warp][slot][NT][32 lanes]
@@ -330,6 +334,10 @@ decode_packed_kernel(const DecPackedParams p) {
     const int step0 = SPLIT ? (int)((long long)p.steps * part / p.split) : 0;
     const int nsteps = SPLIT ? (int)((long long)p.steps * (part + 1) / p.split) - step0 : p.steps;
     float4* mine = sums + (size_t)warp * p.round * (NT * 32) + lane;
+
+    // XS: fragments [token][step][r][t] of 16 bytes, then the inverse scales [token][step]
+    uint8_t* xfrag = reinterpret_cast<uint8_t*>(sums + (size_t)kDpWarps * p.round * (NT * 32));
+    float* xinv = reinterpret_cast<float*>(xfrag + (size_t)p.n * p.x_stride);
 
     pdl_trigger();
     for (int first = 0; first < ntiles; first += p.round) {
@@ -399,7 +407,29 @@ decode_packed_kernel(const DecPackedParams p) {
         for (int i = 0; i < round_n * NT; ++i) mine[i * 32] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (first == 0) pdl_wait();
         load(next);
-        if (first == 0) {
+        if (XS && first == 0) {
+            const int items = p.n * nsteps * 4;  // four lanes hold a step of a token
+            for (int e = threadIdx.x; e < ((items + 31) & ~31); e += kDpThreads) {
+                const int ts = e >> 2, tok = ts / nsteps, st = ts - tok * nsteps;
+                const int kb = (step0 + st) * kDpStepK + tq * 8;
+                const __nv_bfloat16* src = p.X + (long long)tok * p.ldx + kb;
+                uint4 v[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    v[r] = make_uint4(0u, 0u, 0u, 0u);
+                    if (e < items && kb + r * 32 < p.d_in) v[r] = ld(reinterpret_cast<const uint4*>(src + r * 32));
+                }
+                const float inv = scale_fragment(v, kb, 32, p.d_in, (step0 + st) * kDpStepK + kDpStepK > p.d_in);
+                if (e < items) {
+                    uint4* dst = reinterpret_cast<uint4*>(xfrag + (size_t)tok * p.x_stride + st * 256) + tq;
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) dst[4 * r] = v[r];
+                    if (tq == 0) xinv[tok * nsteps + st] = inv;
+                }
+            }
+            __syncthreads();
+        }
+        if (!XS && first == 0) {
             // the activations of the warp's later steps: into L1 while the first step is at work
             // (32 lanes: 16 tokens x two 128-byte lines of a step)
             for (int s = st0 + 1; (s - step0) * round_n < u1; ++s) {
@@ -414,6 +444,15 @@ decode_packed_kernel(const DecPackedParams p) {
         uint4 xb[NT][4];
         float f0[NT], f1[NT];  // inverse scales of the tokens of this lane's sums: 2 t, 2 t + 1
         auto load_x = [&](int st) {
+            if constexpr (XS) {
+                const int at = st - step0;
+                const uint4* src = reinterpret_cast<const uint4*>(xfrag + (size_t)gr * p.x_stride + at * 256) + tq;
+#pragma unroll
+                for (int r = 0; r < 4; ++r) xb[0][r] = gr < p.n ? src[4 * r] : make_uint4(0u, 0u, 0u, 0u);
+                f0[0] = 2 * tq < p.n ? xinv[2 * tq * nsteps + at] : 0.f;
+                f1[0] = 2 * tq + 1 < p.n ? xinv[(2 * tq + 1) * nsteps + at] : 0.f;
+                return;
+            }
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt) {
                 const int tok = nt * 8 + gr;
@@ -758,8 +797,22 @@ size_t deal_tiles(Params& p, int tiles, int* ctas) {
 template <int Q, int NT, int PARTS>
 bcq_status launch_decode_packed(DecPackedParams p, int tiles, cudaStream_t s) {
     int ctas;
-    const size_t smem = deal_tiles<NT>(p, tiles, &ctas);
-    auto kern = p.split > 1 ? decode_packed_kernel<Q, NT, PARTS, true> : decode_packed_kernel<Q, NT, PARTS, false>;
+    size_t smem = deal_tiles<NT>(p, tiles, &ctas);
+    const int steps = ceil_div(p.steps, p.split);  // of a CTA, at most
+    p.x_stride = (uint32_t)steps * 256u + 64u;     // (64 bytes more: tokens next to each other in other banks)
+    const size_t x_bytes = (size_t)p.n * (p.x_stride + steps * sizeof(float));
+    // Activations by way of shared memory: for up to four tokens, where they fit.  With two tokens the CTA's conversion is an eighth
+    // to a quarter of what its warps do otherwise; with four it needs more than one step a warp to be less, with eight it
+    // is as much, behind a barrier; four tables a step (PARTS = 4) leave no registers for it.  q = 4, without and with, us:
+    //   4096 -> 4096   one token 6.12 / 5.84, two 6.18 / 5.99, four 6.22 / 6.17, eight 6.30 / 7.01
+    //   16384 -> 4096, one token 19.0 / 15.6; 4096 -> 16384, one token 13.9 / 13.3; 2048 -> 2048, four tokens 3.27 / 3.38
+    //   2048 -> 2048, g = 32, one token 3.60 / 4.11
+    constexpr bool CAN = NT == 1 && PARTS <= 2;
+    const bool xs = CAN && p.n <= (p.steps > kDpWarps ? 4 : 2) && smem + x_bytes <= kDpMaxSmem;
+    if (xs) smem += x_bytes;
+    void (*kern)(DecPackedParams) = p.split > 1 ? decode_packed_kernel<Q, NT, PARTS, true, false> : decode_packed_kernel<Q, NT, PARTS, false, false>;
+    if constexpr (CAN)
+        if (xs) kern = p.split > 1 ? decode_packed_kernel<Q, NT, PARTS, true, true> : decode_packed_kernel<Q, NT, PARTS, false, true>;
     const bcq_status st = ensure_dynamic_smem(kern, smem);
     if (st != BCQ_OK) return st;
     BCQ_CUDA_TRY(launch_pdl(kern, dim3((unsigned)ctas), kDpThreads, smem, s, (unsigned)p.split, p));

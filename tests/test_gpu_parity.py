@@ -623,6 +623,24 @@ def test_decode_right_after_packing_into_a_used_buffer(d_in, d_out, q, g, n):
         assert torch.equal(out, ref[i % 2]), i
 
 
+@pytest.mark.parametrize("d_in,d_out,q,g", [(100, 40, 2, 100), (2048, 300, 4, 128), (2056, 300, 4, 128), (4104, 2400, 3, 64),
+                                            (16384, 512, 4, 128), (16400, 33, 1, 16400), (128, 60000, 1, 64), (2080, 500, 3, 32)])
+def test_decode_of_few_tokens_is_decode_of_many(d_in, d_out, q, g):
+    # up to two tokens (four, with more than 16 steps of 128) the activations go by way of shared memory, once for the
+    # CTA: the same conversion and the same sums, so to the last bit what the first rows of a larger batch get
+    # (ragged steps, clusters, several rounds of tiles, tables of two and four groups a step)
+    gen = torch.Generator(device="cuda").manual_seed(d_in + d_out)
+    bits, alpha, _ = bcq.quantize(torch.randn((d_out, d_in), generator=gen, device="cuda") * 0.02, q, g)
+    pack = bcq.decode_pack(bits, alpha, d_in, g)
+    X = torch.randn((8, (d_in + 7) // 8 * 8), generator=gen, device="cuda").bfloat16()[:, :d_in]
+    X[1] *= 1e-3
+    Y = bcq.linear_decode_packed(X, pack, d_out, d_in, q, g)
+    ref = (X.double() @ bcq.dequantize(bits, alpha, d_in, g).double().t()).cpu().numpy()
+    assert rel_err(Y.cpu().numpy(), ref) <= TOL
+    for n in (1, 2, 3, 4, 5):
+        assert torch.equal(bcq.linear_decode_packed(X[:n], pack, d_out, d_in, q, g), Y[:n]), n
+
+
 @pytest.mark.parametrize("n", [1, 9])
 @pytest.mark.parametrize("d_in,d_out,q,g", [(4096, 1040, 4, 128), (4224, 1030, 3, 96), (8200, 512, 2, 8200),
                                             (16384, 250, 4, 64), (8192, 16, 6, 128), (4100, 17, 1, 4100)])
