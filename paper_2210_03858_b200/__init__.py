@@ -182,6 +182,15 @@ def _ptr(t):
     return None if t is None else t.data_ptr()
 
 
+def _empty(like, shape, dtype):
+    # (a plain tensor's new_empty is 1.4 us shorter than torch.empty with a device to look up: quantize of a small
+    # layer 11.5 us of the host before, 9.0 now)
+    torch = _torch()
+    if type(like) is torch.Tensor:
+        return like.new_empty(shape, dtype=dtype)
+    return torch.empty(shape, dtype=dtype, device=like.device)
+
+
 def _stream():
     c = _torch()._C
     return c._cuda_getCurrentRawStream(c._cuda_getDevice())
@@ -219,10 +228,9 @@ def quantize(W, q: int, g: int, alt_iters: int = 0, want_sq_err: bool = False):
     assert W.is_cuda and W.dtype == torch.float32 and W.dim() == 2 and W.stride(1) == 1
     d_out, d_in = W.shape
     G = -(-d_in // g) if g > 0 else 1
-    dev = W.device
-    bits = torch.empty((q, d_out, 4 * ((d_in + 127) // 128)), dtype=torch.int32, device=dev)
-    alpha = torch.empty((q, d_out, G), dtype=torch.float32, device=dev)
-    sq_err = torch.empty((d_out, G), dtype=torch.float64, device=dev) if want_sq_err else None
+    bits = _empty(W, (q, d_out, 4 * ((d_in + 127) // 128)), torch.int32)
+    alpha = _empty(W, (q, d_out, G), torch.float32)
+    sq_err = _empty(W, (d_out, G), torch.float64) if want_sq_err else None
     _check(_fn().quantize(d_out, d_in, q, g, _ptr(W), W.stride(0), alt_iters, _ptr(bits),
                               _ptr(alpha), _ptr(sq_err), _stream()), "bcq_quantize")
     return bits, alpha, sq_err
@@ -378,7 +386,7 @@ def linear_bwd_alpha(dY, X, bits, d_in: int, g: int, plane_mask=None, scale: flo
 # ---------------------------------------------------------------------------- the update
 
 def lr_linear_decay(lr0: float, step: int, warmup_steps: int, total_steps: int) -> float:
-    return float(lib().bcq_lr_linear_decay(lr0, step, warmup_steps, total_steps))
+    return _fn().lr_linear_decay(lr0, step, warmup_steps, total_steps)
 
 
 class Segments:
@@ -402,10 +410,11 @@ def alpha_adamw(alpha, dalpha, m, v, step: int, lr: float, beta1: float = 0.9, b
                 eps: float = 1e-8, weight_decay: float = 0.0, grad_scale: float = 1.0, segments: Segments = None):
     """bcq_alpha_adamw on flat fp32 tensors (in place).  Without segments the whole arrays are updated."""
     torch = _torch()
+    n, f32 = alpha.numel(), torch.float32
     for t in (alpha, dalpha, m, v):
-        assert t.is_cuda and t.dtype == torch.float32 and t.is_contiguous() and t.numel() == alpha.numel()
+        assert t.is_cuda and t.dtype == f32 and t.is_contiguous() and t.numel() == n
     if segments is None:
-        count, nseg, b, pfx, sc = alpha.numel(), 0, None, None, None
+        count, nseg, b, pfx, sc = n, 0, None, None, None
     else:
         count, nseg, b, pfx, sc = segments.count, segments.nseg, segments.begin, segments.prefix, segments.scale
     _check(_fn().adamw(count, nseg, _ptr(b), _ptr(pfx), _ptr(sc), _ptr(alpha), _ptr(dalpha), _ptr(m),
@@ -416,7 +425,7 @@ def alpha_adamw(alpha, dalpha, m, v, step: int, lr: float, beta1: float = 0.9, b
 def alpha_pack(alpha_flat, segments: Segments):
     """bcq_alpha_pack: the trained scales as one compact fp32 tensor (the per-task checkpoint)."""
     torch = _torch()
-    out = torch.empty(segments.count, dtype=torch.float32, device=alpha_flat.device)
+    out = _empty(alpha_flat, (segments.count,), torch.float32)
     _check(_fn().pack(segments.count, segments.nseg, _ptr(segments.begin), _ptr(segments.prefix),
                                 _ptr(alpha_flat), _ptr(out), _stream()), "bcq_alpha_pack")
     return out

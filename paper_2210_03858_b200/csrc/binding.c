@@ -21,6 +21,7 @@ typedef int (*bwd_alpha_fn)(int, int, int, int, int, const void*, size_t, const 
 typedef int (*quantize_fn)(int, int, int, int, const void*, size_t, int, void*, void*, void*, void*);
 typedef int (*adamw_fn)(long long, int, const void*, const void*, const void*, void*, const void*, void*, void*, long long, float,
                         float, float, float, float, float, void*);
+typedef float (*lr_fn)(float, long long, long long, long long);
 typedef int (*gather_fn)(long long, int, const void*, const void*, void*, void*, void*);
 
 static fwd_fn f_fwd, f_fwd_prepared, f_decode;
@@ -30,6 +31,7 @@ static bwd_alpha_fn f_bwd_alpha;
 static quantize_fn f_quantize;
 static adamw_fn f_adamw;
 static gather_fn f_pack, f_unpack;
+static lr_fn f_lr;
 
 static inline long long as_int(PyObject* o) { return o == Py_None ? 0 : PyLong_AsLongLong(o); }
 static inline void* as_ptr(PyObject* o) { return o == Py_None ? NULL : PyLong_AsVoidPtr(o); }
@@ -120,6 +122,20 @@ static PyObject* py_adamw(PyObject* self, PyObject* const* args, Py_ssize_t n) {
 GATHER(pack)
 GATHER(unpack)
 
+/* The learning rate of a step (one call per optimiser step; through ctypes 1.1 us, here 0.1).  Steps have to be integers. */
+static PyObject* py_lr_linear_decay(PyObject* self, PyObject* const* args, Py_ssize_t n) {
+    (void)self;
+    if (n != 4 || !PyLong_Check(args[1]) || !PyLong_Check(args[2]) || !PyLong_Check(args[3])) {
+        PyErr_SetString(PyExc_TypeError, "a float and three integers expected");
+        return NULL;
+    }
+    const float lr0 = (float)PyFloat_AsDouble(args[0]);
+    long long k[3];
+    for (int i = 0; i < 3; ++i) k[i] = PyLong_AsLongLong(args[1 + i]);
+    if (PyErr_Occurred() != NULL) return NULL;
+    return PyFloat_FromDouble((double)f_lr(lr0, k[0], k[1], k[2]));
+}
+
 static PyObject* py_load(PyObject* self, PyObject* path) {
     (void)self;
     const char* file = PyUnicode_AsUTF8(path);
@@ -134,7 +150,7 @@ static PyObject* py_load(PyObject* self, PyObject* path) {
         {"bcq_linear_decode_packed", &f_packed}, {"bcq_linear_bwd_x", &f_bwd_x},
         {"bcq_linear_bwd_x_prepared", &f_bwd_x_prepared}, {"bcq_linear_bwd_alpha", &f_bwd_alpha},
         {"bcq_quantize", &f_quantize}, {"bcq_alpha_adamw", &f_adamw}, {"bcq_alpha_pack", &f_pack},
-        {"bcq_alpha_unpack", &f_unpack},
+        {"bcq_alpha_unpack", &f_unpack}, {"bcq_lr_linear_decay", &f_lr},
     };
     for (size_t k = 0; k < sizeof(table) / sizeof(table[0]); ++k) {
         void* sym = dlsym(h, table[k].name);
@@ -150,6 +166,6 @@ static PyObject* py_load(PyObject* self, PyObject* path) {
 #define M(name) {#name, (PyCFunction)(void (*)(void))py_##name, METH_FASTCALL, NULL}
 static PyMethodDef methods[] = {
     M(fwd), M(fwd_prepared), M(decode), M(packed), M(bwd_x), M(bwd_x_prepared), M(bwd_alpha), M(quantize), M(adamw), M(pack),
-    M(unpack), {"load", py_load, METH_O, NULL}, {NULL, NULL, 0, NULL}};
+    M(unpack), M(lr_linear_decay), {"load", py_load, METH_O, NULL}, {NULL, NULL, 0, NULL}};
 static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_bcq_call", NULL, -1, methods, NULL, NULL, NULL, NULL};
 PyMODINIT_FUNC PyInit__bcq_call(void) { return PyModule_Create(&module); }
