@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
             // ---- scales of one plane, 128 rows x alpha_w groups: coalesced reads along the groups (alpha[i][j][c] is
             // contiguous over (j, c)), coalesced writes along the rows (rows past d_out become zeros).  All loads
             // of a thread are in flight at once: a block for all groups of 128 rows, one load at a time, took
-            // 0.8 us for every second group (d_in = 20480, g = 128, 2048 tokens: 70 us for the pre-pass, now 27)
+            // 0.8 us for every second group (d_in = 20480, g = 128, 2048 tokens: 70 us for the pre-pass, now 37)
             const int w = p.alpha_w, shift = __ffs(w) - 1;
             const int cblk = (p.G + w - 1) >> shift;
             const int c0 = (b % cblk) << shift;

@@ -11,9 +11,9 @@
 // this kernel worked before, a plane of 128 weights cost five rounds of 64-bit shuffles and a
 // ballot per 32 weights; now two rounds, and per weight and plane two fp64 additions and one shift
 // that collects the sign.  Measured, before and after: greedy q = 4, g = 128, the four linears of a
-// layer of width 1600 (30.7 M weights) 162 -> 59 us (2.5 TB/s; the logic pipe is 55 % busy, the fp64
-// pipe 21 %); five alternating rounds, q = 3, g = 128, 5120 x 5120: 1119 -> 360 us (instruction fetch of
-// the unrolled rounds and fp64 latency at five warps per scheduler bound it).
+// layer of width 1600 (30.7 M weights) 162 -> 56 us (2.6 TB/s; the logic pipe is 55 % busy, the fp64
+// pipe 21 %); two alternating rounds, q = 3, g = 128, 5120 x 5120: 202 us (instruction fetch of the
+// unrolled rounds and fp64 latency at five warps per scheduler bound it).
 //
 // Sums are fp64 and are reduced in a fixed order, so a result never depends on scheduling.
 //
