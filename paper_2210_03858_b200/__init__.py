@@ -386,7 +386,12 @@ def linear_bwd_alpha(dY, X, bits, d_in: int, g: int, plane_mask=None, scale: flo
 # ---------------------------------------------------------------------------- the update
 
 def lr_linear_decay(lr0: float, step: int, warmup_steps: int, total_steps: int) -> float:
-    return _fn().lr_linear_decay(lr0, step, warmup_steps, total_steps)
+    # (host arithmetic: the shared library alone will do where the extension is not built, and arguments that the extension
+    # leaves to ctypes get its conversions and errors)
+    try:
+        return _fn().lr_linear_decay(lr0, step, warmup_steps, total_steps)
+    except (RuntimeError, TypeError, OverflowError):
+        return float(lib().bcq_lr_linear_decay(lr0, step, warmup_steps, total_steps))
 
 
 class Segments:

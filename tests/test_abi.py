@@ -70,6 +70,22 @@ def test_argument_validation_happens_before_any_launch():
     assert bcq.workspace_bytes(bcq.OP_QUANTIZE, 8, 64, 2, 64, 0) == 0
 
 
+def test_learning_rate_takes_what_the_library_takes(monkeypatch):
+    # every call through the extension has the value, and the error, of the C entry point through ctypes
+    plain = lambda *a: float(bcq.lib().bcq_lr_linear_decay(*a))
+    calls = [(1e-3, 3, 0, 10), (1, 3, 5, 10), (1e-3, True, 0, 10), (1e-3, 2 ** 64 + 3, 0, 10), (1e-3, -2 ** 70 + 4, 2, 2 ** 64 + 9),
+             (C.c_float(0.5), C.c_longlong(2), 0, 8)]
+    refused = [(1e-3, 3.0, 0, 10), ("1", 3, 0, 10), (1e-3, 3, None, 10)]
+    for extension in (True, False):
+        if not extension:
+            monkeypatch.setattr(bcq, "_fn", lambda: (_ for _ in ()).throw(RuntimeError("binding not built")))
+        for a in calls:
+            assert bcq.lr_linear_decay(*a) == plain(*a), a
+        for a in refused:
+            with pytest.raises(C.ArgumentError):
+                bcq.lr_linear_decay(*a)
+
+
 def test_workspace_sizes_are_consistent():
     # decode asks for the room it always asked for (its sums stay on chip); prefill holds its fp16 activations
     assert bcq.workspace_bytes(bcq.OP_DECODE, 4096, 16384, 4, 128, 16) > 0
