@@ -53,8 +53,9 @@ constexpr int kHN = kTN / 2;   // of an epilogue sub-tile, and of the half of B 
 constexpr int kTM = 2 * kBlockM;
 constexpr int kStages = 6;
 constexpr uint32_t kStageBytes = kABytes + kHN * kBlockK * 2;  // 32 KiB
-// sign words of the epilogue's threads, [column chunk of 32][plane of the mask][thread]
+// sign words of the epilogue's threads, [plane of the mask][thread][column chunk of 32]
 constexpr uint32_t kSignBytes = (kHN / 32) * BCQ_MAX_Q * kWorkerWarps * 32 * 4;  // 32 KiB
+static_assert(kHN == 128, "a sub-tile's sign words of a row are one 16-byte load");
 constexpr size_t kDalphaSmem = (size_t)kStages * kStageBytes + 1024 + 256 + kSignBytes;
 static_assert(kDalphaSmem <= 232448, "shared memory of a CTA");
 
@@ -221,7 +222,8 @@ dalpha_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant
         const int half = (warp - kWorkerWarp0) >> 2;
         const int et = (int)threadIdx.x - kWorkerWarp0 * 32;
         constexpr int ET = kWorkerWarps * 32;
-        uint32_t* words = reinterpret_cast<uint32_t*>(ctl_gen + 256) + et;  // this thread's; [chunk * num_planes + plane] * ET
+        uint32_t* mine = reinterpret_cast<uint32_t*>(ctl_gen + 256) + 4 * et;  // this thread's; [plane][thread][chunk]
+        const uint32_t words = ptx::smem_u32(mine);
         const long long plane_words = (long long)p.d_out * p.pitch;
         const int np = p.num_planes;
         bool ok = true;
@@ -235,16 +237,19 @@ dalpha_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant
             const int kbase = k0 + half * HN;
             const int subtile = (k0 / kTN) * 2 + half;
 
-            // the sign words do not depend on the accumulator: fetch them while the main loop runs
+            // The sign words do not depend on the accumulator: they are on their way into shared memory while the main
+            // loop runs, all planes' at once (a row's words of a sub-tile are 16 bytes, aligned).  Loaded plane after
+            // plane through registers they were a chain of as many memory latencies, longer than a short main loop:
+            // 1024 x 1024, 64 tokens, four planes 9.2 us and 8.0 so; 6400 -> 1600, eight planes 30.7 and 27.6.
+            if (j_ok && kbase < p.d_in) {
 #pragma unroll 1
-            for (int i = 0; i < np; ++i) {
-                const uint32_t* src = p.bits + (long long)((p.planes >> (4 * i)) & 15u) * plane_words + (long long)j * p.pitch + (kbase >> 5);
-#pragma unroll
-                for (int ch = 0; ch < NCH; ++ch)
-                    words[(ch * np + i) * ET] = j_ok && (kbase >> 5) + ch < p.pitch ? ~ld(src + ch) : 0u;
+                for (int i = 0; i < np; ++i)
+                    ptx::cp_async_16(words + (uint32_t)i * (ET * 16), p.bits + (long long)((p.planes >> (4 * i)) & 15u) * plane_words +
+                                                                          (long long)j * p.pitch + (kbase >> 5));
             }
 
             ok = wait_bar(ctl.accum + 8 * acc, (uint32_t)(lt >> 1) & 1u, ctl, 16, 512u);
+            ptx::cp_async_wait_all();
             if (!ok) break;
             ptx::tc_fence_after_sync();
             if (kbase < p.d_in) {
@@ -262,13 +267,13 @@ dalpha_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant
                     const bool last = ch == NCH - 1 || kg + 32 >= next_edge;  // of this group in this sub-tile
 #pragma unroll 1
                     for (int i = 0; i < np; ++i) {
-                        const uint32_t w = words[(ch * np + i) * ET];
+                        uint32_t* so_far = mine + i * (4 * ET);
+                        const uint32_t w = ~so_far[ch];
                         float sum = 0.0f;
 #pragma unroll
                         for (int b = 0; b < 32; ++b)
                             sum += __uint_as_float(v[b] ^ ((w << (31 - b)) & 0x80000000u));
                         // the group's sum so far waits in place of the plane's first sign word, which is used up
-                        uint32_t* so_far = words + i * ET;
                         if (!fresh) sum = __uint_as_float(*so_far) + sum;
                         if (!last) {
                             *so_far = __float_as_uint(sum);

@@ -79,6 +79,13 @@ __device__ __forceinline__ void named_bar_sync(uint32_t id, uint32_t threads) {
 // Brings the 128-byte line of `p` into L2.  Reads nothing, so it needs no ordering with the line's writer.
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
+// 16 bytes from global to shared memory, both 16-byte aligned, without a register; this thread's copies have arrived
+// after cp_async_wait_all.
+__device__ __forceinline__ void cp_async_16(uint32_t dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(__cvta_generic_to_global(src)) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // Makes this thread's generic-proxy writes to shared memory visible to the async proxy
 // (TMA and the tensor core read shared memory through it).
 __device__ __forceinline__ void fence_proxy_async_smem() {
