@@ -120,11 +120,15 @@ struct PrepParams {
     int num_counters;
 };
 
-// WPT warps per token row.  A lane keeps up to HELD (four or twelve) 16-byte vectors of the row in registers between finding
-// the row's largest magnitude and writing the scaled fp16 row, so rows of up to 1024 WPT (24576) elements are
-// read once; longer rows are read again from L2.  Four loads of a lane
-// in flight and few registers: the token blocks are bound by memory (n x K x 4 bytes; with a warp per
-// token and two reads, 4096 x 6400 took 21 us and 4096 x 1600 8.5 us).
+// WPT warps per token row.  A lane keeps up to HELD 16-byte vectors of the row in registers between finding the row's
+// largest magnitude and writing the scaled fp16 row.  Rows of up to 1024 WPT elements take HELD = 4 (40 registers), longer
+// ones 8 (62, up to 16384 elements) or 12 (76, up to 24576): all of these are read once.  Rows past that go to <8, 4>
+// and are read again from L2.
+// The token blocks are bound by memory (n x K x 4 bytes; with a warp per token and two reads, 4096 x 6400 took 21 us and
+// 4096 x 1600 8.5 us) and need warps in flight, so registers that no vector comes to cost time.  Whole forward, g = d_in,
+// q = 3, 2048 tokens, with two reads / 12 vectors / the fewest that hold the row, us:
+//   8200 -> 512 43.7 / 50.2 / 42.9    10240 -> 1024 59.9 / 63.8 / 57.9    16384 -> 512 62.8 / 64.7 / 60.3    20480 -> 512 74.0 / 69.1 / 69.1
+// (12 vectors with two blocks of 90 registers an SM instead of three: 20480 -> 512 72.4).
 // Blocks past the activation blocks scan alpha instead.
 constexpr int kPrepWarps = 8;
 
@@ -171,7 +175,8 @@ __device__ __forceinline__ uint4 scale_to_fp16x8(const uint4& x, int k0, int K, 
 }
 
 template <int WPT, int HELD = 4>
-__global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
+__global__ void __launch_bounds__(256, HELD == 12 ? 3 : 0) prepare_kernel(const PrepParams p) {
+    constexpr bool AGAIN = WPT == kPrepWarps && HELD == 4;  // there may be more vectors than are held
     __shared__ uint32_t red[8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     pdl_trigger();
@@ -331,9 +336,13 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
             held[i] = (v < nvec) ? ld(src + v) : make_uint4(0u, 0u, 0u, 0u);
         }
 #pragma unroll
-        for (int i = 0; i < HELD; ++i) m = max(m, max_mag_bf16x8(held[i], (v0 + kThreadsPerToken * i) * 8, p.K));
+        for (int i = 0; i < HELD; ++i) {
+            const int v = v0 + kThreadsPerToken * i;
+            // (HELD = 8 for rows of 1025 to 2048 vectors, so up to three of a lane's eight are not there)
+            if (HELD != 8 || v < nvec) m = max(m, max_mag_bf16x8(held[i], v * 8, p.K));
+        }
         v0 += HELD * kThreadsPerToken;
-    } while (v0 - tl < nvec);
+    } while (AGAIN && v0 - tl < nvec);
     m = __reduce_max_sync(0xffffffffu, m);
     if (WPT > 1) {
         if (lane == 0) red[warp] = m;
@@ -344,7 +353,7 @@ __global__ void __launch_bounds__(256) prepare_kernel(const PrepParams p) {
     const int sh = shift_for(exponent_of_bits(m << 16), 14);
     const float scale = pow2f(sh);
     if (live && tl == 0) p.tok_inv_scale[t] = pow2f(-sh);
-    if (nvec <= HELD * kThreadsPerToken) {
+    if (!AGAIN || nvec <= HELD * kThreadsPerToken) {
 #pragma unroll
         for (int i = 0; i < HELD; ++i) {
             const int v = tl + kThreadsPerToken * i;
@@ -1360,7 +1369,8 @@ bcq_status run_expand(int d_out, int d_in, int q, int g, int n, const void* act,
     const int tok_blocks = ceil_div(n, kPrepWarps / wpt);
     pp.act_blocks = tok_blocks;
     const unsigned pgrid = (unsigned)(tok_blocks + ablocks + pp.bits_blocks + alpha_tr_blocks);
-    auto prep = wpt == 1 ? prepare_kernel<1> : wpt == 2 ? prepare_kernel<2> : wpt == 4 ? prepare_kernel<4> : nvec <= 1024 || nvec > 3072 ? prepare_kernel<8> : prepare_kernel<8, 12>;
+    auto prep = wpt == 1 ? prepare_kernel<1> : wpt == 2 ? prepare_kernel<2> : wpt == 4 ? prepare_kernel<4>
+                : nvec <= 1024 || nvec > 3072 ? prepare_kernel<8> : nvec <= 2048 ? prepare_kernel<8, 8> : prepare_kernel<8, 12>;
     BCQ_CUDA_TRY(launch_pdl(prep, dim3(pgrid), 256, 0, s, 1, pp));
 
     ExpandParams p;

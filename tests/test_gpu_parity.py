@@ -475,6 +475,42 @@ def test_many_tiles_per_cta_around_the_shortest_shared_output(k):
 
 
 # --------------------------------------------------------------------------- dynamic range
+@pytest.mark.parametrize("k", [8200, 16384, 16392, 24576, 24584, 32760])
+def test_pre_pass_of_long_rows(k):
+    # rows that a lane holds in eight vectors, in twelve, and those that are read again; each token's largest element
+    # in another part of its row.  Against a dense fp64 product, as the forward and as the input gradient.
+    n, m, q = 6, 40, 2
+    gen = torch.Generator(device="cuda").manual_seed(k)
+    W = torch.randn((m, k), generator=gen, device="cuda") * 0.02
+    X = torch.randn((n, k), generator=gen, device="cuda").bfloat16()
+    for t in range(n):
+        X[t, (t + 1) * k // n - 1] = 300.0 * (t + 1)
+    bits, alpha, _ = bcq.quantize(W, q, k)
+    ref = (X.double() @ bcq.dequantize(bits, alpha, k, k).double().t()).cpu().numpy()
+    assert rel_err(bcq.linear_fwd(X, bits, alpha, k, k).cpu().numpy(), ref) <= TOL
+    bits, alpha, _ = bcq.quantize(W.t().contiguous(), q, m)
+    ref = (X.double() @ bcq.dequantize(bits, alpha, m, m).double()).cpu().numpy()
+    assert rel_err(bcq.linear_bwd_x(X, bits, alpha, m, m).cpu().numpy(), ref) <= TOL
+
+
+@pytest.mark.parametrize("shift", [1, 2, 3])
+@pytest.mark.parametrize("d_in,d_out,q,g", [(4096, 600, 3, 32), (96, 24, 2, 96)])
+def test_scales_at_any_address(d_in, d_out, q, g, shift):
+    # a linear's scales may be a view of a flat array, four bytes aligned: same results as from an allocation of their own
+    gen = torch.Generator(device="cuda").manual_seed(d_in + shift)
+    bits, alpha, _ = bcq.quantize(torch.randn((d_out, d_in), generator=gen, device="cuda") * 0.02, q, g)
+    alpha[q - 1, d_out - 1, -1] = 3.0  # the largest, and it decides the scaling, is the last
+    flat = torch.empty(alpha.numel() + 4, device="cuda")
+    view = flat[shift:shift + alpha.numel()].view_as(alpha).copy_(alpha)
+    X = torch.randn((64, d_in), generator=gen, device="cuda").bfloat16()
+    dY = torch.randn((64, d_out), generator=gen, device="cuda").bfloat16()
+    assert torch.equal(bcq.linear_fwd(X, bits, view, d_in, g), bcq.linear_fwd(X, bits, alpha, d_in, g))
+    assert torch.equal(bcq.linear_bwd_x(dY, bits, view, d_in, g), bcq.linear_bwd_x(dY, bits, alpha, d_in, g))
+    assert torch.equal(bcq.linear_decode(X[:3], bits, view, d_in, g), bcq.linear_decode(X[:3], bits, alpha, d_in, g))
+    ref = (X.double() @ bcq.dequantize(bits, alpha, d_in, g).double().t()).cpu().numpy()
+    assert rel_err(bcq.linear_fwd(X, bits, view, d_in, g).cpu().numpy(), ref) <= TOL
+
+
 
 def _bf16(x):
     return synth.f32_to_bf16_bits(np.asarray(x, dtype=np.float32))
