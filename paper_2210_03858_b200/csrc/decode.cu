@@ -802,13 +802,13 @@ bcq_status launch_decode_packed(DecPackedParams p, int tiles, cudaStream_t s) {
     p.x_stride = (uint32_t)steps * 256u + 64u;     // (64 bytes more: tokens next to each other in other banks)
     const size_t x_bytes = (size_t)p.n * (p.x_stride + steps * sizeof(float));
     // Activations by way of shared memory: for up to four tokens, where they fit.  With two tokens the CTA's conversion is an eighth
-    // to a quarter of what its warps do otherwise; with four it needs more than one step a warp to be less, with eight it
+    // to a quarter of what its warps do otherwise; with four the CTA needs more than one step a warp for it to be less, with eight it
     // is as much, behind a barrier; four tables a step (PARTS = 4) leave no registers for it.  q = 4, without and with, us:
     //   4096 -> 4096   one token 6.12 / 5.84, two 6.18 / 5.99, four 6.22 / 6.17, eight 6.30 / 7.01
     //   16384 -> 4096, one token 19.0 / 15.6; 4096 -> 16384, one token 13.9 / 13.3; 2048 -> 2048, four tokens 3.27 / 3.38
-    //   2048 -> 2048, g = 32, one token 3.60 / 4.11
+    //   2048 -> 2048, g = 32, one token 3.60 / 4.11; 4096 -> 512, in clusters of two with 16 steps each, four tokens 4.34 / 4.45
     constexpr bool CAN = NT == 1 && PARTS <= 2;
-    const bool xs = CAN && p.n <= (p.steps > kDpWarps ? 4 : 2) && smem + x_bytes <= kDpMaxSmem;
+    const bool xs = CAN && p.n <= (steps > kDpWarps ? 4 : 2) && smem + x_bytes <= kDpMaxSmem;
     if (xs) smem += x_bytes;
     void (*kern)(DecPackedParams) = p.split > 1 ? decode_packed_kernel<Q, NT, PARTS, true, false> : decode_packed_kernel<Q, NT, PARTS, false, false>;
     if constexpr (CAN)

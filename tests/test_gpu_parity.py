@@ -444,37 +444,6 @@ def test_tiles_cut_along_k(n, d_in, d_out, q, g):
         assert rel_err(dX.float().cpu().numpy(), ref) <= tol
 
 
-def test_bwd_x_many_tiles_per_cta_with_short_k():
-    n, d_in, d_out, q, g = 4096, 2560, 64, 4, 128
-    _, X, dY, bits, alpha, _, _ = make_case(811, n, d_in, d_out, q, g)
-    _, dYd, bd, ad = _upload(X, dY, bits, alpha)
-    ref = oracle.bwd_x(dY, bits, alpha, d_in, g)
-    assert rel_err(bcq.linear_bwd_x(dYd, bd, ad, d_in, g, out_dtype=torch.bfloat16).float().cpu().numpy(),
-                   ref) <= TOL + 2.0 ** -8
-    assert rel_err(bcq.linear_bwd_x(dYd, bd, ad, d_in, g).cpu().numpy(), ref) <= TOL
-
-
-@pytest.mark.parametrize("k", [256, 257, 320, 384])
-def test_many_tiles_per_cta_around_the_shortest_shared_output(k):
-    # 4 and 5 stages a tile lie on either side of the line above which the worker warps share the output of a
-    # CTA's last tile; 160 tiles for 74 pairs, so accumulators are reused.  Against a dense fp64 product.
-    n, m = 4096, 2560
-    gen = torch.Generator(device="cuda").manual_seed(k)
-    X = torch.randn((n, (k + 7) // 8 * 8), generator=gen, device="cuda").bfloat16()[:, :k]
-    W = torch.randn((m, k), generator=gen, device="cuda") * 0.02
-    bits, alpha, _ = bcq.quantize(W, 3, k)
-    ref = X.double() @ bcq.dequantize(bits, alpha, k, k).double().t()
-    bits_t, alpha_t, _ = bcq.quantize(W.t().contiguous(), 3, 128)
-    ref_t = X.double() @ bcq.dequantize(bits_t, alpha_t, m, 128).double()
-    for dt, tol in ((torch.float32, TOL), (torch.bfloat16, TOL + 2.0 ** -8)):
-        for _ in range(3):
-            Y = bcq.linear_fwd(X, bits, alpha, k, k, out_dtype=dt)
-            assert float((Y.double() - ref).abs().max() / ref.abs().max()) <= tol
-            dX = bcq.linear_bwd_x(X, bits_t, alpha_t, m, 128, out_dtype=dt)
-            assert float((dX.double() - ref_t).abs().max() / ref_t.abs().max()) <= tol
-
-
-# --------------------------------------------------------------------------- dynamic range
 @pytest.mark.parametrize("k", [8200, 16384, 16392, 24576, 24584, 32760])
 def test_pre_pass_of_long_rows(k):
     # rows that a lane holds in eight vectors, in twelve, and those that are read again; each token's largest element
@@ -542,6 +511,37 @@ def test_token_with_one_huge_channel():
                 assert np.abs(Yd[t] - refd[t]).max() <= TOL * np.abs(refd[t]).max()
 
 
+def test_bwd_x_many_tiles_per_cta_with_short_k():
+    n, d_in, d_out, q, g = 4096, 2560, 64, 4, 128
+    _, X, dY, bits, alpha, _, _ = make_case(811, n, d_in, d_out, q, g)
+    _, dYd, bd, ad = _upload(X, dY, bits, alpha)
+    ref = oracle.bwd_x(dY, bits, alpha, d_in, g)
+    assert rel_err(bcq.linear_bwd_x(dYd, bd, ad, d_in, g, out_dtype=torch.bfloat16).float().cpu().numpy(),
+                   ref) <= TOL + 2.0 ** -8
+    assert rel_err(bcq.linear_bwd_x(dYd, bd, ad, d_in, g).cpu().numpy(), ref) <= TOL
+
+
+@pytest.mark.parametrize("k", [256, 257, 320, 384])
+def test_many_tiles_per_cta_around_the_shortest_shared_output(k):
+    # 4 and 5 stages a tile lie on either side of the line above which the worker warps share the output of a
+    # CTA's last tile; 160 tiles for 74 pairs, so accumulators are reused.  Against a dense fp64 product.
+    n, m = 4096, 2560
+    gen = torch.Generator(device="cuda").manual_seed(k)
+    X = torch.randn((n, (k + 7) // 8 * 8), generator=gen, device="cuda").bfloat16()[:, :k]
+    W = torch.randn((m, k), generator=gen, device="cuda") * 0.02
+    bits, alpha, _ = bcq.quantize(W, 3, k)
+    ref = X.double() @ bcq.dequantize(bits, alpha, k, k).double().t()
+    bits_t, alpha_t, _ = bcq.quantize(W.t().contiguous(), 3, 128)
+    ref_t = X.double() @ bcq.dequantize(bits_t, alpha_t, m, 128).double()
+    for dt, tol in ((torch.float32, TOL), (torch.bfloat16, TOL + 2.0 ** -8)):
+        for _ in range(3):
+            Y = bcq.linear_fwd(X, bits, alpha, k, k, out_dtype=dt)
+            assert float((Y.double() - ref).abs().max() / ref.abs().max()) <= tol
+            dX = bcq.linear_bwd_x(X, bits_t, alpha_t, m, 128, out_dtype=dt)
+            assert float((dX.double() - ref_t).abs().max() / ref_t.abs().max()) <= tol
+
+
+# --------------------------------------------------------------------------- dynamic range
 def test_tiny_output_gradients():
     # dY ~ 1e-6: far below the smallest normal fp16 number unless each token row is rescaled
     n, d_in, d_out, q, g = 200, 384, 256, 4, 128
