@@ -529,6 +529,9 @@ decode_packed_kernel(const DecPackedParams p) {
 // fp32 sums of +-alpha_i.  Levels carry a power of two per (row, step) that brings the largest sum of
 // |alpha_i| to [2^13, 2^14), taken out of the sums again in fp32.
 // This replaced a tcgen05 kernel with a split over K and a second kernel that added the parts.
+//
+// Weights are on their way one unit ahead, as in the kernel above, or (DEEP, see launch_decode_planes) two units ahead in
+// two register sets that take turns.
 
 struct DecPlanesParams {
     int d_out, d_in, q, g, G, n;
@@ -608,7 +611,7 @@ struct RowExpand {
     }
 };
 
-template <int NQ, int NT, bool SPLIT>
+template <int NQ, int NT, bool SPLIT, bool DEEP>
 __global__ void __launch_bounds__(kDpThreads, 1)
 decode_planes_kernel(const DecPlanesParams p) {
     extern __shared__ float4 sums[];  // [warp][tile][NT][32 lanes]
@@ -657,8 +660,9 @@ decode_planes_kernel(const DecPlanesParams p) {
                 l_c = group_of(++l_st);
             }
         };
-        PlaneWords<NQ> next;
+        PlaneWords<NQ> next, after;
         load(next);
+        if (DEEP) load(after);
         for (int i = 0; i < round_n * NT; ++i) mine[i * 32] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (first == 0) {
             for (int s = st0 + 1; (s - step0) * round_n < u1; ++s) {
@@ -749,7 +753,14 @@ decode_planes_kernel(const DecPlanesParams p) {
 #pragma unroll 1
         for (int u = u0; u < u1; ++u) {
             if (fresh) load_x(u_st);
-            if (NQ == 8) {  // one unit's registers are all there is room for
+            if (DEEP) {
+                unit(next);
+                load(next);
+                if (++u == u1) break;
+                if (fresh) load_x(u_st);
+                unit(after);
+                load(after);
+            } else if (NQ == 8) {  // one unit's registers are all there is room for
                 unit(next);
                 load(next);
             } else {
@@ -835,7 +846,19 @@ template <int NQ, int NT>
 bcq_status launch_decode_planes(DecPlanesParams p, cudaStream_t s) {
     int ctas;
     const size_t smem = deal_tiles<NT>(p, ceil_div(p.d_out, kDpRows), &ctas);
-    auto kern = p.split > 1 ? decode_planes_kernel<NQ, NT, true> : decode_planes_kernel<NQ, NT, false>;
+    void (*kern)(DecPlanesParams) = p.split > 1 ? decode_planes_kernel<NQ, NT, true, false> : decode_planes_kernel<NQ, NT, false, false>;
+    // Two units ahead (DEEP) where a warp has few units and the start of its loads counts for more than a loop that is there
+    // once.  us, one ahead / two ahead, one token; in front: units of a CTA, to be dealt to its 16 warps:
+    //   q = 3   6   768 -> 768 2.78 / 2.67        16  2048 -> 2048 3.80 / 3.62   20  1280 -> 5120 5.46 / 5.04   39  1600 -> 4800 6.07 / 5.70
+    //           50  6400 -> 1600 8.88 / 8.54      64  4096 -> 4096 8.74 / 8.73   256 16384 -> 4096 27.8 / 28.6
+    //   q = 4   12  768 -> 3072 3.82 / 3.93       16  2048 -> 2048 4.79 / 4.81   20  1280 -> 4096 6.34 / 5.93   25  3200 -> 1600 6.32 / 6.05
+    //           32  2048 -> 4096 6.50 / 6.97      33  1408 -> 6400 6.92 / 6.63   39  1600 -> 4800 7.26 / 7.07   40  5120 -> 1280 9.32 / 9.66
+    // and with nine tokens and more one ahead is the faster (q = 3, 1024 -> 1024, 16 tokens 4.38 / 4.72).
+    if constexpr (NQ < 8 && NT == 1) {
+        const int units = p.round * ceil_div(p.steps, p.split);
+        const bool deep = NQ == 3 ? units < 4 * kDpWarps : units > kDpWarps && 2 * units < 5 * kDpWarps && units % kDpWarps != 0;
+        if (deep) kern = p.split > 1 ? decode_planes_kernel<NQ, NT, true, true> : decode_planes_kernel<NQ, NT, false, true>;
+    }
     const bcq_status st = ensure_dynamic_smem(kern, smem);
     if (st != BCQ_OK) return st;
     BCQ_CUDA_TRY(launch_pdl(kern, dim3((unsigned)ctas), kDpThreads, smem, s, (unsigned)p.split, p));
