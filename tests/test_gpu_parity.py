@@ -111,7 +111,7 @@ def test_quantize_matches_oracle(d_out, d_in, q, g, alt, outl):
     np.testing.assert_allclose(sq_err[same], sq_ref[same], rtol=1e-6, atol=1e-18)
 
 
-@pytest.mark.parametrize("alt", [0, 3])
+@pytest.mark.parametrize("alt", [0, 2, 3])
 @pytest.mark.parametrize("d_in,g", [(96, 32), (200, 64), (420, 96), (520, 160), (900, 256), (1100, 512), (1023, 1023),
                                     (2050, 2050), (5000, 2528), (8192, 8192), (12001, 12001), (20000, 20000)])
 def test_quantize_team_sizes_with_exact_ties(d_in, g, alt):
@@ -134,10 +134,12 @@ def test_quantize_team_sizes_with_exact_ties(d_in, g, alt):
             np.testing.assert_allclose(sq.cpu().numpy(), sq_ref, rtol=1e-6, atol=1e-12)
 
 
-@pytest.mark.parametrize("d_in,g", [(420, 96), (260, 128), (1023, 1023), (1582, 1582)])
-def test_quantize_alternating_short_and_long_problems(d_in, g):
+@pytest.mark.parametrize("alt", [2, 3])
+@pytest.mark.parametrize("d_in,g", [(100, 32), (420, 96), (260, 128), (700, 256), (1023, 1023), (1582, 1582)])
+def test_quantize_alternating_short_and_long_problems(d_in, g, alt):
     # The size of the team depends on how much there is to do: the same five rows alone and repeated past
     # the line (30720 weights per SM).  Values as in the test above, so the bits are the oracle's exactly.
+    # (Groups of up to 256 are taken by teams with two rounds, with three by lanes on sorted magnitudes.)
     rng = np.random.default_rng(d_in)
     W = (rng.integers(-6, 7, size=(5, d_in)) / 64.0).astype(np.float32)
     W[0, ::3] = -0.0
@@ -146,9 +148,9 @@ def test_quantize_alternating_short_and_long_problems(d_in, g):
     reps = 30720 * sms // (5 * -(-d_in // g) * g) + 1
     Wd = torch.from_numpy(W).cuda()
     for q in (1, 2, 3, 4):
-        bits_ref, alpha_ref, sq_ref, _ = oracle.quantize(W, q, g, alt_iters=3)
+        bits_ref, alpha_ref, sq_ref, _ = oracle.quantize(W, q, g, alt_iters=alt)
         for r in (1, reps):
-            bits, alpha, sq = bcq.quantize(Wd.repeat(r, 1), q, g, 3, want_sq_err=True)
+            bits, alpha, sq = bcq.quantize(Wd.repeat(r, 1), q, g, alt, want_sq_err=True)
             np.testing.assert_array_equal(host_bits(bits), np.tile(bits_ref, (1, r, 1)))
             np.testing.assert_allclose(alpha.cpu().numpy(), np.tile(alpha_ref, (1, r, 1)), rtol=1e-6, atol=1e-9)
             np.testing.assert_allclose(sq.cpu().numpy(), np.tile(sq_ref, (r, 1)), rtol=1e-6, atol=1e-12)
@@ -180,18 +182,19 @@ def test_quantize_a_row_alone_and_among_many(d_in, g):
     rows = 30720 * sms // (-(-d_in // g) * g) + 1                    # past the line between the team sizes
     W = torch.randn((rows, d_in), generator=gen, device="cuda") * 0.02
     pick = slice(rows // 2, rows // 2 + 600)
-    for q, alt in ((1, 3), (2, 3), (3, 3), (4, 3), (4, 0)):
+    for q, alt in ((1, 3), (2, 3), (3, 3), (4, 3), (4, 0), (2, 2), (3, 2), (4, 2)):
         bits, alpha, sq = bcq.quantize(W, q, g, alt, want_sq_err=True)
         b, a, s = bcq.quantize(W[pick].contiguous(), q, g, alt, want_sq_err=True)
         assert torch.equal(b, bits[:, pick]) and torch.equal(a, alpha[:, pick]) and torch.equal(s, sq[pick])
 
 
 @pytest.mark.parametrize("alt", [3, 15])
-@pytest.mark.parametrize("d_in,g", [(32, 32), (64, 64), (130, 64), (288, 96), (420, 128), (256, 256), (1001, 256)])
+@pytest.mark.parametrize("d_in,g", [(32, 32), (64, 64), (130, 64), (288, 96), (420, 128), (256, 256), (1001, 256),
+                                    (500, 160), (580, 192), (450, 224)])
 def test_quantize_rounds_on_sorted_magnitudes(d_in, g, alt):
     # Values whose sums are exact in fp64 (see above), so that the bits are the oracle's: ties with a scale and with a
     # midpoint, groups of one magnitude, of zeros, with one weight far above the rest, infinities and NaNs; rows
-    # that are no multiple of a warp's share, aligned and not, alone and 150 times.
+    # that are no multiple of a warp's share, aligned and not, alone and 150 times, and in rows whose padding is not to be read.
     rng = np.random.default_rng(d_in + alt)
     W = (rng.integers(-40, 41, size=(13, d_in)) / 64.0).astype(np.float32)
     W[0, ::3], W[1], W[2] = -0.0, 0.0, np.where(rng.random(d_in) < 0.5, 0.25, -0.25)
@@ -201,13 +204,41 @@ def test_quantize_rounds_on_sorted_magnitudes(d_in, g, alt):
     W[10, 0] = np.array([0x7FFFFFFF], np.uint32).view(np.float32)[0]
     odd = torch.zeros((13, d_in + 1), dtype=torch.float32, device="cuda")[:, 1:]
     odd.copy_(torch.from_numpy(W))
+    padded = torch.full((13, -(-d_in // 4) * 4 + 4), 7e4, dtype=torch.float32, device="cuda")[:, :d_in]
+    padded.copy_(torch.from_numpy(W))
     for q in (2, 3, 4):
         bits_ref, alpha_ref, sq_ref, _ = oracle.quantize(W, q, g, alt_iters=alt)
-        for src, r in ((odd, 1), (torch.from_numpy(W).cuda(), 1), (torch.from_numpy(W).cuda().repeat(150, 1), 150)):
+        for src, r in ((odd, 1), (padded, 1), (torch.from_numpy(W).cuda(), 1), (torch.from_numpy(W).cuda().repeat(150, 1), 150)):
             bits, alpha, sq = bcq.quantize(src, q, g, alt, want_sq_err=True)
             np.testing.assert_array_equal(host_bits(bits), np.tile(bits_ref, (1, r, 1)))
             np.testing.assert_allclose(alpha.cpu().numpy(), np.tile(alpha_ref, (1, r, 1)), rtol=1e-6, atol=1e-9, equal_nan=True)
             np.testing.assert_allclose(sq.cpu().numpy(), np.tile(sq_ref, (r, 1)), rtol=1e-6, atol=1e-12, equal_nan=True)
+
+
+@pytest.mark.parametrize("d_in,g", [(32, 32), (130, 64), (288, 96), (420, 128), (1001, 256)])
+def test_quantize_sorted_rounds_in_blocks_of_four_warps(d_in, g):
+    # From 24 warps an SM on, four warps of 32 groups (16 with more than 128 weights) share a block.  The last block's warps
+    # past the last group repeat it; its row, the last, is not finite.  What every copy of the rows becomes is what they
+    # become alone (which the test above compares with the oracle).
+    rng = np.random.default_rng(d_in)
+    W = (rng.integers(-40, 41, size=(13, d_in)) / 64.0).astype(np.float32)
+    W[0, ::3], W[1] = -0.0, 0.0
+    W[4, 3], W[12, [0, d_in - 1]] = np.inf, (np.inf, np.nan)
+    Wd = torch.from_numpy(W).cuda()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    G, share = -(-d_in // g), 32 if g <= 128 else 16
+    reps = 24 * sms * share // (13 * G) + 1
+    while -(-13 * reps * G // share) % 4 == 0:
+        reps += 1
+    for q in (2, 3, 4):
+        one = bcq.quantize(Wd, q, g, 4, want_sq_err=True)
+        many = bcq.quantize(Wd.repeat(reps, 1), q, g, 4, want_sq_err=True)
+        for a, b, rows in zip(one, many, (1, 1, 0)):
+            want = a.repeat((1, reps, 1) if rows else (reps, 1))
+            if a.dtype == torch.int32:
+                assert torch.equal(want, b)
+            else:
+                assert torch.equal(want.nan_to_num(nan=1.5, posinf=2.5, neginf=3.5), b.nan_to_num(nan=1.5, posinf=2.5, neginf=3.5))
 
 
 def test_quantize_strided_input_and_determinism():
@@ -511,6 +542,37 @@ def test_many_tiles_per_cta_around_the_shortest_shared_output(k):
 
 
 # --------------------------------------------------------------------------- dynamic range
+
+def _bf16(x):
+    return synth.f32_to_bf16_bits(np.asarray(x, dtype=np.float32))
+
+
+def test_token_with_one_huge_channel():
+    # one channel of one token is 1e4 among N(0,1): the per-token power-of-two scale has to keep
+    # both the outlier and the ordinary channels inside the fp16 operands' range
+    n, d_in, d_out, q, g = 96, 512, 256, 3, 128
+    _, X, dY, bits, alpha, _, _ = make_case(900, n, d_in, d_out, q, g)
+    Xf = synth.bf16_bits_to_f32(X)
+    Xf[5, 77] = 1.0e4
+    Xf[40, 300] = -3.0e4
+    X = _bf16(Xf)
+    Xd, _, bd, ad = _upload(X, dY, bits, alpha)
+    ref = oracle.fwd(X, bits, alpha, d_in, g)
+    Y = bcq.linear_fwd(Xd, bd, ad, d_in, g).cpu().numpy()
+    assert np.isfinite(Y).all()
+    # per token, since the two outlier tokens dwarf the others
+    for t in (0, 5, 40, 95):
+        assert np.abs(Y[t] - ref[t]).max() <= TOL * np.abs(ref[t]).max()
+    pack = bcq.decode_pack(bd, ad, d_in, g)
+    for nn in (1, 16):
+        refd = ref[:nn * 6:6]
+        Xs = Xd[:nn * 6:6].contiguous()
+        for Yd in (bcq.linear_decode(Xs, bd, ad, d_in, g).cpu().numpy(),
+                   bcq.linear_decode_packed(Xs, pack, d_out, d_in, q, g).cpu().numpy()):
+            for t in range(nn):
+                assert np.abs(Yd[t] - refd[t]).max() <= TOL * np.abs(refd[t]).max()
+
+
 def test_tiny_output_gradients():
     # dY ~ 1e-6: far below the smallest normal fp16 number unless each token row is rescaled
     n, d_in, d_out, q, g = 200, 384, 256, 4, 128
@@ -629,9 +691,10 @@ def test_decode_right_after_packing_into_a_used_buffer(d_in, d_out, q, g, n):
 
 
 @pytest.mark.parametrize("d_in,d_out,q,g", [(100, 40, 2, 100), (2048, 300, 4, 128), (2056, 300, 4, 128), (4104, 2400, 3, 64),
-                                            (16384, 512, 4, 128), (16400, 33, 1, 16400), (128, 60000, 1, 64), (2080, 500, 3, 32)])
+                                            (16384, 512, 4, 128), (16400, 33, 1, 16400), (128, 60000, 1, 64), (2080, 500, 3, 32),
+                                            (4096, 512, 4, 128), (6144, 500, 3, 64)])
 def test_decode_of_few_tokens_is_decode_of_many(d_in, d_out, q, g):
-    # up to two tokens (four, with more than 16 steps of 128) the activations go by way of shared memory, once for the
+    # up to two tokens (four, with more than 16 steps of 128 to a CTA) the activations go by way of shared memory, once for the
     # CTA: the same conversion and the same sums, so to the last bit what the first rows of a larger batch get
     # (ragged steps, clusters, several rounds of tiles, tables of two and four groups a step)
     gen = torch.Generator(device="cuda").manual_seed(d_in + d_out)
@@ -644,6 +707,26 @@ def test_decode_of_few_tokens_is_decode_of_many(d_in, d_out, q, g):
     assert rel_err(Y.cpu().numpy(), ref) <= TOL
     for n in (1, 2, 3, 4, 5):
         assert torch.equal(bcq.linear_decode_packed(X[:n], pack, d_out, d_in, q, g), Y[:n]), n
+
+
+@pytest.mark.parametrize("d_in,d_out,q,g", [(128, 300, 3, 128), (768, 760, 3, 768), (1608, 4790, 2, 64), (6400, 1600, 1, 6400),
+                                            (4096, 512, 3, 64), (3200, 1600, 4, 128), (1408, 6390, 4, 1408), (1280, 4096, 4, 32),
+                                            (4480, 1000, 4, 128), (128, 60000, 2, 64), (128, 60000, 4, 64)])
+def test_decode_from_planes_two_units_ahead(d_in, d_out, q, g):
+    # few units of 16 rows x 128 columns to a warp (none to four; one, two or four CTAs to a tile; two rounds of tiles): up to eight
+    # tokens take the weights two units ahead, sixteen one, with the same sums where a CTA's tiles fit one round.
+    # Against a dense fp64 product.
+    gen = torch.Generator(device="cuda").manual_seed(d_in + d_out)
+    bits, alpha, _ = bcq.quantize(torch.randn((d_out, d_in), generator=gen, device="cuda") * 0.02, q, g)
+    X = torch.randn((16, d_in), generator=gen, device="cuda").bfloat16()
+    ref = (X.double() @ bcq.dequantize(bits, alpha, d_in, g).double().t()).cpu().numpy()
+    Y = bcq.linear_decode(X, bits, alpha, d_in, g)
+    assert rel_err(Y.cpu().numpy(), ref) <= TOL
+    for n in (1, 8):
+        few = bcq.linear_decode(X[:n], bits, alpha, d_in, g)
+        assert rel_err(few.cpu().numpy(), ref[:n]) <= TOL
+        if d_out < 20000:
+            assert torch.equal(few, Y[:n]), n
 
 
 @pytest.mark.parametrize("n", [1, 9])
