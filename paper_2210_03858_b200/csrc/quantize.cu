@@ -1070,14 +1070,16 @@ sorted_quantize_kernel(const QuantParams p, int batch) {
     };
     // Weight 4 i + e of a lane: 16 i + e after its first.
     const int kt = (tl >> 2) * (16 * NI) + (tl & 3) * 4;
-    // pieces 4 from .. of a lane
+    // Pieces 4 from .. of a lane, whole ones wherever the group's size is a multiple of four (g = 224, q = 2, three rounds, 3200 x 5376:
+    // 119.5 us with such groups' weights one by one, 108.6 so).
     auto load = [&](const Place& x, int from, auto& w) {
         constexpr int COUNT = sizeof(w) / sizeof(float);
         const float* src = p.W + (long long)x.j * p.ldw + x.c * p.g + kt + 16 * from;
-        if (x.m == C && p.vec) {
+        if (p.vec && (x.m & 3) == 0) {
 #pragma unroll
             for (int i = 0; i < COUNT / 4; ++i) {
-                const float4 v = bcq::ld(reinterpret_cast<const float4*>(src + 16 * i));
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (kt + 16 * (from + i) < x.m) v = bcq::ld(reinterpret_cast<const float4*>(src + 16 * i));
                 w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
             }
         } else {
