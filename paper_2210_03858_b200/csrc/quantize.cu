@@ -582,9 +582,11 @@ __device__ __noinline__ void fit_not_finite(const QuantParams p, long long item)
 // holds a short group goes another way for all its groups; row by row that were 61 % of the warps at 1600 columns and
 // g = 128 (6400 rows, q = 4: 20.1 us row by row and 18.2 with the short groups last; 2222 x 3331, q = 3: 18.9 and 15.6).  An
 // instance of its own, because the order costs matrices without short groups 3 to 6 %.
+// Blocks to an SM: with four planes and 8 weights a lane four, since the 80 registers of six are too few (512 x 512, g = 32, two
+// rounds: 17.1 us with six and 13.5 with four; 5120 x 5120 539 and 522; with three, 170 registers, 12.9 and 592).
 template <int NI, int L, int TW, int Q, bool TAILS>
 __global__ void __launch_bounds__(TW == 1 ? 128 : TW * 32,
-                                  TW == 1   ? (NI == 2 || (Q == 0 && NI == 4) ? 6 : Q == 0 || NI == 4 ? 5 : 3)
+                                  TW == 1   ? ((NI == 2 && Q < 4) || (Q == 0 && NI == 4) ? 6 : NI == 2 ? 4 : Q == 0 || NI == 4 ? 5 : 3)
                                   : TW <= 4 ? (NI == 4 ? 20 : 12) / TW
                                             : 1)
 team_quantize_kernel(const QuantParams p) {
