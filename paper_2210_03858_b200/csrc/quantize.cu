@@ -1033,7 +1033,10 @@ struct SortedShape {
 
 constexpr int kSortWarps = 4;  // of a block, at most
 
-template <int NI, int L, int Q>
+// PIECES: the full groups leave some of the lanes' 16-byte pieces empty.  An instance of its own, because asking for each piece
+// costs full lanes 1 % (5120 x 5120, g = 128, q = 3, five rounds 166.7 us and 168.4), and taking such groups one weight at a
+// time, as short last groups of an odd size are taken, costs more (g = 224, q = 2, three rounds, 3200 x 5376: 118.8 and 108.7).
+template <int NI, int L, int Q, bool PIECES>
 __global__ void __launch_bounds__(32 * kSortWarps, 2)
 sorted_quantize_kernel(const QuantParams p, int batch) {
     using Sh = SortedShape<NI, L>;
@@ -1072,20 +1075,19 @@ sorted_quantize_kernel(const QuantParams p, int batch) {
     };
     // Weight 4 i + e of a lane: 16 i + e after its first.
     const int kt = (tl >> 2) * (16 * NI) + (tl & 3) * 4;
-    // Pieces 4 from .. of a lane, whole ones wherever the group's size is a multiple of four (g = 224, q = 2, three rounds, 3200 x 5376:
-    // 119.5 us with such groups' weights one by one, 108.6 so).
+    // pieces from .. of a lane
     auto load = [&](const Place& x, int from, auto& w) {
         constexpr int COUNT = sizeof(w) / sizeof(float);
         const float* src = p.W + (long long)x.j * p.ldw + x.c * p.g + kt + 16 * from;
-        if (p.vec && (x.m & 3) == 0) {
+        const int left = x.m - kt - 16 * from;
+        if (p.vec && (PIECES ? (x.m & 3) == 0 : x.m == C)) {
 #pragma unroll
             for (int i = 0; i < COUNT / 4; ++i) {
                 float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (kt + 16 * (from + i) < x.m) v = bcq::ld(reinterpret_cast<const float4*>(src + 16 * i));
+                if (!PIECES || 16 * i < left) v = bcq::ld(reinterpret_cast<const float4*>(src + 16 * i));
                 w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
             }
         } else {
-            const int left = x.m - kt - 16 * from;
 #pragma unroll
             for (int e = 0; e < COUNT; ++e) w[e] = 16 * (e / 4) + e % 4 < left ? bcq::ld(src + 16 * (e / 4) + e % 4) : 0.0f;
         }
@@ -1579,7 +1581,9 @@ sorted_quantize_kernel(const QuantParams p, int batch) {
 template <int NI, int L, int Q>
 cudaError_t launch_sorted(const QuantParams& p, cudaStream_t stream) {
     using Sh = SortedShape<NI, L>;
-    const auto kern = sorted_quantize_kernel<NI, L, Q>;
+    void (*kern)(const QuantParams, int) = sorted_quantize_kernel<NI, L, Q, false>;
+    if constexpr (NI == 8 && Q < 4)  // (q = 4: no difference, the rounds are most of the time)
+        if (p.g < Sh::C && p.vec) kern = sorted_quantize_kernel<NI, L, Q, true>;
     const bcq_status st = bcq::ensure_dynamic_smem(kern, kSortWarps * Sh::bytes);
     if (st != BCQ_OK) return cudaErrorUnknown;
     const long long places = 9ll * bcq::sm_count();
