@@ -1622,27 +1622,29 @@ cudaError_t launch_team(QuantParams p, cudaStream_t stream) {
 // Greedy: the smallest team that holds a group at 32 weights a thread (8 or 16 for groups of 32 or 64).
 // Alternating: a thread goes through its weights one after the other in every round, so a problem that
 // is over in a few waves takes as long as one thread does, and fewer weights a thread are better;
-// more lanes mean more shuffles and more copies of the solve, which a long one pays for.  Measured, five
-// rounds, at 32 / 16 / 8 weights a thread:
-//   g = 128, q = 4   512 x 512 56 / 37 / 28 us   2048 x 1536 209 / 138 / 118   3000 x 4096 401 / 333 / 401
-//                    5120 x 5120 711 / 653 / 851
-//   g = 128, q = 3   512 x 512 31 / 20 / 21 us   1406 x 1582 93 / 55 / 58   5120 x 5120 357 / 345 / 468
-//   g = 128, 1600 x 1600, 16 / 8 a thread: q = 1 18.6 / 15.5 us, q = 2 37.9 / 33.4, q = 3 72.7 / 63.8;
-//                    64 x 512, q = 3 13.0 / 10.1 (so for every q, though two problems of q = 3 above lose 5 %)
-//   g = 256, q = 3   1406 x 1582 106 / 57 us     5120 x 5120 355 / 346
-//   a row, q = 3     1024 x 1024 80 / 53 us      2048 x 1536 128 / 98       3000 x 4096 231 / 288
-// From three rounds on groups of up to 256 go to the sorted kernel, which takes about 110 us for 5120 x 5120 before the
-// first round and 12 (q = 3) for each, where the team kernel takes 90 and 55 (one round, q = 2 / 3 / 4: 84 / 145 / 237
-// us here, 98 / 130 / 203 there; three 140 / 258 / 461 and 108 / 147 / 245; 1600 x 1600, one round 15 / 25 / 41 and 22 / 28 / 47,
-// three 22 / 40 / 81 and 24 / 31 / 45).  Problems of a few hundred groups are chains of latencies in both and lose 1 - 5 us there
-// (64 x 512, q = 3, five rounds 12.8 and 14.1).
-// The line between "few waves" and "long" is 30720 weights per SM (4.5 M on 148, three waves of the
-// 16-weight teams).
+// more lanes mean more shuffles and more copies of the solve, which a long one pays for.  Measured, us a call:
+//   g = 128, two rounds, 8 / 16 weights a thread (groups of q > 1 come here with one or two rounds, see below)
+//     q = 1   64 x 512 2.3 / 2.4   512 x 512 3.2 / 2.8    1600 x 1600 10.4 / 9.2    5120 x 5120 77.6 / 57.3
+//     q = 2   64 x 512 3.6 / 4.3   1024 x 1024 8.7 / 9.2    1600 x 1600 17.7 / 15.6   5120 x 5120 143 / 106
+//     q = 3   512 x 512 9.2 / 9.8   1024 x 1024 14.5 / 15.7   1600 x 1600 29.8 / 24.9   5120 x 5120 249 / 190
+//     q = 4   512 x 512 12.1 / 15.9   1024 x 1024 22.5 / 24.6   1600 x 1600 52.4 / 43.1   5120 x 5120 458 / 318
+//   g = 256, two rounds, 16 / 32 weights a thread: q = 3 512 x 512 10.4 / 15.1   1600 x 1600 26.9 / 29.7   5120 x 5120 186 / 158
+//   a row, five rounds, 16 / 32 weights a thread
+//     q = 3   1024 x 1024 30.8 / 35.7   2000 x 1024 44.0 / 48.9   3000 x 1024 59.0 / 57.2   1500 x 2048 63.2 / 60.0   4000 x 2048 142 / 116
+//     q = 4   2000 x 1024 72.2 / 79.8   3000 x 1024 102 / 101   1024 x 2048 79.3 / 91.1   1500 x 2048 105 / 97.5
+// The line between "few waves" and "long" is thus 18432 weights per SM for rows (2.7 M on 148) and 8192 for groups of
+// 65 to 128 (1.2 M; 1024 with one plane, whose rounds are short).
+// From three rounds on groups of up to 256 go to the sorted kernel.  5120 x 5120, g = 128, q = 2 / 3 / 4: one round 82 / 139 / 218 us
+// here and 100 / 129 / 189 there, two 107 / 192 / 320 and 105 / 140 / 210, three 132 / 239 / 413 and 109 / 146 / 231, five 178 / 331 / 599 and
+// 118 / 167 / 278.  Small problems are chains of latencies in both, and there sorting costs: 1600 x 1600, three rounds
+// 19 / 32 / 58 and 24 / 33 / 52; 512 x 512, five rounds 9.3 / 16.2 / 22.0 and 10.1 / 14.8 / 27.7; 64 x 512, three rounds 4.3 / 6.7 / 10.5 and
+// 7.5 / 11.1 / 19.8.  They go there all the same: the choice may not depend on the number of rows, because the two kernels add in
+// different orders and a row gets the same scales whatever else is in the call.
 template <int Q>
 cudaError_t launch_team_size(const QuantParams& p, cudaStream_t s) {
     const int g = p.g;
-    const bool few = Q > 0 && p.items * g <= 30720ll * bcq::sm_count();
-    // (the choice must not depend on the number of rows: the two kernels add in different orders)
+    const bool few = Q > 0 && p.items * g <= (g > 128 ? 18432ll : Q == 1 ? 1024ll : 8192ll) * bcq::sm_count();
+    // (whatever the number of rows, see above)
     if constexpr (Q > 1)
         if (p.alt_iters >= 3) {
             if (g <= 32) return launch_sorted<2, 4, Q>(p, s);

@@ -138,7 +138,7 @@ def test_quantize_team_sizes_with_exact_ties(d_in, g, alt):
 @pytest.mark.parametrize("d_in,g", [(100, 32), (420, 96), (260, 128), (700, 256), (1023, 1023), (1582, 1582)])
 def test_quantize_alternating_short_and_long_problems(d_in, g, alt):
     # The size of the team depends on how much there is to do: the same five rows alone and repeated past
-    # the line (30720 weights per SM).  Values as in the test above, so the bits are the oracle's exactly.
+    # the line (18432 weights per SM at most).  Values as in the test above, so the bits are the oracle's exactly.
     # (Groups of up to 256 are taken by teams with two rounds, with three by lanes on sorted magnitudes.)
     rng = np.random.default_rng(d_in)
     W = (rng.integers(-6, 7, size=(5, d_in)) / 64.0).astype(np.float32)
@@ -179,7 +179,7 @@ def test_quantize_a_row_alone_and_among_many(d_in, g):
     # in the call, to the last bit, though the teams that share a group differ in size.
     gen = torch.Generator(device="cuda").manual_seed(d_in)
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    rows = 30720 * sms // (-(-d_in // g) * g) + 1                    # past the line between the team sizes
+    rows = 30720 * sms // (-(-d_in // g) * g) + 1                    # past every line between the team sizes
     W = torch.randn((rows, d_in), generator=gen, device="cuda") * 0.02
     pick = slice(rows // 2, rows // 2 + 600)
     for q, alt in ((1, 3), (2, 3), (3, 3), (4, 3), (4, 0), (2, 2), (3, 2), (4, 2)):
