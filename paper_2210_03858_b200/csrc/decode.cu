@@ -849,16 +849,15 @@ bcq_status launch_decode_planes(DecPlanesParams p, cudaStream_t s) {
     void (*kern)(DecPlanesParams) = p.split > 1 ? decode_planes_kernel<NQ, NT, true, false> : decode_planes_kernel<NQ, NT, false, false>;
     // Two units ahead (DEEP) where a warp has few units and the start of its loads counts for more than a loop that is there
     // once.  us, one ahead / two ahead, one token; in front: units of a CTA, to be dealt to its 16 warps:
-    //   q = 3   6   768 -> 768 2.78 / 2.67        16  2048 -> 2048 3.80 / 3.62   20  1280 -> 5120 5.46 / 5.04   39  1600 -> 4800 6.07 / 5.70
-    //           50  6400 -> 1600 8.88 / 8.54      64  4096 -> 4096 8.74 / 8.73   256 16384 -> 4096 27.8 / 28.6
-    //   q = 4   12  768 -> 3072 3.82 / 3.93       16  2048 -> 2048 4.79 / 4.81   20  1280 -> 4096 6.34 / 5.93   25  3200 -> 1600 6.32 / 6.05
-    //           32  2048 -> 4096 6.50 / 6.97      33  1408 -> 6400 6.92 / 6.63   39  1600 -> 4800 7.26 / 7.07   40  5120 -> 1280 9.32 / 9.66
-    // and with nine tokens and more one ahead is the faster (q = 3, 1024 -> 1024, 16 tokens 4.38 / 4.72).
-    if constexpr (NQ < 8 && NT == 1) {
-        const int units = p.round * ceil_div(p.steps, p.split);
-        const bool deep = NQ == 3 ? units < 4 * kDpWarps : units > kDpWarps && 2 * units < 5 * kDpWarps && units % kDpWarps != 0;
-        if (deep) kern = p.split > 1 ? decode_planes_kernel<NQ, NT, true, true> : decode_planes_kernel<NQ, NT, false, true>;
-    }
+    //   q = 3   6   768 -> 768 2.78 / 2.67      16   2048 -> 2048 3.80 / 3.62   20  1280 -> 5120 5.46 / 5.04   39  1600 -> 4800 6.07 / 5.70
+    //           50  6400 -> 1600 8.88 / 8.54    64   4096 -> 4096 8.74 / 8.73   256 16384 -> 4096 27.8 / 28.6
+    // With nine tokens and more one ahead is the faster (1024 -> 1024, 16 tokens 4.38 / 4.72).  q = 4 is left alone: two ahead
+    // gains where the units do not divide evenly among the warps (33  1408 -> 6400 6.92 / 6.63) and loses where they do (32  2048 -> 4096
+    // 6.50 / 6.97), and a layer whose linears then take turns in two kernels fetches the code of both (the four linears of width
+    // 1600, four tokens 30.4 us, with a rule of that kind 30.7).
+    if constexpr (NQ == 3 && NT == 1)
+        if (p.round * ceil_div(p.steps, p.split) < 4 * kDpWarps)
+            kern = p.split > 1 ? decode_planes_kernel<NQ, NT, true, true> : decode_planes_kernel<NQ, NT, false, true>;
     const bcq_status st = ensure_dynamic_smem(kern, smem);
     if (st != BCQ_OK) return st;
     BCQ_CUDA_TRY(launch_pdl(kern, dim3((unsigned)ctas), kDpThreads, smem, s, (unsigned)p.split, p));

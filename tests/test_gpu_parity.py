@@ -713,8 +713,9 @@ def test_decode_of_few_tokens_is_decode_of_many(d_in, d_out, q, g):
                                             (4096, 512, 3, 64), (3200, 1600, 4, 128), (1408, 6390, 4, 1408), (1280, 4096, 4, 32),
                                             (4480, 1000, 4, 128), (128, 60000, 2, 64), (128, 60000, 4, 64)])
 def test_decode_from_planes_two_units_ahead(d_in, d_out, q, g):
-    # few units of 16 rows x 128 columns to a warp (none to four; one, two or four CTAs to a tile; two rounds of tiles): up to eight
-    # tokens take the weights two units ahead, sixteen one, with the same sums where a CTA's tiles fit one round.
+    # few units of 16 rows x 128 columns to a warp (none to four; one, two or four CTAs to a tile; two rounds of tiles): with up to
+    # three planes and eight tokens the weights are taken two units ahead, else one, with the same sums where a CTA's tiles
+    # fit one round.
     # Against a dense fp64 product.
     gen = torch.Generator(device="cuda").manual_seed(d_in + d_out)
     bits, alpha, _ = bcq.quantize(torch.randn((d_out, d_in), generator=gen, device="cuda") * 0.02, q, g)
