@@ -12,7 +12,7 @@
 // ballot per 32 weights; now two rounds, and per weight and plane two fp64 additions and one shift
 // that collects the sign.  Measured, before and after: greedy q = 4, g = 128, the four linears of a
 // layer of width 1600 (30.7 M weights) 162 -> 56 us (2.6 TB/s; the logic pipe is 55 % busy, the fp64
-// pipe 21 %); two alternating rounds, q = 3, g = 128, 5120 x 5120: 202 us (instruction fetch of the
+// pipe 21 %); two alternating rounds, q = 3, g = 128, 5120 x 5120: 190 us (instruction fetch of the
 // unrolled rounds and fp64 latency at five warps per scheduler bound it).
 //
 // Sums are fp64 and are reduced in a fixed order, so a result never depends on scheduling.
@@ -944,14 +944,14 @@ team_quantize_kernel(const QuantParams p) {
 //
 // A warp takes up to 32 groups.  (1) In teams of L lanes it loads 32 / L groups at a time, sorts them in registers
 // (a network in each lane, then merges across the lanes) and puts keys and running sums into shared memory.
-// (2) Lane k does all rounds of group k, so a least-squares solve is done once per group and not by every lane
-// of a team.  (3) In teams again, the weights are read once more (from L2), find their levels and are
+// (2) Lane k does all rounds of group k (or four lanes do, see SHARE), so a least-squares solve is done once per group
+// and not by every lane of a team.  (3) In teams again, the weights are read once more (from L2), find their levels and are
 // written as planes.  Warps are blocks of their own, so that some sort while others wait for the chains of fp64
 // divisions of (2); eight or nine fit an SM (25 KiB each).
 //
 // The team kernel keeps a group in registers and goes through its weights in every round, and all lanes of a team solve.
-// Measured, that and this: 5120 x 5120, g = 128, q = 3: five rounds 364 and 169 us, fifteen 905 and 270; q = 4 689
-// and 297.  What bounds it now: min and max of the sort run at half rate (the logic pipe), and the code, 15 to 30 KiB for
+// Measured, that and this: 5120 x 5120, g = 128, five rounds: q = 3 331 and 167 us, q = 4 599 and 278 (launch_team_size has
+// more).  What bounds it now: min and max of the sort run at half rate (the logic pipe), and the code, 15 to 30 KiB for
 // a pass, comes slowly to eight warps an SM (stall no_instruction; 4.2 an issue with everything unrolled, 250 us).
 //
 // Key of a weight: its magnitude's bits shifted left by one, below them 1 where it is not negative: integers in the
@@ -1031,12 +1031,16 @@ struct SortedShape {
     static constexpr size_t bytes = (size_t)C * GROUPS * 4 + (size_t)(RUNS + 1) * GROUPS * 8;
 };
 
-constexpr int kSortWarps = 4;  // of a block, at most
+constexpr int kSortWarps = 4;         // of a block, at most
+constexpr long long kSortPlaces = 9;  // warps that an SM holds
 
 // PIECES: the full groups leave some of the lanes' 16-byte pieces empty.  An instance of its own, because asking for each piece
 // costs full lanes 1 % (5120 x 5120, g = 128, q = 3, five rounds 166.7 us and 168.4), and taking such groups one weight at a
 // time, as short last groups of an odd size are taken, costs more (g = 224, q = 2, three rounds, 3200 x 5376: 118.8 and 108.7).
-template <int NI, int L, int Q, bool PIECES>
+// SHARE: four lanes to a group in (2), for calls that give a warp at most eight, whose other lanes would be idle: each looks for
+// every fourth cut, and all do the rest alike.  One lane goes through the cuts one instruction at a time, which a chip
+// full of warps hides and a small call does not: 512 x 512, g = 256, q = 4, five rounds 27.4 us and 22.5, q = 3 15.9 and 15.1.
+template <int NI, int L, int Q, bool PIECES, bool SHARE>
 __global__ void __launch_bounds__(32 * kSortWarps, 2)
 sorted_quantize_kernel(const QuantParams p, int batch) {
     using Sh = SortedShape<NI, L>;
@@ -1168,8 +1172,16 @@ sorted_quantize_kernel(const QuantParams p, int batch) {
     }
     __syncwarp();
 
-    // ---- (2) rounds: a group per lane
-    const int grp = min(lane, count - 1);
+    // ---- (2) rounds: a group per lane, or per four
+    constexpr int SHARES = SHARE ? 4 : 1, OWN = (N - 1 + SHARES - 1) / SHARES;  // cuts that a lane looks for: s = share + 1, + SHARES, ...
+    const int slot = SHARE ? lane & 7 : lane, share = SHARE ? lane >> 3 : 0;
+    const int grp = min(slot, count - 1);
+    auto own = [&](const auto& of_cut, int o) {  // (of the last cut again, where there are fewer)
+        auto v = of_cut[min(SHARES * o + 1, N - 1)];
+#pragma unroll
+        for (int k = 1; k < SHARES; ++k) v = share == k ? of_cut[min(SHARES * o + 1 + k, N - 1)] : v;
+        return v;
+    };
     const long long item = first + grp;
     float a[Q], a_cut[Q];  // scales; the scales that the last cuts were made for
     LevelSearch<Q> ls;
@@ -1327,11 +1339,11 @@ sorted_quantize_kernel(const QuantParams p, int batch) {
 #pragma unroll
                 for (int i = 0; i < Q; ++i) {
                     const double d = warp_sum(dS[i]);
-                    if (lane == f) S[i] += d;
+                    if (slot == f) S[i] += d;
 #pragma unroll
                     for (int l = i + 1; l < Q; ++l) {
                         const int n = __reduce_add_sync(0xffffffffu, dagree[i][l]);
-                        if (lane == f) agree[i][l] += n;
+                        if (slot == f) agree[i][l] += n;
                     }
                 }
             }
@@ -1364,8 +1376,16 @@ sorted_quantize_kernel(const QuantParams p, int batch) {
 #pragma unroll
             for (int s = 1; s < N; ++s) at[s] = __float_as_uint(ls.mid[s]) << 1;
             }
+            int own_cut[OWN];
+            double own_below[OWN];
 #pragma unroll
-            for (int s = 1; s < N; ++s) cuts[s] = cut(at[s], below[s]);
+            for (int o = 0; o < OWN; ++o) own_cut[o] = cut(own(at, o), own_below[o]);
+#pragma unroll
+            for (int s = 1; s < N; ++s) {
+                const int o = (s - 1) / SHARES, from = slot + 8 * ((s - 1) % SHARES);
+                cuts[s] = SHARE ? __shfl_sync(0xffffffffu, own_cut[o], from) : own_cut[o];
+                below[s] = SHARE ? __shfl_sync(0xffffffffu, own_below[o], from) : own_below[o];
+            }
             if (it < 0) {
                 const int plane = it + Q;
                 double S = 0.0;
@@ -1397,9 +1417,14 @@ sorted_quantize_kernel(const QuantParams p, int batch) {
             } else {
                 float near = tiny;
 #pragma unroll
-                for (int s = 1; s < N; ++s) {
-                    if (cuts[s] > 0) near = fminf(near, ls.mid[s] - key_magnitude(key(cuts[s] - 1)));
-                    if (cuts[s] < m) near = fminf(near, key_magnitude(key(cuts[s])) - ls.mid[s]);
+                for (int o = 0; o < OWN; ++o) {
+                    const float mid = own(ls.mid, o);
+                    if (own_cut[o] > 0) near = fminf(near, mid - key_magnitude(key(own_cut[o] - 1)));
+                    if (own_cut[o] < m) near = fminf(near, key_magnitude(key(own_cut[o])) - mid);
+                }
+                if (SHARE) {
+                    near = fminf(near, __shfl_xor_sync(0xffffffffu, near, 8));
+                    near = fminf(near, __shfl_xor_sync(0xffffffffu, near, 16));
                 }
                 // fp32 decides where a weight is 2^-22 of the largest level away from the midpoint, which is rounded by
                 // 2^-24 of itself; half of ls.delta keeps the neighbourhoods of two midpoints apart
@@ -1581,14 +1606,16 @@ sorted_quantize_kernel(const QuantParams p, int batch) {
 template <int NI, int L, int Q>
 cudaError_t launch_sorted(const QuantParams& p, cudaStream_t stream) {
     using Sh = SortedShape<NI, L>;
-    void (*kern)(const QuantParams, int) = sorted_quantize_kernel<NI, L, Q, false>;
-    if constexpr (NI == 8 && Q < 4)  // (q = 4: no difference, the rounds are most of the time)
-        if (p.g < Sh::C && p.vec) kern = sorted_quantize_kernel<NI, L, Q, true>;
-    const bcq_status st = bcq::ensure_dynamic_smem(kern, kSortWarps * Sh::bytes);
-    if (st != BCQ_OK) return cudaErrorUnknown;
-    const long long places = 9ll * bcq::sm_count();
+    const long long places = kSortPlaces * bcq::sm_count();
     int batch = std::max(Sh::TEAMS, 4);
     while (batch < Sh::GROUPS && (p.items + batch - 1) / batch > places) batch *= 2;
+    void (*kern)(const QuantParams, int) = sorted_quantize_kernel<NI, L, Q, false, false>;
+    if constexpr (NI == 8 && Q < 4)  // (q = 4: no difference, the rounds are most of the time)
+        if (p.g < Sh::C && p.vec) kern = sorted_quantize_kernel<NI, L, Q, true, false>;
+    if constexpr (Q > 2)  // (q = 2 has one cut)
+        if (batch <= 8) kern = sorted_quantize_kernel<NI, L, Q, false, true>;
+    const bcq_status st = bcq::ensure_dynamic_smem(kern, kSortWarps * Sh::bytes);
+    if (st != BCQ_OK) return cudaErrorUnknown;
     const long long warps = (p.items + batch - 1) / batch;
     const int per_block = warps >= 24ll * bcq::sm_count() ? kSortWarps : 1;
     return bcq::launch_pdl(kern, dim3((unsigned)((warps + per_block - 1) / per_block)), 32 * per_block, per_block * Sh::bytes, stream, 1, p, batch);
@@ -1637,8 +1664,8 @@ cudaError_t launch_team(QuantParams p, cudaStream_t stream) {
 // From three rounds on groups of up to 256 go to the sorted kernel.  5120 x 5120, g = 128, q = 2 / 3 / 4: one round 82 / 139 / 218 us
 // here and 100 / 129 / 189 there, two 107 / 192 / 320 and 105 / 140 / 210, three 132 / 239 / 413 and 109 / 146 / 231, five 178 / 331 / 599 and
 // 118 / 167 / 278.  Small problems are chains of latencies in both, and there sorting costs: 1600 x 1600, three rounds
-// 19 / 32 / 58 and 24 / 33 / 52; 512 x 512, five rounds 9.3 / 16.2 / 22.0 and 10.1 / 14.8 / 27.7; 64 x 512, three rounds 4.3 / 6.7 / 10.5 and
-// 7.5 / 11.1 / 19.8.  They go there all the same: the choice may not depend on the number of rows, because the two kernels add in
+// 19 / 32 / 58 and 24 / 33 / 52; 512 x 512, five rounds 9.3 / 16.2 / 22.0 and 8.6 / 12.4 / 20.6; 64 x 512, three rounds 4.3 / 6.7 / 10.5 and
+// 6.4 / 9.5 / 15.4.  They go there all the same: the choice may not depend on the number of rows, because the two kernels add in
 // different orders and a row gets the same scales whatever else is in the call.
 template <int Q>
 cudaError_t launch_team_size(const QuantParams& p, cudaStream_t s) {
@@ -1649,7 +1676,10 @@ cudaError_t launch_team_size(const QuantParams& p, cudaStream_t s) {
         if (p.alt_iters >= 3) {
             if (g <= 32) return launch_sorted<2, 4, Q>(p, s);
             if (g <= 64) return launch_sorted<4, 4, Q>(p, s);
-            if (g <= 128) return launch_sorted<8, 4, Q>(p, s);
+            // Groups of 65 to 128 in eight lanes, as long as warps of four groups find their places at once: half the weights to
+            // sort in a lane (512 x 512, g = 128, three rounds, q = 2 / 3 / 4: 8.2 / 11.6 / 18.5 us in four lanes, 6.8 / 9.7 / 16.2 in eight;
+            // 1024 x 1024 9.7 / 13.7 / 22.4 and 10.3 / 14.3 / 22.9; groups of 256 in sixteen 8.8 / 12.0 / 18.2 and 9.1 / 12.7 / 19.0)
+            if (g <= 128) return p.items <= 4 * kSortPlaces * bcq::sm_count() ? launch_sorted<4, 8, Q>(p, s) : launch_sorted<8, 4, Q>(p, s);
             if (g <= 256) return launch_sorted<8, 8, Q>(p, s);
         }
     if (g <= 32) return launch_team<2, 4, 1, Q>(p, s);
