@@ -564,7 +564,7 @@ def quantize_numbers(bcq, torch, dev, peaks):
         gbs = weights * (4 + q / 8 + 4 * q / g) / (ms * 1e-3) / 1e9
         out[tag] = {"ms": ms, "Gweights/s": weights / (ms * 1e-3) / 1e9, "GB/s": gbs,
                     "frac_of_hbm": gbs / peaks["hbm_gbs"],
-                    "bound": "hbm" if alt == 0 else "instruction fetch and fp64 latency (the alternating rounds), not memory"}
+                    "bound": "hbm" if alt == 0 else "the sort (min and max at half rate), instruction fetch and chains of fp64 divisions, not memory"}
         del Ws
 
     for name, d_in, d_out in block(1600, 6400):
