@@ -1036,7 +1036,7 @@ constexpr long long kSortPlaces = 9;  // warps that an SM holds
 
 // PIECES: the full groups leave some of the lanes' 16-byte pieces empty.  An instance of its own, because asking for each piece
 // costs full lanes 1 % (5120 x 5120, g = 128, q = 3, five rounds 166.7 us and 168.4), and taking such groups one weight at a
-// time, as short last groups of an odd size are taken, costs more (g = 224, q = 2, three rounds, 3200 x 5376: 118.8 and 108.7).
+// time, as short last groups of an odd size are taken, costs more (g = 224, q = 3, three rounds, 3200 x 5376: 146.4 and 138.4).
 // SHARE: four lanes to a group in (2), for calls that give a warp at most eight, whose other lanes would be idle: each looks for
 // every fourth cut, and all do the rest alike.  One lane goes through the cuts one instruction at a time, which a chip
 // full of warps hides and a small call does not: 512 x 512, g = 256, q = 4, five rounds 27.4 us and 22.5, q = 3 15.9 and 15.1.
@@ -1655,13 +1655,18 @@ cudaError_t launch_team(QuantParams p, cudaStream_t stream) {
 //     q = 2   64 x 512 3.6 / 4.3   1024 x 1024 8.7 / 9.2    1600 x 1600 17.7 / 15.6   5120 x 5120 143 / 106
 //     q = 3   512 x 512 9.2 / 9.8   1024 x 1024 14.5 / 15.7   1600 x 1600 29.8 / 24.9   5120 x 5120 249 / 190
 //     q = 4   512 x 512 12.1 / 15.9   1024 x 1024 22.5 / 24.6   1600 x 1600 52.4 / 43.1   5120 x 5120 458 / 318
-//   g = 256, two rounds, 16 / 32 weights a thread: q = 3 512 x 512 10.4 / 15.1   1600 x 1600 26.9 / 29.7   5120 x 5120 186 / 158
+//   g = 256, two rounds, 16 / 32 weights a thread (g = 512 is alike)
+//     q = 2   1600 x 1600 16.3 / 17.9   2560 x 2560 30.7 / 29.7   3200 x 3072 43.7 / 40.6   5120 x 5120 108 / 94.4
+//     q = 3   512 x 512 10.4 / 15.1   2048 x 2048 35.0 / 35.4   2560 x 2560 52.6 / 50.6   3200 x 3072 73.9 / 67.2   5120 x 5120 187 / 160
+//     q = 4   2048 x 2048 58.8 / 57.8   3200 x 3072 125 / 113   5120 x 5120 315 / 282
+//     q = 1, five rounds   3200 x 3072 36.1 / 36.8   4096 x 4096 60.4 / 60.9   5120 x 5120 87.7 / 82.5
 //   a row, five rounds, 16 / 32 weights a thread
 //     q = 3   1024 x 1024 30.8 / 35.7   2000 x 1024 44.0 / 48.9   3000 x 1024 59.0 / 57.2   1500 x 2048 63.2 / 60.0   4000 x 2048 142 / 116
 //     q = 4   2000 x 1024 72.2 / 79.8   3000 x 1024 102 / 101   1024 x 2048 79.3 / 91.1   1500 x 2048 105 / 97.5
-// The line between "few waves" and "long" is thus 18432 weights per SM for rows (2.7 M on 148) and 8192 for groups of
-// 65 to 128 (1.2 M; 1024 with one plane, whose rounds are short).
-// From three rounds on groups of up to 256 go to the sorted kernel.  5120 x 5120, g = 128, q = 2 / 3 / 4: one round 82 / 139 / 218 us
+// The line between "few waves" and "long" is thus 18432 weights per SM for rows (2.7 M on 148), 49152 for groups of 129 to 512
+// (7.3 M; with one plane 98304) and 8192 for groups of 65 to 128 (1.2 M; with one plane, whose rounds are short, 1024).
+// From three rounds on groups of up to 256 go to the sorted kernel, with two planes groups of more than 128 from four on
+// (g = 256, three rounds: 64 x 512 4.9 us here and 8.0 there, 1600 x 1600 20.2 / 28.3, 3200 x 3072 50.2 / 58.2, 5120 x 5120 119 / 125).  5120 x 5120, g = 128, q = 2 / 3 / 4: one round 82 / 139 / 218 us
 // here and 100 / 129 / 189 there, two 107 / 192 / 320 and 105 / 140 / 210, three 132 / 239 / 413 and 109 / 146 / 231, five 178 / 331 / 599 and
 // 118 / 167 / 278.  Small problems are chains of latencies in both, and there sorting costs: 1600 x 1600, three rounds
 // 19 / 32 / 58 and 24 / 33 / 52; 512 x 512, five rounds 9.3 / 16.2 / 22.0 and 8.6 / 12.4 / 20.6; 64 x 512, three rounds 4.3 / 6.7 / 10.5 and
@@ -1670,10 +1675,11 @@ cudaError_t launch_team(QuantParams p, cudaStream_t stream) {
 template <int Q>
 cudaError_t launch_team_size(const QuantParams& p, cudaStream_t s) {
     const int g = p.g;
-    const bool few = Q > 0 && p.items * g <= (g > 128 ? 18432ll : Q == 1 ? 1024ll : 8192ll) * bcq::sm_count();
+    const long long line = g > 512 ? 18432 : g > 128 ? (Q == 1 ? 98304 : 49152) : Q == 1 ? 1024 : 8192;  // weights per SM
+    const bool few = Q > 0 && p.items * g <= line * bcq::sm_count();
     // (whatever the number of rows, see above)
     if constexpr (Q > 1)
-        if (p.alt_iters >= 3) {
+        if (p.alt_iters >= (Q == 2 && g > 128 ? 4 : 3)) {
             if (g <= 32) return launch_sorted<2, 4, Q>(p, s);
             if (g <= 64) return launch_sorted<4, 4, Q>(p, s);
             // Groups of 65 to 128 in eight lanes, as long as warps of four groups find their places at once: half the weights to
@@ -1686,8 +1692,8 @@ cudaError_t launch_team_size(const QuantParams& p, cudaStream_t s) {
     if (g <= 64) return launch_team<4, 4, 1, Q>(p, s);
     if constexpr (Q > 0) {
         if (g <= 128) return few ? launch_team<2, 16, 1, Q>(p, s) : launch_team<4, 8, 1, Q>(p, s);
-        if (g <= 256) return launch_team<4, 16, 1, Q>(p, s);
-        if (g <= 512) return launch_team<4, 32, 1, Q>(p, s);
+        if (g <= 256) return few ? launch_team<4, 16, 1, Q>(p, s) : launch_team<8, 8, 1, Q>(p, s);
+        if (g <= 512) return few ? launch_team<4, 32, 1, Q>(p, s) : launch_team<8, 16, 1, Q>(p, s);
         if (g <= 1024 && few) return launch_team<4, 32, 2, Q>(p, s);
         if (g <= 2048 && few) return launch_team<4, 32, 4, Q>(p, s);
     } else {

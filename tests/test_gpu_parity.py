@@ -135,17 +135,17 @@ def test_quantize_team_sizes_with_exact_ties(d_in, g, alt):
 
 
 @pytest.mark.parametrize("alt", [2, 3])
-@pytest.mark.parametrize("d_in,g", [(100, 32), (420, 96), (260, 128), (700, 256), (1023, 1023), (1582, 1582)])
+@pytest.mark.parametrize("d_in,g", [(100, 32), (420, 96), (260, 128), (700, 256), (900, 512), (1023, 1023), (1582, 1582)])
 def test_quantize_alternating_short_and_long_problems(d_in, g, alt):
     # The size of the team depends on how much there is to do: the same five rows alone and repeated past
-    # the line (18432 weights per SM at most).  Values as in the test above, so the bits are the oracle's exactly.
+    # every line (98304 weights per SM at most).  Values as in the test above, so the bits are the oracle's exactly.
     # (Groups of up to 256 are taken by teams with two rounds, with three by lanes on sorted magnitudes.)
     rng = np.random.default_rng(d_in)
     W = (rng.integers(-6, 7, size=(5, d_in)) / 64.0).astype(np.float32)
     W[0, ::3] = -0.0
     W[2, : d_in // 2] = 0.25
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    reps = 30720 * sms // (5 * -(-d_in // g) * g) + 1
+    reps = (99000 if 128 < g <= 512 else 30720) * sms // (5 * -(-d_in // g) * g) + 1
     Wd = torch.from_numpy(W).cuda()
     for q in (1, 2, 3, 4):
         bits_ref, alpha_ref, sq_ref, _ = oracle.quantize(W, q, g, alt_iters=alt)
@@ -173,16 +173,16 @@ def test_quantize_weights_that_are_not_finite(d_in, g, alt):
         np.testing.assert_allclose(sq.cpu().numpy(), sq_ref, rtol=1e-6, atol=1e-12, equal_nan=True)
 
 
-@pytest.mark.parametrize("d_in,g", [(64, 32), (256, 64), (640, 128), (1000, 256), (700, 700), (1500, 1500)])
+@pytest.mark.parametrize("d_in,g", [(64, 32), (256, 64), (640, 128), (1000, 256), (1700, 512), (700, 700), (1500, 1500)])
 def test_quantize_a_row_alone_and_among_many(d_in, g):
     # Every (row, group) is a problem of its own: what a row becomes must not depend on how many others are
     # in the call, to the last bit, though the teams that share a group differ in size.
     gen = torch.Generator(device="cuda").manual_seed(d_in)
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    rows = 30720 * sms // (-(-d_in // g) * g) + 1                    # past every line between the team sizes
+    rows = (99000 if 128 < g <= 512 else 30720) * sms // (-(-d_in // g) * g) + 1  # past every line between the team sizes
     W = torch.randn((rows, d_in), generator=gen, device="cuda") * 0.02
     pick = slice(rows // 2, rows // 2 + 600)
-    for q, alt in ((1, 3), (2, 3), (3, 3), (4, 3), (4, 0), (2, 2), (3, 2), (4, 2)):
+    for q, alt in ((1, 3), (2, 3), (3, 3), (4, 3), (4, 0), (2, 2), (3, 2), (4, 2), (2, 4)):
         bits, alpha, sq = bcq.quantize(W, q, g, alt, want_sq_err=True)
         b, a, s = bcq.quantize(W[pick].contiguous(), q, g, alt, want_sq_err=True)
         assert torch.equal(b, bits[:, pick]) and torch.equal(a, alpha[:, pick]) and torch.equal(s, sq[pick])
